@@ -1077,8 +1077,7 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
 }  // namespace
 
 bool attn_fwd_tc_supported(const fbl_plan* p) {
-  return p->d.dtype == FBL_DTYPE_BF16 && (p->d.head_dim == 64 || p->d.head_dim == 128) && p->n_pad >= 128 &&
-         p->n_pad_kv >= 128;
+  return p->d.dtype == FBL_DTYPE_BF16 && (p->d.head_dim == 64 || p->d.head_dim == 128);   // boxes past the last row load zeros
 }
 bool attn_bwd_tc_supported(const fbl_plan* p) { return attn_fwd_tc_supported(p); }
 

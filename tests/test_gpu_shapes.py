@@ -1,0 +1,32 @@
+"""Shapes at the edges of the kernels' dispatch rules (partly filled tiles, remainders, smallest and largest of a range),
+each against the float64 oracle."""
+import pytest
+
+from fbl_inputs import LayerConfig, MlpConfig, XattnConfig
+
+import test_gpu_layer
+import test_gpu_mlp
+import test_gpu_xattn
+
+pytestmark = pytest.mark.gpu
+
+
+def check(cfg):
+    if isinstance(cfg, MlpConfig):
+        test_gpu_mlp.run_and_compare(cfg, guard_bytes=4096)
+    elif isinstance(cfg, XattnConfig):
+        test_gpu_xattn.run_and_compare(cfg, guard_bytes=4096)
+    else:
+        test_gpu_layer.run_and_compare(cfg, affine_noise=True, guard_bytes=4096)
+
+
+@pytest.mark.parametrize("cfg", [
+    # fewer token rows than one tile, one 64-wide key head, one memory tile beside many query rows
+    LayerConfig("sh1", 1, 121, 128, 2, 1, 64, "bf16", "layernorm", True, True, True, 1e-5, 201, 0.05),
+    LayerConfig("sh2", 3, 17, 192, 3, 1, 128, "bf16", "rmsnorm", False, False, False, 1e-5, 202, 0.05),
+    LayerConfig("sh3", 2, 150, 320, 5, 1, 64, "bf16", "rmsnorm", True, False, True, 1e-5, 203, 0.05),
+    MlpConfig("sh4", 1, 40, 64, 192, "bf16", "layernorm", "swiglu", True, True, 1e-5, 204, 0.05),
+    XattnConfig("sh5", 1, 130, 9, 128, 64, 2, 1, 64, "bf16", "layernorm", True, True, 1e-5, 205, 0.05),
+], ids=lambda c: c.name)
+def test_tensor_core_kernels_on_partly_filled_tiles(cfg):
+    check(cfg)
