@@ -423,7 +423,6 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
   const bool bias = p->d.has_bias;
   const int n = (int)p->n_pad, D = p->d.d_model;
 
-  if (!norm_fwd_resets_status(p)) FBL_CUDA(cudaMemsetAsync(status, 0, FBL_ALIGN, st));
   FBL_PROF_BEGIN();
   FBL_STEP("norm_fwd", 1, launch_norm_fwd(p, X, gamma, beta, Xn, stats, status, st));
   {
@@ -597,17 +596,11 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     cg.src[0] = (const float*)(sc + p->sb_acc_o); cg.dst[0] = dWo; cg.n[0] = up8(p->dq) * (int64_t)D; cg.count = 1;
     FBL_STEP("dW round", 1, launch_convert_f32_group(cg, st));
   }
-  // every bias gradient is a token-axis column sum: the four of them share their launches, and the second stage
-  // shares the norm backward's second kernel where that kernel exists
+  // every bias gradient is a token-axis column sum: the four of them ride in the norm backward's two launches
   const void* M4[4] = {dY, dQ, dK, dV};
   float* O4[4] = {dbo, dbq, dbk, dbv};
   const int C4[4] = {D, p->dq, p->dkv, p->dkv};
-  if (bias && norm_bwd_takes_colsums(p)) {
-    FBL_STEP("db+norm_bwd", 2, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, (float*)part, st, 4, M4, C4, O4));
-    return FBL_OK;
-  }
-  if (bias) FBL_STEP("db", 2, launch_colsum_group(p->d.dtype, 4, M4, p->n_pad, C4, O4, (float*)part, st));
-  FBL_STEP("norm_bwd", norm_bwd_takes_colsums(p) ? 2 : 1, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, (float*)part, st));
+  FBL_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, (float*)part, st, bias ? 4 : 0, M4, C4, O4));
   return FBL_OK;
 }
 

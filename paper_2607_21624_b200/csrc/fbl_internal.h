@@ -126,10 +126,9 @@ void fbl_note_cuda_error(cudaError_t e, const char* where);
 cudaError_t launch_pack(int dtype, int unpack, const void* src, void* dst, int64_t outer, int64_t rows,
                         int64_t rows_pad, int cols, cudaStream_t st);
 cudaError_t launch_rope(const fbl_plan* p, void* A, int heads_a, void* B, int heads_b, int inverse, cudaStream_t st);
-bool norm_fwd_resets_status(const fbl_plan* p);   // the forward norm kernel for this plan zeroes the status word itself
 cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
                             float* stats, int32_t* status, cudaStream_t st);
-bool norm_bwd_takes_colsums(const fbl_plan* p);
+// counts its own launches in p->launches (one to three)
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                             const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
                             cudaStream_t st, int bias_count = 0, const void* const* bias_m = nullptr,

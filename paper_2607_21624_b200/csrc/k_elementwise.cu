@@ -27,13 +27,6 @@ __device__ __forceinline__ void store16(T* p, const float (&v)[Vec16<T>::N]) {
   *reinterpret_cast<uint4*>(p) = raw;
 }
 
-__device__ __forceinline__ float group8_sum(float v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  return v;
-}
-
 // ------------------------------------------------------------------------------------------
 // pack / unpack: the only layout conversions, used at the graph boundary.
 // ------------------------------------------------------------------------------------------
@@ -68,273 +61,437 @@ __global__ void unpack_kernel(const T* __restrict__ src, T* __restrict__ dst, in
 }
 
 // ------------------------------------------------------------------------------------------
-// Pre-norm forward: row (feature-axis) reductions.  32 token rows per block.
-// stats[2r] = mean (0 for RMSNorm), stats[2r+1] = rstd.  Padding rows get zeros.
+// Pre-norm forward and backward for every width and both dtypes.  A thread owns the same 16-byte column vectors (NV of
+// them, `tpr` threads a row apart) of every row it meets, so gamma, beta and the token-axis sums of its columns stay in
+// registers and X (and dXn, dY) cross memory exactly once.  A row is `tpr` threads (a power of two up to a warp, whole
+// warps above); a block holds as many rows side by side as fit 256 threads.  What bounds both is bytes in flight against
+// the chain load -> row sums -> store, and next to it instruction issue (hence two-wide arithmetic).
+//   Forward: the next PF rows' vectors are in flight in registers; a row stays within a warp up to 96 vectors.
+//   Backward: R consecutive rows make a pass (R 128-byte pieces that lie behind each other in every column panel, one
+//   exchange between a row's warps for all of them), and the next pass is on its way to a ring in shared memory meanwhile:
+//   every thread copies to slots of its own and reads them back itself, which needs no barrier and no registers.
+// Measured stand-alone, warm caches, against a warp-register kernel at eight widths and two- and three-pass kernels with
+// shared-memory atomics elsewhere and in fp32 (us, before -> now, forward / backward with its reduction):
+//   2048 x 768 2.9 -> 2.4 / 9.0 -> 7.6;  6304 x 768 5.5 -> 4.5 / 15.0 -> 13.1;  6304 x 768 fp32 13.9 -> 10.4 / 43 -> 21;
+//   896 x 1280 10.4 -> 2.9 / 35 -> 7.0;  2977 x 2880 32 -> 11.4 / 90 -> 20.3;  8192 x 4096 34 -> 35 / 60 -> 42.
 // ------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) norm_fwd_kernel(const T* __restrict__ X, const float* __restrict__ gamma,
-                                                       const float* __restrict__ beta, T* __restrict__ Xn,
-                                                       float* __restrict__ stats, int64_t n_pad, int d, int seq,
-                                                       int t_pad, int rms, float eps) {
-  constexpr int TW = tile_w_of<T>::value;
-  constexpr int V = Vec16<T>::N;
-  const int64_t r = (int64_t)blockIdx.x * 32 + threadIdx.x / 8;
-  const int l8 = threadIdx.x % 8;
-  if (r >= n_pad) return;                       // whole 8-lane groups leave together
-  const bool pad = (int)(r % t_pad) >= seq;
-  const int panels = d / TW;
-  float v[V];
-  float mean = 0.f;
-  if (!rms) {
-    float s = 0.f;
-    for (int p = 0; p < panels; ++p) {
-      load16(X + ((int64_t)p * n_pad + r) * TW + l8 * V, v);
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool live) {     // zeros where not live
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(live ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__host__ __device__ constexpr int norm_stages(int r, int nv) { return r * nv > 4 ? 1 : r * nv == 4 ? 2 : 3; }   // passes in the ring: at most 192 KB
+
+// Two-wide fp32 arithmetic (one instruction for two elements): these kernels issue about as many instructions as their
+// bytes take cycles.
+template <typename T> __device__ __forceinline__ float2 pair_of(const uint4& raw, int i);      // elements 2i, 2i + 1
+template <> __device__ __forceinline__ float2 pair_of<float>(const uint4& raw, int i) { return reinterpret_cast<const float2*>(&raw)[i]; }
+template <> __device__ __forceinline__ float2 pair_of<__nv_bfloat16>(const uint4& raw, int i) {
+  const uint32_t u = reinterpret_cast<const uint32_t*>(&raw)[i];
+  return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+}
+// The V consecutive values of a vector of gamma or beta (plain fp32 arrays, normally 16-byte aligned).
+template <int V>
+__device__ __forceinline__ void load_params(const float* __restrict__ p, int c0, bool live, float2 (&v)[V / 2]) {
+  if (!live) {
 #pragma unroll
-      for (int i = 0; i < V; ++i) s += v[i];
+    for (int i = 0; i < V / 2; ++i) v[i] = make_float2(0.f, 0.f);
+  } else if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+#pragma unroll
+    for (int i = 0; i < V; i += 4) {
+      const float4 t = *reinterpret_cast<const float4*>(p + c0 + i);
+      v[i / 2] = make_float2(t.x, t.y); v[i / 2 + 1] = make_float2(t.z, t.w);
     }
-    mean = group8_sum(s) / (float)d;
-  }
-  float q = 0.f;
-  for (int p = 0; p < panels; ++p) {
-    load16(X + ((int64_t)p * n_pad + r) * TW + l8 * V, v);
+  } else {
 #pragma unroll
-    for (int i = 0; i < V; ++i) { float c = v[i] - mean; q += c * c; }
-  }
-  float rstd = rsqrtf(group8_sum(q) / (float)d + eps);
-  if (pad) { mean = 0.f; rstd = 0.f; }
-  if (l8 == 0) { stats[2 * r] = mean; stats[2 * r + 1] = rstd; }
-  for (int p = 0; p < panels; ++p) {
-    const int64_t off = ((int64_t)p * n_pad + r) * TW + l8 * V;
-    load16(X + off, v);
-    const int c0 = p * TW + l8 * V;
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-      float y = (v[i] - mean) * rstd * gamma[c0 + i] + (beta ? beta[c0 + i] : 0.f);
-      v[i] = pad ? 0.f : y;
-    }
-    store16(Xn + off, v);
+    for (int i = 0; i < V / 2; ++i) v[i] = make_float2(p[c0 + 2 * i], p[c0 + 2 * i + 1]);
   }
 }
-
-// ------------------------------------------------------------------------------------------
-// Pre-norm backward.  Row reductions mean(g), mean(g*xhat) with g = dXn*gamma give dX; the
-// token-axis reductions dgamma = sum dXn*xhat and dbeta = sum dXn are accumulated per block in
-// shared memory (a reduction over the block's 4 storage tiles) and added to the fp32 outputs.
-// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 template <typename T>
-__global__ void __launch_bounds__(256) norm_bwd_kernel(const T* __restrict__ dXn, const T* __restrict__ X,
-                                                       const T* __restrict__ dY, const float* __restrict__ stats,
-                                                       const float* __restrict__ gamma, T* __restrict__ dX,
-                                                       float* __restrict__ dgamma, float* __restrict__ dbeta,
-                                                       int64_t n_pad, int d, int rms) {
-  constexpr int TW = tile_w_of<T>::value;
-  constexpr int V = Vec16<T>::N;
-  extern __shared__ float sh[];                 // [2][d]
-  float* s_dg = sh;
-  float* s_db = sh + d;
-  for (int i = threadIdx.x; i < 2 * d; i += blockDim.x) sh[i] = 0.f;
-  __syncthreads();
-  const int64_t r = (int64_t)blockIdx.x * 32 + threadIdx.x / 8;
-  const int l8 = threadIdx.x % 8;
-  const bool live = r < n_pad;
-  const int panels = d / TW;
-  float mean = 0.f, rstd = 0.f;
-  if (live) { mean = stats[2 * r]; rstd = stats[2 * r + 1]; }
-  float xv[V], gv[V];
-  float s1 = 0.f, s2 = 0.f;
-  for (int p = 0; p < panels; ++p) {
-    const int c0 = p * TW + l8 * V;
-    float pg[V], pb[V];
-    if (live) {
-      const int64_t off = ((int64_t)p * n_pad + r) * TW + l8 * V;
-      load16(X + off, xv);
-      load16(dXn + off, gv);
+__device__ __forceinline__ void store_pairs(T* p, const float2 (&v)[Vec16<T>::N / 2]) {
+  store16(p, reinterpret_cast<const float(&)[Vec16<T>::N]>(v));
+}
+
+struct NormShape { int nv, tpr, groups, r; };   // vectors per thread, threads per row, rows side by side, rows per pass
+
+static NormShape norm_shape(int nvec, int nv) {
+  NormShape s;
+  s.nv = nv;
+  const int per = (nvec + nv - 1) / nv;
+  if (per <= 32) { s.tpr = 8; while (s.tpr < per) s.tpr *= 2; }
+  else s.tpr = (per + 31) / 32 * 32;
+  s.groups = s.tpr >= 256 ? 1 : 256 / s.tpr;
+  s.r = 1;
+  return s;
+}
+// Forward: a row within one warp up to 96 vectors; then two or three vectors per thread, whichever leaves fewer idle
+// lanes (three where equal: fewer warps to a row); above 512 vectors four or eight.
+static NormShape norm_fwd_shape(int nvec) {
+  if (nvec <= 96) return norm_shape(nvec, (nvec + 31) / 32);
+  if (nvec > 512) return norm_shape(nvec, nvec <= 2048 ? 4 : 8);
+  const NormShape two = norm_shape(nvec, 2), three = norm_shape(nvec, 3);
+  return two.tpr * 2 < three.tpr * 3 ? two : three;
+}
+// Backward: one vector per thread up to 256 (the token-axis sums of one vector are 16 registers), with as many rows per
+// pass (1, 2 or 4) as the rows leave for two blocks on every SM; wider rows two vectors and two rows, then four or eight.
+static NormShape norm_bwd_shape(int nvec, int64_t n_pad, int sm_count) {
+  NormShape s = norm_shape(nvec, nvec <= 256 ? 1 : nvec <= 1024 ? 2 : nvec <= 2048 ? 4 : 8);
+  const int64_t slots = (int64_t)2 * sm_count * s.groups, want = (n_pad + slots - 1) / slots;
+  s.r = want >= 3 ? 4 : (want == 2 ? 2 : 1);
+  while (s.r * s.nv > 4 && s.r > 1) s.r /= 2;
+  return s;
+}
+
+// Sums of K values over the tpr threads of a row, returned to all of them.  Up to a warp: shuffles.  Whole warps: the
+// K sums of a warp by exchanging halves (K / 2 + K / 4 + ... shuffles, then the rest on one value), one exchange of
+// the warps' sums through shared memory behind a barrier of the row's own.  Successive calls alternate between two
+// exchange buffers: a warp that writes a buffer again has passed the barrier of the call in between, which every
+// reader of the earlier values reached after reading them.
+constexpr int NORM_EX = 16 * 8;                              // floats of one exchange buffer of a block: warps x values
+// TPR > 0: tpr at compile time.
+template <int K, int TPR = 0>
+__device__ __forceinline__ void row_sums(float (&v)[K], int tpr, int group, float* ex, int& buf) {
+  const int lane = threadIdx.x & 31;
+  if (TPR == 32) {
 #pragma unroll
-      for (int i = 0; i < V; ++i) {
-        float xh = (xv[i] - mean) * rstd;
-        float g = gv[i] * gamma[c0 + i];
-        s1 += g;
-        s2 += g * xh;
-        pg[i] = gv[i] * xh;
-        pb[i] = gv[i];
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    return;
+  }
+  if (TPR == 0 && tpr <= 32) {
+    for (int o = tpr / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    return;
+  }
+  float* e = ex + buf * NORM_EX;
+  buf ^= 1;
+  int idx = 0;
+#pragma unroll
+  for (int n = K, o = 16; n > 1; n /= 2, o >>= 1) {          // lanes with bit o keep the upper half of the values
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < n / 2; ++k) {
+      const float send = up ? v[k] : v[k + n / 2], keep = up ? v[k + n / 2] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    idx = idx * 2 + (up ? 1 : 0);
+  }
+#pragma unroll
+  for (int o = 16 / K; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  const int warp = threadIdx.x / 32, wpr = (TPR ? TPR : tpr) / 32, w0 = group * wpr;
+  if ((lane & (32 / K - 1)) == 0) e[warp * K + idx] = v[0];
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(tpr) : "memory");
+#pragma unroll
+  for (int k = 0; k < K; ++k) v[k] = 0.f;
+#pragma unroll 8
+  for (int w = 0; w < wpr; ++w) {
+    if constexpr (K % 4 == 0) {
+#pragma unroll
+      for (int k = 0; k < K; k += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(e + (w0 + w) * K + k);
+        v[k] += t.x; v[k + 1] += t.y; v[k + 2] += t.z; v[k + 3] += t.w;
       }
     } else {
 #pragma unroll
-      for (int i = 0; i < V; ++i) { pg[i] = 0.f; pb[i] = 0.f; }
-    }
-    // sum the 4 rows of this warp, then one shared-memory add per column per warp
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-      pg[i] += __shfl_xor_sync(0xffffffffu, pg[i], 8);
-      pg[i] += __shfl_xor_sync(0xffffffffu, pg[i], 16);
-      pb[i] += __shfl_xor_sync(0xffffffffu, pb[i], 8);
-      pb[i] += __shfl_xor_sync(0xffffffffu, pb[i], 16);
-    }
-    if ((threadIdx.x & 31) < 8) {
-#pragma unroll
-      for (int i = 0; i < V; ++i) {
-        atomicAdd(&s_dg[c0 + i], pg[i]);
-        atomicAdd(&s_db[c0 + i], pb[i]);
-      }
+      for (int k = 0; k < K; ++k) v[k] += e[(w0 + w) * K + k];
     }
   }
-  s1 = group8_sum(s1) / (float)d;
-  s2 = group8_sum(s2) / (float)d;
-  if (rms) s1 = 0.f;
-  if (live) {
-    for (int p = 0; p < panels; ++p) {
-      const int64_t off = ((int64_t)p * n_pad + r) * TW + l8 * V;
-      const int c0 = p * TW + l8 * V;
-      load16(X + off, xv);
-      load16(dXn + off, gv);
-      float rv[V];
-      if (dY) load16(dY + off, rv);
-#pragma unroll
-      for (int i = 0; i < V; ++i) {
-        float xh = (xv[i] - mean) * rstd;
-        float o = rstd * (gv[i] * gamma[c0 + i] - s1 - xh * s2);
-        xv[i] = dY ? o + rv[i] : o;
-      }
-      store16(dX + off, xv);
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    atomicAdd(&dgamma[i], s_dg[i]);
-    if (dbeta) atomicAdd(&dbeta[i], s_db[i]);
-  }
 }
 
-
-// ------------------------------------------------------------------------------------------
-// Register-resident norm kernels for bf16 rows (NV vectors of 16 bytes per lane, WPR warps per row, d_model =
-// 256 NV WPR up to 4096): a warp owns a row or a contiguous part of it, lane l holds vectors l, l + 32, ... of it (each warp-level load covers four
-// whole 128-byte tile rows, one per column panel), so X (and dXn) cross HBM exactly once.
-// ------------------------------------------------------------------------------------------
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// WPR warps share a row (d_model = NV * 256 * WPR columns): the row statistics are combined through shared memory.
-// The warps of a row meet at a named barrier of their own (rows of one block do not wait for each other), and
-// successive reductions alternate between two exchange buffers: a warp that writes buffer b again has passed the
-// barrier of the reduction in between, which every reader of the earlier value reached after reading it.
-template <int WPR>
-__device__ __forceinline__ float row_sum(float v, float* s_part, int slot, int part, int& buf) {
-  v = warp_sum(v);
-  if (WPR == 1) return v;
-  float* ex = s_part + buf * 8;
-  buf ^= 1;
-  if ((threadIdx.x & 31) == 0) ex[slot * WPR + part] = v;
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + slot), "r"(WPR * 32) : "memory");
-  float t = 0.f;
-#pragma unroll
-  for (int i = 0; i < WPR; ++i) t += ex[slot * WPR + i];
-  return t;
-}
-
-// Two sums in one exchange.
-template <int WPR>
-__device__ __forceinline__ void row_sum2(float& a, float& b, float* s_part, int slot, int part, int& buf) {
-  a = warp_sum(a);
-  b = warp_sum(b);
-  if (WPR == 1) return;
-  float* ex = s_part + buf * 16;
-  buf ^= 1;
-  if ((threadIdx.x & 31) == 0) { ex[(slot * WPR + part) * 2] = a; ex[(slot * WPR + part) * 2 + 1] = b; }
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + slot), "r"(WPR * 32) : "memory");
-  a = 0.f; b = 0.f;
-#pragma unroll
-  for (int i = 0; i < WPR; ++i) { a += ex[(slot * WPR + i) * 2]; b += ex[(slot * WPR + i) * 2 + 1]; }
-}
-
-template <int NV, int WPR>
-__global__ void __launch_bounds__(256, 2) norm_fwd_rows_kernel(const __nv_bfloat16* __restrict__ X,
-                                                            const float* __restrict__ gamma,
-                                                            const float* __restrict__ beta,
-                                                            __nv_bfloat16* __restrict__ Xn, float* __restrict__ stats,
-                                                            int64_t n_pad, int seq, int t_pad, int rms, float eps,
-                                                            int32_t* __restrict__ status) {
-  constexpr int D = NV * 256 * WPR;
-  constexpr int RPB = 8 / WPR;                       // rows per block pass
-  __shared__ float s_part[16];
+template <typename T, int NV, int PF, int TPR>
+__global__ void __launch_bounds__(512) norm_fwd_kernel(const T* __restrict__ X, const float* __restrict__ gamma,
+                                                       const float* __restrict__ beta, T* __restrict__ Xn,
+                                                       float* __restrict__ stats, int64_t n_pad, int d, int tpr_rt, int64_t per_block,
+                                                       int seq, int t_pad, int rms, float eps, int32_t* __restrict__ status) {
+  constexpr int V = Vec16<T>::N, TW = tile_w_of<T>::value;
+  __shared__ __align__(16) float s_ex[2 * NORM_EX];
   // First kernel of the forward pass: it resets the pass's status word (later kernels only write it after a
   // bounded wait of about a second has expired), which saves a fill node in front of the pass.
-  if (status && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
-  const int lane = threadIdx.x % 32, wib = threadIdx.x / 32;
-  const int slot = wib / WPR, part = wib % WPR;
-  int buf = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
   pdl_launch_dependents();
-  // gamma and beta are inputs of the step: in registers before waiting for the previous kernel
-  float gm[NV][8], bt[NV][8];
+  const int tpr = TPR ? TPR : tpr_rt;
+  const int group = threadIdx.x / tpr, lt = threadIdx.x % tpr, groups = blockDim.x / tpr;
+  const float inv_d = 1.f / (float)d;
+  int buf = 0;
+  bool on[NV];
+  float2 gm[NV][V / 2], bt[NV][V / 2];                       // inputs of the step: read before waiting for the kernel in front
 #pragma unroll
   for (int j = 0; j < NV; ++j) {
-    const int c0 = ((part * NV + j) * 32 + lane) * 8;
-    const float4 g0 = *reinterpret_cast<const float4*>(gamma + c0), g1 = *reinterpret_cast<const float4*>(gamma + c0 + 4);
-    float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
-    if (beta) { b0 = *reinterpret_cast<const float4*>(beta + c0); b1 = *reinterpret_cast<const float4*>(beta + c0 + 4); }
-    gm[j][0] = g0.x; gm[j][1] = g0.y; gm[j][2] = g0.z; gm[j][3] = g0.w; gm[j][4] = g1.x; gm[j][5] = g1.y; gm[j][6] = g1.z; gm[j][7] = g1.w;
-    bt[j][0] = b0.x; bt[j][1] = b0.y; bt[j][2] = b0.z; bt[j][3] = b0.w; bt[j][4] = b1.x; bt[j][5] = b1.y; bt[j][6] = b1.z; bt[j][7] = b1.w;
+    const int c0 = (lt + j * tpr) * V;
+    on[j] = c0 < d;
+    load_params<V>(gamma, c0, on[j], gm[j]);
+    load_params<V>(beta, c0, on[j] && beta, bt[j]);
   }
   pdl_wait();
-  // Each block owns a contiguous range of rows and walks it in order: the PF rows in flight are then neighbours,
-  // i.e. in every 64-column panel PF adjacent 128-byte pieces (with a grid-stride walk every piece stood alone).
-  constexpr int64_t stride = RPB;
-  const int64_t per_block = ((n_pad + gridDim.x - 1) / gridDim.x + RPB - 1) / RPB * RPB;
   const int64_t r_end = min(n_pad, ((int64_t)blockIdx.x + 1) * per_block);
-  // lane's vectors of a row: vector index v -> panel v / 8, chunk v % 8
-  auto vec_off = [&](int j, int64_t r) {
-    const int v = (part * NV + j) * 32 + lane;
-    return ((int64_t)(v / 8) * n_pad + r) * 64 + (v % 8) * 8;
-  };
-  // PF rows ahead are in flight per warp (raw vectors in registers): with one row ahead a block waited ~1.4 us
-  // per row on the load of the next one; HBM needs about 10 MB in flight across the GPU
-  constexpr int PF = NV == 3 ? 3 : 4;
-  int64_t r = (int64_t)blockIdx.x * per_block + slot;
-  uint4 ring[PF][NV];
+  auto fetch = [&](uint4 (&raw)[NV], int64_t r) {
 #pragma unroll
-  for (int k = 0; k < PF; ++k) {
-    if (r + k * stride < r_end) {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) ring[k][j] = *reinterpret_cast<const uint4*>(X + vec_off(j, r + k * stride));
+    for (int j = 0; j < NV; ++j) {
+      const int v = lt + j * tpr;
+      raw[j] = make_uint4(0u, 0u, 0u, 0u);
+      if (on[j] && r < r_end) raw[j] = *reinterpret_cast<const uint4*>(X + ((int64_t)(v / 8) * n_pad + r) * TW + (v % 8) * V);
     }
-  }
-  bool more = r < r_end;
-  while (more) {
+  };
+  uint4 ring[PF][NV];
+  const int64_t base = (int64_t)blockIdx.x * per_block;
+#pragma unroll
+  for (int k = 0; k < PF; ++k) fetch(ring[k], base + group + k * groups);
+  for (int64_t rb = base; rb < r_end;) {                     // block-uniform: every thread takes part in the row sums
 #pragma unroll
     for (int k = 0; k < PF; ++k) {
-      if (r >= r_end) { more = false; break; }
+      if (rb >= r_end) break;
+      const int64_t r = rb + group;
       const bool pad = (int)(r % t_pad) >= seq;
-      float x[NV][8];
-      float s = 0.f;
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&ring[k][j]);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { x[j][i] = __bfloat162float(e[i]); s += x[j][i]; }
-      }
-      if (r + PF * stride < r_end) {
-#pragma unroll
-        for (int j = 0; j < NV; ++j) ring[k][j] = *reinterpret_cast<const uint4*>(X + vec_off(j, r + PF * stride));
-      }
-      const float mean = rms ? 0.f : row_sum<WPR>(s, s_part, slot, part, buf) * (1.f / D);
-      float q = 0.f;
+      float2 x[NV][V / 2];
+      float2 t = both(0.f);
 #pragma unroll
       for (int j = 0; j < NV; ++j)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { const float c = x[j][i] - mean; q += c * c; }
-      const float rstd = rsqrtf(row_sum<WPR>(q, s_part, slot, part, buf) * (1.f / D) + eps);
-      if (lane == 0 && part == 0) { stats[2 * r] = pad ? 0.f : mean; stats[2 * r + 1] = pad ? 0.f : rstd; }
+        for (int i = 0; i < V / 2; ++i) { x[j][i] = pair_of<T>(ring[k][j], i); t = __fadd2_rn(t, x[j][i]); }
+      fetch(ring[k], r + PF * groups);
+      float mean[1] = {0.f}, q[1];
+      if (!rms) {
+        mean[0] = t.x + t.y;
+        row_sums<1, TPR>(mean, tpr, group, s_ex, buf);
+        mean[0] *= inv_d;
+      }
+      t = both(0.f);
 #pragma unroll
       for (int j = 0; j < NV; ++j) {
-        float y[8];
+        if (!on[j]) continue;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) y[i] = pad ? 0.f : (x[j][i] - mean) * rstd * gm[j][i] + bt[j][i];
-        store16(Xn + vec_off(j, r), y);
+        for (int i = 0; i < V / 2; ++i) { x[j][i] = __fadd2_rn(x[j][i], both(-mean[0])); t = __ffma2_rn(x[j][i], x[j][i], t); }
       }
-      r += stride;
+      q[0] = t.x + t.y;
+      row_sums<1, TPR>(q, tpr, group, s_ex, buf);
+      const float rstd = rsqrtf(q[0] * inv_d + eps);
+      if (r < r_end) {
+        if (lt == 0) *reinterpret_cast<float2*>(stats + 2 * r) = pad ? make_float2(0.f, 0.f) : make_float2(mean[0], rstd);
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          if (!on[j]) continue;
+          float2 y[V / 2];
+#pragma unroll
+          for (int i = 0; i < V / 2; ++i) y[i] = pad ? both(0.f) : __ffma2_rn(__fmul2_rn(x[j][i], both(rstd)), gm[j][i], bt[j][i]);
+          const int v = lt + j * tpr;
+          store_pairs(Xn + ((int64_t)(v / 8) * n_pad + r) * TW + (v % 8) * V, y);
+        }
+      }
+      rb += groups;
+    }
+  }
+}
+
+constexpr int COLSUM_SLAB = 256;
+
+struct ColsumGroup {
+  const void* m[4];
+  float* out[4];
+  int cols[4];
+  int64_t part_off[4];      // float offset of each matrix's partials inside the scratch area
+  int count;
+};
+
+// First stage of a token-axis column sum: the block's (128-byte column panel p, slab of 256 rows) of matrix `which`,
+// 32 storage tiles, reduced to one row of partials.  Any block of whole warps up to 512 threads; `red` has a row per warp.
+template <typename T>
+__device__ __forceinline__ void colsum_slab(const ColsumGroup& G, int64_t rows, float* __restrict__ part_base, int p,
+                                            int slab, int which, float (*red)[tile_w_of<T>::value + 1]) {
+  constexpr int TW = tile_w_of<T>::value;
+  constexpr int V = Vec16<T>::N;
+  const int cols = G.cols[which];
+  if (p * TW >= cols) return;
+  const T* M = (const T*)G.m[which];
+  float* part = part_base + G.part_off[which];
+  const int rr = threadIdx.x / 8, l8 = threadIdx.x % 8, rstep = blockDim.x / 8;
+  float acc[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) acc[i] = 0.f;
+  const int64_t r_end = min((int64_t)(slab + 1) * COLSUM_SLAB, rows);
+#pragma unroll 8                              // all of a thread's loads of the slab in flight together
+  for (int64_t r = (int64_t)slab * COLSUM_SLAB + rr; r < r_end; r += rstep) {
+    float v[V];
+    load16(M + ((int64_t)p * rows + r) * TW + l8 * V, v);
+#pragma unroll
+    for (int i = 0; i < V; ++i) acc[i] += v[i];
+  }
+  // a warp holds four rows of eight vectors: add them, then one row per warp through shared memory
+#pragma unroll
+  for (int i = 0; i < V; ++i) {
+    acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 8);
+    acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+  }
+  const int warp = threadIdx.x / 32, warps = blockDim.x / 32;
+  if ((threadIdx.x & 31) < 8) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) red[warp][l8 * V + i] = acc[i];
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < TW; c += blockDim.x) {
+    float s = 0.f;
+    for (int k = 0; k < warps; ++k) s += red[k][c];
+    part[(int64_t)slab * cols + p * TW + c] = s;
+  }
+}
+
+// Backward.  Row sums mean(g) and mean(g xhat) with g = dXn gamma give dX; dgamma = sum dXn xhat and dbeta = sum dXn of
+// the thread's own columns accumulate in registers over the block's rows, are added over the block's row groups at the
+// end and leave as one partial row per block (the second kernel adds the blocks' rows: no atomics, the result does not
+// depend on their order).  partials = nullptr: the norm's parameters are frozen, only dX is formed.
+template <typename T, int NV, int R>
+__global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn, const T* __restrict__ X, const T* __restrict__ dY,
+                                                       const float* __restrict__ stats, const float* __restrict__ gamma,
+                                                       T* __restrict__ dX, float* __restrict__ partials, int64_t n_pad, int d,
+                                                       int tpr, int64_t per_block, int rms, int n_norm,
+                                                       const __grid_constant__ ColsumGroup CG,
+                                                       float* __restrict__ cs_part, int cs_panels, int cs_slabs) {
+  constexpr int V = Vec16<T>::N, TW = tile_w_of<T>::value;
+  // exchange buffers of the row sums; the column-sum blocks use it as well
+  __shared__ __align__(16) float s_ex[16 * (TW + 1) > 2 * NORM_EX ? 16 * (TW + 1) : 2 * NORM_EX];
+  // Blocks behind the first n_norm ones do the first stage of the bias gradients' column sums (one launch less):
+  // block n_norm + (which * slabs + slab) * panels + p
+  if ((int)blockIdx.x >= n_norm) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int idx = (int)blockIdx.x - n_norm;
+    colsum_slab<T>(CG, n_pad, cs_part, idx % cs_panels, (idx / cs_panels) % cs_slabs, idx / (cs_panels * cs_slabs),
+                   reinterpret_cast<float(*)[TW + 1]>(s_ex));
+    return;
+  }
+  pdl_launch_dependents();
+  const int group = threadIdx.x / tpr, lt = threadIdx.x % tpr, groups = blockDim.x / tpr;
+  const float inv_d = 1.f / (float)d;
+  int buf = 0;
+  bool on[NV];
+  float2 gm[NV][V / 2], ag[NV][V / 2], ab[NV][V / 2];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    const int c0 = (lt + j * tpr) * V;
+    on[j] = c0 < d;
+    load_params<V>(gamma, c0, on[j], gm[j]);
+#pragma unroll
+    for (int i = 0; i < V / 2; ++i) ag[j][i] = ab[j][i] = both(0.f);
+  }
+  pdl_wait();
+  constexpr int S = norm_stages(R, NV);
+  extern __shared__ __align__(16) uint8_t s_ring[];          // [stage][X, dXn, (dY)][row][vector][thread]
+  const int arrays = dY ? 3 : 2;
+  const uint4* ring = reinterpret_cast<const uint4*>(s_ring) + threadIdx.x;
+  const uint32_t ring_addr = (uint32_t)__cvta_generic_to_shared(s_ring) + threadIdx.x * 16;
+  const int64_t first = (int64_t)blockIdx.x * per_block + group * R, r_end = min(n_pad, ((int64_t)blockIdx.x + 1) * per_block);
+  auto fetch = [&](int64_t r0, int stage) {
+#pragma unroll
+    for (int k = 0; k < R; ++k)
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        const int v = lt + j * tpr;
+        const bool live = on[j] && r0 + k < r_end;
+        const int64_t off = live ? ((int64_t)(v / 8) * n_pad + r0 + k) * TW + (v % 8) * V : 0;
+        const uint32_t dst = ring_addr + ((stage * arrays * R + k) * NV + j) * blockDim.x * 16, step = R * NV * blockDim.x * 16;
+        cp_async16(dst, X + off, live);
+        cp_async16(dst + step, dXn + off, live);
+        if (dY) cp_async16(dst + 2 * step, dY + off, live);
+      }
+    cp_async_commit();
+  };
+  float2 stn[R];                                             // mean and rstd of the next pass's rows
+  auto fetch_stats = [&](int64_t r0) {
+#pragma unroll
+    for (int k = 0; k < R; ++k) stn[k] = r0 + k < r_end ? *reinterpret_cast<const float2*>(stats + 2 * (r0 + k)) : make_float2(0.f, 0.f);
+  };
+#pragma unroll
+  for (int i = 0; i < S - 1; ++i) fetch(first + (int64_t)i * groups * R, i);
+  fetch_stats(first);
+  int stage = 0;
+  for (int64_t r0 = first; r0 - group * R < r_end; r0 += groups * R) {
+    fetch(r0 + (int64_t)(S - 1) * groups * R, stage == 0 ? S - 1 : stage - 1);      // the stage read a pass ago
+    float2 st[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) st[k] = stn[k];
+    fetch_stats(r0 + groups * R);
+    cp_async_wait<S - 1>();
+    const uint4* xs = ring + stage * arrays * R * NV * blockDim.x;
+    const uint4* gs = xs + R * NV * blockDim.x;
+    const uint4* ys = gs + R * NV * blockDim.x;
+    stage = stage == S - 1 ? 0 : stage + 1;
+    float s[2 * R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      float2 t1 = both(0.f), t2 = both(0.f);
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        const uint4 xr = xs[(k * NV + j) * blockDim.x], gr = gs[(k * NV + j) * blockDim.x];
+#pragma unroll
+        for (int i = 0; i < V / 2; ++i) {
+          const float2 xh = __fmul2_rn(__fadd2_rn(pair_of<T>(xr, i), both(-st[k].x)), both(st[k].y));
+          const float2 gv = pair_of<T>(gr, i), g = __fmul2_rn(gv, gm[j][i]);
+          ag[j][i] = __ffma2_rn(gv, xh, ag[j][i]);
+          ab[j][i] = __fadd2_rn(ab[j][i], gv);
+          t1 = __fadd2_rn(t1, g);
+          t2 = __ffma2_rn(g, xh, t2);
+        }
+      }
+      s[2 * k] = t1.x + t1.y;
+      s[2 * k + 1] = t2.x + t2.y;
+    }
+    row_sums<2 * R>(s, tpr, group, s_ex, buf);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const int64_t r = r0 + k;
+      if (r >= r_end) break;
+      const float s1 = rms ? 0.f : s[2 * k] * inv_d, s2 = s[2 * k + 1] * inv_d;
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        if (!on[j]) continue;
+        const uint4 xr = xs[(k * NV + j) * blockDim.x], gr = gs[(k * NV + j) * blockDim.x];
+        const uint4 yr = dY ? ys[(k * NV + j) * blockDim.x] : make_uint4(0u, 0u, 0u, 0u);
+        float2 o[V / 2];
+#pragma unroll
+        for (int i = 0; i < V / 2; ++i) {
+          const float2 xh = __fmul2_rn(__fadd2_rn(pair_of<T>(xr, i), both(-st[k].x)), both(st[k].y));
+          const float2 g = __ffma2_rn(pair_of<T>(gr, i), gm[j][i], both(-s1));
+          o[i] = __ffma2_rn(both(st[k].y), __ffma2_rn(xh, both(-s2), g), pair_of<T>(yr, i));
+        }
+        const int v = lt + j * tpr;
+        store_pairs(dX + ((int64_t)(v / 8) * n_pad + r) * TW + (v % 8) * V, o);
+      }
+    }
+  }
+  cp_async_wait<0>();
+  if (!partials) return;
+  float* mine = partials + (int64_t)blockIdx.x * 2 * d;
+  const int width = tpr * NV * V;
+  if (groups > 1) {
+    float* s_sum = reinterpret_cast<float*>(s_ring);         // [groups][2][row width], over the ring
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+#pragma unroll
+      for (int i = 0; i < V; i += 4) {
+        float* p = s_sum + (size_t)group * 2 * width + (lt + j * tpr) * V + i;
+        *reinterpret_cast<float4*>(p) = make_float4(ag[j][i / 2].x, ag[j][i / 2].y, ag[j][i / 2 + 1].x, ag[j][i / 2 + 1].y);
+        *reinterpret_cast<float4*>(p + width) = make_float4(ab[j][i / 2].x, ab[j][i / 2].y, ab[j][i / 2 + 1].x, ab[j][i / 2 + 1].y);
+      }
+    __syncthreads();
+    for (int c = threadIdx.x; c < (rms ? d : 2 * d); c += blockDim.x) {
+      const int at = c < d ? c : width + c - d;
+      float t = 0.f;
+      for (int q = 0; q < groups; ++q) t += s_sum[(size_t)q * 2 * width + at];
+      mine[c] = t;
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    if (!on[j]) continue;
+    const int c0 = (lt + j * tpr) * V;
+#pragma unroll
+    for (int i = 0; i < V; i += 4) {
+      *reinterpret_cast<float4*>(mine + c0 + i) = make_float4(ag[j][i / 2].x, ag[j][i / 2].y, ag[j][i / 2 + 1].x, ag[j][i / 2 + 1].y);
+      if (!rms) *reinterpret_cast<float4*>(mine + d + c0 + i) = make_float4(ab[j][i / 2].x, ab[j][i / 2].y, ab[j][i / 2 + 1].x, ab[j][i / 2 + 1].y);
     }
   }
 }
@@ -388,217 +545,12 @@ __global__ void __launch_bounds__(256) rope_kernel(T* __restrict__ A, int heads_
   }
 }
 
-constexpr int COLSUM_SLAB = 256;
-
-struct ColsumGroup {
-  const void* m[4];
-  float* out[4];
-  int cols[4];
-  int64_t part_off[4];      // float offset of each matrix's partials inside the scratch area
-  int count;
-};
-
-// First stage of a token-axis column sum: the block's (64-column panel p, slab of 256 rows) of matrix `which`,
-// 32 storage tiles, reduced to one row of partials.  `red` is 32 x (tile width + 1) floats of shared memory.
-template <typename T>
-__device__ __forceinline__ void colsum_slab(const ColsumGroup& G, int64_t rows, float* __restrict__ part_base, int p,
-                                            int slab, int which, float (*red)[tile_w_of<T>::value + 1]) {
-  constexpr int TW = tile_w_of<T>::value;
-  constexpr int V = Vec16<T>::N;
-  const int cols = G.cols[which];
-  if (p * TW >= cols) return;
-  const T* M = (const T*)G.m[which];
-  float* part = part_base + G.part_off[which];
-  const int rr = threadIdx.x / 8, l8 = threadIdx.x % 8;
-  float acc[V];
-#pragma unroll
-  for (int i = 0; i < V; ++i) acc[i] = 0.f;
-  const int64_t r_end = min((int64_t)(slab + 1) * COLSUM_SLAB, rows);
-#pragma unroll 8                              // a slab is eight 32-row steps: all their loads in flight together
-  for (int64_t r = (int64_t)slab * COLSUM_SLAB + rr; r < r_end; r += 32) {
-    float v[V];
-    load16(M + ((int64_t)p * rows + r) * TW + l8 * V, v);
-#pragma unroll
-    for (int i = 0; i < V; ++i) acc[i] += v[i];
-  }
-#pragma unroll
-  for (int i = 0; i < V; ++i) red[rr][l8 * V + i] = acc[i];
-  __syncthreads();
-  if (threadIdx.x < TW) {
-    float s = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) s += red[k][threadIdx.x];
-    part[(int64_t)slab * cols + p * TW + threadIdx.x] = s;
-  }
-}
-
-// Shared memory of the kernel below: per warp its private token-axis sums (dgamma and dbeta parts of its columns,
-// as float4 slots [which][2 NV][32 lanes]: consecutive lanes, consecutive slots, conflict-free), then gamma.
-template <int NV, int WPR>
-struct NormBwdSmem {
-  static constexpr int D = NV * 256 * WPR;
-  static constexpr int ACC_F4_PER_WARP = 2 * 2 * NV * 32;
-  static constexpr size_t ACC_BYTES = (size_t)8 * ACC_F4_PER_WARP * 16;
-  static constexpr size_t BYTES = ACC_BYTES + (size_t)D * 4;
-};
-
-// A warp (or WPR warps) owns a row; the row's X and dXn stay in registers as raw bf16 vectors, and the next row's
-// are requested before the current row's two reductions, so X and dXn cross HBM exactly once with a row in flight
-// per warp at all times.  The token-axis sums (dgamma, dbeta) of a warp's rows accumulate in its private
-// shared-memory slots (registers are better spent on the row in flight).
-template <int NV, int WPR>
-__global__ void __launch_bounds__(256, 2) norm_bwd_rows_kernel(const __nv_bfloat16* __restrict__ dXn,
-                                                            const __nv_bfloat16* __restrict__ X,
-                                                            const __nv_bfloat16* __restrict__ dY,
-                                                            const float* __restrict__ stats,
-                                                            const float* __restrict__ gamma,
-                                                            __nv_bfloat16* __restrict__ dX, float* __restrict__ partials,
-                                                            int64_t n_pad, int rms, int n_norm, ColsumGroup CG,
-                                                            float* __restrict__ cs_part, int cs_panels, int cs_slabs) {
-  using SMEM = NormBwdSmem<NV, WPR>;
-  constexpr int D = SMEM::D;
-  constexpr int RPB = 8 / WPR;
-  extern __shared__ __align__(16) uint8_t norm_smem[];
-  __shared__ float s_part[32];
-  // Blocks behind the first n_norm ones do the first stage of the bias gradients' column sums (one launch less):
-  // block n_norm + (which * slabs + slab) * panels + p
-  if ((int)blockIdx.x >= n_norm) {
-    __shared__ float cs_red[32][65];
-    pdl_launch_dependents();
-    pdl_wait();
-    const int idx = (int)blockIdx.x - n_norm;
-    colsum_slab<__nv_bfloat16>(CG, n_pad, cs_part, idx % cs_panels, (idx / cs_panels) % cs_slabs, idx / (cs_panels * cs_slabs), cs_red);
-    return;
-  }
-  float4* s_acc = reinterpret_cast<float4*>(norm_smem);
-  float* s_gamma = reinterpret_cast<float*>(norm_smem + SMEM::ACC_BYTES);
-  const int lane = threadIdx.x % 32, wib = threadIdx.x / 32;
-  const int slot = wib / WPR, part = wib % WPR;
-  int buf = 0;
-  // gamma is an input of the step: into shared memory before waiting for the GEMM in front; the sums start at zero
-  for (int i = threadIdx.x; i < D; i += 256) s_gamma[i] = gamma[i];
-  for (int i = threadIdx.x; i < 8 * SMEM::ACC_F4_PER_WARP; i += 256) s_acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  __syncthreads();
-  pdl_launch_dependents();
-  float4* my_acc = s_acc + wib * SMEM::ACC_F4_PER_WARP;       // [which][2 j + h][lane]
-  auto vec_off = [&](int j, int64_t r) {
-    const int v = (part * NV + j) * 32 + lane;
-    return ((int64_t)(v / 8) * n_pad + r) * 64 + (v % 8) * 8;
-  };
-  pdl_wait();
-  // each block owns a contiguous range of rows (neighbouring 128-byte pieces in every panel)
-  const int64_t per_block = ((n_pad + n_norm - 1) / n_norm + RPB - 1) / RPB * RPB;
-  const int64_t r_end = min(n_pad, ((int64_t)blockIdx.x + 1) * per_block);
-  int64_t r = (int64_t)blockIdx.x * per_block + slot;
-  uint4 xr[NV], gr[NV];
-  float2 st = make_float2(0.f, 0.f);
-  if (r < r_end) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      xr[j] = *reinterpret_cast<const uint4*>(X + vec_off(j, r));
-      gr[j] = *reinterpret_cast<const uint4*>(dXn + vec_off(j, r));
-    }
-    st = *reinterpret_cast<const float2*>(stats + 2 * r);
-  }
-  while (r < r_end) {
-    const int64_t rn = r + RPB;
-    uint4 xn[NV], gn[NV], yr[NV];
-    float2 stn = make_float2(0.f, 0.f);
-    if (rn < r_end) {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        xn[j] = *reinterpret_cast<const uint4*>(X + vec_off(j, rn));
-        gn[j] = *reinterpret_cast<const uint4*>(dXn + vec_off(j, rn));
-      }
-      stn = *reinterpret_cast<const float2*>(stats + 2 * rn);
-    }
-    if (dY) {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) yr[j] = *reinterpret_cast<const uint4*>(dY + vec_off(j, r));
-    }
-    const float mean = st.x, rstd = st.y;
-    float s1 = 0.f, s2 = 0.f;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      const __nv_bfloat16* xe = reinterpret_cast<const __nv_bfloat16*>(&xr[j]);
-      const __nv_bfloat16* ge = reinterpret_cast<const __nv_bfloat16*>(&gr[j]);
-      const int c0 = ((part * NV + j) * 32 + lane) * 8;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float4 gm = *reinterpret_cast<const float4*>(s_gamma + c0 + 4 * h);
-        const float gmv[4] = {gm.x, gm.y, gm.z, gm.w};
-        float4 ag = my_acc[(2 * j + h) * 32 + lane], ab = my_acc[(2 * NV + 2 * j + h) * 32 + lane];
-        float* agv = reinterpret_cast<float*>(&ag);
-        float* abv = reinterpret_cast<float*>(&ab);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float xh = (__bfloat162float(xe[4 * h + i]) - mean) * rstd;
-          const float gv = __bfloat162float(ge[4 * h + i]);
-          const float g = gv * gmv[i];
-          agv[i] = fmaf(gv, xh, agv[i]);
-          abv[i] += gv;
-          s1 += g;
-          s2 = fmaf(g, xh, s2);
-        }
-        my_acc[(2 * j + h) * 32 + lane] = ag;
-        my_acc[(2 * NV + 2 * j + h) * 32 + lane] = ab;
-      }
-    }
-    row_sum2<WPR>(s1, s2, s_part, slot, part, buf);
-    s1 = rms ? 0.f : s1 * (1.f / D);
-    s2 *= (1.f / D);
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      const __nv_bfloat16* xe = reinterpret_cast<const __nv_bfloat16*>(&xr[j]);
-      const __nv_bfloat16* ge = reinterpret_cast<const __nv_bfloat16*>(&gr[j]);
-      const __nv_bfloat16* ye = reinterpret_cast<const __nv_bfloat16*>(&yr[j]);
-      const int c0 = ((part * NV + j) * 32 + lane) * 8;
-      float o[8];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float4 gm = *reinterpret_cast<const float4*>(s_gamma + c0 + 4 * h);
-        const float gmv[4] = {gm.x, gm.y, gm.z, gm.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float xh = (__bfloat162float(xe[4 * h + i]) - mean) * rstd;
-          const float g = __bfloat162float(ge[4 * h + i]) * gmv[i];
-          const float dx = rstd * (g - s1 - xh * s2);
-          o[4 * h + i] = dY ? __bfloat162float(ye[4 * h + i]) + dx : dx;
-        }
-      }
-      store16(dX + vec_off(j, r), o);
-    }
-#pragma unroll
-    for (int j = 0; j < NV; ++j) { xr[j] = xn[j]; gr[j] = gn[j]; }
-    st = stn;
-    r = rn;
-  }
-  __syncthreads();
-  // this block's token-axis partial sums: the RPB warps that share a column range are added, and the row goes to
-  // row blockIdx.x of partials[blocks][2][D]; a second kernel adds the rows
-  float* mine = partials + (int64_t)blockIdx.x * 2 * D;
-  const float* accf = reinterpret_cast<const float*>(s_acc);
-  for (int c = threadIdx.x; c < D; c += 256) {
-    const int v = c / 8, i = c % 8, ln = v % 32, pj = v / 32, pt = pj / NV, j = pj % NV;
-    float sg = 0.f, sb = 0.f;
-#pragma unroll
-    for (int sl = 0; sl < RPB; ++sl) {
-      const float* w = accf + (size_t)(sl * WPR + pt) * SMEM::ACC_F4_PER_WARP * 4;
-      sg += w[((2 * j + i / 4) * 32 + ln) * 4 + i % 4];
-      sb += w[((2 * NV + 2 * j + i / 4) * 32 + ln) * 4 + i % 4];
-    }
-    mine[c] = sg;
-    if (!rms) mine[D + c] = sb;
-  }
-}
-
-
 // dgamma[c] (y = 0) or dbeta[c] (y = 1) = sum over the first kernel's blocks of their partial rows.  Blocks with
 // y >= ny_norm finish the bias column sums instead (matrix y - ny_norm: the tree over its slab partials), so that
 // the step's two small final reductions share one launch.
 __global__ void __launch_bounds__(256) norm_bwd_reduce_kernel(const float* __restrict__ part, int blocks, int d,
                                                               float* __restrict__ dgamma, float* __restrict__ dbeta,
-                                                              int ny_norm, ColsumGroup G, const float* __restrict__ cpart,
+                                                              int ny_norm, const __grid_constant__ ColsumGroup G, const float* __restrict__ cpart,
                                                               int n_slabs) {
   __shared__ float red[8][33];
   pdl_launch_dependents();
@@ -640,74 +592,68 @@ __global__ void __launch_bounds__(256) norm_bwd_reduce_kernel(const float* __res
   }
 }
 
-template <int NV, int WPR>
-void norm_fwd_rows_launch(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
-                          float* stats, int rms, int32_t* status, cudaStream_t st) {
-  const int blocks = (int)min((int64_t)p->sm_count * 2, p->n_pad / (8 / WPR));
-  launch_pdl(norm_fwd_rows_kernel<NV, WPR>, dim3(blocks), dim3(256), 0, st, (const __nv_bfloat16*)X, gamma,
-             rms ? (const float*)nullptr : beta, (__nv_bfloat16*)Xn, stats, p->n_pad, p->d.seq, p->t_pad, rms, p->d.eps, status);
-}
-template <int NV, int WPR>
-void norm_bwd_rows_launch(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
-                          const float* gamma, void* dX, float* dgamma, float* dbeta, float* part, int rms,
-                          const ColsumGroup& cg, const float* cpart, int n_slabs, cudaStream_t st) {
-  const int blocks = (int)min((int64_t)p->sm_count * 2, p->n_pad / (8 / WPR));
-  int cs_panels = 0;
-  for (int i = 0; i < cg.count; ++i) cs_panels = cg.cols[i] / 64 > cs_panels ? cg.cols[i] / 64 : cs_panels;
-  const int cs_blocks = cs_panels * n_slabs * cg.count;
-  constexpr size_t smem = NormBwdSmem<NV, WPR>::BYTES;
-  cudaFuncSetAttribute(norm_bwd_rows_kernel<NV, WPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  launch_pdl(norm_bwd_rows_kernel<NV, WPR>, dim3(blocks + cs_blocks), dim3(256), smem, st, (const __nv_bfloat16*)dXn,
-             (const __nv_bfloat16*)X, (const __nv_bfloat16*)dY, stats, gamma, (__nv_bfloat16*)dX, part, p->n_pad, rms,
-             blocks, cg, const_cast<float*>(cpart), cs_panels, n_slabs);
-  const int ny = rms ? 1 : 2;
-  launch_pdl(norm_bwd_reduce_kernel, dim3((p->d.d_model + 31) / 32, ny + cg.count), dim3(256), 0, st, (const float*)part,
-             blocks, p->d.d_model, dgamma, dbeta, ny, cg, cpart, n_slabs);
-}
-
-// d_model -> (vectors per lane, warps per row) of the register-resident kernels; false if there is none.  At most
-// three vectors per lane: the backward keeps five values per column in registers, and two blocks should fit an SM.
-bool norm_rows_shape(int d, int* nv, int* wpr) {
-  if (d % 256 != 0) return false;
-  switch (d / 256) {
-    case 1: *nv = 1; *wpr = 1; return true;
-    case 2: *nv = 2; *wpr = 1; return true;
-    case 3: *nv = 3; *wpr = 1; return true;
-    case 4: *nv = 2; *wpr = 2; return true;
-    case 6: *nv = 3; *wpr = 2; return true;
-    case 8: *nv = 2; *wpr = 4; return true;
-    case 12: *nv = 3; *wpr = 4; return true;
-    case 16: *nv = 2; *wpr = 8; return true;
-    default: return false;
-  }
-}
-
-#define FBL_NORM_DISPATCH(CALL)                                        \
-  do {                                                                 \
-    if (wpr == 1) {                                                    \
-      if (nv == 1) CALL(1, 1); else if (nv == 2) CALL(2, 1); else CALL(3, 1); \
-    } else if (wpr == 2) {                                             \
-      if (nv == 2) CALL(2, 2); else CALL(3, 2);                        \
-    } else if (wpr == 4) {                                             \
-      if (nv == 2) CALL(2, 4); else CALL(3, 4);                        \
-    } else {                                                           \
-      CALL(2, 8);                                                      \
-    }                                                                  \
-  } while (0)
-
-// ------------------------------------------------------------------------------------------
-// Token-axis column sums, two stages over tiles: (1) one block per (panel, slab of 256 rows)
-// reduces its 32 storage tiles to one row of partials, (2) a tree over slabs.
-// ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) colsum_stage1(ColsumGroup G, int64_t rows, float* __restrict__ part_base) {
-  __shared__ float red[32][tile_w_of<T>::value + 1];
+__global__ void __launch_bounds__(256) colsum_stage1(const __grid_constant__ ColsumGroup G, int64_t rows, float* __restrict__ part_base) {
+  __shared__ float red[8][tile_w_of<T>::value + 1];
   pdl_launch_dependents();
   pdl_wait();
   colsum_slab<T>(G, rows, part_base, blockIdx.x, blockIdx.y, blockIdx.z, red);
 }
 
-__global__ void colsum_stage2(ColsumGroup G, const float* __restrict__ part_base, int n_slabs) {
+template <typename T, int NV, int PF, int TPR>
+cudaError_t norm_fwd_launch(const fbl_plan* p, const NormShape& s, const void* X, const float* gamma, const float* beta,
+                            void* Xn, float* stats, int32_t* status, cudaStream_t st) {
+  const int64_t blocks = min((int64_t)p->sm_count * (NV == 1 ? 4 : 2), (p->n_pad + s.groups - 1) / s.groups);
+  const int64_t per_block = ((p->n_pad + blocks - 1) / blocks + s.groups - 1) / s.groups * s.groups;
+  return launch_pdl(norm_fwd_kernel<T, NV, PF, TPR>, dim3((unsigned)((p->n_pad + per_block - 1) / per_block)), dim3(s.tpr * s.groups), 0, st,
+                    (const T*)X, gamma, beta, (T*)Xn, stats, p->n_pad, p->d.d_model, s.tpr, per_block, p->d.seq, p->t_pad,
+                    (int)(p->d.norm == FBL_NORM_RMSNORM), p->d.eps, status);
+}
+
+template <typename T, int NV, int R>
+cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* dXn, const void* X, const void* dY,
+                            const float* stats, const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
+                            const ColsumGroup& cg, float* cpart, int n_slabs, cudaStream_t st) {
+  constexpr int V = Vec16<T>::N;
+  const int d = p->d.d_model, rms = p->d.norm == FBL_NORM_RMSNORM;
+  const int64_t pass = (int64_t)s.groups * R;
+  // at most two blocks per SM: the partial-sum area holds that many rows, and the second kernel adds them all
+  const int64_t most = min((int64_t)p->sm_count * 2, (p->n_pad + pass - 1) / pass);
+  const int64_t per_block = ((p->n_pad + most - 1) / most + pass - 1) / pass * pass;
+  const int blocks = (int)((p->n_pad + per_block - 1) / per_block);
+  const size_t ring = (size_t)norm_stages(R, NV) * (dY ? 3 : 2) * R * NV * s.tpr * s.groups * 16;
+  int cs_panels = 0;
+  for (int i = 0; i < cg.count; ++i) cs_panels = cg.cols[i] / tile_w_of<T>::value > cs_panels ? cg.cols[i] / tile_w_of<T>::value : cs_panels;
+  // The column sums' first stage shares this launch while it is a few blocks for each that fits an SM beside the ring's
+  // shared memory, which those blocks occupy without using it; beyond that a launch of its own is cheaper (91 us
+  // together, 40 us apart for four 2977 x 2880 matrices; 4 us dearer apart for a 2048 x 768 and a 2048 x 3072 one).
+  int cs_blocks = cs_panels * n_slabs * cg.count;
+  if (cs_blocks > (ring <= 56 * 1024 ? 8 : 4) * p->sm_count) {
+    cudaError_t ce = launch_pdl(colsum_stage1<T>, dim3(cs_panels, n_slabs, cg.count), dim3(256), 0, st, cg, p->n_pad, cpart);
+    if (ce != cudaSuccess) return ce;
+    p->launches++;
+    cs_blocks = 0;
+  }
+  const size_t sums = (size_t)s.groups * 2 * s.tpr * NV * V * sizeof(float), smem = ring > sums ? ring : sums;
+  cudaError_t e = cudaSuccess;
+  if (smem > 40 * 1024) e = cudaFuncSetAttribute(norm_bwd_kernel<T, NV, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(norm_bwd_kernel<T, NV, R>, dim3(blocks + cs_blocks), dim3(s.tpr * s.groups), smem, st,
+                             (const T*)dXn, (const T*)X, (const T*)dY, stats, gamma, (T*)dX, dgamma ? part : (float*)nullptr, p->n_pad,
+                             d, s.tpr, per_block, rms, blocks, cg, cpart, cs_panels, n_slabs);
+  if (e != cudaSuccess) return e;
+  const int ny = !dgamma ? 0 : rms ? 1 : 2;
+  p->launches += ny + cg.count == 0 ? 1 : 2;
+  if (ny + cg.count == 0) return cudaSuccess;
+  return launch_pdl(norm_bwd_reduce_kernel, dim3((d + 31) / 32, ny + cg.count), dim3(256), 0, st, (const float*)part,
+                    blocks, d, dgamma, dbeta, ny, cg, (const float*)cpart, n_slabs);
+}
+
+// ------------------------------------------------------------------------------------------
+// Token-axis column sums, two stages over tiles: (1) one block per (panel, slab of 256 rows)
+// reduces its 32 storage tiles to one row of partials, (2) a tree over slabs.
+// ------------------------------------------------------------------------------------------
+__global__ void colsum_stage2(const __grid_constant__ ColsumGroup G, const float* __restrict__ part_base, int n_slabs) {
   pdl_launch_dependents();
   pdl_wait();
   const int which = blockIdx.y;
@@ -752,94 +698,67 @@ cudaError_t launch_rope(const fbl_plan* p, void* A, int heads_a, void* B, int he
                     (__nv_bfloat16*)B, heads_b, p->n_pad, p->d.seq, p->t_pad, hd, k, inverse ? -1.f : 1.f);
 }
 
-bool norm_fwd_resets_status(const fbl_plan* p) {
-  int nv, wpr;
-  return p->d.dtype == FBL_DTYPE_BF16 && norm_rows_shape(p->d.d_model, &nv, &wpr);
+template <typename T>
+cudaError_t norm_fwd_dispatch(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
+                              float* stats, int32_t* status, cudaStream_t st) {
+  const NormShape s = norm_fwd_shape(p->d.d_model / Vec16<T>::N);
+#define FBL_CALL(NV_, PF_, TPR_) norm_fwd_launch<T, NV_, PF_, TPR_>(p, s, X, gamma, beta, Xn, stats, status, st)
+  switch (s.nv) {
+    case 1: return s.tpr == 32 ? FBL_CALL(1, 4, 32) : FBL_CALL(1, 4, 0);
+    case 2:
+      return s.tpr == 32 ? FBL_CALL(2, 4, 32) : s.tpr == 64 ? FBL_CALL(2, 4, 64) : s.tpr == 128 ? FBL_CALL(2, 4, 128)
+                         : s.tpr == 256 ? FBL_CALL(2, 4, 256) : FBL_CALL(2, 4, 0);
+    case 3: return s.tpr == 32 ? FBL_CALL(3, 3, 32) : FBL_CALL(3, 3, 0);
+    case 4: return sizeof(T) == 4 ? FBL_CALL(4, 2, 0) : FBL_CALL(4, 1, 0);
+  }
+  if constexpr (sizeof(T) == 4) return FBL_CALL(8, 1, 0);
+  return cudaErrorInvalidValue;                // bf16: d_model <= 16384 needs at most four vectors
+#undef FBL_CALL
 }
 
 cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
                             float* stats, int32_t* status, cudaStream_t st) {
-  const int blocks = (int)((p->n_pad + 31) / 32);
-  const int rms = p->d.norm == FBL_NORM_RMSNORM;
-  int nv, wpr;
-  if (p->d.dtype == FBL_DTYPE_BF16 && norm_rows_shape(p->d.d_model, &nv, &wpr)) {
-#define FBL_CALL(NV_, WPR_) norm_fwd_rows_launch<NV_, WPR_>(p, X, gamma, beta, Xn, stats, rms, status, st)
-    FBL_NORM_DISPATCH(FBL_CALL);
-#undef FBL_CALL
-    return cudaGetLastError();
+  if (p->d.norm == FBL_NORM_RMSNORM) beta = nullptr;
+  return p->d.dtype == FBL_DTYPE_FP32 ? norm_fwd_dispatch<float>(p, X, gamma, beta, Xn, stats, status, st)
+                                      : norm_fwd_dispatch<__nv_bfloat16>(p, X, gamma, beta, Xn, stats, status, st);
+}
+
+template <typename T>
+cudaError_t norm_bwd_dispatch(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
+                              const float* gamma, void* dX, float* dgamma, float* dbeta, float* npart,
+                              const ColsumGroup& cg, float* cpart, int n_slabs, cudaStream_t st) {
+  const NormShape s = norm_bwd_shape(p->d.d_model / Vec16<T>::N, p->n_pad, p->sm_count);
+#define FBL_CALL(NV_, R_) norm_bwd_launch<T, NV_, R_>(p, s, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, cpart, n_slabs, st)
+  switch (s.nv) {
+    case 1: return s.r == 4 ? FBL_CALL(1, 4) : s.r == 2 ? FBL_CALL(1, 2) : FBL_CALL(1, 1);
+    case 2: return s.r == 2 ? FBL_CALL(2, 2) : FBL_CALL(2, 1);
+    case 4: return FBL_CALL(4, 1);
   }
-  if (p->d.dtype == FBL_DTYPE_FP32)
-    norm_fwd_kernel<float><<<blocks, 256, 0, st>>>((const float*)X, gamma, rms ? nullptr : beta, (float*)Xn, stats,
-                                                   p->n_pad, p->d.d_model, p->d.seq, p->t_pad, rms, p->d.eps);
-  else
-    norm_fwd_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)X, gamma, rms ? nullptr : beta,
-                                                           (__nv_bfloat16*)Xn, stats, p->n_pad, p->d.d_model,
-                                                           p->d.seq, p->t_pad, rms, p->d.eps);
-  return cudaGetLastError();
+  if constexpr (sizeof(T) == 4) return FBL_CALL(8, 1);
+  return cudaErrorInvalidValue;                // bf16: d_model <= 16384 needs at most four vectors
+#undef FBL_CALL
 }
 
-// Norm backward, and with it (bias_count > 0, register-resident bf16 path only) the bias column sums of up to four
-// matrices: their first stage runs as extra blocks of the norm's rows kernel, their second stage inside the norm's
-// own second kernel.
-// `part` holds the column-sum slab partials first and the norm's per-block partial rows behind them.
-bool norm_bwd_takes_colsums(const fbl_plan* p) {
-  int nv, wpr;
-  return p->d.dtype == FBL_DTYPE_BF16 && norm_rows_shape(p->d.d_model, &nv, &wpr);
-}
-
+// Norm backward (dgamma = nullptr: only dX, the norm's parameters are frozen), and with it (bias_count > 0) the bias
+// column sums of up to four matrices: their first stage runs as extra blocks of the first kernel, their second stage
+// inside the second.  `part` holds the column-sum slab partials first and the norm's per-block partial rows behind them.
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                             const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
                             cudaStream_t st, int bias_count, const void* const* bias_m, const int* bias_cols,
                             float* const* bias_out) {
-  const int blocks = (int)((p->n_pad + 31) / 32);
-  const int d = p->d.d_model;
-  const int rms = p->d.norm == FBL_NORM_RMSNORM;
-  const size_t sh = 2 * (size_t)d * sizeof(float);
-  int nv, wpr;
-  if (p->d.dtype == FBL_DTYPE_BF16 && norm_rows_shape(d, &nv, &wpr)) {
-    ColsumGroup cg;
-    memset(&cg, 0, sizeof(cg));
-    const int n_slabs = (int)((p->n_pad + COLSUM_SLAB - 1) / COLSUM_SLAB);
-    float* npart = part;
-    if (bias_count > 0) {
-      if (bias_count > 4) return cudaErrorInvalidValue;
-      int max_cols = 0;
-      int64_t off = 0;
-      for (int i = 0; i < bias_count; ++i) {
-        cg.m[i] = bias_m[i]; cg.out[i] = bias_out[i]; cg.cols[i] = bias_cols[i]; cg.part_off[i] = off;
-        off += (int64_t)n_slabs * bias_cols[i];
-        max_cols = bias_cols[i] > max_cols ? bias_cols[i] : max_cols;
-      }
-      cg.count = bias_count;                // their first stage rides in the rows kernel's launch, as extra blocks
-      (void)max_cols;
-      npart = part + (off + 255) / 256 * 256;
-    }
-    // token-axis sums in two steps over `npart` (no atomics: the result does not depend on block order)
-#define FBL_CALL(NV_, WPR_) norm_bwd_rows_launch<NV_, WPR_>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, rms, cg, part, n_slabs, st)
-    FBL_NORM_DISPATCH(FBL_CALL);
-#undef FBL_CALL
-    return cudaGetLastError();
+  ColsumGroup cg;
+  memset(&cg, 0, sizeof(cg));
+  const int n_slabs = (int)((p->n_pad + COLSUM_SLAB - 1) / COLSUM_SLAB);
+  if (bias_count > 4) return cudaErrorInvalidValue;
+  int64_t off = 0;
+  for (int i = 0; i < bias_count; ++i) {
+    cg.m[i] = bias_m[i]; cg.out[i] = bias_out[i]; cg.cols[i] = bias_cols[i]; cg.part_off[i] = off;
+    off += (int64_t)n_slabs * bias_cols[i];
   }
-  if (bias_count > 0) return cudaErrorInvalidValue;      // callers ask norm_bwd_takes_colsums first
-  cudaError_t e = cudaMemsetAsync(dgamma, 0, d * sizeof(float), st);
-  if (e != cudaSuccess) return e;
-  if (dbeta) {
-    e = cudaMemsetAsync(dbeta, 0, d * sizeof(float), st);
-    if (e != cudaSuccess) return e;
-  }
-  if (p->d.dtype == FBL_DTYPE_FP32) {
-    auto k = norm_bwd_kernel<float>;
-    if (sh > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-    k<<<blocks, 256, sh, st>>>((const float*)dXn, (const float*)X, (const float*)dY, stats, gamma, (float*)dX, dgamma,
-                               rms ? nullptr : dbeta, p->n_pad, d, rms);
-  } else {
-    using B = __nv_bfloat16;
-    auto k = norm_bwd_kernel<B>;
-    if (sh > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-    k<<<blocks, 256, sh, st>>>((const B*)dXn, (const B*)X, (const B*)dY, stats, gamma, (B*)dX, dgamma,
-                               rms ? nullptr : dbeta, p->n_pad, d, rms);
-  }
-  return cudaGetLastError();
+  cg.count = bias_count;
+  float* npart = part + (off + 255) / 256 * 256;
+  if (p->d.dtype == FBL_DTYPE_FP32) return norm_bwd_dispatch<float>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, part, n_slabs, st);
+  return norm_bwd_dispatch<__nv_bfloat16>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, part, n_slabs, st);
 }
 
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols) {

@@ -143,7 +143,6 @@ int fbl_layer_fwd_lora(const fbl_plan* p, const void* X, const float* gamma, con
   const int n = (int)p->n_pad, D = p->d.d_model;
   int k = 0;
 
-  if (!norm_fwd_resets_status(p)) LORA_CUDA(cudaMemsetAsync(status, 0, FBL_ALIGN, st));
   if (p->prof_on) { p->prof_n = 0; LORA_CUDA(cudaEventRecord(p->prof_ev[0], st)); }
   LORA_STEP("norm_fwd", 1, launch_norm_fwd(p, X, gamma, beta, Xn, stats, status, st));
   {
@@ -214,9 +213,11 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
   void* dA = sc + p->sb_da; float* dvec = (float*)(sc + p->sb_dvec); float* dqacc = (float*)(sc + p->sb_dqacc);
   void* dQ = sc + p->sb_dq; void* dK = sc + p->sb_dk; void* dV = sc + p->sb_dv; void* dXn = sc + p->sb_dxn;
   void* dT = sc + p->sb_dt; float* part = (float*)(sc + p->sb_part);
-  float* frozen = (float*)(sc + p->sb_frozen);                 // where the unused gradients of a frozen norm go
-  if (!dgamma) dgamma = frozen;
-  if (!dbeta) dbeta = frozen + p->d.d_model;
+  if (dgamma || dbeta) {                                       // one of the two asked for: the other goes to a spare place
+    float* frozen = (float*)(sc + p->sb_frozen);
+    if (!dgamma) dgamma = frozen;
+    if (!dbeta) dbeta = frozen + p->d.d_model;
+  }
   const int n = (int)p->n_pad, D = p->d.d_model;
   const int cols[3] = {p->dq, p->dkv, p->dkv};
   int k = 0;
@@ -277,7 +278,7 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     LORA_STEP("dB+dXn+dA", 0, cudaSuccess);
     p->launches += k;
   }
-  LORA_STEP("norm_bwd", norm_bwd_takes_colsums(p) ? 2 : 1, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st));
+  LORA_STEP("norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st));
   return FBL_OK;
 }
 

@@ -242,7 +242,7 @@ int fbl_mlp_set_kernel_path(fbl_mlp_plan* plan, int path) {
   if (!plan) return FBL_ERR_INVALID_ARG;
   return fbl_plan_set_kernel_path(plan->base, path);
 }
-int64_t fbl_mlp_launch_count(const fbl_mlp_plan* plan) { return plan ? plan->launches : -1; }
+int64_t fbl_mlp_launch_count(const fbl_mlp_plan* plan) { return plan ? plan->launches + plan->base->launches : -1; }
 
 int fbl_mlp_tensor_bytes(const fbl_mlp_plan* plan, int matrix_id, size_t* bytes) {
   int64_t outer, rows, rows_pad; int cols;
@@ -314,7 +314,6 @@ int fbl_mlp_fwd(const fbl_mlp_plan* p, const void* X, const float* gamma, const 
   void* Xn = sv + p->sv_xn; void* U = sv + p->sv_u; void* G = sv + p->sv_g; void* H = sv + p->sv_h;
   const int n = (int)p->n_pad, D = p->d.d_model, F = p->d.d_ff;
 
-  if (!norm_fwd_resets_status(bp)) MLP_CUDA(cudaMemsetAsync(status, 0, FBL_ALIGN, st));
   MLP_STEP(1, launch_norm_fwd(bp, X, gamma, beta, Xn, stats, status, st));
   {
     GemmArgs gs[2];
@@ -455,17 +454,12 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
     p->launches += k;
   }
   if (cg.count > 0) MLP_STEP(1, launch_convert_f32_group(cg, st));
-  // bias gradients: token-axis column sums of dY, dU (and dG), sharing the norm backward's launches where they can
+  // bias gradients: token-axis column sums of dY, dU (and dG), riding in the norm backward's launches
   const void* M3[3] = {dY, dU, dG};
   float* O3[3] = {db2, db1, dbg};
   const int C3[3] = {D, F, F};
   const int nb = gated ? 3 : 2;
-  if (bias && norm_bwd_takes_colsums(bp)) {
-    MLP_STEP(2, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st, nb, M3, C3, O3));
-    return FBL_OK;
-  }
-  if (bias) MLP_STEP(2, launch_colsum_group(p->d.dtype, nb, M3, p->n_pad, C3, O3, part, st));
-  MLP_STEP(norm_bwd_takes_colsums(bp) ? 2 : 1, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st));
+  MLP_STEP(0, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st, bias ? nb : 0, M3, C3, O3));
   return FBL_OK;
 }
 

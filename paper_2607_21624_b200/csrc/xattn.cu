@@ -59,7 +59,6 @@ int fbl_xattn_fwd(const fbl_plan* p, const void* X, const void* M, const float* 
   const bool bias = p->d.has_bias;
   const int n = (int)p->n_pad, nk = (int)p->n_pad_kv, D = p->d.d_model, Dm = p->d_mem;
 
-  if (!norm_fwd_resets_status(p)) XA_CUDA(cudaMemsetAsync(status, 0, FBL_ALIGN, st));
   XA_PROF_BEGIN();
   XA_STEP("norm_fwd", 1, launch_norm_fwd(p, X, gamma, beta, Xn, stats, status, st));
   {
@@ -238,12 +237,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
   float* Ok[2] = {dbk, dbv};
   const int Ck[2] = {p->dkv, p->dkv};
   if (bias) XA_STEP("db_kv", 2, launch_colsum_group(p->d.dtype, 2, Mk, p->n_pad_kv, Ck, Ok, part_kv, st));
-  if (bias && norm_bwd_takes_colsums(p)) {
-    XA_STEP("db+norm_bwd", 2, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st, 2, Mq, Cq, Oq));
-    return FBL_OK;
-  }
-  if (bias) XA_STEP("db", 2, launch_colsum_group(p->d.dtype, 2, Mq, p->n_pad, Cq, Oq, part, st));
-  XA_STEP("norm_bwd", norm_bwd_takes_colsums(p) ? 2 : 1, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st));
+  XA_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st, bias ? 2 : 0, Mq, Cq, Oq));
   return FBL_OK;
 }
 

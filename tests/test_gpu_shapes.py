@@ -30,3 +30,18 @@ def check(cfg):
 ], ids=lambda c: c.name)
 def test_tensor_core_kernels_on_partly_filled_tiles(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # row widths of the norm kernels: part of a warp, a ragged last warp, several warps, more than one vector per thread
+    # (fp32 above 2048 columns, bf16 above 4096); one, two and four rows per pass, with a short last block
+    LayerConfig("nw1", 1, 9, 64, 1, 1, 64, "bf16", "layernorm", False, True, True, 1e-5, 211, 0.05),
+    LayerConfig("nw2", 2, 613, 192, 2, 1, 64, "bf16", "rmsnorm", True, True, False, 1e-5, 212, 0.05),
+    LayerConfig("nw3", 3, 401, 320, 2, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 213, 0.05),
+    LayerConfig("nw4", 1, 70, 4160, 1, 1, 64, "bf16", "layernorm", False, False, True, 1e-5, 214, 0.02),
+    LayerConfig("nw5", 2, 45, 96, 1, 1, 32, "fp32", "layernorm", True, True, True, 1e-5, 215, 0.1),
+    LayerConfig("nw6", 1, 700, 160, 1, 1, 32, "fp32", "rmsnorm", False, True, False, 1e-5, 216, 0.1),
+    LayerConfig("nw7", 1, 20, 2080, 1, 1, 32, "fp32", "layernorm", False, False, False, 1e-5, 217, 0.02),
+], ids=lambda c: c.name)
+def test_norm_row_widths(cfg):
+    check(cfg)
