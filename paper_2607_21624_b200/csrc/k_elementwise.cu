@@ -30,33 +30,36 @@ __device__ __forceinline__ void store16(T* p, const float (&v)[Vec16<T>::N]) {
 // ------------------------------------------------------------------------------------------
 // pack / unpack: the only layout conversions, used at the graph boundary.
 // ------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void pack_kernel(const T* __restrict__ src, T* __restrict__ dst, int64_t outer, int64_t rows,
-                            int64_t rows_pad, int cols, int64_t total) {
-  constexpr int TW = tile_w_of<T>::value;
-  const int64_t r_pad = outer * rows_pad;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t panel = i / (r_pad * TW);
-    int64_t rem = i - panel * r_pad * TW;
-    int64_t r = rem / TW;
-    int c = (int)(panel * TW + rem % TW);
-    int64_t o = r / rows_pad, row = r - o * rows_pad;
-    T v = from_f<T>(0.f);
-    if (row < rows) v = src[(o * rows + row) * cols + c];
-    dst[i] = v;
-  }
-}
-
-template <typename T>
-__global__ void unpack_kernel(const T* __restrict__ src, T* __restrict__ dst, int64_t outer, int64_t rows,
-                              int64_t rows_pad, int cols, int64_t total) {
-  constexpr int TW = tile_w_of<T>::value;
-  const int64_t r_pad = outer * rows_pad;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t orow = i / cols;
-    int c = (int)(i - orow * cols);
-    int64_t o = orow / rows, row = orow - o * rows;
-    dst[i] = src[rt_off<TW>(r_pad, o * rows_pad + row, c)];
+// A block converts PACK_UNITS / (units per row) whole padded rows, or one; a thread's accesses are PACK_UNITS / 256 units
+// in flight.  A unit is 16 bytes (eight consecutive threads are one 128-byte tile row on the tiled side and 128 consecutive
+// bytes on the row-major side), or one element where the row-major pointer is not 16-byte aligned.  HBM-bound: two passes
+// of 3 MB take 2.4 us, where one element per thread and 64-bit divisions took 11 us.
+// (No early trigger for the kernel behind: it may request weights before it waits, and this may be what packs them.)
+constexpr int PACK_UNITS = 1024;
+template <typename U, bool PACK>
+__global__ void __launch_bounds__(256) pack_kernel(const U* __restrict__ src, U* __restrict__ dst, uint32_t rows,
+                                                   uint32_t rows_pad, uint32_t r_pad, uint32_t units, uint32_t rows_per_block) {
+  constexpr uint32_t TU = 128 / sizeof(U);                   // units per tile row
+  const uint32_t r0 = blockIdx.x * rows_per_block, n = min(rows_per_block, r_pad - r0) * units;
+  pdl_wait();
+  for (uint32_t i0 = threadIdx.x; i0 < n; i0 += PACK_UNITS) {
+    U v[PACK_UNITS / 256];
+    int64_t to[PACK_UNITS / 256];
+#pragma unroll
+    for (int k = 0; k < PACK_UNITS / 256; ++k) {
+      const uint32_t i = i0 + k * 256;
+      to[k] = -1;
+      if (i >= n) continue;
+      const uint32_t r = r0 + i / units, u = i % units, o = r / rows_pad, row = r - o * rows_pad;
+      const int64_t tiled = ((int64_t)(u / TU) * r_pad + r) * TU + u % TU, flat = ((int64_t)o * rows + row) * units + u;
+      const bool live = row < rows;
+      v[k] = U{};
+      if (live) v[k] = src[PACK ? flat : tiled];
+      if (PACK || live) to[k] = PACK ? tiled : flat;
+    }
+#pragma unroll
+    for (int k = 0; k < PACK_UNITS / 256; ++k)
+      if (to[k] >= 0) dst[to[k]] = v[k];
   }
 }
 
@@ -669,20 +672,24 @@ __global__ void colsum_stage2(const __grid_constant__ ColsumGroup G, const float
 
 }  // namespace
 
+template <typename U>
+static cudaError_t pack_launch(int unpack, const void* src, void* dst, int64_t outer, int64_t rows, int64_t rows_pad,
+                               int64_t row_bytes, cudaStream_t st) {
+  const uint32_t units = (uint32_t)(row_bytes / sizeof(U)), r_pad = (uint32_t)(outer * rows_pad);
+  const uint32_t per_block = units >= PACK_UNITS ? 1 : PACK_UNITS / units;
+  const dim3 grid((r_pad + per_block - 1) / per_block);
+  return unpack ? launch_pdl(pack_kernel<U, false>, grid, dim3(256), 0, st, (const U*)src, (U*)dst, (uint32_t)rows, (uint32_t)rows_pad, r_pad, units, per_block)
+                : launch_pdl(pack_kernel<U, true>, grid, dim3(256), 0, st, (const U*)src, (U*)dst, (uint32_t)rows, (uint32_t)rows_pad, r_pad, units, per_block);
+}
+
 cudaError_t launch_pack(int dtype, int unpack, const void* src, void* dst, int64_t outer, int64_t rows,
                         int64_t rows_pad, int cols, cudaStream_t st) {
-  const int64_t total = unpack ? outer * rows * cols : outer * rows_pad * cols;
-  if (total == 0) return cudaSuccess;
-  const int blocks = (int)min((int64_t)148 * 16, (total + 255) / 256);
-  if (dtype == FBL_DTYPE_FP32) {
-    if (unpack) unpack_kernel<float><<<blocks, 256, 0, st>>>((const float*)src, (float*)dst, outer, rows, rows_pad, cols, total);
-    else pack_kernel<float><<<blocks, 256, 0, st>>>((const float*)src, (float*)dst, outer, rows, rows_pad, cols, total);
-  } else {
-    using B = __nv_bfloat16;
-    if (unpack) unpack_kernel<B><<<blocks, 256, 0, st>>>((const B*)src, (B*)dst, outer, rows, rows_pad, cols, total);
-    else pack_kernel<B><<<blocks, 256, 0, st>>>((const B*)src, (B*)dst, outer, rows, rows_pad, cols, total);
-  }
-  return cudaGetLastError();
+  if (outer * rows * cols == 0) return cudaSuccess;
+  const int64_t row_bytes = (int64_t)cols * (dtype == FBL_DTYPE_FP32 ? 4 : 2);
+  if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0)
+    return pack_launch<uint4>(unpack, src, dst, outer, rows, rows_pad, row_bytes, st);
+  if (dtype == FBL_DTYPE_FP32) return pack_launch<uint32_t>(unpack, src, dst, outer, rows, rows_pad, row_bytes, st);
+  return pack_launch<uint16_t>(unpack, src, dst, outer, rows, rows_pad, row_bytes, st);
 }
 
 cudaError_t launch_rope(const fbl_plan* p, void* A, int heads_a, void* B, int heads_b, int inverse, cudaStream_t st) {

@@ -45,3 +45,24 @@ def test_tensor_core_kernels_on_partly_filled_tiles(cfg):
 ], ids=lambda c: c.name)
 def test_norm_row_widths(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("offset", [0, 1], ids=["aligned", "element-aligned"])
+@pytest.mark.parametrize("b,t,d,dtype", [(1, 1, 64, "bf16"), (3, 13, 192, "bf16"), (2, 37, 96, "fp32"), (1, 9, 16384, "bf16"), (5, 130, 64, "fp32")])
+def test_pack_and_unpack(b, t, d, dtype, offset):
+    import torch
+    from paper_2607_21624_b200 import LayerRunner
+    from paper_2607_21624_b200.binding import TENSOR
+    w = 64 if dtype == "bf16" else 32
+    run = LayerRunner(LayerConfig("pk", b, t, d, 1, 1, w, dtype, "layernorm", True, False, False, 1e-5, 0, 0.02), guard_bytes=4096)
+    n, stream, t_pad = b * t * d, torch.cuda.current_stream().cuda_stream, (t + 7) // 8 * 8
+    src = torch.randn(n + 1, device="cuda").to(run.tdtype)[offset:offset + n]
+    run.buf["X"].fill_(255)
+    run.plan.pack(TENSOR["X"], src.data_ptr(), run.buf["X"].data_ptr(), stream)
+    tiled = run.buf["X"].view(run.tdtype).view(d // w, b, t_pad, w)
+    want = src.view(b, t, d // w, w).permute(2, 0, 1, 3)
+    assert torch.equal(tiled[:, :, :t], want) and not tiled[:, :, t:].any()
+    back = torch.full((n + 2,), 7.0, device="cuda").to(run.tdtype)
+    run.plan.unpack(TENSOR["X"], run.buf["X"].data_ptr(), back[offset:].data_ptr(), stream)
+    assert torch.equal(back[offset:offset + n], src) and (back[offset + n:] == 7).all() and (back[:offset] == 7).all()
+    assert run.guards_intact() == []
