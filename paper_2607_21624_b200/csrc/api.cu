@@ -62,16 +62,19 @@ thread_local char g_detail[256] = "";
     }                                                              \
   } while (0)
 
+// A group of GEMM problems as one step; run_gemm_group says how many kernels it took.
+#define FBL_GEMM_STEP(name, gs, count, launch_id)                               \
+  do {                                                                          \
+    int k__ = 0;                                                                \
+    FBL_CUDA(run_gemm_group(p, gs, count, status, st, launch_id, &k__));        \
+    FBL_STEP(name, k__, cudaSuccess);                                           \
+  } while (0)
+
 #define FBL_PROF_BEGIN()                                           \
   do {                                                             \
     const fbl_plan* mp__ = p;                                      \
     if (mp__->prof_on) { mp__->prof_n = 0; FBL_CUDA(cudaEventRecord(mp__->prof_ev[0], st)); } \
   } while (0)
-
-cudaError_t run_gemm(const fbl_plan* p, const GemmArgs& g, int32_t* status, cudaStream_t st, int launch_id = -1) {
-  if (p->use_tc && gemm_tc_supported(p, g)) return launch_gemm_tc_group(p, &g, 1, status, st, launch_id);
-  return launch_gemm_simt(p->d.dtype, g, st);
-}
 
 }  // namespace
 
@@ -431,7 +434,6 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
     const float* B[3] = {bq, bk, bv};
     const int cols[3] = {p->dq, p->dkv, p->dkv};
     GemmArgs gs[3];
-    bool tc = p->use_tc != 0;
     for (int i = 0; i < 3; ++i) {
       GemmArgs& g = gs[i];
       g = GemmArgs{};
@@ -440,14 +442,8 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
       g.b_static = 1;
       g.c = O[i]; g.c_rpad = p->n_pad; g.bias = bias ? B[i] : nullptr;
       g.seq = p->d.seq; g.t_pad = p->t_pad;
-      tc = tc && gemm_tc_supported(p, g);
     }
-    if (tc) {
-      FBL_STEP("proj_qkv", 1, launch_gemm_tc_group(p, gs, 3, status, st, FBL_GEMM_PROJ_QKV));   // one launch, blockIdx.z picks Q, K or V
-    } else {
-      for (int i = 0; i < 3; ++i)
-        FBL_STEP(i == 0 ? "proj_q" : i == 1 ? "proj_k" : "proj_v", 1, launch_gemm_simt(p->d.dtype, gs[i], st));
-    }
+    FBL_GEMM_STEP("proj_qkv", gs, 3, FBL_GEMM_PROJ_QKV);
   }
   if (p->rope_base > 0.f) FBL_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
   if (p->use_tc && attn_fwd_tc_supported(p)) FBL_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
@@ -460,7 +456,7 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
     g.c = Y; g.c_rpad = p->n_pad; g.bias = bias ? bo : nullptr;
     g.residual = p->d.residual ? X : nullptr;
     g.seq = p->d.seq; g.t_pad = p->t_pad;
-    FBL_STEP("proj_o", 1, run_gemm(p, g, status, st, FBL_GEMM_PROJ_O));
+    FBL_GEMM_STEP("proj_o", &g, 1, FBL_GEMM_PROJ_O);
   }
   return FBL_OK;
 }
@@ -524,24 +520,23 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     ga.t[0] = {dY, p->n_pad, 0, Wo, p->dq, 1, D};
     ga.b_static = 1;
     ga.c = dA; ga.c_rpad = p->n_pad; ga.seq = p->d.seq; ga.t_pad = p->t_pad;
-    if (p->use_tc && gemm_tc_supported(p, gw) && gemm_tc_supported(p, ga)) {
-      // D = rowsum(dO * O) per head comes out of the dA epilogue, from the fp32 accumulator
+    if (gemm_fuses_dot(p, ga)) {
+      // D = rowsum(dO * O) per head comes out of the dA epilogue
       ga.dot_with = A; ga.dot_out = dvec; ga.dot_hd = p->d.head_dim; ga.dot_hq = p->d.n_q_heads;
       dvec_ready = true;
+    }
+    if (gemm_group_tc(p, gs, 2)) {
       if (split_o) { gw.ksplit = p->ksplit_o; gw.acc = (float*)(sc + p->sb_acc_o); }
       if (first_gemm_fills) {
         gs[0].zero_ptr = dqacc; gs[0].zero_bytes = p->zero_bytes - p->sb_dqacc;
         gs[0].reset_status = 1; gs[0].serial = 1;
       }
-      FBL_STEP("dWo+dA", 1, launch_gemm_tc_group(p, gs, 2, status, st, FBL_GEMM_DWO_DA));
       dwo_round = split_o;        // nothing in the step reads dWo: its rounding joins that of dWq, dWk, dWv below
-    } else {
-      FBL_STEP("dA", 1, run_gemm(p, ga, status, st));
-      FBL_STEP("dWo", 1, run_gemm(p, gw, status, st));
     }
+    FBL_GEMM_STEP("dWo+dA", gs, 2, FBL_GEMM_DWO_DA);
   }
   if (p->use_tc && attn_bwd_tc_supported(p)) FBL_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));   // dqacc: zero already
-  else FBL_STEP("attn_bwd", 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, st));
+  else FBL_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   // back through the rotation of Q and K: its transpose is the rotation by the opposite angle
   if (p->rope_base > 0.f) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   {
@@ -549,14 +544,12 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     void* DW[3] = {dWq, dWk, dWv};
     const int cols[3] = {p->dq, p->dkv, p->dkv};
     GemmArgs gs[4];
-    bool tc = p->use_tc != 0;
     for (int i = 0; i < 3; ++i) {   // dW* = Xn^T d* : token-axis reductions, Xn's tiles read MN-major
       GemmArgs& g = gs[i];
       g = GemmArgs{};
       g.m = D; g.n = cols[i]; g.n_terms = 1;
       g.t[0] = {Xn, p->n_pad, 1, G[i], p->n_pad, 0, n};
       g.c = DW[i]; g.c_rpad = D;
-      tc = tc && gemm_tc_supported(p, g);
     }
     GemmArgs& gx = gs[3];           // dXn = dQ Wq^T + dK Wk^T + dV Wv^T : one accumulator, three reduction loops
     gx = GemmArgs{};
@@ -566,9 +559,8 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     gx.t[1] = {dK, p->n_pad, 0, Wk, D, 1, p->dkv};
     gx.t[2] = {dV, p->n_pad, 0, Wv, D, 1, p->dkv};
     gx.c = dXn; gx.c_rpad = p->n_pad; gx.seq = p->d.seq; gx.t_pad = p->t_pad;
-    tc = tc && gemm_tc_supported(p, gx);
-    if (tc) {
-      ConvertGroup cg = {};
+    ConvertGroup cg = {};
+    if (gemm_group_tc(p, gs, 4)) {
       if (split_qkv) {
         float* acc = (float*)(sc + p->sb_acc_qkv);
         for (int i = 0; i < 3; ++i) {
@@ -583,13 +575,9 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
         cg.count++;
         dwo_round = false;
       }
-      FBL_STEP("dWqkv+dXn", 1, launch_gemm_tc_group(p, gs, 4, status, st, FBL_GEMM_DWQKV_DXN));
-      if (cg.count > 0) FBL_STEP("dW round", 1, launch_convert_f32_group(cg, st));     // one rounding launch for all sliced GEMMs
-    } else {
-      FBL_STEP("dXn", 1, run_gemm(p, gx, status, st));
-      for (int i = 0; i < 3; ++i)
-        FBL_STEP(i == 0 ? "dWq" : i == 1 ? "dWk" : "dWv", 1, run_gemm(p, gs[i], status, st));
     }
+    FBL_GEMM_STEP("dWqkv+dXn", gs, 4, FBL_GEMM_DWQKV_DXN);
+    if (cg.count > 0) FBL_STEP("dW round", 1, launch_convert_f32_group(cg, st));     // one rounding launch for all sliced GEMMs
   }
   if (dwo_round) {
     ConvertGroup cg = {};

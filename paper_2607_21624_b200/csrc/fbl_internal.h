@@ -112,10 +112,25 @@ struct GemmArgs {
   int epi; const void* aux1; void* c2;
 };
 
-cudaError_t launch_gemm_simt(int dtype, const GemmArgs& g, cudaStream_t st);
+cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
 bool gemm_tc_supported(const fbl_plan* p, const GemmArgs& g);
 cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st,
                                  int launch_id = -1);
+bool gemm_ffma_supported(const fbl_plan* p, const GemmArgs& g);
+cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st);
+// Every problem of the group can run on the tensor-core kernel and the plan wants it to.
+static inline bool gemm_group_tc(const fbl_plan* p, const GemmArgs* gs, int count) {
+  bool tc = p->use_tc != 0;
+  for (int i = 0; i < count; ++i) tc = tc && gemm_tc_supported(p, gs[i]);
+  return tc;
+}
+// One launch on the tensor-core kernel (bf16) or on the FFMA kernel (fp32), else one per problem on the plain FFMA kernel
+// (bf16 storage, the cross-check path).  *kernels: how many were enqueued.
+cudaError_t run_gemm_group(const fbl_plan* p, GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int launch_id, int* kernels);
+// The product that forms dA can form D = rowsum(dA * A) per head on the way.
+static inline bool gemm_fuses_dot(const fbl_plan* p, const GemmArgs& ga) {
+  return p->d.dtype == FBL_DTYPE_FP32 ? p->d.head_dim <= 64 && gemm_ffma_supported(p, ga) : p->use_tc && gemm_tc_supported(p, ga);
+}
 struct GemmShape { int64_t m; int n; int kblocks; int splittable; };
 int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count);
 cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles, cudaStream_t st);
@@ -143,7 +158,7 @@ cudaError_t launch_attn_fwd_simt(const fbl_plan* p, const void* Q, const void* K
                                  cudaStream_t st);
 cudaError_t launch_attn_bwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,
                                  const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
-                                 void* dV, cudaStream_t st);
+                                 void* dV, bool dvec_ready, cudaStream_t st);
 cudaError_t launch_attn_bwd_pre(const fbl_plan* p, const void* A, const void* dA, float* dvec, float* dqacc,
                                 bool dvec_ready, cudaStream_t st);
 struct ConvertGroup { const float* src[4]; void* dst[4]; int64_t n[4]; int count; };

@@ -8,7 +8,8 @@
 namespace {
 
 // ------------------------------------------------------------------------------------------
-// GEMM: C[m,n] = sum_terms A_t[m,:] . B_t[:,n] (+ bias[n]) (+ residual), 64x64 tile per block.
+// GEMM: C[m,n] = sum_terms A_t[m,:] . B_t[:,n] (+ bias[n]) (+ residual), 64x64 tile per block (bf16 storage only: the
+// cross-check of the tensor-core kernels; fp32 storage has a kernel of its own).
 // ------------------------------------------------------------------------------------------
 constexpr int GB = 64, GK = 16;
 
@@ -418,10 +419,9 @@ cudaError_t attn_bwd_launch(const fbl_plan* p, const void* Q, const void* K, con
 
 }  // namespace
 
-cudaError_t launch_gemm_simt(int dtype, const GemmArgs& g, cudaStream_t st) {
+cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {
   dim3 grid((g.n + GB - 1) / GB, (g.m + GB - 1) / GB);
-  if (dtype == FBL_DTYPE_FP32) gemm_simt_kernel<float><<<grid, 256, 0, st>>>(g);
-  else gemm_simt_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g);
+  gemm_simt_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g);
   return cudaGetLastError();
 }
 
@@ -471,9 +471,9 @@ cudaError_t launch_convert_f32_group(const ConvertGroup& g, cudaStream_t st) {
 
 cudaError_t launch_attn_bwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,
                                  const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
-                                 void* dV, cudaStream_t st) {
+                                 void* dV, bool dvec_ready, cudaStream_t st) {
   const int hd = p->d.head_dim;
-  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, false, st);
+  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, dvec_ready, st);
   if (e != cudaSuccess) return e;
   e = cudaErrorInvalidValue;
   if (p->d.dtype == FBL_DTYPE_FP32) {

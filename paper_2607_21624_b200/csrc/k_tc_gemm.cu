@@ -801,16 +801,24 @@ cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles
   return cudaGetLastError();
 }
 
-bool fbl_encode_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels) {
+static bool encode_panels(CUtensorMap* map, CUtensorMapDataType type, int width, const void* base, int64_t r_pad, int panels,
+                          int box_rows, int box_panels) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[3] = {64, (cuuint64_t)r_pad, (cuuint64_t)panels};
+  cuuint64_t dims[3] = {(cuuint64_t)width, (cuuint64_t)r_pad, (cuuint64_t)panels};
   cuuint64_t strides[2] = {128, (cuuint64_t)r_pad * 128};
-  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_panels};
+  cuuint32_t box[3] = {(cuuint32_t)width, (cuuint32_t)box_rows, (cuuint32_t)box_panels};
   cuuint32_t estr[3] = {1, 1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+  return fn(map, type, 3, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool fbl_encode_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels) {
+  return encode_panels(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, base, r_pad, panels, box_rows, box_panels);
+}
+bool fbl_encode_f32_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels) {
+  return encode_panels(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 32, base, r_pad, panels, box_rows, box_panels);
 }
 
 // fp32 accumulator [n_pad, cols] stored in the bf16 tile order (64-column panels, 256-byte rows), viewed as

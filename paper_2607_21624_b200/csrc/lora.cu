@@ -81,18 +81,6 @@ inline const char* colblock(const fbl_plan* p, const void* base, int64_t r_pad, 
   return (const char*)base + (size_t)off[i] * (size_t)r_pad * p->e;     // whole 64 (32) column panels: panel stride r_pad * tw
 }
 
-cudaError_t run_group(const fbl_plan* p, GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int* kernels) {
-  bool tc = p->use_tc != 0;
-  for (int i = 0; i < count; ++i) tc = tc && gemm_tc_supported(p, gs[i]);
-  if (tc) { *kernels = 1; return launch_gemm_tc_group(p, gs, count, status, st); }
-  *kernels = count;
-  for (int i = 0; i < count; ++i) {
-    cudaError_t e = launch_gemm_simt(p->d.dtype, gs[i], st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 }  // namespace
 
 extern "C" {
@@ -151,7 +139,7 @@ int fbl_layer_fwd_lora(const fbl_plan* p, const void* X, const float* gamma, con
     g.t[0] = {Xn, p->n_pad, 0, A_all, up8(D), 0, D};
     g.b_static = 1;
     g.c = T; g.c_rpad = p->n_pad; g.seq = p->d.seq; g.t_pad = p->t_pad;
-    LORA_CUDA(run_group(p, &g, 1, status, st, &k));
+    LORA_CUDA(run_gemm_group(p, &g, 1, status, st, -1, &k));
     LORA_STEP("lora_T", 0, cudaSuccess);
     p->launches += k;
   }
@@ -171,7 +159,7 @@ int fbl_layer_fwd_lora(const fbl_plan* p, const void* X, const float* gamma, con
       g.c = O[i]; g.c_rpad = p->n_pad; g.bias = bias ? B[i] : nullptr;
       g.seq = p->d.seq; g.t_pad = p->t_pad;
     }
-    LORA_CUDA(run_group(p, gs, 3, status, st, &k));
+    LORA_CUDA(run_gemm_group(p, gs, 3, status, st, -1, &k));
     LORA_STEP("proj_qkv", 0, cudaSuccess);
     p->launches += k;
   }
@@ -186,7 +174,7 @@ int fbl_layer_fwd_lora(const fbl_plan* p, const void* X, const float* gamma, con
     g.c = Y; g.c_rpad = p->n_pad; g.bias = bias ? bo : nullptr;
     g.residual = p->d.residual ? X : nullptr;
     g.seq = p->d.seq; g.t_pad = p->t_pad;
-    LORA_CUDA(run_group(p, &g, 1, status, st, &k));
+    LORA_CUDA(run_gemm_group(p, &g, 1, status, st, -1, &k));
     LORA_STEP("proj_o", 0, cudaSuccess);
     p->launches += k;
   }
@@ -231,16 +219,16 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     ga.t[0] = {dY, p->n_pad, 0, Wo, up8(p->dq), 1, D};
     ga.b_static = 1;
     ga.c = dA; ga.c_rpad = p->n_pad; ga.seq = p->d.seq; ga.t_pad = p->t_pad;
-    if (p->use_tc && gemm_tc_supported(p, ga)) {
+    if (gemm_fuses_dot(p, ga)) {
       ga.dot_with = A; ga.dot_out = dvec; ga.dot_hd = p->d.head_dim; ga.dot_hq = p->d.n_q_heads;
       dvec_ready = true;
     }
-    LORA_CUDA(run_group(p, &ga, 1, status, st, &k));
+    LORA_CUDA(run_gemm_group(p, &ga, 1, status, st, -1, &k));
     LORA_STEP("dA", 0, cudaSuccess);
     p->launches += k;
   }
   if (p->use_tc && attn_bwd_tc_supported(p)) LORA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
-  else LORA_STEP("attn_bwd", 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, st));
+  else LORA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   if (p->rope_base > 0.f) LORA_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   const void* G[3] = {dQ, dK, dV};
   {
@@ -248,7 +236,7 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     g.m = n; g.n = RA; g.n_terms = 3;      // its zero blocks keep each gradient in its own adapter's columns
     for (int i = 0; i < 3; ++i) g.t[i] = {G[i], p->n_pad, 0, colblock(p, B_all, RA, i), RA, 1, cols[i]};
     g.c = dT; g.c_rpad = p->n_pad; g.seq = p->d.seq; g.t_pad = p->t_pad;
-    LORA_CUDA(run_group(p, &g, 1, status, st, &k));
+    LORA_CUDA(run_gemm_group(p, &g, 1, status, st, -1, &k));
     LORA_STEP("lora_dT", 0, cudaSuccess);
     p->launches += k;
   }
@@ -274,7 +262,7 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     g.m = D; g.n = RA; g.n_terms = 1;
     g.t[0] = {Xn, p->n_pad, 1, dT, p->n_pad, 0, n};
     g.c = dA_all; g.c_rpad = up8(D);
-    LORA_CUDA(run_group(p, gs, 5, status, st, &k));
+    LORA_CUDA(run_gemm_group(p, gs, 5, status, st, -1, &k));
     LORA_STEP("dB+dXn+dA", 0, cudaSuccess);
     p->launches += k;
   }

@@ -138,21 +138,6 @@ cudaError_t act(const fbl_mlp_plan* p, bool bwd, const void* a, const void* U, c
                                       : act_launch<__nv_bfloat16>(p, bwd, a, U, G, o1, o2, st);
 }
 
-// One launch for a group of problems on the tensor-core kernel if every one of them can run there, else one FFMA
-// launch per problem.  Returns the number of kernels enqueued in *kernels.
-cudaError_t run_group(const fbl_mlp_plan* p, GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int* kernels) {
-  bool tc = p->base->use_tc != 0;
-  for (int i = 0; i < count; ++i) tc = tc && gemm_tc_supported(p->base, gs[i]);
-  if (tc) { *kernels = 1; return launch_gemm_tc_group(p->base, gs, count, status, st); }
-  *kernels = count;
-  for (int i = 0; i < count; ++i) {
-    gs[i].ksplit = 0; gs[i].acc = nullptr;
-    cudaError_t e = launch_gemm_simt(p->d.dtype, gs[i], st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 bool mshape(const fbl_mlp_plan* p, int id, int64_t* outer, int64_t* rows, int64_t* rows_pad, int* cols) {
   const fbl_mlp_desc& d = p->d;
   switch (id) {
@@ -334,17 +319,17 @@ int fbl_mlp_fwd(const fbl_mlp_plan* p, const void* X, const float* gamma, const 
     if (tc && !gated) {
       // the activation rides in the up projection's epilogue: U and H = gelu(U) leave the same accumulator tile
       gs[0].epi = 1; gs[0].c2 = H;
-      MLP_CUDA(run_group(p, gs, 1, status, st, &k));
+      MLP_CUDA(run_gemm_group(bp, gs, 1, status, st, -1, &k));
       p->launches += k;
     } else if (tc) {
       // gated: U first, then the gate projection, whose epilogue reads U's tile and writes G and H = silu(G) * U
-      MLP_CUDA(run_group(p, &gs[0], 1, status, st, &k));
+      MLP_CUDA(run_gemm_group(bp, &gs[0], 1, status, st, -1, &k));
       p->launches += k;
       gs[1].epi = 3; gs[1].residual = U; gs[1].c2 = H;
-      MLP_CUDA(run_group(p, &gs[1], 1, status, st, &k));
+      MLP_CUDA(run_gemm_group(bp, &gs[1], 1, status, st, -1, &k));
       p->launches += k;
     } else {
-      MLP_CUDA(run_group(p, gs, cnt, status, st, &k));
+      MLP_CUDA(run_gemm_group(bp, gs, cnt, status, st, -1, &k));
       p->launches += k;
       MLP_STEP(1, act(p, false, nullptr, U, G, H, nullptr, st));
     }
@@ -358,7 +343,7 @@ int fbl_mlp_fwd(const fbl_mlp_plan* p, const void* X, const float* gamma, const 
     g.residual = p->d.residual ? X : nullptr;
     g.seq = p->d.seq; g.t_pad = bp->t_pad;
     int k = 0;
-    MLP_CUDA(run_group(p, &g, 1, status, st, &k));
+    MLP_CUDA(run_gemm_group(bp, &g, 1, status, st, -1, &k));
     p->launches += k;
   }
   return FBL_OK;
@@ -412,10 +397,10 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
       // the activation's derivative rides in the dH product's epilogue: dU (and dG) leave the accumulator tile, dH
       // itself is never stored
       gh.epi = gated ? 4 : 2; gh.residual = U; gh.aux1 = gated ? G : nullptr; gh.c = dU; gh.c2 = gated ? dG : nullptr;
-      MLP_CUDA(run_group(p, gs, 2, status, st, &k));
+      MLP_CUDA(run_gemm_group(bp, gs, 2, status, st, -1, &k));
       p->launches += k;
     } else {
-      MLP_CUDA(run_group(p, gs, 2, status, st, &k));
+      MLP_CUDA(run_gemm_group(bp, gs, 2, status, st, -1, &k));
       p->launches += k;
       MLP_STEP(1, act(p, true, dH, U, G, dU, dG, st));
     }
@@ -450,7 +435,7 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
       }
     }
     int k = 0;
-    MLP_CUDA(run_group(p, gs, nw + 1, status, st, &k));
+    MLP_CUDA(run_gemm_group(bp, gs, nw + 1, status, st, -1, &k));
     p->launches += k;
   }
   if (cg.count > 0) MLP_STEP(1, launch_convert_f32_group(cg, st));

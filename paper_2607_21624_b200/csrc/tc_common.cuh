@@ -313,4 +313,5 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 
 // Host side: encode a 3-D tensor map over an R-Tile bf16 matrix viewed as [panels][rows][64].
 bool fbl_encode_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels);
+bool fbl_encode_f32_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels);   // fp32: [panels][rows][32]
 bool fbl_encode_f32_panel_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_halves = 2);

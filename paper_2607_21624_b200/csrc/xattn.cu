@@ -29,13 +29,15 @@ inline int64_t up8(int64_t v) { return (v + 7) / 8 * 8; }
       p->prof_n++;                                                       \
     }                                                                    \
   } while (0)
+// A group of GEMM problems as one step; run_gemm_group says how many kernels it took.
+#define XA_GEMM_STEP(name, gs, count)                                   \
+  do {                                                                  \
+    int k__ = 0;                                                        \
+    XA_CUDA(run_gemm_group(p, gs, count, status, st, -1, &k__));        \
+    XA_STEP(name, k__, cudaSuccess);                                    \
+  } while (0)
 #define XA_PROF_BEGIN() \
   do { if (p->prof_on) { p->prof_n = 0; XA_CUDA(cudaEventRecord(p->prof_ev[0], st)); } } while (0)
-
-cudaError_t run_gemm(const fbl_plan* p, const GemmArgs& g, int32_t* status, cudaStream_t st) {
-  if (p->use_tc && gemm_tc_supported(p, g)) return launch_gemm_tc_group(p, &g, 1, status, st);
-  return launch_gemm_simt(p->d.dtype, g, st);
-}
 
 }  // namespace
 
@@ -78,14 +80,8 @@ int fbl_xattn_fwd(const fbl_plan* p, const void* X, const void* M, const float* 
       g.t[0] = {M, p->n_pad_kv, 0, W[i], up8(Dm), 0, Dm};
       g.c = O[i]; g.c_rpad = p->n_pad_kv; g.bias = bias ? B[i] : nullptr; g.seq = p->seq_kv; g.t_pad = p->t_pad_kv;
     }
-    bool tc = p->use_tc != 0;
-    for (int i = 0; i < 3; ++i) { gs[i].b_static = 1; tc = tc && gemm_tc_supported(p, gs[i]); }
-    if (tc) {
-      XA_STEP("proj_qkv", 1, launch_gemm_tc_group(p, gs, 3, status, st));
-    } else {
-      for (int i = 0; i < 3; ++i)
-        XA_STEP(i == 0 ? "proj_q" : i == 1 ? "proj_k" : "proj_v", 1, run_gemm(p, gs[i], status, st));
-    }
+    for (int i = 0; i < 3; ++i) gs[i].b_static = 1;
+    XA_GEMM_STEP("proj_qkv", gs, 3);
   }
   if (p->use_tc && attn_fwd_tc_supported(p)) XA_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
   else XA_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
@@ -97,7 +93,7 @@ int fbl_xattn_fwd(const fbl_plan* p, const void* X, const void* M, const float* 
     g.c = Y; g.c_rpad = p->n_pad; g.bias = bias ? bo : nullptr;
     g.residual = p->d.residual ? X : nullptr;
     g.seq = p->d.seq; g.t_pad = p->t_pad;
-    XA_STEP("proj_o", 1, run_gemm(p, g, status, st));
+    XA_GEMM_STEP("proj_o", &g, 1);
   }
   return FBL_OK;
 }
@@ -150,21 +146,18 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     ga.t[0] = {dY, p->n_pad, 0, Wo, up8(p->dq), 1, D};
     ga.b_static = 1;
     ga.c = dA; ga.c_rpad = p->n_pad; ga.seq = p->d.seq; ga.t_pad = p->t_pad;
-    if (p->use_tc && gemm_tc_supported(p, gw) && gemm_tc_supported(p, ga)) {
+    if (gemm_fuses_dot(p, ga)) {
       ga.dot_with = A; ga.dot_out = dvec; ga.dot_hd = p->d.head_dim; ga.dot_hq = p->d.n_q_heads;
       dvec_ready = true;
-      if (split_o) {
-        gw.ksplit = p->ksplit_o; gw.acc = (float*)(sc + p->sb_acc_o);
-        cg.src[cg.count] = gw.acc; cg.dst[cg.count] = dWo; cg.n[cg.count] = up8(p->dq) * (int64_t)D; cg.count++;
-      }
-      XA_STEP("dWo+dA", 1, launch_gemm_tc_group(p, gs, 2, status, st));
-    } else {
-      XA_STEP("dA", 1, run_gemm(p, ga, status, st));
-      XA_STEP("dWo", 1, run_gemm(p, gw, status, st));
     }
+    if (split_o && gemm_group_tc(p, gs, 2)) {
+      gw.ksplit = p->ksplit_o; gw.acc = (float*)(sc + p->sb_acc_o);
+      cg.src[cg.count] = gw.acc; cg.dst[cg.count] = dWo; cg.n[cg.count] = up8(p->dq) * (int64_t)D; cg.count++;
+    }
+    XA_GEMM_STEP("dWo+dA", gs, 2);
   }
   if (p->use_tc && attn_bwd_tc_supported(p)) XA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
-  else XA_STEP("attn_bwd", 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, st));
+  else XA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   {
     // query side: dWq = Xn^T dQ (token-axis reduction), dXn = dQ Wq^T
     // memory side: dWk = M^T dK, dWv = M^T dV (reductions over the memory's tokens), dM = dK Wk^T + dV Wv^T
@@ -192,41 +185,23 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     gk[2].b_static = 1;
     gk[2].t[1] = {dV, p->n_pad_kv, 0, Wv, up8(Dm), 1, p->dkv};
     gk[2].c = dM; gk[2].c_rpad = p->n_pad_kv; gk[2].seq = p->seq_kv; gk[2].t_pad = p->t_pad_kv;
-    bool tc_q = p->use_tc != 0, tc_k = p->use_tc != 0;
-    for (int i = 0; i < 2; ++i) tc_q = tc_q && gemm_tc_supported(p, gq[i]);
-    for (int i = 0; i < 3; ++i) tc_k = tc_k && gemm_tc_supported(p, gk[i]);
-    if (tc_q && split_q) {
-      gq[0].ksplit = p->ksplit_qkv; gq[0].acc = (float*)(sc + p->sb_acc_qkv);
-      cg.src[cg.count] = gq[0].acc; cg.dst[cg.count] = dWq; cg.n[cg.count] = up8(D) * (int64_t)p->dq; cg.count++;
+    // both sides in one launch: the three token-axis reductions first in the work list (longest loops), then the two
+    // input gradients
+    GemmArgs all[5] = {gq[0], gk[0], gk[1], gq[1], gk[2]};
+    const bool tc = gemm_group_tc(p, all, 5);
+    if (tc && split_q) {
+      all[0].ksplit = p->ksplit_qkv; all[0].acc = (float*)(sc + p->sb_acc_qkv);
+      cg.src[cg.count] = all[0].acc; cg.dst[cg.count] = dWq; cg.n[cg.count] = up8(D) * (int64_t)p->dq; cg.count++;
     }
-    if (tc_k && split_kv) {
+    if (tc && split_kv) {
       float* acc = (float*)(sc + p->sb_acc_kv);
       for (int i = 0; i < 2; ++i) {
-        gk[i].ksplit = p->ksplit_kv; gk[i].acc = acc;
+        all[1 + i].ksplit = p->ksplit_kv; all[1 + i].acc = acc;
         cg.src[cg.count] = acc; cg.dst[cg.count] = DW[i]; cg.n[cg.count] = up8(Dm) * (int64_t)p->dkv; cg.count++;
         acc += up8(Dm) * (int64_t)p->dkv;
       }
     }
-    if (tc_q && tc_k) {
-      // both sides in one launch: the three token-axis reductions first in the work list (longest loops), then the
-      // two input gradients
-      GemmArgs all[5] = {gq[0], gk[0], gk[1], gq[1], gk[2]};
-      XA_STEP("dWqkv+dXn+dM", 1, launch_gemm_tc_group(p, all, 5, status, st));
-    } else {
-    if (tc_q) {
-      XA_STEP("dWq+dXn", 1, launch_gemm_tc_group(p, gq, 2, status, st));
-    } else {
-      XA_STEP("dXn", 1, run_gemm(p, gq[1], status, st));
-      XA_STEP("dWq", 1, run_gemm(p, gq[0], status, st));
-    }
-    if (tc_k) {
-      XA_STEP("dWkv+dM", 1, launch_gemm_tc_group(p, gk, 3, status, st));
-    } else {
-      XA_STEP("dM", 1, run_gemm(p, gk[2], status, st));
-      XA_STEP("dWk", 1, run_gemm(p, gk[0], status, st));
-      XA_STEP("dWv", 1, run_gemm(p, gk[1], status, st));
-    }
-    }
+    XA_GEMM_STEP("dWqkv+dXn+dM", all, 5);
     if (cg.count > 0) XA_STEP("dW round", 1, launch_convert_f32_group(cg, st));
   }
   // bias gradients: column sums over the query tokens (dY, dQ) and over the memory's tokens (dK, dV)

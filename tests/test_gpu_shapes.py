@@ -66,3 +66,18 @@ def test_pack_and_unpack(b, t, d, dtype, offset):
     run.plan.unpack(TENSOR["X"], run.buf["X"].data_ptr(), back[offset:].data_ptr(), stream)
     assert torch.equal(back[offset:offset + n], src) and (back[offset + n:] == 7).all() and (back[:offset] == 7).all()
     assert run.guards_intact() == []
+
+
+@pytest.mark.parametrize("cfg", [
+    # fp32 products: partly filled 64 x 64 tiles both ways, reductions of one to many 32-wide blocks (1 to 8 slices), all
+    # operand orientations, heads of 32, 64 and 128
+    LayerConfig("ff1", 1, 5, 32, 1, 1, 32, "fp32", "layernorm", True, True, True, 1e-5, 221, 0.2),
+    LayerConfig("ff2", 3, 67, 160, 5, 1, 32, "fp32", "rmsnorm", True, True, False, 1e-5, 222, 0.1),
+    LayerConfig("ff3", 2, 129, 1056, 3, 3, 64, "fp32", "layernorm", False, False, True, 1e-5, 223, 0.03),
+    LayerConfig("ff4", 1, 200, 96, 2, 1, 128, "fp32", "rmsnorm", True, True, True, 1e-5, 224, 0.1),
+    MlpConfig("ff5", 2, 70, 96, 416, "fp32", "layernorm", "swiglu", True, True, 1e-5, 225, 0.1),
+    MlpConfig("ff6", 1, 1100, 64, 256, "fp32", "rmsnorm", "gelu", True, False, 1e-5, 226, 0.1),
+    XattnConfig("ff7", 2, 33, 90, 64, 224, 4, 2, 32, "fp32", "layernorm", True, True, 1e-5, 227, 0.1),
+], ids=lambda c: c.name)
+def test_fp32_gemm_tiles_and_slices(cfg):
+    check(cfg)
