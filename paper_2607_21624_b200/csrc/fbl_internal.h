@@ -74,6 +74,8 @@ struct fbl_plan {
   // bookkeeping of the enqueue calls (they take the plan as const): kernels enqueued so far, optional per-step
   // event timing.  Calls on one plan are not thread-safe; give each host thread its own plan.
   mutable int64_t launches;
+  static constexpr int TILE_MEMO = 16;      // GEMM launches by shape: the output tile chosen for each
+  mutable struct { uint64_t key; int kind; } tile_memo[TILE_MEMO];
   mutable int prof_on, prof_n;
   mutable cudaEvent_t prof_ev[FBL_PROF_MAX + 1];
   mutable const char* prof_name[FBL_PROF_MAX];

@@ -961,80 +961,110 @@ cudaError_t launch_group_pair(const fbl_plan* p, const GemmArgs* gs, int count, 
                       : launch_pdl(k, dim3(2 * pairs), dim3(192), SP::TOTAL, st, G);
 }
 
+namespace {
+
+// Output tiles a launch may use: 128 x 128 or 128 x 256 on one CTA, 256 x 256 on a CTA pair.
+enum TileKind { TILE_NARROW = 0, TILE_WIDE, TILE_PAIR };
+struct TileCost { int m, n; double kb, unit, epilogue, fixed; };      // extents; clocks per k-block, per unit, of an epilogue, per launch
+// Clocks from a sweep of the four launches of a layer over 64 to 6300 tokens and widths of 320 to 3264 columns.  A
+// k-block of a wide tile costs less than two of a narrow one (operands are re-read half as often per flop), a pair's
+// less still, but pairs start later; with few k-blocks the epilogue of the tile before is what a tile waits for.
+const TileCost TILE_COST[3] = {{128, 128, 545, 800, 1600, 0}, {128, 256, 710, 900, 3600, 0}, {256, 256, 675, 900, 3600, 3500}};
+struct TileWork { long long m; int n, kb, split; };
+
+// Clocks of the longest block (pair) when the persistent kernel deals the units of a group's problems out in turn.
+double tile_makespan(const TileCost& c, const TileWork* w, int count, int slots) {
+  std::vector<double> load((size_t)slots, 0.0);
+  long long dealt = 0;
+  for (int i = 0; i < count; ++i) {
+    const long long units = ((w[i].m + c.m - 1) / c.m) * ((w[i].n + c.n - 1) / c.n) * w[i].split;
+    const double main = ((w[i].kb + w[i].split - 1) / w[i].split + (w[i].split > 1 ? 2 : 0)) * c.kb + c.unit;
+    const double len = main > c.epilogue ? main : c.epilogue;
+    const int first = (int)(dealt % slots), extra = (int)(units % slots);
+    for (int s = 0; s < slots; ++s) {
+      const int turn = s >= first ? s - first : s - first + slots;       // this slot's place among the problem's first units
+      load[(size_t)s] += (double)(units / slots + (turn < extra ? 1 : 0)) * len;
+    }
+    dealt += units;
+  }
+  double longest = 0;
+  for (double l : load) longest = l > longest ? l : longest;
+  return longest + (dealt <= slots ? 0.5 : 1.0) * c.epilogue + c.fixed;
+}
+
+int best_tile(const TileWork* w, int count, int sm_count, bool pairs, double* clocks) {
+  int kind = TILE_NARROW;
+  *clocks = 1e300;
+  for (int k = TILE_NARROW; k <= (pairs ? TILE_PAIR : TILE_WIDE); ++k) {
+    const double t = tile_makespan(TILE_COST[k], w, count, k == TILE_PAIR ? sm_count / 2 : sm_count);
+    if (t < *clocks) { *clocks = t; kind = k; }
+  }
+  return kind;
+}
+
+}  // namespace
+
 cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st,
                                  int launch_id) {
   if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
   fbl_plan::GemmChoice ch = {0, -1, 0};
   if (launch_id >= 0 && launch_id < FBL_GEMM_LAUNCH_COUNT) ch = p->choice[launch_id];
-  bool wide = true;                       // 128 x 256 tiles when every problem's N is whole 256-column blocks
-  int tiles_wide = 0;
-  for (int i = 0; i < count; ++i) {
-    wide = wide && gs[i].n % 256 == 0;
-    tiles_wide += ((gs[i].m + BM - 1) / BM) * ((gs[i].n + 255) / 256) * (gs[i].ksplit > 1 ? gs[i].ksplit : 1);
-  }
-  const bool wide_legal = wide;
-  // with too few wide tiles to occupy the SMs, narrower tiles (twice as many) finish sooner
-  if (wide && tiles_wide * 3 < p->sm_count * 2) wide = false;
-  // CTA pairs on 256 x 256 tiles for large problems (several rounds of tiles per SM pair): measured 2-6 % faster
-  // on the workload 5 GEMMs, no gain or a loss below that
   bool any_epi = false;
   for (int i = 0; i < count; ++i) any_epi = any_epi || gs[i].epi != 0;
-  // an offline choice for this launch overrides the heuristics below wherever its tile shape is legal
-  if (ch.bn == 128) wide = false;
-  else if (ch.bn == 256 && wide_legal) wide = true;
-  const int pair_mode = ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 whenever legal, -1 by size
-  if (pair_mode == 1 && wide_legal && !any_epi) return launch_group_pair(p, gs, count, status, st);
-  if (wide && pair_mode != 0 && !any_epi) {
-    long long pair_tiles = 0;
-    for (int i = 0; i < count; ++i)
-      pair_tiles += (long long)((gs[i].m + 255) / 256) * (gs[i].n / 256) * (gs[i].ksplit > 1 ? gs[i].ksplit : 1);
-    if (pair_tiles >= 4 * (p->sm_count / 2)) return launch_group_pair(p, gs, count, status, st);
+  // The tile whose slowest block finishes first; an offline choice for this launch, or the pair knob, comes before it.
+  // (N need not be whole tiles: panels past it are loaded as zeros and not stored.)
+  const int pair_mode = any_epi ? 0 : ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 always, -1 by cost
+  int kind = TILE_NARROW;
+  if (pair_mode == 1) {
+    kind = TILE_PAIR;
+  } else if (ch.bn) {
+    kind = ch.bn == 128 ? TILE_NARROW : TILE_WIDE;
+  } else {
+    // the same few launches come again on every pass of a plan: their tiles are remembered by shape
+    TileWork w[MAX_PROBLEMS];
+    uint64_t key = 1469598103934665603ull ^ (uint64_t)(pair_mode != 0);
+    for (int i = 0; i < count; ++i) {
+      w[i] = {gs[i].m, gs[i].n, 0, gs[i].ksplit > 1 ? gs[i].ksplit : 1};
+      for (int t = 0; t < gs[i].n_terms; ++t) w[i].kb += (gs[i].t[t].k + BK - 1) / BK;
+      for (uint64_t v : {(uint64_t)w[i].m, (uint64_t)w[i].n, (uint64_t)w[i].kb, (uint64_t)w[i].split}) key = (key ^ v) * 1099511628211ull;
+    }
+    int at = 0;
+    while (at < fbl_plan::TILE_MEMO && p->tile_memo[at].key && p->tile_memo[at].key != key) ++at;
+    if (at < fbl_plan::TILE_MEMO && p->tile_memo[at].key) {
+      kind = p->tile_memo[at].kind;
+    } else {
+      double clocks;
+      kind = best_tile(w, count, p->sm_count, pair_mode != 0, &clocks);
+      if (at < fbl_plan::TILE_MEMO) p->tile_memo[at] = {key, kind};
+    }
   }
-  if (wide) return launch_group_bn<256, 4>(p, gs, count, status, st, ch.esets);
+  if (kind == TILE_PAIR) return launch_group_pair(p, gs, count, status, st);
+  if (kind == TILE_WIDE) return launch_group_bn<256, 4>(p, gs, count, status, st, ch.esets);
   return launch_group_bn<128, 6>(p, gs, count, status, st, ch.esets);
 }
 
 // How many slices to cut the reduction loops of the splittable problems of a group into (the same number for all
 // of them).  The persistent kernel deals work units to its blocks round-robin, so a few long units beside many
-// short ones leave most SMs idle: this replays the dealing for each candidate and keeps the one whose longest
-// block finishes first, charging the fp32 detour (zero-fill, bulk reductions, rounding pass) as extra k-blocks.
+// short ones leave most SMs idle: this asks, for each candidate, when the longest block of the best tile finishes,
+// charging the fp32 detour (zero-fill, bulk reductions, rounding pass) as extra k-blocks and a fixed cost.
 int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count) {
   static const int cand[] = {1, 2, 3, 4, 6, 8, 12, 16};
   double base_cost = 0.0, best_cost = 0.0;
   int best = 1;
-  for (int ci = 0; ci < (int)(sizeof(cand) / sizeof(cand[0])); ++ci) {
-    const int S = cand[ci];
-    bool wide = true;
-    long long tiles_wide = 0;
-    bool any_split = false;
+  for (int S : cand) {
+    TileWork w[MAX_PROBLEMS];
+    bool too_short = false, any_split = false;
     for (int i = 0; i < count; ++i) {
-      wide = wide && sh[i].n % 256 == 0;
-      const int s_i = (sh[i].splittable && S > 1) ? S : 1;
-      if (s_i > 1 && sh[i].kblocks / s_i < 8) { any_split = false; tiles_wide = -1; break; }   // slices too short
-      any_split = any_split || s_i > 1;
-      tiles_wide += (long long)((sh[i].m + BM - 1) / BM) * ((sh[i].n + 255) / 256) * s_i;
+      w[i] = {sh[i].m, sh[i].n, sh[i].kblocks, sh[i].splittable ? S : 1};
+      too_short = too_short || (w[i].split > 1 && sh[i].kblocks / S < 8);
+      any_split = any_split || w[i].split > 1;
     }
-    if (tiles_wide < 0 || (S > 1 && !any_split)) continue;
-    if (wide && tiles_wide * 3 < (long long)sm_count * 2) wide = false;
-    const int bn = wide ? 256 : 128;
-    const double per_kb = wide ? 1.32 : 1.0;               // a k-block of a 128 x 256 tile takes about 660 clk, of 128 x 128 about 500
-    long long units = 0;
-    for (int i = 0; i < count; ++i)
-      units += (long long)((sh[i].m + BM - 1) / BM) * ((sh[i].n + bn - 1) / bn) * ((sh[i].splittable && S > 1) ? S : 1);
-    const int grid = (int)(units < sm_count ? units : sm_count);
-    std::vector<double> load((size_t)grid, 0.0);
-    long long w = 0;
-    for (int i = 0; i < count; ++i) {
-      const int s_i = (sh[i].splittable && S > 1) ? S : 1;
-      const long long n_i = (long long)((sh[i].m + BM - 1) / BM) * ((sh[i].n + bn - 1) / bn) * s_i;
-      const double len = ((sh[i].kblocks + s_i - 1) / s_i + (s_i > 1 ? 2 : 0) + 3) * per_kb;   // + pipeline fill and epilogue
-      for (long long u = 0; u < n_i; ++u, ++w) load[w % grid] += len;
-    }
-    double mk = 0;
-    for (int b = 0; b < grid; ++b) mk = load[b] > mk ? load[b] : mk;
-    if (S > 1) mk += 16;                                   // zero-fill and rounding pass
-    if (ci == 0) { base_cost = mk; best_cost = mk; }
-    else if (mk < 0.85 * base_cost && mk < best_cost) { best = S; best_cost = mk; }   // worth it only with a clear gain
+    if (too_short || (S > 1 && !any_split)) continue;
+    double cost;
+    best_tile(w, count, sm_count, true, &cost);
+    if (S > 1) cost += 8000;                               // zero-fill and rounding pass
+    if (S == 1) base_cost = best_cost = cost;
+    else if (cost < 0.85 * base_cost && cost < best_cost) { best = S; best_cost = cost; }   // worth it only with a clear gain
   }
   return best;
 }

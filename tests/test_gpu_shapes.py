@@ -81,3 +81,15 @@ def test_pack_and_unpack(b, t, d, dtype, offset):
 ], ids=lambda c: c.name)
 def test_fp32_gemm_tiles_and_slices(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("pair", ["-1", "1"], ids=["by-cost", "pairs"])
+@pytest.mark.parametrize("cfg", [
+    # columns that are not whole tiles, on every tile shape: one to a few tiles of rows, an odd number of 64-wide panels
+    LayerConfig("rg1", 1, 300, 192, 5, 1, 64, "bf16", "layernorm", True, True, True, 1e-5, 241, 0.05),
+    LayerConfig("rg2", 2, 500, 1088, 17, 17, 64, "bf16", "rmsnorm", True, False, False, 1e-5, 242, 0.02),
+    MlpConfig("rg3", 3, 333, 448, 1216, "bf16", "layernorm", "gelu", True, True, 1e-5, 243, 0.03),
+], ids=lambda c: getattr(c, "name", ""))
+def test_ragged_columns_on_every_gemm_tile(cfg, pair, monkeypatch):
+    monkeypatch.setenv("FBL_GEMM_PAIR", pair)
+    check(cfg)
