@@ -138,6 +138,13 @@ int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count);
 cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles, cudaStream_t st);
 bool attn_fwd_tc_supported(const fbl_plan* p);
 bool attn_bwd_tc_supported(const fbl_plan* p);
+bool attn_bwd_tc_direct(const fbl_plan* p);    // the tensor-core backward writes dQ itself: no fp32 accumulator to zero and round
+// Leading bytes of the backward scratch a step starts by zero-filling: status word and sliced products' accumulation areas,
+// and behind them the dQ accumulator where the attention backward adds into it.
+static inline size_t bwd_zero_bytes(const fbl_plan* p) {
+  return p->use_tc && attn_bwd_tc_supported(p) && attn_bwd_tc_direct(p) ? p->sb_dqacc : p->zero_bytes;
+}
+static inline int attn_bwd_tc_launches(const fbl_plan* p, bool dvec_ready) { return (dvec_ready ? 1 : 2) + (attn_bwd_tc_direct(p) ? 0 : 1); }
 void fbl_note_cuda_error(cudaError_t e, const char* where);
 
 cudaError_t launch_pack(int dtype, int unpack, const void* src, void* dst, int64_t outer, int64_t rows,

@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
         }
         mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
         // lazy running max: move it only when the tile's max beats it by more than the threshold
-        moved = mx > m + tau || m == -INFINITY;
+        moved = mx > m + tau;                       // (a first finite maximum always does)
         const float m_new = moved ? fmaxf(m, mx) : m;
         alpha = (m == -INFINITY) ? 0.f : tc::fast_exp2((m - m_new) * c);
         mc = (m_new == -INFINITY) ? 0.f : m_new * c;
@@ -340,9 +340,14 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
         tc::tmem_st32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
         tc::tmem_st32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
       } else {
-        // At most 128 registers here (two blocks per SM): two passes over the scores in tensor memory, four
-        // 32-column loads each, instead of holding the row.
+        // At most 128 registers here (two blocks per SM): two passes over the scores in tensor memory in 32-column
+        // loads instead of holding the row, and only as many as the warp attends to.
+        // 32-key chunks of this tile that any row of the warp attends to (the rest: beyond the keys, above the diagonal;
+        // none for a warp of padding rows).  P is zero in the others, and their scores are not looked at.
+        const int gw = gi - lane, key_end = gw >= P.seq ? 0 : P.causal ? min(P.seq_k, gw + 32) : P.seq_k;
+        const int n_ch = min(4, max(0, key_end - j0 + 31) / 32);
         auto mask_chunk = [&](float* sc, int cc) {
+          if (j0 + cc * 32 + 32 <= P.seq_k && (!P.causal || j0 + cc * 32 + 31 <= gw)) return;
 #pragma unroll
           for (int k = 0; k < 32; ++k) {
             const int gj = j0 + cc * 32 + k;
@@ -351,7 +356,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
         };
         float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
 #pragma unroll 1
-        for (int cc = 0; cc < 4; ++cc) {
+        for (int cc = 0; cc < n_ch; ++cc) {
           uint32_t sr[32];
           tc::tmem_ld32(s_addr + cc * 32, sr);
           tc::tmem_ld_wait();
@@ -364,7 +369,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
           }
         }
         mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
-        moved = mx > m + tau || m == -INFINITY;
+        moved = mx > m + tau;                       // (a first finite maximum always does)
         const float m_new = moved ? fmaxf(m, mx) : m;
         alpha = (m == -INFINITY) ? 0.f : tc::fast_exp2((m - m_new) * c);
         mc = (m_new == -INFINITY) ? 0.f : m_new * c;
@@ -390,7 +395,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
         // pass 2: P packed to bf16 over the score columns already consumed (32 scores become 16 packed columns;
         // the thread owns the lane, so nobody else's data is overwritten)
 #pragma unroll 1
-        for (int cc = 0; cc < 4; ++cc) {
+        for (int cc = 0; cc < n_ch; ++cc) {
           uint32_t sr[32];
           tc::tmem_ld32(s_addr + cc * 32, sr);
           tc::tmem_ld_wait();
@@ -408,11 +413,17 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
           }
           tc::tmem_st16(s_addr + cc * 16, pk);
         }
+        const uint32_t zero[16] = {};
+#pragma unroll 1
+        for (int cc = n_ch; cc < 4; ++cc) tc::tmem_st16(s_addr + cc * 16, zero);
       }
       if (moved) l *= alpha;
       l += (sum01.x + sum01.y) + (sum23.x + sum23.y);
       tc::tmem_st_wait();
       tc::tc_fence_before();
+      // With rotating buffers a tile's scores say nothing about its last P V product, and a wait that has let a phase of
+      // that barrier pass unseen would take an older one for it: see every phase before the next one can complete.
+      if (ROT && j > 0 && !tc::mbar_wait(bar(B_PVDONE + w), (j - 1) & 1, status, 211)) { ok = false; break; }
       tc::mbar_arrive(bar(B_PFULL + sbuf));
     }
     if (ok && n_kvw > 0) ok = tc::mbar_wait(bar(B_PVDONE + w), (n_kvw - 1) & 1, status, 210);
@@ -499,6 +510,7 @@ struct alignas(64) AttnBwdParams {
   const float* lse;      // [B, Hq, t_pad]
   const float* dvec;     // [B, Hq, t_pad]   D = rowsum(dO * O)
   float* dqacc;          // fp32 [n_pad, dq] in the bf16 tile order
+  __nv_bfloat16* dq;     // where dQ goes at once when a block sees all keys of its queries
   __nv_bfloat16* dk;
   __nv_bfloat16* dv;
   long long n_pad, n_pad_k;          // rows of the query-side (Q, dO, dQ) and key-side (K, V, dK, dV) buffers
@@ -535,10 +547,32 @@ struct BwdSmem {
 
 enum { BB_KVFULL = 0, BB_QFULL = 1, BB_QEMPTY = 4, BB_DOFULL = 7, BB_DOEMPTY = 9, BB_SFULL = 11, BB_PDSFULL, BB_DQFULL, BB_DQDRAINED, BB_DQSTAGED, BB_STAGEFREE = BB_DQSTAGED + 2, BB_SREAD = BB_STAGEFREE + 2, BB_DVDONE, BB_DPFULL };
 
+// No (query, key) pair of nq queries from i and the 32 keys from j takes part.
+__device__ __forceinline__ bool warp_masked(int i, int nq, int j, const AttnBwdParams& P) {
+  return i >= P.seq || j >= P.seq_k || (P.causal && i + nq - 1 < j);
+}
+
+// NC accumulator columns of one row, scaled and rounded, to columns col .. of row `row` of an R-Tile matrix.
+template <int NC>
+__device__ __forceinline__ void store_cols(__nv_bfloat16* m, long long rows, long long row, int col, const uint32_t (&o)[NC], float f) {
+  __nv_bfloat16* dst = m + ((long long)(col / 64) * rows + row) * 64 + (col % 64);
+#pragma unroll
+  for (int k = 0; k < NC / 8; ++k) {
+    uint4 v;
+    v.x = tc::pack_bf16(__uint_as_float(o[k * 8 + 0]) * f, __uint_as_float(o[k * 8 + 1]) * f);
+    v.y = tc::pack_bf16(__uint_as_float(o[k * 8 + 2]) * f, __uint_as_float(o[k * 8 + 3]) * f);
+    v.z = tc::pack_bf16(__uint_as_float(o[k * 8 + 4]) * f, __uint_as_float(o[k * 8 + 5]) * f);
+    v.w = tc::pack_bf16(__uint_as_float(o[k * 8 + 6]) * f, __uint_as_float(o[k * 8 + 7]) * f);
+    *reinterpret_cast<uint4*>(dst + 8 * k) = v;
+  }
+}
+
 constexpr int BWD_THREADS = 608;     // warp 0 TMA loads, warp 1 MMA, warps 2-17 softmax (four per TMEM lane quarter), warp 18 dQ reductions
 constexpr int BWD_SM_THREADS = 512;
 
-template <int HD>
+// DIRECT: the sequence has a single key tile, so a block's dQ tile is complete and goes out rounded, without the fp32
+// accumulator, its zero-fill and the rounding pass.
+template <int HD, bool DIRECT>
 __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __grid_constant__ AttnBwdParams P) {
   using SM = BwdSmem<HD>;
   constexpr bool PIPE = SM::PIPE;
@@ -594,7 +628,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
     // This thread is the TMA producer: K, V and the first Q tile (forward-pass data) are requested right here, so
     // that their latency overlaps the tensor-memory allocation and the block-wide barrier below.
     tc::tma_prefetch_desc(&P.tk); tc::tma_prefetch_desc(&P.tv); tc::tma_prefetch_desc(&P.tq);
-    tc::tma_prefetch_desc(&P.tdo); tc::tma_prefetch_desc(&P.tdq);
+    tc::tma_prefetch_desc(&P.tdo);
+    if (!DIRECT) tc::tma_prefetch_desc(&P.tdq);
     tc::mbar_expect_tx(bar(BB_KVFULL), 2 * SM::TILE);
     tc::tma_load_3d(base + SM::K_OFF, &P.tk, bar(BB_KVFULL), 0, row0k + j0, g * (int)PANELS);
     tc::tma_load_3d(base + SM::V_OFF, &P.tv, bar(BB_KVFULL), 0, row0k + j0, g * (int)PANELS);
@@ -761,7 +796,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       // arrival, on the barrier the pipelined variant uses for dV, tells the epilogue that they are complete
       if (ok && n_it > 0) tc::mma_commit(bar(BB_DVDONE));
     }
-  } else if (warp == 18) {
+  } else if (!DIRECT && warp == 18) {
     // ---- dQ reduction warp: adds each staged dQ tile to the fp32 accumulator with bulk tensor reductions ----
     if (lane == 0) {
       pdl_wait();                                    // the accumulator's zero-fill precedes the kernel before this one
@@ -779,7 +814,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       }
       tc::bulk_wait_group0();
     }
-  } else if (warp >= 2) {
+  } else if (warp >= 2 && warp < 18) {
     // ---- softmax warps: thread = (key row, one quarter of the 128 query columns) -----------------------
     const int q = warp % 4;                         // TMEM lane quarter
     const int part = (warp - 2) / 4;                // which 32 query columns (and which quarter of HD later)
@@ -809,6 +844,11 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       tc::tmem_ld_wait();
       tc::tc_fence_before();
       tc::mbar_arrive(bar(BB_DQDRAINED));            // TMEM side done: the tensor pipe may reuse the columns
+      if constexpr (DIRECT) {
+        const int h = g * P.group + dit / per_head, gi = (qt_begin + dit % per_head) * BQ + r;
+        if (gi < P.t_pad) store_cols<NC>(P.dq, P.n_pad, row0 + gi, h * HD + c0, o, P.scale);
+        return true;
+      }
       // Only now wait for the staging buffer (its previous tile must have been read by its bulk reduction, which
       // takes a few thousand cycles): the values sit in registers meanwhile and the columns are already free.
       if (dit >= (int)NS && !stage_is_alt(dit) && !tc::mbar_wait(bar(BB_STAGEFREE + (dit % NS)), (dit / (int)NS - 1) & 1, status, 310)) return false;
@@ -861,10 +901,15 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       auto chunk = [&](int cc, auto masked_tag) {
         constexpr bool MASKED = decltype(masked_tag)::value;
         const int c0 = part * 32 + cc * 16;
+        uint32_t pp[8], dd[8];
+        // a warp whose 32 keys x 16 queries are all masked (beyond a sequence, above the diagonal) only writes zeros
+        if (MASKED && warp_masked(i0 + c0, 16, j0 + q * 32, P)) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) pp[k] = dd[k] = 0u;
+        } else {
         uint32_t dpv[16];
         tc::tmem_ld16(lane_addr + DP_COL + c0, dpv);
         tc::tmem_ld_wait();
-        uint32_t pp[8], dd[8];
 #pragma unroll
         for (int k = 0; k < 16; k += 4) {
           const float4 l4 = *reinterpret_cast<const float4*>(&s_lse[c0 + k]);
@@ -896,6 +941,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
           pp[k / 2 + 1] = tc::pack_bf16(pv[2], pv[3]);
           dd[k / 2] = tc::pack_bf16(gv[0], gv[1]);
           dd[k / 2 + 1] = tc::pack_bf16(gv[2], gv[3]);
+        }
         }
         if (PIPE && cc == 0 && it > 0) {
           // P^T has its own columns, single-buffered: the dV product of the previous tile must have read them.
@@ -1024,17 +1070,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
           tc::tmem_ld16(lane_addr + (which ? DK_COL : DV_COL) + c0, o);   // warp-collective: no lane may skip it
           tc::tmem_ld_wait();
           if (gj < P.t_pad_k) {
-            const int col = g * HD + c0;
-            __nv_bfloat16* dst = out + ((long long)(col / 64) * P.n_pad_k + row0k + gj) * 64 + (col % 64);
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              uint4 v;
-              v.x = tc::pack_bf16(__uint_as_float(o[k * 8 + 0]) * f, __uint_as_float(o[k * 8 + 1]) * f);
-              v.y = tc::pack_bf16(__uint_as_float(o[k * 8 + 2]) * f, __uint_as_float(o[k * 8 + 3]) * f);
-              v.z = tc::pack_bf16(__uint_as_float(o[k * 8 + 4]) * f, __uint_as_float(o[k * 8 + 5]) * f);
-              v.w = tc::pack_bf16(__uint_as_float(o[k * 8 + 6]) * f, __uint_as_float(o[k * 8 + 7]) * f);
-              *reinterpret_cast<uint4*>(dst + 8 * k) = v;
-            }
+            store_cols<16>(out, P.n_pad_k, row0k + gj, g * HD + c0, o, f);
           }
         }
       }
@@ -1045,26 +1081,273 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
   if (warp == 1) tc::tmem_dealloc(tmem_base, TMEM_COLS);
 }
 
-template <int HD>
-cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* dA,
-                       const float* lse, const float* dvec, float* dqacc, void* dK, void* dV, int32_t* status,
-                       cudaStream_t st) {
-  AttnBwdParams P;
-  memset(&P, 0, sizeof(P));
-  const int panels = HD / 64;
-  if (!fbl_encode_rtile_map(&P.tq, Q, p->n_pad, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
-  if (!fbl_encode_rtile_map(&P.tdo, dA, p->n_pad, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
-  if (!fbl_encode_rtile_map(&P.tk, K, p->n_pad_kv, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
-  if (!fbl_encode_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
-  if (!fbl_encode_f32_panel_map(&P.tdq, dqacc, p->n_pad, p->dq / 64, BQ)) return cudaErrorInvalidValue;
-  P.lse = lse; P.dvec = dvec; P.dqacc = dqacc; P.dk = (__nv_bfloat16*)dK; P.dv = (__nv_bfloat16*)dV;
-  P.n_pad = p->n_pad; P.seq = p->d.seq; P.t_pad = p->t_pad; P.hq = p->d.n_q_heads; P.group = p->group;
-  P.causal = p->d.causal; P.dkv = p->dkv; P.scale = p->scale; P.status = status;
-  P.n_pad_k = p->n_pad_kv; P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;
-  auto k = attn_bwd_tc_kernel<HD>;
+// ---------------------------------------------------------------------------------------------------
+// Backward of short sequences (two key tiles, at most two query tiles, head_dim 64, a KV head per query head): one block
+// per (head, sequence) takes all their tile pairs.  K, V, Q and dO are loaded once and stay in shared memory; dQ of both
+// query tiles accumulates in tensor memory over the key tiles and goes out rounded, so there is no fp32 accumulator, no
+// zero-fill and no rounding pass; dV and dK of a key tile are copied out while the next key tile's scores are at work.
+// The roles and the per-tile schedule are those of the pipelined variant above, except that P^T goes through shared
+// memory like dS^T: tensor memory is full (S^T, dP^T, dV, dK and two dQ tiles are 512 columns).
+// Bound: start-up and drain of a block against its three or four tiles of softmax arithmetic; one block does both key
+// tiles' with one start-up, half the loads and no bulk reductions.
+// ---------------------------------------------------------------------------------------------------
+struct ShortSmem {
+  static constexpr uint32_t TILE = 16384;                                // 128 rows x 64 bf16
+  static constexpr uint32_t K_OFF = 0, V_OFF = 2 * TILE, Q_OFF = 4 * TILE, DO_OFF = 6 * TILE;
+  static constexpr uint32_t DS_OFF = 8 * TILE, P_OFF = DS_OFF + 2 * 32768;
+  static constexpr uint32_t LSE_OFF = P_OFF + 32768, D_OFF = LSE_OFF + 2 * 512, BAR_OFF = D_OFF + 2 * 512;
+  static constexpr uint32_t N_BARS = 16, TOTAL = BAR_OFF + 8 * N_BARS + 16;
+};
+enum { SB_KVFULL = 0, SB_QFULL = 2, SB_DOFULL = 4, SB_SFULL = 6, SB_SREAD, SB_PDSFULL, SB_DVDONE, SB_DQDONE, SB_DKDONE, SB_KVDRAINED, SB_FINAL };
+constexpr int SHORT_THREADS = 576;       // warp 0 TMA loads, warp 1 MMA, warps 2-17 softmax
+
+__global__ void __launch_bounds__(SHORT_THREADS, 1) attn_bwd_short_kernel(const __grid_constant__ AttnBwdParams P) {
+  using SM = ShortSmem;
+  constexpr int HD = 64;
+  constexpr uint32_t S_COL = 0, DP_COL = 128, DV_COL = 256, DK_COL = 320, DQ_COL = 384, TMEM_COLS = 512;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t base = tc::smem_u32(smem_raw);
+  const uint32_t bars = base + SM::BAR_OFF, slot = bars + 8 * SM::N_BARS;
+  auto bar = [&](int i) { return bars + 8u * i; };
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int h = blockIdx.x % P.hq, b = blockIdx.x / P.hq;
+  const int row0 = b * P.t_pad, row0k = b * P.t_pad_k;
+  const int n_qt = (P.seq + BQ - 1) / BQ, n_kt = (P.seq_k + BKV - 1) / BKV;
+  const int i1 = P.causal ? 1 : 0;                                       // first query tile of key tile 1
+  const int n0 = n_qt, n_it = n0 + (n_kt > 1 ? n_qt - i1 : 0);           // tile pairs: key tile 0's, then key tile 1's
+  auto key_tile = [&](int it) { return it < n0 ? 0 : 1; };
+  auto query_tile = [&](int it) { return it < n0 ? it : it - n0 + i1; };
+  int32_t* status = P.status;
+  if ((base & 1023u) != 0) {
+    if (threadIdx.x == 0) atomicCAS(status, 0, 398);
+    return;
+  }
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < 2; ++s) {
+      tc::mbar_init(bar(SB_KVFULL + s), 1);
+      tc::mbar_init(bar(SB_QFULL + s), 1);
+      tc::mbar_init(bar(SB_DOFULL + s), 1);
+    }
+    tc::mbar_init(bar(SB_SFULL), 1);
+    tc::mbar_init(bar(SB_SREAD), BWD_SM_THREADS);
+    tc::mbar_init(bar(SB_PDSFULL), BWD_SM_THREADS);
+    tc::mbar_init(bar(SB_DVDONE), 1);
+    tc::mbar_init(bar(SB_DQDONE), 1);
+    tc::mbar_init(bar(SB_DKDONE), 1);
+    tc::mbar_init(bar(SB_KVDRAINED), BWD_SM_THREADS);
+    tc::mbar_init(bar(SB_FINAL), 1);
+    tc::fence_barrier_init();
+    // forward-pass data: requested before the allocation, the block barrier and the wait for the kernel in front
+    tc::tma_prefetch_desc(&P.tk); tc::tma_prefetch_desc(&P.tv); tc::tma_prefetch_desc(&P.tq); tc::tma_prefetch_desc(&P.tdo);
+    for (int t = 0; t < 2; ++t) {
+      if (t < n_kt) {
+        tc::mbar_expect_tx(bar(SB_KVFULL + t), 2 * SM::TILE);
+        tc::tma_load_3d(base + SM::K_OFF + t * SM::TILE, &P.tk, bar(SB_KVFULL + t), 0, row0k + t * BKV, h);
+        tc::tma_load_3d(base + SM::V_OFF + t * SM::TILE, &P.tv, bar(SB_KVFULL + t), 0, row0k + t * BKV, h);
+      }
+      if (t < n_qt) {
+        tc::mbar_expect_tx(bar(SB_QFULL + t), SM::TILE + 512);
+        tc::tma_load_3d(base + SM::Q_OFF + t * SM::TILE, &P.tq, bar(SB_QFULL + t), 0, row0 + t * BQ, h);
+        tc::bulk_load(base + SM::LSE_OFF + t * 512, P.lse + ((long long)b * P.hq + h) * P.t_pad + t * BQ, 512, bar(SB_QFULL + t));
+      }
+    }
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(slot, TMEM_COLS);
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  uint32_t tmem_base;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  pdl_launch_dependents();
+
+  if (warp == 0 && lane == 0) {
+    pdl_wait();                                          // dO and D come from the kernel in front
+    for (int t = 0; t < n_qt; ++t) {
+      tc::mbar_expect_tx(bar(SB_DOFULL + t), SM::TILE + 512);
+      tc::tma_load_3d(base + SM::DO_OFF + t * SM::TILE, &P.tdo, bar(SB_DOFULL + t), 0, row0 + t * BQ, h);
+      tc::bulk_load(base + SM::D_OFF + t * 512, P.dvec + ((long long)b * P.hq + h) * P.t_pad + t * BQ, 512, bar(SB_DOFULL + t));
+    }
+  } else if (warp == 1 && lane == 0) {
+    // ---- MMA issuer ----
+    const uint32_t idesc_s = tc::idesc_bf16(BKV, BQ, 0, 0), idesc_kv = tc::idesc_bf16(BKV, HD, 0, 1), idesc_dq = tc::idesc_bf16(BQ, HD, 1, 1);
+    const uint32_t hi = tc::smem_desc_hi(1024), TW = SM::TILE >> 4;
+    const uint32_t k_km = tc::smem_desc_lo(base + SM::K_OFF, 16), k_mn = tc::smem_desc_lo(base + SM::K_OFF, 16384);
+    const uint32_t v_km = tc::smem_desc_lo(base + SM::V_OFF, 16);
+    const uint32_t q_km = tc::smem_desc_lo(base + SM::Q_OFF, 16), q_mn = tc::smem_desc_lo(base + SM::Q_OFF, 16384);
+    const uint32_t do_km = tc::smem_desc_lo(base + SM::DO_OFF, 16), do_mn = tc::smem_desc_lo(base + SM::DO_OFF, 16384);
+    const uint32_t ds_km = tc::smem_desc_lo(base + SM::DS_OFF, 16), ds_mn = tc::smem_desc_lo(base + SM::DS_OFF, 16384);
+    const uint32_t p_km = tc::smem_desc_lo(base + SM::P_OFF, 16);
+    auto scores = [&](uint32_t col, uint32_t a, uint32_t q) {            // S^T = K Q^T, dP^T = V dO^T
+#pragma unroll
+      for (uint32_t kk = 0; kk < 4; ++kk) tc::mma_bf16_ss_w(tmem_base + col, a + kk * 2, hi, q + kk * 2, hi, idesc_s, kk > 0);
+    };
+    auto product = [&](uint32_t col, uint32_t a, uint32_t q, bool more) {  // dV += P^T dO, dK += dS^T Q
+#pragma unroll
+      for (uint32_t kk = 0; kk < 8; ++kk)
+        tc::mma_bf16_ss_w(tmem_base + col, a + (kk / 4) * 1024 + (kk % 4) * 2, hi, q + kk * 128, hi, idesc_kv, more || kk > 0);
+    };
+    bool ok = tc::mbar_wait(bar(SB_KVFULL), 0, status, 321) && tc::mbar_wait(bar(SB_QFULL), 0, status, 322) &&
+              tc::mbar_wait(bar(SB_DOFULL), 0, status, 323);
+    if (ok) {
+      tc::tc_fence_after();
+      scores(S_COL, k_km, q_km);
+      scores(DP_COL, v_km, do_km);
+      tc::mma_commit(bar(SB_SFULL));
+    }
+    for (int it = 0; it < n_it && ok; ++it) {
+      const int j = key_tile(it), i = query_tile(it);
+      const bool next = it + 1 < n_it;
+      const int jn = next ? key_tile(it + 1) : 0, in = next ? query_tile(it + 1) : 0;
+      if (next) {                                        // S^T of the next pair once every warp holds this one's scores
+        if (!tc::mbar_wait(bar(SB_SREAD), it & 1, status, 324)) break;
+        if (!tc::mbar_wait(bar(SB_QFULL + in), 0, status, 322) || !tc::mbar_wait(bar(SB_KVFULL + jn), 0, status, 321)) break;
+        tc::tc_fence_after();
+        scores(S_COL, k_km + jn * TW, q_km + in * TW);
+      }
+      if (!tc::mbar_wait(bar(SB_PDSFULL), it & 1, status, 325)) break;
+      tc::tc_fence_after();
+      if (next) {
+        if (!tc::mbar_wait(bar(SB_DOFULL + in), 0, status, 323)) break;
+        tc::tc_fence_after();
+        scores(DP_COL, v_km + jn * TW, do_km + in * TW);
+        tc::mma_commit(bar(SB_SFULL));
+      }
+      if (it == n0 && !tc::mbar_wait(bar(SB_KVDRAINED), 0, status, 326)) break;   // key tile 0's dV, dK are copied out
+      tc::tc_fence_after();
+      const bool more = it != 0 && it != n0;
+      product(DV_COL, p_km, do_mn + i * TW, more);
+      tc::mma_commit(bar(SB_DVDONE));
+      product(DK_COL, ds_km + (it & 1) * 2048, q_mn + i * TW, more);
+      if (it + 1 == n0) tc::mma_commit(bar(SB_DKDONE));
+#pragma unroll
+      for (uint32_t kk = 0; kk < 8; ++kk)                // dQ += dS K: the dS^T tile read MN-major
+        tc::mma_bf16_ss_w(tmem_base + DQ_COL + i * 64, ds_mn + (it & 1) * 2048 + kk * 128, hi, k_mn + j * TW + kk * 128, hi, idesc_dq,
+                          (j > 0 || kk > 0) ? 1u : 0u);
+      tc::mma_commit(bar(SB_DQDONE));
+      if (!next) tc::mma_commit(bar(SB_FINAL));
+    }
+  } else if (warp >= 2) {
+    // ---- softmax warps: thread = (key row, one quarter of the 128 query columns) ----
+    const int q = warp % 4, part = (warp - 2) / 4, r = q * 32 + lane;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    const float c = P.scale * LOG2E;
+    const float* s_lse = reinterpret_cast<const float*>(smem_raw + SM::LSE_OFF);
+    const float* s_d = reinterpret_cast<const float*>(smem_raw + SM::D_OFF);
+    pdl_wait();                                          // before this role writes anything
+    bool ok = true;
+    auto copy_kv = [&](int j) {                          // dV, dK of key tile j: 16 columns each per thread
+      const int gj = j * BKV + r;
+      const bool live = gj < P.seq_k;
+#pragma unroll 1
+      for (int which = 0; which < 2; ++which) {
+        uint32_t o[16];
+        tc::tmem_ld16(lane_addr + (which ? DK_COL : DV_COL) + part * 16, o);
+        tc::tmem_ld_wait();
+        if (gj < P.t_pad_k) store_cols<16>(which ? P.dk : P.dv, P.n_pad_k, row0k + gj, h * HD + part * 16, o, live ? (which ? P.scale : 1.f) : 0.f);
+      }
+    };
+    for (int it = 0; it < n_it && ok; ++it) {
+      const int j0 = key_tile(it) * BKV, i = query_tile(it), i0 = i * BQ, gj = j0 + r;
+      if (!tc::mbar_wait(bar(SB_SFULL), it & 1, status, 327)) { ok = false; break; }
+      tc::tc_fence_after();
+      const bool need_mask = (P.causal && i0 < j0 + BKV - 1) || j0 + BKV > P.seq_k || i0 + BQ > P.seq;
+      uint32_t sv[32];
+      tc::tmem_ld32(lane_addr + S_COL + part * 32, sv);
+      tc::tmem_ld_wait();
+      tc::tc_fence_before();
+      tc::mbar_arrive(bar(SB_SREAD));
+      const uint32_t row_off = (uint32_t)(part / 2) * 16384 + r * 128;
+      auto chunk = [&](int cc, auto masked_tag) {
+        constexpr bool MASKED = decltype(masked_tag)::value;
+        const int c0 = part * 32 + cc * 16;
+        uint32_t pp[8], dd[8];
+        if (MASKED && warp_masked(i0 + c0, 16, j0 + q * 32, P)) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) pp[k] = dd[k] = 0u;
+        } else {
+          uint32_t dpv[16];
+          tc::tmem_ld16(lane_addr + DP_COL + c0, dpv);
+          tc::tmem_ld_wait();
+          const float2 c2 = make_float2(c, c), nl2e = make_float2(-LOG2E, -LOG2E), neg1 = make_float2(-1.f, -1.f);
+#pragma unroll
+          for (int k = 0; k < 16; k += 2) {
+            const float2 l = *reinterpret_cast<const float2*>(&s_lse[i * 128 + c0 + k]);
+            const float2 d = *reinterpret_cast<const float2*>(&s_d[i * 128 + c0 + k]);
+            const float2 x = __ffma2_rn(make_float2(__uint_as_float(sv[cc * 16 + k]), __uint_as_float(sv[cc * 16 + k + 1])), c2, __fmul2_rn(l, nl2e));
+            float pv[2] = {tc::fast_exp2(x.x), tc::fast_exp2(x.y)};
+            const float2 gd = __ffma2_rn(d, neg1, make_float2(__uint_as_float(dpv[k]), __uint_as_float(dpv[k + 1])));
+            float gv[2] = {pv[0] * gd.x, pv[1] * gd.y};
+            if (MASKED) {                                // LSE / D of rows past the sequence end are not defined
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const int gi = i0 + c0 + k + u;
+                if (gj >= P.seq_k || gi >= P.seq || (P.causal && gi < gj)) pv[u] = gv[u] = 0.f;
+              }
+            }
+            pp[k / 2] = tc::pack_bf16(pv[0], pv[1]);
+            dd[k / 2] = tc::pack_bf16(gv[0], gv[1]);
+          }
+        }
+        if (cc == 0 && it > 0) {                         // dV of the pair before has read P^T
+          if (!tc::mbar_wait(bar(SB_DVDONE), (it - 1) & 1, status, 328)) { ok = false; return; }
+        }
+        const uint32_t ds = base + SM::DS_OFF + (it & 1) * 32768 + row_off, pt = base + SM::P_OFF + row_off;
+#pragma unroll
+        for (int ch = 0; ch < 2; ++ch) {
+          const uint32_t at = (((uint32_t)((part % 2) * 4 + cc * 2 + ch) ^ (uint32_t)(r & 7)) * 16);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(pt + at), "r"(pp[ch * 4]), "r"(pp[ch * 4 + 1]), "r"(pp[ch * 4 + 2]), "r"(pp[ch * 4 + 3]) : "memory");
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ds + at), "r"(dd[ch * 4]), "r"(dd[ch * 4 + 1]), "r"(dd[ch * 4 + 2]), "r"(dd[ch * 4 + 3]) : "memory");
+        }
+      };
+      if (need_mask) {
+        chunk(0, std::true_type{});
+        if (ok) chunk(1, std::true_type{});
+      } else {
+        chunk(0, std::false_type{});
+        if (ok) chunk(1, std::false_type{});
+      }
+      if (!ok) break;
+      // dK and dQ of the pair before are complete before this pair's products can be issued: the dS^T buffer of the pair
+      // after this one is free, and no warp falls a phase behind on this barrier
+      if (it > 0 && !tc::mbar_wait(bar(SB_DQDONE), (it - 1) & 1, status, 329)) { ok = false; break; }
+      tc::fence_proxy_async();
+      tc::tc_fence_before();
+      tc::mbar_arrive(bar(SB_PDSFULL));
+      if (it == n0) {                                    // key tile 0's sums, while the tensor pipe has the next scores to do
+        if (!tc::mbar_wait(bar(SB_DKDONE), 0, status, 330)) { ok = false; break; }
+        tc::tc_fence_after();
+        copy_kv(0);
+        tc::tc_fence_before();
+        tc::mbar_arrive(bar(SB_KVDRAINED));
+      }
+    }
+    if (ok) ok = tc::mbar_wait(bar(SB_FINAL), 0, status, 331);
+    tc::tc_fence_after();
+    if (ok) {
+      copy_kv(n_kt - 1);
+      for (int i = 0; i < n_qt; ++i) {
+        const int gi = i * BQ + r;
+        uint32_t o[16];
+        tc::tmem_ld16(lane_addr + DQ_COL + i * 64 + part * 16, o);
+        tc::tmem_ld_wait();
+        if (gi < P.t_pad) store_cols<16>(P.dq, P.n_pad, row0 + gi, h * HD + part * 16, o, P.scale);
+      }
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) tc::tmem_dealloc(tmem_base, TMEM_COLS);
+}
+
+
+template <int HD, bool DIRECT>
+cudaError_t bwd_launch_t(const fbl_plan* p, AttnBwdParams& P, cudaStream_t st) {
+  auto k = attn_bwd_tc_kernel<HD, DIRECT>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwdSmem<HD>::TOTAL);
   if (e != cudaSuccess) return e;
-  P.batch = p->d.batch;
   // Q, dO (bf16) and the fp32 dQ accumulator of the query heads of one KV head.  The HD = 128 variant waits for
   // its single-buffered Q / dO tiles on the critical path, so it keeps the blocks that share those tiles close
   // together (small chunks: L2 hits); the pipelined HD = 64 variant hides that latency and prefers balance.
@@ -1074,7 +1357,39 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   return launch_pdl(k, grid, dim3(BWD_THREADS), BwdSmem<HD>::TOTAL, st, P);
 }
 
+template <int HD>
+cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* dA,
+                       const float* lse, const float* dvec, float* dqacc, void* dQ, void* dK, void* dV, int32_t* status,
+                       cudaStream_t st) {
+  AttnBwdParams P;
+  memset(&P, 0, sizeof(P));
+  const int panels = HD / 64;
+  if (!fbl_encode_rtile_map(&P.tq, Q, p->n_pad, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
+  if (!fbl_encode_rtile_map(&P.tdo, dA, p->n_pad, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
+  if (!fbl_encode_rtile_map(&P.tk, K, p->n_pad_kv, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
+  if (!fbl_encode_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
+  const bool direct = attn_bwd_tc_direct(p);
+  if (!direct && !fbl_encode_f32_panel_map(&P.tdq, dqacc, p->n_pad, p->dq / 64, BQ)) return cudaErrorInvalidValue;
+  P.lse = lse; P.dvec = dvec; P.dqacc = dqacc; P.dq = (__nv_bfloat16*)dQ; P.dk = (__nv_bfloat16*)dK; P.dv = (__nv_bfloat16*)dV;
+  P.n_pad = p->n_pad; P.seq = p->d.seq; P.t_pad = p->t_pad; P.hq = p->d.n_q_heads; P.group = p->group;
+  P.causal = p->d.causal; P.dkv = p->dkv; P.scale = p->scale; P.status = status;
+  P.n_pad_k = p->n_pad_kv; P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;
+  P.batch = p->d.batch;
+  if (!direct) return bwd_launch_t<HD, false>(p, P, st);
+  if (p->t_pad_kv <= BKV) return bwd_launch_t<HD, true>(p, P, st);
+  cudaError_t e = cudaFuncSetAttribute(attn_bwd_short_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ShortSmem::TOTAL);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(attn_bwd_short_kernel, dim3((unsigned)(P.hq * P.batch)), dim3(SHORT_THREADS), ShortSmem::TOTAL, st, P);
+}
+
 }  // namespace
+
+// Every block of the backward sees all keys of its queries, and writes dQ itself: sequences of one key tile, or of two key
+// and at most two query tiles where every query head has its own keys and head_dim is 64 (attn_bwd_short_kernel).
+bool attn_bwd_tc_direct(const fbl_plan* p) {
+  if (p->t_pad_kv <= BKV) return true;
+  return p->d.head_dim == 64 && p->group == 1 && p->t_pad_kv <= 2 * BKV && p->t_pad <= 2 * BQ;
+}
 
 bool attn_fwd_tc_supported(const fbl_plan* p) {
   return p->d.dtype == FBL_DTYPE_BF16 && (p->d.head_dim == 64 || p->d.head_dim == 128);   // boxes past the last row load zeros
@@ -1091,12 +1406,12 @@ cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, 
 cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,
                                const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
                                void* dV, bool dvec_ready, int32_t* status, cudaStream_t st) {
-  // dQ accumulator := 0, and D = rowsum(dO * O) unless the dA GEMM's epilogue already produced it
+  // D = rowsum(dO * O) unless the dA GEMM's epilogue already produced it
   cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, dvec_ready, st);
   if (e != cudaSuccess) return e;
-  if (p->d.head_dim == 64) e = bwd_launch<64>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, status, st);
-  else if (p->d.head_dim == 128) e = bwd_launch<128>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, status, st);
+  if (p->d.head_dim == 64) e = bwd_launch<64>(p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status, st);
+  else if (p->d.head_dim == 128) e = bwd_launch<128>(p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status, st);
   else e = cudaErrorInvalidValue;
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || attn_bwd_tc_direct(p)) return e;
   return launch_attn_bwd_post(p, dqacc, dQ, st);                      // fp32 accumulator -> storage dtype
 }

@@ -210,7 +210,7 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
   const int cols[3] = {p->dq, p->dkv, p->dkv};
   int k = 0;
 
-  LORA_CUDA(cudaMemsetAsync(status, 0, p->zero_bytes, st));    // status word and the dQ accumulator
+  LORA_CUDA(cudaMemsetAsync(status, 0, bwd_zero_bytes(p), st));    // status word and the dQ accumulator
   if (p->prof_on) { p->prof_n = 0; LORA_CUDA(cudaEventRecord(p->prof_ev[0], st)); }
   bool dvec_ready = false;
   {
@@ -227,7 +227,7 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     LORA_STEP("dA", 0, cudaSuccess);
     p->launches += k;
   }
-  if (p->use_tc && attn_bwd_tc_supported(p)) LORA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
+  if (p->use_tc && attn_bwd_tc_supported(p)) LORA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
   else LORA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   if (p->rope_base > 0.f) LORA_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   const void* G[3] = {dQ, dK, dV};

@@ -127,7 +127,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
   // one fill: status word, the accumulation areas of sliced weight-gradient products, the dQ accumulator.  It is
   // also the barrier between the forward pass's kernels and the backward's, which the attention backward relies on
   // when it requests forward-pass data before waiting for the kernel in front of it.
-  XA_CUDA(cudaMemsetAsync(status, 0, p->zero_bytes, st));
+  XA_CUDA(cudaMemsetAsync(status, 0, bwd_zero_bytes(p), st));
   XA_PROF_BEGIN();
   const bool split_o = p->use_tc && p->ksplit_o > 1, split_q = p->use_tc && p->ksplit_qkv > 1,
              split_kv = p->use_tc && p->ksplit_kv > 1;
@@ -156,7 +156,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     }
     XA_GEMM_STEP("dWo+dA", gs, 2);
   }
-  if (p->use_tc && attn_bwd_tc_supported(p)) XA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
+  if (p->use_tc && attn_bwd_tc_supported(p)) XA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
   else XA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   {
     // query side: dWq = Xn^T dQ (token-axis reduction), dXn = dQ Wq^T

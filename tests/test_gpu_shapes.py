@@ -93,3 +93,23 @@ def test_fp32_gemm_tiles_and_slices(cfg):
 def test_ragged_columns_on_every_gemm_tile(cfg, pair, monkeypatch):
     monkeypatch.setenv("FBL_GEMM_PAIR", pair)
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # one key tile (dQ straight from the block), with one and several query tiles, grouped heads, both head widths
+    LayerConfig("sa1", 2, 128, 128, 4, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 251, 0.05),
+    LayerConfig("sa2", 2, 97, 256, 2, 1, 128, "bf16", "rmsnorm", False, False, False, 1e-5, 252, 0.05),
+    XattnConfig("sa3", 2, 300, 120, 128, 64, 2, 1, 64, "bf16", "layernorm", True, True, 1e-5, 253, 0.05),
+    XattnConfig("sa4", 1, 129, 33, 128, 64, 2, 1, 128, "bf16", "layernorm", False, True, 1e-5, 254, 0.05),
+    # two key tiles and one or two query tiles in one block: full, ragged at either end, causal and not; then one past it
+    LayerConfig("sa5", 2, 256, 128, 2, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 255, 0.05),
+    LayerConfig("sa6", 2, 129, 192, 3, 3, 64, "bf16", "rmsnorm", True, False, False, 1e-5, 256, 0.05),
+    LayerConfig("sa7", 3, 255, 128, 2, 2, 64, "bf16", "layernorm", False, True, False, 1e-5, 257, 0.05),
+    LayerConfig("sa8", 2, 131, 128, 2, 2, 64, "bf16", "layernorm", False, False, True, 1e-5, 258, 0.05),
+    XattnConfig("sa9", 2, 60, 200, 128, 64, 2, 2, 64, "bf16", "layernorm", True, True, 1e-5, 259, 0.05),
+    XattnConfig("sa10", 2, 256, 130, 128, 192, 2, 2, 64, "bf16", "rmsnorm", True, True, 1e-5, 260, 0.05),
+    LayerConfig("sa11", 2, 257, 128, 2, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 261, 0.05),
+    XattnConfig("sa12", 2, 257, 256, 128, 64, 2, 2, 64, "bf16", "layernorm", True, True, 1e-5, 262, 0.05),
+], ids=lambda c: c.name)
+def test_attention_backward_of_short_sequences(cfg):
+    check(cfg)
