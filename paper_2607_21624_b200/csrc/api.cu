@@ -204,7 +204,8 @@ static int plan_build(const fbl_layer_desc* desc, int cross, int seq_kv_in, int 
   p->zero_bytes = o;
   p->sb_da = o;    o += mat(p->dq);
   p->sb_dvec = o;  o += fbl_align_up(rows_bh * sizeof(float), FBL_ALIGN);
-  p->sb_dq = o;    o += mat(p->dq);
+  if (d.dtype == FBL_DTYPE_FP32) p->sb_dq = p->sb_dqacc;      // fp32: the accumulator is dQ itself
+  else { p->sb_dq = o; o += mat(p->dq); }
   p->sb_dk = o;    o += mat_kv(p->dkv);
   p->sb_dv = o;    o += mat_kv(p->dkv);
   p->sb_dxn = o;   o += mat(d.d_model);
@@ -447,6 +448,7 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
   }
   if (p->rope_base > 0.f) FBL_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
   if (p->use_tc && attn_fwd_tc_supported(p)) FBL_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
+  else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
   else FBL_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
   {
     GemmArgs g = {};
@@ -536,6 +538,7 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     FBL_GEMM_STEP("dWo+dA", gs, 2, FBL_GEMM_DWO_DA);
   }
   if (p->use_tc && attn_bwd_tc_supported(p)) FBL_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));   // dqacc: zero already
+  else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
   else FBL_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   // back through the rotation of Q and K: its transpose is the rotation by the opposite angle
   if (p->rope_base > 0.f) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));

@@ -163,6 +163,13 @@ size_t colsum_scratch_bytes(int64_t rows, int64_t cols);
 cudaError_t launch_colsum_group(int dtype, int count, const void* const* M, int64_t rows, const int* cols,
                                 float* const* out, float* partials, cudaStream_t st);
 
+// fp32 storage (k_ffma_attn.cu); the backward adds into dQ, zeroed by the caller
+cudaError_t launch_attn_fwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
+                                 int32_t* status, cudaStream_t st);
+cudaError_t launch_attn_bwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A, const void* dA,
+                                 const float* lse, float* dvec, void* dQ, void* dK, void* dV, bool dvec_ready, int32_t* status,
+                                 cudaStream_t st);
+// bf16 storage in fp32 arithmetic (cross-check)
 cudaError_t launch_attn_fwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                  cudaStream_t st);
 cudaError_t launch_attn_bwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,

@@ -1,7 +1,7 @@
-// FP32-arithmetic kernels (plain FFMA, no tensor cores) on R-Tile matrices: the projection GEMMs and
-// the fused attention forward/backward.  They are the fp32 storage path (single-pass TF32 cannot
-// hold a 1e-4 relative bound) and accept bf16 storage too.  Every operand is addressed through the
-// R-Tile element map; "transposed" operands are the same tiles read with swapped index roles.
+// FP32-arithmetic kernels (plain FFMA, no tensor cores) for bf16 storage: the projection GEMM and the fused attention
+// forward/backward that cross-check the tensor-core kernels on the device (fp32 storage has kernels of its own), and the
+// small conversions of the backward.  Every operand is addressed through the R-Tile element map; "transposed" operands
+// are the same tiles read with swapped index roles.
 #include "fbl_internal.h"
 #include "pdl.cuh"
 
@@ -427,15 +427,8 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {
 
 cudaError_t launch_attn_fwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                  cudaStream_t st) {
-  const int hd = p->d.head_dim;
-  if (p->d.dtype == FBL_DTYPE_FP32) {
-    if (hd == 32) return attn_fwd_launch<float, 32>(p, Q, K, V, A, lse, st);
-    if (hd == 64) return attn_fwd_launch<float, 64>(p, Q, K, V, A, lse, st);
-    if (hd == 128) return attn_fwd_launch<float, 128>(p, Q, K, V, A, lse, st);
-  } else {
-    if (hd == 64) return attn_fwd_launch<__nv_bfloat16, 64>(p, Q, K, V, A, lse, st);
-    if (hd == 128) return attn_fwd_launch<__nv_bfloat16, 128>(p, Q, K, V, A, lse, st);
-  }
+  if (p->d.head_dim == 64) return attn_fwd_launch<__nv_bfloat16, 64>(p, Q, K, V, A, lse, st);
+  if (p->d.head_dim == 128) return attn_fwd_launch<__nv_bfloat16, 128>(p, Q, K, V, A, lse, st);
   return cudaErrorInvalidValue;
 }
 
@@ -457,8 +450,6 @@ cudaError_t launch_attn_bwd_pre(const fbl_plan* p, const void* A, const void* dA
 cudaError_t launch_attn_bwd_post(const fbl_plan* p, const float* dqacc, void* dQ, cudaStream_t st) {
   const int64_t nq = p->n_pad * p->dq;
   const int blocks = (int)min((int64_t)148 * 8, (nq / 4 + 255) / 256);
-  if (p->d.dtype == FBL_DTYPE_FP32)
-    return launch_pdl(convert_f32_kernel<float>, dim3(blocks), dim3(256), 0, st, dqacc, (float*)dQ, nq);
   return launch_pdl(convert_f32_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, dqacc, (__nv_bfloat16*)dQ, nq);
 }
 
@@ -475,15 +466,9 @@ cudaError_t launch_attn_bwd_simt(const fbl_plan* p, const void* Q, const void* K
   const int hd = p->d.head_dim;
   cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, dvec_ready, st);
   if (e != cudaSuccess) return e;
-  e = cudaErrorInvalidValue;
-  if (p->d.dtype == FBL_DTYPE_FP32) {
-    if (hd == 32) e = attn_bwd_launch<float, 32>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
-    else if (hd == 64) e = attn_bwd_launch<float, 64>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
-    else if (hd == 128) e = attn_bwd_launch<float, 128>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
-  } else {
-    if (hd == 64) e = attn_bwd_launch<__nv_bfloat16, 64>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
-    else if (hd == 128) e = attn_bwd_launch<__nv_bfloat16, 128>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
-  }
+  if (hd == 64) e = attn_bwd_launch<__nv_bfloat16, 64>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
+  else if (hd == 128) e = attn_bwd_launch<__nv_bfloat16, 128>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
+  else e = cudaErrorInvalidValue;
   if (e != cudaSuccess) return e;
   return launch_attn_bwd_post(p, dqacc, dQ, st);
 }

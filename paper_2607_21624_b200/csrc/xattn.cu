@@ -84,6 +84,7 @@ int fbl_xattn_fwd(const fbl_plan* p, const void* X, const void* M, const float* 
     XA_GEMM_STEP("proj_qkv", gs, 3);
   }
   if (p->use_tc && attn_fwd_tc_supported(p)) XA_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
+  else if (p->d.dtype == FBL_DTYPE_FP32) XA_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
   else XA_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
   {
     GemmArgs g = {};
@@ -157,6 +158,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     XA_GEMM_STEP("dWo+dA", gs, 2);
   }
   if (p->use_tc && attn_bwd_tc_supported(p)) XA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
+  else if (p->d.dtype == FBL_DTYPE_FP32) XA_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
   else XA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   {
     // query side: dWq = Xn^T dQ (token-axis reduction), dXn = dQ Wq^T

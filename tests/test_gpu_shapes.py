@@ -113,3 +113,16 @@ def test_ragged_columns_on_every_gemm_tile(cfg, pair, monkeypatch):
 ], ids=lambda c: c.name)
 def test_attention_backward_of_short_sequences(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # fp32 attention: one to many 32-row tiles, 64-key / 64-query tiles full, half and ragged, groups, all head widths
+    LayerConfig("fa1", 2, 33, 64, 2, 1, 32, "fp32", "layernorm", True, True, True, 1e-5, 271, 0.2),
+    LayerConfig("fa2", 1, 224, 64, 2, 2, 64, "fp32", "rmsnorm", True, False, False, 1e-5, 272, 0.1),
+    LayerConfig("fa3", 2, 161, 64, 4, 2, 64, "fp32", "layernorm", False, True, True, 1e-5, 273, 0.1),
+    LayerConfig("fa4", 2, 117, 64, 2, 1, 128, "fp32", "layernorm", True, True, False, 1e-5, 274, 0.1),
+    XattnConfig("fa5", 2, 97, 31, 64, 96, 2, 2, 128, "fp32", "layernorm", True, True, 1e-5, 275, 0.1),
+    XattnConfig("fa6", 2, 1, 130, 64, 64, 2, 1, 64, "fp32", "rmsnorm", True, True, 1e-5, 276, 0.1),
+], ids=lambda c: c.name)
+def test_fp32_attention_tiles(cfg):
+    check(cfg)
