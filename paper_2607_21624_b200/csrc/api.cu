@@ -158,6 +158,8 @@ static int plan_build(const fbl_layer_desc* desc, int cross, int seq_kv_in, int 
   p->sv_v = o;     o += mat_kv(p->dkv);
   p->sv_a = o;     o += mat(p->dq);
   p->sv_lse = o;   o += fbl_align_up(rows_bh * sizeof(float) + 512, FBL_ALIGN);   // + one 128-float copy window past the last row
+  p->sv_rope = o;
+  if (!cross) o += fbl_align_up((size_t)p->t_pad * (d.head_dim / 2) * sizeof(float2), FBL_ALIGN);
   p->saved_bytes = o;
 
   // Partial-sum area of the backward's token-axis reductions: the slab partials of the four bias column sums
@@ -423,12 +425,13 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
   int32_t* status = (int32_t*)sc;
   float* stats = (float*)(sv + p->sv_stats);
   void* Xn = sv + p->sv_xn; void* Q = sv + p->sv_q; void* K = sv + p->sv_k; void* V = sv + p->sv_v;
-  void* A = sv + p->sv_a; float* lse = (float*)(sv + p->sv_lse);
+  void* A = sv + p->sv_a; float* lse = (float*)(sv + p->sv_lse); float2* rope = (float2*)(sv + p->sv_rope);
   const bool bias = p->d.has_bias;
   const int n = (int)p->n_pad, D = p->d.d_model;
 
   FBL_PROF_BEGIN();
-  FBL_STEP("norm_fwd", 1, launch_norm_fwd(p, X, gamma, beta, Xn, stats, status, st));
+  FBL_STEP("norm_fwd", 1, launch_norm_fwd(p, X, gamma, beta, Xn, stats, status, st, p->rope_base > 0.f ? rope : nullptr));
+  bool rotated = false;
   {
     const void* W[3] = {Wq, Wk, Wv};
     void* O[3] = {Q, K, V};
@@ -444,9 +447,10 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
       g.c = O[i]; g.c_rpad = p->n_pad; g.bias = bias ? B[i] : nullptr;
       g.seq = p->d.seq; g.t_pad = p->t_pad;
     }
+    rotated = rope_in_projection(p, gs, rope);
     FBL_GEMM_STEP("proj_qkv", gs, 3, FBL_GEMM_PROJ_QKV);
   }
-  if (p->rope_base > 0.f) FBL_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
+  if (p->rope_base > 0.f && !rotated) FBL_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
   if (p->use_tc && attn_fwd_tc_supported(p)) FBL_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
   else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
   else FBL_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
@@ -485,6 +489,7 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
   void* dA = sc + p->sb_da; float* dvec = (float*)(sc + p->sb_dvec); float* dqacc = (float*)(sc + p->sb_dqacc);
   void* dQ = sc + p->sb_dq; void* dK = sc + p->sb_dk; void* dV = sc + p->sb_dv; void* dXn = sc + p->sb_dxn;
   void* part = sc + p->sb_part;
+  const float2* rope = p->rope_base > 0.f ? (const float2*)(sv + p->sv_rope) : nullptr;
   const bool bias = p->d.has_bias;
   const int n = (int)p->n_pad, D = p->d.d_model;
 
@@ -537,11 +542,11 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     }
     FBL_GEMM_STEP("dWo+dA", gs, 2, FBL_GEMM_DWO_DA);
   }
-  if (p->use_tc && attn_bwd_tc_supported(p)) FBL_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));   // dqacc: zero already
+  if (p->use_tc && attn_bwd_tc_supported(p)) FBL_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope));   // dqacc: zero already
   else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
   else FBL_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   // back through the rotation of Q and K: its transpose is the rotation by the opposite angle
-  if (p->rope_base > 0.f) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
+  if (p->rope_base > 0.f && !(p->use_tc && attn_bwd_tc_supported(p))) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   {
     const void* G[3] = {dQ, dK, dV};
     void* DW[3] = {dWq, dWk, dWv};

@@ -45,7 +45,7 @@ struct fbl_plan {
   int sm_count;
   int use_tc;   // 1: tensor-core (tcgen05) kernels where one exists for the shape; 0: FFMA kernels only
   // byte offsets inside `saved`
-  size_t sv_stats, sv_xn, sv_q, sv_k, sv_v, sv_a, sv_lse, saved_bytes;
+  size_t sv_stats, sv_xn, sv_q, sv_k, sv_v, sv_a, sv_lse, sv_rope, saved_bytes;   // sv_rope: the rotary embedding's table
   // byte offsets inside the backward scratch
   size_t sb_da, sb_dvec, sb_dqacc, sb_dq, sb_dk, sb_dv, sb_dxn, sb_part, scratch_bwd_bytes;
   size_t scratch_fwd_bytes;
@@ -111,7 +111,8 @@ struct GemmArgs {
   // fused activation of the feed-forward block (tensor-core kernel only): 0 none, 1 GELU forward (c = U, c2 = gelu(U)),
   // 2 GELU backward (c = value * gelu'(U), U in `residual`), 3 gated forward (c = G, c2 = silu(G) * U, U in `residual`),
   // 4 gated backward (c = value * silu(G), c2 = value * U * silu'(G); U in `residual`, G in `aux1`)
-  int epi; const void* aux1; void* c2;
+  // 5 rotary embedding of whole heads of rope_hd columns, with the table launch_norm_fwd leaves (see there)
+  int epi; const void* aux1; void* c2; const float2* rope; int rope_hd;
 };
 
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
@@ -133,6 +134,12 @@ cudaError_t run_gemm_group(const fbl_plan* p, GemmArgs* gs, int count, int32_t* 
 static inline bool gemm_fuses_dot(const fbl_plan* p, const GemmArgs& ga) {
   return p->d.dtype == FBL_DTYPE_FP32 ? p->d.head_dim <= 64 && gemm_ffma_supported(p, ga) : p->use_tc && gemm_tc_supported(p, ga);
 }
+// The rotary embedding in the epilogue of the Q and K projections (gs[0], gs[1] of three): true if it goes there.
+static inline bool rope_in_projection(const fbl_plan* p, GemmArgs* gs, const float2* table) {
+  if (!(p->rope_base > 0.f) || !gemm_group_tc(p, gs, 3)) return false;
+  for (int i = 0; i < 2; ++i) { gs[i].epi = 5; gs[i].rope = table; gs[i].rope_hd = p->d.head_dim; }
+  return true;
+}
 struct GemmShape { int64_t m; int n; int kblocks; int splittable; };
 int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count);
 cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles, cudaStream_t st);
@@ -144,14 +151,19 @@ bool attn_bwd_tc_direct(const fbl_plan* p);    // the tensor-core backward write
 static inline size_t bwd_zero_bytes(const fbl_plan* p) {
   return p->use_tc && attn_bwd_tc_supported(p) && attn_bwd_tc_direct(p) ? p->sb_dqacc : p->zero_bytes;
 }
-static inline int attn_bwd_tc_launches(const fbl_plan* p, bool dvec_ready) { return (dvec_ready ? 1 : 2) + (attn_bwd_tc_direct(p) ? 0 : 1); }
+static inline int attn_bwd_tc_launches(const fbl_plan* p, bool dvec_ready) {
+  return (dvec_ready ? 1 : 2) + (attn_bwd_tc_direct(p) && !(p->rope_base > 0.f) ? 0 : 1);
+}
 void fbl_note_cuda_error(cudaError_t e, const char* where);
 
 cudaError_t launch_pack(int dtype, int unpack, const void* src, void* dst, int64_t outer, int64_t rows,
                         int64_t rows_pad, int cols, cudaStream_t st);
+// fp32 dQ sums -> dQ in bf16, and dK in place, both turned back by the table's angles
+cudaError_t launch_rope_bwd_round(const fbl_plan* p, const float* acc, void* dQ, void* dK, const float2* rope, cudaStream_t st);
 cudaError_t launch_rope(const fbl_plan* p, void* A, int heads_a, void* B, int heads_b, int inverse, cudaStream_t st);
+// rope: where to leave the rotary embedding's table, [head_dim / 2][t_pad] (cosine, sine) of token t * base^(-2i/head_dim)
 cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
-                            float* stats, int32_t* status, cudaStream_t st);
+                            float* stats, int32_t* status, cudaStream_t st, float2* rope = nullptr);
 // counts its own launches in p->launches (one to three)
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                             const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
@@ -184,4 +196,4 @@ cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, 
                                int32_t* status, cudaStream_t st);
 cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,
                                const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
-                               void* dV, bool dvec_ready, int32_t* status, cudaStream_t st);
+                               void* dV, bool dvec_ready, int32_t* status, cudaStream_t st, const float2* rope = nullptr);

@@ -208,13 +208,24 @@ template <typename T, int NV, int PF, int TPR>
 __global__ void __launch_bounds__(512) norm_fwd_kernel(const T* __restrict__ X, const float* __restrict__ gamma,
                                                        const float* __restrict__ beta, T* __restrict__ Xn,
                                                        float* __restrict__ stats, int64_t n_pad, int d, int tpr_rt, int64_t per_block,
-                                                       int seq, int t_pad, int rms, float eps, int32_t* __restrict__ status) {
+                                                       int seq, int t_pad, int rms, float eps, int32_t* __restrict__ status,
+                                                       int n_norm, float2* __restrict__ rope, int rope_half, float rope_k) {
   constexpr int V = Vec16<T>::N, TW = tile_w_of<T>::value;
   __shared__ __align__(16) float s_ex[2 * NORM_EX];
   // First kernel of the forward pass: it resets the pass's status word (later kernels only write it after a
   // bounded wait of about a second has expired), which saves a fill node in front of the pass.
   if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
   pdl_launch_dependents();
+  if ((int)blockIdx.x >= n_norm) {                           // blocks behind the norm's: the rotary embedding's table
+    pdl_wait();
+    const int i = ((int)blockIdx.x - n_norm) * (int)blockDim.x + (int)threadIdx.x;
+    if (i < rope_half * t_pad) {
+      float sn, cs;
+      sincosf((float)(i % t_pad) * exp2f((float)(i / t_pad) * rope_k), &sn, &cs);
+      rope[i] = make_float2(cs, sn);
+    }
+    return;
+  }
   const int tpr = TPR ? TPR : tpr_rt;
   const int group = threadIdx.x / tpr, lt = threadIdx.x % tpr, groups = blockDim.x / tpr;
   const float inv_d = 1.f / (float)d;
@@ -285,6 +296,47 @@ __global__ void __launch_bounds__(512) norm_fwd_kernel(const T* __restrict__ X, 
       }
       rb += groups;
     }
+  }
+}
+
+// The rotation back of dQ, on its way from the fp32 accumulator to bf16, and of dK in place: one launch for both and the
+// rounding.  A thread takes 8 columns of a head's low half and the matching 8 of its high half.
+__global__ void __launch_bounds__(256) rope_bwd_round_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, int heads_q,
+                                                             __nv_bfloat16* __restrict__ dk, int heads_k, int64_t n_pad, int seq,
+                                                             int t_pad, int hd, const float2* __restrict__ rope) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int half = hd / 2, vec = half / 8;
+  const int64_t per_q = n_pad * heads_q * vec, total = per_q + n_pad * heads_k * vec;
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
+    const bool is_k = idx >= per_q;
+    int64_t rem = is_k ? idx - per_q : idx;
+    const int v = (int)(rem % vec);
+    rem /= vec;
+    const int64_t r = rem % n_pad;
+    const int h = (int)(rem / n_pad), t = (int)(r % t_pad);
+    const int64_t lo_off = rt_off<64>(n_pad, r, h * hd + v * 8), hi_off = rt_off<64>(n_pad, r, h * hd + half + v * 8);
+    float lo[8], hi[8];
+    if (is_k) {
+      load16(dk + lo_off, lo);
+      load16(dk + hi_off, hi);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; i += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(acc + lo_off + i), b = *reinterpret_cast<const float4*>(acc + hi_off + i);
+        lo[i] = a.x; lo[i + 1] = a.y; lo[i + 2] = a.z; lo[i + 3] = a.w;
+        hi[i] = b.x; hi[i + 1] = b.y; hi[i + 2] = b.z; hi[i + 3] = b.w;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float2 cs = rope[(int64_t)(v * 8 + i) * t_pad + t];
+      const float a = lo[i], b = hi[i];
+      lo[i] = a * cs.x + b * cs.y;
+      hi[i] = b * cs.x - a * cs.y;
+    }
+    store16((is_k ? dk : dq) + lo_off, lo);
+    store16((is_k ? dk : dq) + hi_off, hi);
   }
 }
 
@@ -605,12 +657,15 @@ __global__ void __launch_bounds__(256) colsum_stage1(const __grid_constant__ Col
 
 template <typename T, int NV, int PF, int TPR>
 cudaError_t norm_fwd_launch(const fbl_plan* p, const NormShape& s, const void* X, const float* gamma, const float* beta,
-                            void* Xn, float* stats, int32_t* status, cudaStream_t st) {
+                            void* Xn, float* stats, int32_t* status, float2* rope, cudaStream_t st) {
   const int64_t blocks = min((int64_t)p->sm_count * (NV == 1 ? 4 : 2), (p->n_pad + s.groups - 1) / s.groups);
   const int64_t per_block = ((p->n_pad + blocks - 1) / blocks + s.groups - 1) / s.groups * s.groups;
-  return launch_pdl(norm_fwd_kernel<T, NV, PF, TPR>, dim3((unsigned)((p->n_pad + per_block - 1) / per_block)), dim3(s.tpr * s.groups), 0, st,
+  const int threads = s.tpr * s.groups, n_norm = (int)((p->n_pad + per_block - 1) / per_block), half = p->d.head_dim / 2;
+  const int extra = rope ? (half * p->t_pad + threads - 1) / threads : 0;
+  return launch_pdl(norm_fwd_kernel<T, NV, PF, TPR>, dim3((unsigned)(n_norm + extra)), dim3(threads), 0, st,
                     (const T*)X, gamma, beta, (T*)Xn, stats, p->n_pad, p->d.d_model, s.tpr, per_block, p->d.seq, p->t_pad,
-                    (int)(p->d.norm == FBL_NORM_RMSNORM), p->d.eps, status);
+                    (int)(p->d.norm == FBL_NORM_RMSNORM), p->d.eps, status, n_norm, rope, half,
+                    rope ? -2.f * log2f(p->rope_base) / (float)p->d.head_dim : 0.f);
 }
 
 template <typename T, int NV, int R>
@@ -707,9 +762,9 @@ cudaError_t launch_rope(const fbl_plan* p, void* A, int heads_a, void* B, int he
 
 template <typename T>
 cudaError_t norm_fwd_dispatch(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
-                              float* stats, int32_t* status, cudaStream_t st) {
+                              float* stats, int32_t* status, float2* rope, cudaStream_t st) {
   const NormShape s = norm_fwd_shape(p->d.d_model / Vec16<T>::N);
-#define FBL_CALL(NV_, PF_, TPR_) norm_fwd_launch<T, NV_, PF_, TPR_>(p, s, X, gamma, beta, Xn, stats, status, st)
+#define FBL_CALL(NV_, PF_, TPR_) norm_fwd_launch<T, NV_, PF_, TPR_>(p, s, X, gamma, beta, Xn, stats, status, rope, st)
   switch (s.nv) {
     case 1: return s.tpr == 32 ? FBL_CALL(1, 4, 32) : FBL_CALL(1, 4, 0);
     case 2:
@@ -723,11 +778,18 @@ cudaError_t norm_fwd_dispatch(const fbl_plan* p, const void* X, const float* gam
 #undef FBL_CALL
 }
 
+cudaError_t launch_rope_bwd_round(const fbl_plan* p, const float* acc, void* dQ, void* dK, const float2* rope, cudaStream_t st) {
+  const int64_t total = p->n_pad * (int64_t)(p->d.n_q_heads + p->d.n_kv_heads) * (p->d.head_dim / 16);
+  const int blocks = (int)min((int64_t)p->sm_count * 16, (total + 255) / 256);
+  return launch_pdl(rope_bwd_round_kernel, dim3(blocks), dim3(256), 0, st, acc, (__nv_bfloat16*)dQ, p->d.n_q_heads, (__nv_bfloat16*)dK,
+                    p->d.n_kv_heads, p->n_pad, p->d.seq, p->t_pad, p->d.head_dim, rope);
+}
+
 cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
-                            float* stats, int32_t* status, cudaStream_t st) {
+                            float* stats, int32_t* status, cudaStream_t st, float2* rope) {
   if (p->d.norm == FBL_NORM_RMSNORM) beta = nullptr;
-  return p->d.dtype == FBL_DTYPE_FP32 ? norm_fwd_dispatch<float>(p, X, gamma, beta, Xn, stats, status, st)
-                                      : norm_fwd_dispatch<__nv_bfloat16>(p, X, gamma, beta, Xn, stats, status, st);
+  return p->d.dtype == FBL_DTYPE_FP32 ? norm_fwd_dispatch<float>(p, X, gamma, beta, Xn, stats, status, rope, st)
+                                      : norm_fwd_dispatch<__nv_bfloat16>(p, X, gamma, beta, Xn, stats, status, rope, st);
 }
 
 template <typename T>

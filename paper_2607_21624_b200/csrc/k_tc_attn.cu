@@ -1405,13 +1405,17 @@ cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, 
 
 cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,
                                const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
-                               void* dV, bool dvec_ready, int32_t* status, cudaStream_t st) {
+                               void* dV, bool dvec_ready, int32_t* status, cudaStream_t st, const float2* rope) {
   // D = rowsum(dO * O) unless the dA GEMM's epilogue already produced it
   cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, dvec_ready, st);
   if (e != cudaSuccess) return e;
   if (p->d.head_dim == 64) e = bwd_launch<64>(p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status, st);
   else if (p->d.head_dim == 128) e = bwd_launch<128>(p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status, st);
   else e = cudaErrorInvalidValue;
-  if (e != cudaSuccess || attn_bwd_tc_direct(p)) return e;
-  return launch_attn_bwd_post(p, dqacc, dQ, st);                      // fp32 accumulator -> storage dtype
+  if (e != cudaSuccess) return e;
+  // dQ: fp32 accumulator -> storage dtype where the kernel has not written it; with the rotary embedding (`rope`: the
+  // forward's table) dQ and dK are turned back by the opposite angle on the way
+  if (attn_bwd_tc_direct(p)) return rope ? launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st) : cudaSuccess;
+  if (rope) return launch_rope_bwd_round(p, dqacc, dQ, dK, rope, st);
+  return launch_attn_bwd_post(p, dqacc, dQ, st);
 }

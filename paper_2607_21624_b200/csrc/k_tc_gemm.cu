@@ -43,6 +43,9 @@ struct alignas(64) TcProblem {
   // operand U instead of a residual, `aux1` at the second one, G; `tc2` is the second output's map):
   //   1 GELU forward    C = v (U), C2 = gelu(v)           2 GELU backward    C = v gelu'(U)
   //   3 gated forward   C = v (G), C2 = silu(v) U          4 gated backward   C = v silu(G), C2 = v U silu'(G)
+  //   5 rotary embedding C = v with each head's (i, i + rope_hd / 2) pairs turned by the table's angle of the row's token
+  const float2* rope;      // [rope_hd / 2][t_pad] cosine and sine
+  int rope_hd;
   int epi;
   const __nv_bfloat16* aux1;
   CUtensorMap tc2;
@@ -104,10 +107,6 @@ __device__ __forceinline__ bool tile_at(const TcGroup& G, int w, TileCoord* tc_o
   return false;
 }
 
-// Persistent kernel: one block per SM walks the work list with stride gridDim.x.  Warp 0 feeds the
-// shared-memory ring by TMA, warp 1 issues the MMAs into one of two TMEM accumulators, warps 2-5 drain the
-// other accumulator (bias, residual, padding-row mask, bf16 rows in R-Tile order), so the epilogue of
-// one tile overlaps the main loop of the next.
 __device__ __forceinline__ float tanh_fast(float x) {
   float y;
   asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -120,7 +119,284 @@ __device__ __forceinline__ float gelu_grad_fast(float u) {
 }
 __device__ __forceinline__ float sigmoid_fast(float g) { return __fdividef(1.f, 1.f + __expf(-g)); }
 
-template <int BN, int STAGES, int ESETS, bool EPI = false>
+// One output tile of a CTA's 128 accumulator rows: TMEM -> registers -> swizzled staging -> bulk tensor store.  Each warp
+// owns the 32 rows of its TMEM lane quarter and its staging tiles, and issues its own stores: no block-wide hand-off per
+// panel, and the store of one panel overlaps the conversion of the next.  `acc`: the warp's lanes of the accumulator;
+// `wait`: waits until it is complete (what does not depend on it is requested first).
+// ESETS = 2 (launches in which every block has a single tile, so that nothing overlaps its epilogue): two sets of four
+// warps share the tile's 64-column panels, first and second half, and the epilogue takes half as long.  Each warp then
+// has one staging tile instead of two (the staging area is the same size).
+// EPI: what the instantiation can fuse besides bias, residual and the row reduction.
+enum { EPI_NONE = 0, EPI_ACT, EPI_ROPE };
+template <int BN, int ESETS, int EPI, typename Wait>
+__device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0, uint32_t acc, uint32_t stg0, int& pc, Wait wait) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, q = warp % 4, set = (warp - 2) / 4;
+  constexpr int PPS = BN / 64 / ESETS;              // panels per set
+  const int row = m0 + q * 32 + lane;               // row of the problem owned by this thread
+  const bool pad = P.t_pad > 0 && (row % P.t_pad) >= P.seq;
+  const bool has_res = P.residual && row < P.m;
+  // a head of the fused row reduction, or of the rotation, must stay within one warp: where it spans more panels than a set has, the
+  // first set takes the whole tile
+  const bool whole = ESETS == 2 && ((P.dot_with && P.dot_hd > 64 * PPS) || (EPI == EPI_ROPE && P.epi == 5 && P.rope_hd > 64 * PPS));
+  const int pn_begin = set == 0 ? 0 : (whole ? BN / 64 : PPS);
+  const int pn_end = ESETS == 1 ? BN / 64 : (set == 0 ? (whole ? BN / 64 : PPS) : BN / 64);
+  uint4 rv[8];                                    // residual values of the next panel, requested a panel ahead
+  if (has_res && pn_begin < pn_end && n0 + pn_begin * 64 < P.n) {
+    const __nv_bfloat16* rp = P.residual + ((long long)(n0 / 64 + pn_begin) * P.c_rpad + row) * 64;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
+  }
+  uint4 rv2[EPI == EPI_ACT ? 8 : 1];                         // second extra operand of a fused activation, likewise
+  if constexpr (EPI == EPI_ACT) {
+    if (P.epi == 4 && row < P.m && pn_begin < pn_end && n0 + pn_begin * 64 < P.n) {
+      const __nv_bfloat16* rp = P.aux1 + ((long long)(n0 / 64 + pn_begin) * P.c_rpad + row) * 64;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) rv2[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
+    }
+  }
+  const float* bias = P.bias;
+  float bl[BN / 32];                              // this tile's bias: lane l holds columns l*BN/32 ... (requested
+  if (bias) {                                     // while the MMAs run, handed out by shuffles below)
+#pragma unroll
+    for (int k = 0; k < BN / 32; ++k) {
+      const int c = n0 + lane * (BN / 32) + k;
+      bl[k] = c < P.n ? bias[c] : 0.f;
+    }
+  }
+  if (!wait()) return false;
+  tc::tc_fence_after();
+  float dot_acc = 0.f;
+#pragma unroll 1
+  for (int pn = pn_begin; pn < pn_end; ++pn) {
+    const int n = n0 + pn * 64;
+    if (n >= P.n) break;                           // uniform: N is whole 64-column panels
+    uint32_t v[64];
+    tc::tmem_ld32(acc + pn * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+    tc::tmem_ld32(acc + pn * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+    tc::tmem_ld_wait();
+    if (P.ksplit > 1) {
+      // partial sums of a reduction slice: two 32-column halves of the panel, fp32, added to the accumulation
+      // buffer by bulk tensor reductions (same staging tiles and swizzle as the bf16 rows below)
+#pragma unroll 1
+      for (int hf = 0; hf < 2; ++hf) {
+        const uint32_t stg = stg0 + (ESETS == 2 ? (uint32_t)(warp - 2) : (uint32_t)(q * 2 + (pc & 1))) * 4096u;
+        if (ESETS == 2 && lane == 0) tc::bulk_wait_group_read0();     // the single staging tile's previous contents have been read
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
+                       "r"(hf ? v[32 + 4 * j] : v[4 * j]), "r"(hf ? v[33 + 4 * j] : v[4 * j + 1]),
+                       "r"(hf ? v[34 + 4 * j] : v[4 * j + 2]), "r"(hf ? v[35 + 4 * j] : v[4 * j + 3]) : "memory");
+        tc::fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+          tc::tma_reduce_add_4d(&P.tacc, stg, 0, hf, m0 + q * 32, n / 64);
+          tc::bulk_commit_group();
+          if (ESETS == 1) tc::bulk_wait_group_read1();
+        }
+        ++pc;
+      }
+      continue;
+    }
+    if constexpr (EPI == EPI_ACT) {
+      if (P.epi != 0) {
+        // ---- fused activation: one or two outputs from this panel ------------------------------------
+        if (bias) {
+#pragma unroll
+          for (int j = 0; j < 64; ++j)
+            v[j] = __float_as_uint(__uint_as_float(v[j]) + __shfl_sync(0xffffffffu, bl[j % (BN / 32)], (pn * 64 + j) / (BN / 32)));
+        }
+        uint4 o1[8], o2[8];
+        uint32_t* w1 = reinterpret_cast<uint32_t*>(o1);
+        uint32_t* w2 = reinterpret_cast<uint32_t*>(o2);
+        const bool live = !pad && row < P.m;
+        const __nv_bfloat16* a0 = reinterpret_cast<const __nv_bfloat16*>(rv);
+        const __nv_bfloat16* a1 = reinterpret_cast<const __nv_bfloat16*>(rv2);
+        const float keep = live ? 1.f : 0.f;            // padding rows and rows past the matrix are written as zero
+        if (P.epi == 1) {
+#pragma unroll
+          for (int j = 0; j < 64; j += 2) {
+            const float x0 = __uint_as_float(v[j]) * keep, x1 = __uint_as_float(v[j + 1]) * keep;
+            w1[j / 2] = tc::pack_bf16(x0, x1);
+            w2[j / 2] = tc::pack_bf16(gelu_fast(x0), gelu_fast(x1));
+          }
+        } else if (P.epi == 2) {
+#pragma unroll
+          for (int j = 0; j < 64; j += 2) {
+            const float x0 = __uint_as_float(v[j]) * keep, x1 = __uint_as_float(v[j + 1]) * keep;
+            w1[j / 2] = tc::pack_bf16(x0 * gelu_grad_fast(__bfloat162float(a0[j])), x1 * gelu_grad_fast(__bfloat162float(a0[j + 1])));
+          }
+        } else if (P.epi == 3) {
+#pragma unroll
+          for (int j = 0; j < 64; j += 2) {
+            const float x0 = __uint_as_float(v[j]) * keep, x1 = __uint_as_float(v[j + 1]) * keep;
+            w1[j / 2] = tc::pack_bf16(x0, x1);
+            w2[j / 2] = tc::pack_bf16(x0 * sigmoid_fast(x0) * __bfloat162float(a0[j]), x1 * sigmoid_fast(x1) * __bfloat162float(a0[j + 1]));
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 64; j += 2) {
+            float y1[2], y2[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const float x = __uint_as_float(v[j + u]) * keep;
+              const float uu = __bfloat162float(a0[j + u]), gg = __bfloat162float(a1[j + u]), sg = sigmoid_fast(gg);
+              y1[u] = x * gg * sg;
+              y2[u] = x * uu * sg * (1.f + gg * (1.f - sg));
+            }
+            w1[j / 2] = tc::pack_bf16(y1[0], y1[1]);
+            w2[j / 2] = tc::pack_bf16(y2[0], y2[1]);
+          }
+        }
+        // the next panel's extra operands, requested while this panel's stores are under way
+        if (pn + 1 < pn_end && n + 64 < P.n && row < P.m) {
+          if (P.epi >= 2) {
+            const __nv_bfloat16* rp = P.residual + ((long long)(n / 64 + 1) * P.c_rpad + row) * 64;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
+          }
+          if (P.epi == 4) {
+            const __nv_bfloat16* rp = P.aux1 + ((long long)(n / 64 + 1) * P.c_rpad + row) * 64;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) rv2[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
+          }
+        }
+        const int n_out = (P.epi == 2) ? 1 : 2;
+#pragma unroll 1
+        for (int oi = 0; oi < n_out; ++oi) {
+          const uint4* ov = oi ? o2 : o1;
+          const uint32_t stg = stg0 + (ESETS == 2 ? (uint32_t)(warp - 2) : (uint32_t)(q * 2 + (pc & 1))) * 4096u;
+          if (ESETS == 2 && lane == 0) tc::bulk_wait_group_read0();
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
+                         "r"(ov[j].x), "r"(ov[j].y), "r"(ov[j].z), "r"(ov[j].w) : "memory");
+          tc::fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) {
+            tc::tma_store_3d(oi ? &P.tc2 : &P.tc, stg, 0, m0 + q * 32, n / 64);
+            tc::bulk_commit_group();
+            if (ESETS == 1) tc::bulk_wait_group_read1();
+          }
+          ++pc;
+        }
+        continue;
+      }
+    }
+    bool bias_left = bias != nullptr;
+    if constexpr (EPI == EPI_ROPE) {
+      if (P.epi == 5) {
+        // rotation of a head's (i, i + hd / 2) column pairs; the table has a frequency's tokens next to each other, as
+        // the lanes have their rows
+        const float2* tab = P.rope + row % P.t_pad;
+        if (bias) {
+#pragma unroll
+          for (int j = 0; j < 64; ++j)
+            v[j] = __float_as_uint(__uint_as_float(v[j]) + __shfl_sync(0xffffffffu, bl[j % (BN / 32)], (pn * 64 + j) / (BN / 32)));
+          bias_left = false;
+        }
+        if (P.rope_hd == 64) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const float2 cs = tab[(long long)j * P.t_pad];
+            const float a = __uint_as_float(v[j]), b = __uint_as_float(v[j + 32]);
+            v[j] = __float_as_uint(a * cs.x - b * cs.y);
+            v[j + 32] = __float_as_uint(b * cs.x + a * cs.y);
+          }
+        } else {                                     // 128: the partner is the same column of the neighbouring panel
+          const float sign = (n / 64) & 1 ? 1.f : -1.f;
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t w[32];
+            tc::tmem_ld32(acc + (pn ^ 1) * 64 + hf * 32, w);
+            tc::tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const float2 cs = tab[(long long)(hf * 32 + j) * P.t_pad];
+              float b = __uint_as_float(w[j]);
+              if (bias) b += __shfl_sync(0xffffffffu, bl[(hf * 32 + j) % (BN / 32)], ((pn ^ 1) * 64 + hf * 32 + j) / (BN / 32));
+              v[hf * 32 + j] = __float_as_uint(__uint_as_float(v[hf * 32 + j]) * cs.x + sign * b * cs.y);
+            }
+          }
+        }
+      }
+    }
+    uint4 outv[8];
+    uint32_t* ow = reinterpret_cast<uint32_t*>(outv);
+    if (has_res) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const __nv_bfloat16* rb = reinterpret_cast<const __nv_bfloat16*>(&rv[j]);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[8 * j + k] = __float_as_uint(__uint_as_float(v[8 * j + k]) + __bfloat162float(rb[k]));
+      }
+      if (pn + 1 < pn_end && n + 64 < P.n) {
+        const __nv_bfloat16* rp = P.residual + ((long long)(n / 64 + 1) * P.c_rpad + row) * 64;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
+      }
+    }
+    if (bias_left) {
+#pragma unroll
+      for (int j = 0; j < 64; j += 2) {
+        // column pn*64 + j is register (j % (BN/32)) of lane (pn*64 + j) / (BN/32)
+        const float b0 = __shfl_sync(0xffffffffu, bl[j % (BN / 32)], (pn * 64 + j) / (BN / 32));
+        const float b1 = __shfl_sync(0xffffffffu, bl[(j + 1) % (BN / 32)], (pn * 64 + j + 1) / (BN / 32));
+        ow[j / 2] = tc::pack_bf16(pad ? 0.f : __uint_as_float(v[j]) + b0, pad ? 0.f : __uint_as_float(v[j + 1]) + b1);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 64; j += 2)
+        ow[j / 2] = tc::pack_bf16(pad ? 0.f : __uint_as_float(v[j]), pad ? 0.f : __uint_as_float(v[j + 1]));
+    }
+    if (P.dot_with && row < P.m) {
+      // Row reduction over this head's columns, on the ROUNDED values the attention backward will read:
+      // sum_j dS_ij = 0 (softmax shift invariance) holds only if D matches the dP that kernel forms.
+      const __nv_bfloat16* ap = P.dot_with + ((long long)(n / 64) * P.c_rpad + row) * 64;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint4 av = *reinterpret_cast<const uint4*>(ap + 8 * j);
+        const __nv_bfloat16* ab16 = reinterpret_cast<const __nv_bfloat16*>(&av);
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+          const uint32_t w2 = ow[4 * j + k / 2];        // two bf16: low half = even column
+          dot_acc = fmaf(__uint_as_float(w2 << 16), __bfloat162float(ab16[k]), dot_acc);
+          dot_acc = fmaf(__uint_as_float(w2 & 0xffff0000u), __bfloat162float(ab16[k + 1]), dot_acc);
+        }
+      }
+      if ((n + 64) % P.dot_hd == 0) {                 // last panel of a head
+        const int hh = n / P.dot_hd, bb = row / P.t_pad, tt = row % P.t_pad;
+        P.dot_out[((long long)bb * P.dot_hq + hh) * P.t_pad + tt] = dot_acc;
+        dot_acc = 0.f;
+      }
+    }
+    // Staging tile (pc & 1) of this warp: its previous store (two panels ago) has been read, since lane 0
+    // waited for that after committing the store of the panel before this one.
+    const uint32_t stg = stg0 + (ESETS == 2 ? (uint32_t)(warp - 2) : (uint32_t)(q * 2 + (pc & 1))) * 4096u;
+    if (ESETS == 2 && lane == 0) tc::bulk_wait_group_read0();    // one staging tile: the store before has read it
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
+                   "r"(outv[j].x), "r"(outv[j].y), "r"(outv[j].z), "r"(outv[j].w) : "memory");
+    tc::fence_proxy_async();
+    __syncwarp();
+    if (lane == 0) {
+      tc::tma_store_3d(&P.tc, stg, 0, m0 + q * 32, n / 64);
+      tc::bulk_commit_group();
+      if (ESETS == 1) tc::bulk_wait_group_read1();  // the store before this one has read its staging tile
+    }
+    ++pc;
+  }
+  return true;
+}
+
+// Persistent kernel: one block per SM walks the work list with stride gridDim.x.  Warp 0 feeds the
+// shared-memory ring by TMA, warp 1 issues the MMAs into one of two TMEM accumulators, warps 2-5 drain the
+// other accumulator (bias, residual, padding-row mask, bf16 rows in R-Tile order), so the epilogue of
+// one tile overlaps the main loop of the next.
+template <int BN, int STAGES, int ESETS, int EPI>
 __global__ void __launch_bounds__(64 + 128 * ESETS, 1) gemm_tc_kernel(const __grid_constant__ TcGroup G) {
   using SP = SmemPlan<BN, STAGES>;
   extern __shared__ uint8_t smem_raw[];
@@ -241,243 +517,20 @@ __global__ void __launch_bounds__(64 + 128 * ESETS, 1) gemm_tc_kernel(const __gr
       if (ok) tc::mma_commit(acc_full(ab));
     }
   } else if (warp >= 2) {
-    // ---- epilogue: TMEM -> registers -> swizzled staging -> bulk tensor store.  Each warp owns the 32 rows of
-    // its TMEM lane quarter and two 32 x 64 staging tiles, and issues its own stores: no block-wide hand-off per
-    // panel, and the store of one panel overlaps the conversion of the next. ---------------------------------
+    // ---- epilogue warps ---------------------------------------------------------------------------
     pdl_wait();                                       // the previous kernel may still be reading what we overwrite
     group_chores(G, threadIdx.x - 64, 128 * ESETS);
     const int q = warp % 4;                           // the TMEM lane quarter this warp may access
-    // ESETS = 2 (launches in which every block has a single tile, so that nothing overlaps its epilogue): two sets
-    // of four warps share the tile's 64-column panels, first and second half, and the epilogue takes half as long.
-    // Each warp then has one staging tile instead of two (the staging area is the same size).
-    const int set = (warp - 2) / 4;
-    constexpr int PPS = BN / 64 / ESETS;              // panels per set
-    const int r = q * 32 + lane;                      // row of the tile owned by this thread
     int ti = 0, pc = 0;                               // tiles and panels done by this warp
     bool ok = true;
     TileCoord tcd;
     for (int w = blockIdx.x; ok && tile_at<BN>(G, w, &tcd); w += gridDim.x, ++ti) {
       const TcProblem& P = G.p[tcd.prob];
       const int ab = ti & 1;
-      const int row = tcd.m0 + r;
-      const bool pad = P.t_pad > 0 && (row % P.t_pad) >= P.seq;
-      const bool has_res = P.residual && row < P.m;
-      // a head of the fused row reduction must stay within one warp: where it spans more panels than a set has, the
-      // first set takes the whole tile
-      const bool whole = ESETS == 2 && P.dot_with && P.dot_hd > 64 * PPS;
-      const int pn_begin = set == 0 ? 0 : (whole ? BN / 64 : PPS);
-      const int pn_end = ESETS == 1 ? BN / 64 : (set == 0 ? (whole ? BN / 64 : PPS) : BN / 64);
-      uint4 rv[8];                                    // residual values of the next panel, requested a panel ahead
-      if (has_res && pn_begin < pn_end && tcd.n0 + pn_begin * 64 < P.n) {
-        const __nv_bfloat16* rp = P.residual + ((long long)(tcd.n0 / 64 + pn_begin) * P.c_rpad + row) * 64;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
-      }
-      uint4 rv2[EPI ? 8 : 1];                         // second extra operand of a fused activation, likewise
-      if constexpr (EPI) {
-        if (P.epi == 4 && row < P.m && pn_begin < pn_end && tcd.n0 + pn_begin * 64 < P.n) {
-          const __nv_bfloat16* rp = P.aux1 + ((long long)(tcd.n0 / 64 + pn_begin) * P.c_rpad + row) * 64;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) rv2[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
-        }
-      }
-      const float* bias = P.bias;
-      float bl[BN / 32];                              // this tile's bias: lane l holds columns l*BN/32 ... (requested
-      if (bias) {                                     // while the MMAs run, handed out by shuffles below)
-#pragma unroll
-        for (int k = 0; k < BN / 32; ++k) {
-          const int c = tcd.n0 + lane * (BN / 32) + k;
-          bl[k] = c < P.n ? bias[c] : 0.f;
-        }
-      }
-      if (!tc::mbar_wait(acc_full(ab), (ti >> 1) & 1, status, 103)) { ok = false; break; }
-      tc::tc_fence_after();
-      float dot_acc = 0.f;
-#pragma unroll 1
-      for (int pn = pn_begin; pn < pn_end; ++pn) {
-        const int n = tcd.n0 + pn * 64;
-        if (n >= P.n) break;                           // uniform: N is whole 64-column panels
-        uint32_t v[64];
-        tc::tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN + pn * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-        tc::tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN + pn * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-        tc::tmem_ld_wait();
-        if (P.ksplit > 1) {
-          // partial sums of a reduction slice: two 32-column halves of the panel, fp32, added to the accumulation
-          // buffer by bulk tensor reductions (same staging tiles and swizzle as the bf16 rows below)
-#pragma unroll 1
-          for (int hf = 0; hf < 2; ++hf) {
-            const uint32_t stg = base + SP::STG_OFF + (ESETS == 2 ? (uint32_t)(warp - 2) : (uint32_t)(q * 2 + (pc & 1))) * 4096u;
-            if (ESETS == 2 && lane == 0) tc::bulk_wait_group_read0();     // the single staging tile's previous contents have been read
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
-                           "r"(hf ? v[32 + 4 * j] : v[4 * j]), "r"(hf ? v[33 + 4 * j] : v[4 * j + 1]),
-                           "r"(hf ? v[34 + 4 * j] : v[4 * j + 2]), "r"(hf ? v[35 + 4 * j] : v[4 * j + 3]) : "memory");
-            tc::fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) {
-              tc::tma_reduce_add_4d(&P.tacc, stg, 0, hf, tcd.m0 + q * 32, n / 64);
-              tc::bulk_commit_group();
-              if (ESETS == 1) tc::bulk_wait_group_read1();
-            }
-            ++pc;
-          }
-          continue;
-        }
-        if constexpr (EPI) {
-          if (P.epi != 0) {
-            // ---- fused activation: one or two outputs from this panel ------------------------------------
-            if (bias) {
-#pragma unroll
-              for (int j = 0; j < 64; ++j)
-                v[j] = __float_as_uint(__uint_as_float(v[j]) + __shfl_sync(0xffffffffu, bl[j % (BN / 32)], (pn * 64 + j) / (BN / 32)));
-            }
-            uint4 o1[8], o2[8];
-            uint32_t* w1 = reinterpret_cast<uint32_t*>(o1);
-            uint32_t* w2 = reinterpret_cast<uint32_t*>(o2);
-            const bool live = !pad && row < P.m;
-            const __nv_bfloat16* a0 = reinterpret_cast<const __nv_bfloat16*>(rv);
-            const __nv_bfloat16* a1 = reinterpret_cast<const __nv_bfloat16*>(rv2);
-            const float keep = live ? 1.f : 0.f;            // padding rows and rows past the matrix are written as zero
-            if (P.epi == 1) {
-#pragma unroll
-              for (int j = 0; j < 64; j += 2) {
-                const float x0 = __uint_as_float(v[j]) * keep, x1 = __uint_as_float(v[j + 1]) * keep;
-                w1[j / 2] = tc::pack_bf16(x0, x1);
-                w2[j / 2] = tc::pack_bf16(gelu_fast(x0), gelu_fast(x1));
-              }
-            } else if (P.epi == 2) {
-#pragma unroll
-              for (int j = 0; j < 64; j += 2) {
-                const float x0 = __uint_as_float(v[j]) * keep, x1 = __uint_as_float(v[j + 1]) * keep;
-                w1[j / 2] = tc::pack_bf16(x0 * gelu_grad_fast(__bfloat162float(a0[j])), x1 * gelu_grad_fast(__bfloat162float(a0[j + 1])));
-              }
-            } else if (P.epi == 3) {
-#pragma unroll
-              for (int j = 0; j < 64; j += 2) {
-                const float x0 = __uint_as_float(v[j]) * keep, x1 = __uint_as_float(v[j + 1]) * keep;
-                w1[j / 2] = tc::pack_bf16(x0, x1);
-                w2[j / 2] = tc::pack_bf16(x0 * sigmoid_fast(x0) * __bfloat162float(a0[j]), x1 * sigmoid_fast(x1) * __bfloat162float(a0[j + 1]));
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 64; j += 2) {
-                float y1[2], y2[2];
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                  const float x = __uint_as_float(v[j + u]) * keep;
-                  const float uu = __bfloat162float(a0[j + u]), gg = __bfloat162float(a1[j + u]), sg = sigmoid_fast(gg);
-                  y1[u] = x * gg * sg;
-                  y2[u] = x * uu * sg * (1.f + gg * (1.f - sg));
-                }
-                w1[j / 2] = tc::pack_bf16(y1[0], y1[1]);
-                w2[j / 2] = tc::pack_bf16(y2[0], y2[1]);
-              }
-            }
-            // the next panel's extra operands, requested while this panel's stores are under way
-            if (pn + 1 < pn_end && n + 64 < P.n && row < P.m) {
-              if (P.epi >= 2) {
-                const __nv_bfloat16* rp = P.residual + ((long long)(n / 64 + 1) * P.c_rpad + row) * 64;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
-              }
-              if (P.epi == 4) {
-                const __nv_bfloat16* rp = P.aux1 + ((long long)(n / 64 + 1) * P.c_rpad + row) * 64;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) rv2[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
-              }
-            }
-            const int n_out = (P.epi == 2) ? 1 : 2;
-#pragma unroll 1
-            for (int oi = 0; oi < n_out; ++oi) {
-              const uint4* ov = oi ? o2 : o1;
-              const uint32_t stg = base + SP::STG_OFF + (ESETS == 2 ? (uint32_t)(warp - 2) : (uint32_t)(q * 2 + (pc & 1))) * 4096u;
-              if (ESETS == 2 && lane == 0) tc::bulk_wait_group_read0();
-              __syncwarp();
-#pragma unroll
-              for (int j = 0; j < 8; ++j)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
-                             "r"(ov[j].x), "r"(ov[j].y), "r"(ov[j].z), "r"(ov[j].w) : "memory");
-              tc::fence_proxy_async();
-              __syncwarp();
-              if (lane == 0) {
-                tc::tma_store_3d(oi ? &P.tc2 : &P.tc, stg, 0, tcd.m0 + q * 32, n / 64);
-                tc::bulk_commit_group();
-                if (ESETS == 1) tc::bulk_wait_group_read1();
-              }
-              ++pc;
-            }
-            continue;
-          }
-        }
-        uint4 outv[8];
-        uint32_t* ow = reinterpret_cast<uint32_t*>(outv);
-        if (has_res) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const __nv_bfloat16* rb = reinterpret_cast<const __nv_bfloat16*>(&rv[j]);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[8 * j + k] = __float_as_uint(__uint_as_float(v[8 * j + k]) + __bfloat162float(rb[k]));
-          }
-          if (pn + 1 < pn_end && n + 64 < P.n) {
-            const __nv_bfloat16* rp = P.residual + ((long long)(n / 64 + 1) * P.c_rpad + row) * 64;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
-          }
-        }
-        if (bias) {
-#pragma unroll
-          for (int j = 0; j < 64; j += 2) {
-            // column pn*64 + j is register (j % (BN/32)) of lane (pn*64 + j) / (BN/32)
-            const float b0 = __shfl_sync(0xffffffffu, bl[j % (BN / 32)], (pn * 64 + j) / (BN / 32));
-            const float b1 = __shfl_sync(0xffffffffu, bl[(j + 1) % (BN / 32)], (pn * 64 + j + 1) / (BN / 32));
-            ow[j / 2] = tc::pack_bf16(pad ? 0.f : __uint_as_float(v[j]) + b0, pad ? 0.f : __uint_as_float(v[j + 1]) + b1);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 64; j += 2)
-            ow[j / 2] = tc::pack_bf16(pad ? 0.f : __uint_as_float(v[j]), pad ? 0.f : __uint_as_float(v[j + 1]));
-        }
-        if (P.dot_with && row < P.m) {
-          // Row reduction over this head's columns, on the ROUNDED values the attention backward will read:
-          // sum_j dS_ij = 0 (softmax shift invariance) holds only if D matches the dP that kernel forms.
-          const __nv_bfloat16* ap = P.dot_with + ((long long)(n / 64) * P.c_rpad + row) * 64;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const uint4 av = *reinterpret_cast<const uint4*>(ap + 8 * j);
-            const __nv_bfloat16* ab16 = reinterpret_cast<const __nv_bfloat16*>(&av);
-#pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-              const uint32_t w2 = ow[4 * j + k / 2];        // two bf16: low half = even column
-              dot_acc = fmaf(__uint_as_float(w2 << 16), __bfloat162float(ab16[k]), dot_acc);
-              dot_acc = fmaf(__uint_as_float(w2 & 0xffff0000u), __bfloat162float(ab16[k + 1]), dot_acc);
-            }
-          }
-          if ((n + 64) % P.dot_hd == 0) {                 // last panel of a head
-            const int hh = n / P.dot_hd, bb = row / P.t_pad, tt = row % P.t_pad;
-            P.dot_out[((long long)bb * P.dot_hq + hh) * P.t_pad + tt] = dot_acc;
-            dot_acc = 0.f;
-          }
-        }
-        // Staging tile (pc & 1) of this warp: its previous store (two panels ago) has been read, since lane 0
-        // waited for that after committing the store of the panel before this one.
-        const uint32_t stg = base + SP::STG_OFF + (ESETS == 2 ? (uint32_t)(warp - 2) : (uint32_t)(q * 2 + (pc & 1))) * 4096u;
-        if (ESETS == 2 && lane == 0) tc::bulk_wait_group_read0();    // one staging tile: the store before has read it
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
-                       "r"(outv[j].x), "r"(outv[j].y), "r"(outv[j].z), "r"(outv[j].w) : "memory");
-        tc::fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) {
-          tc::tma_store_3d(&P.tc, stg, 0, tcd.m0 + q * 32, n / 64);
-          tc::bulk_commit_group();
-          if (ESETS == 1) tc::bulk_wait_group_read1();  // the store before this one has read its staging tile
-        }
-        ++pc;
-      }
+      const bool ready = epilogue_tile<BN, ESETS, EPI>(P, tcd.m0, tcd.n0, tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN, base + SP::STG_OFF, pc, [&] {
+        return tc::mbar_wait(acc_full(ab), (ti >> 1) & 1, status, 103);
+      });
+      if (!ready) { ok = false; break; }
       tc::tc_fence_before();
       tc::mbar_arrive(acc_empty(ab));             // this accumulator may be overwritten by the tile after next
     }
@@ -527,6 +580,7 @@ __device__ __forceinline__ bool pair_tile_at(const TcGroup& G, int w, TileCoord*
   return false;
 }
 
+template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair_kernel(const __grid_constant__ TcGroup G) {
   using SP = PairSmem;
   constexpr int STAGES = PAIR_STAGES, BN = PAIR_BN;
@@ -632,7 +686,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair
     pdl_wait();
     group_chores(G, threadIdx.x - 64, 128);
     const int q = warp % 4;
-    const int r = q * 32 + lane;
     int ti = 0, pc = 0;
     bool ok = true;
     TileCoord tcd;
@@ -640,117 +693,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair
       const TcProblem& P = G.p[tcd.prob];
       const int ab = ti & 1;
       const int m0 = tcd.m0 + (int)rank * 128;
-      const int row = m0 + r;
-      const bool pad = P.t_pad > 0 && (row % P.t_pad) >= P.seq;
-      const bool has_res = P.residual && row < P.m;
-      uint4 rv[8];
-      if (has_res) {
-        const __nv_bfloat16* rp = P.residual + ((long long)(tcd.n0 / 64) * P.c_rpad + row) * 64;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
-      }
-      const float* bias = P.bias;
-      float bl[BN / 32];
-      if (bias) {
-#pragma unroll
-        for (int k = 0; k < BN / 32; ++k) {
-          const int c = tcd.n0 + lane * (BN / 32) + k;
-          bl[k] = c < P.n ? bias[c] : 0.f;
-        }
-      }
-      if (!tc::mbar_wait(acc_full(ab), (ti >> 1) & 1, status, 113)) { ok = false; break; }
-      tc::tc_fence_after();
-      float dot_acc = 0.f;
-#pragma unroll 1
-      for (int pn = 0; pn < BN / 64; ++pn) {
-        const int n = tcd.n0 + pn * 64;
-        if (n >= P.n) break;
-        uint32_t v[64];
-        tc::tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN + pn * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-        tc::tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN + pn * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-        tc::tmem_ld_wait();
-        if (P.ksplit > 1) {
-#pragma unroll 1
-          for (int hf = 0; hf < 2; ++hf) {
-            const uint32_t stg = base + SP::STG_OFF + (uint32_t)(q * 2 + (pc & 1)) * 4096u;
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
-                           "r"(hf ? v[32 + 4 * j] : v[4 * j]), "r"(hf ? v[33 + 4 * j] : v[4 * j + 1]),
-                           "r"(hf ? v[34 + 4 * j] : v[4 * j + 2]), "r"(hf ? v[35 + 4 * j] : v[4 * j + 3]) : "memory");
-            tc::fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) {
-              tc::tma_reduce_add_4d(&P.tacc, stg, 0, hf, m0 + q * 32, n / 64);
-              tc::bulk_commit_group();
-              tc::bulk_wait_group_read1();
-            }
-            ++pc;
-          }
-          continue;
-        }
-        uint4 outv[8];
-        uint32_t* ow = reinterpret_cast<uint32_t*>(outv);
-        if (has_res) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const __nv_bfloat16* rb = reinterpret_cast<const __nv_bfloat16*>(&rv[j]);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[8 * j + k] = __float_as_uint(__uint_as_float(v[8 * j + k]) + __bfloat162float(rb[k]));
-          }
-          if (pn + 1 < BN / 64 && n + 64 < P.n) {
-            const __nv_bfloat16* rp = P.residual + ((long long)(n / 64 + 1) * P.c_rpad + row) * 64;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) rv[j] = *reinterpret_cast<const uint4*>(rp + 8 * j);
-          }
-        }
-        if (bias) {
-#pragma unroll
-          for (int j = 0; j < 64; j += 2) {
-            const float b0 = __shfl_sync(0xffffffffu, bl[j % (BN / 32)], (pn * 64 + j) / (BN / 32));
-            const float b1 = __shfl_sync(0xffffffffu, bl[(j + 1) % (BN / 32)], (pn * 64 + j + 1) / (BN / 32));
-            ow[j / 2] = tc::pack_bf16(pad ? 0.f : __uint_as_float(v[j]) + b0, pad ? 0.f : __uint_as_float(v[j + 1]) + b1);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 64; j += 2)
-            ow[j / 2] = tc::pack_bf16(pad ? 0.f : __uint_as_float(v[j]), pad ? 0.f : __uint_as_float(v[j + 1]));
-        }
-        if (P.dot_with && row < P.m) {
-          const __nv_bfloat16* ap = P.dot_with + ((long long)(n / 64) * P.c_rpad + row) * 64;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const uint4 av = *reinterpret_cast<const uint4*>(ap + 8 * j);
-            const __nv_bfloat16* ab16 = reinterpret_cast<const __nv_bfloat16*>(&av);
-#pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-              const uint32_t w2 = ow[4 * j + k / 2];
-              dot_acc = fmaf(__uint_as_float(w2 << 16), __bfloat162float(ab16[k]), dot_acc);
-              dot_acc = fmaf(__uint_as_float(w2 & 0xffff0000u), __bfloat162float(ab16[k + 1]), dot_acc);
-            }
-          }
-          if ((n + 64) % P.dot_hd == 0) {
-            const int hh = n / P.dot_hd, bb = row / P.t_pad, tt = row % P.t_pad;
-            P.dot_out[((long long)bb * P.dot_hq + hh) * P.t_pad + tt] = dot_acc;
-            dot_acc = 0.f;
-          }
-        }
-        const uint32_t stg = base + SP::STG_OFF + (uint32_t)(q * 2 + (pc & 1)) * 4096u;
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg + lane * 128 + (((uint32_t)j ^ (uint32_t)(lane & 7)) * 16)),
-                       "r"(outv[j].x), "r"(outv[j].y), "r"(outv[j].z), "r"(outv[j].w) : "memory");
-        tc::fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) {
-          tc::tma_store_3d(&P.tc, stg, 0, m0 + q * 32, n / 64);
-          tc::bulk_commit_group();
-          tc::bulk_wait_group_read1();
-        }
-        ++pc;
-      }
+      const bool ready = epilogue_tile<BN, 1, EPI>(P, m0, tcd.n0, tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN, base + SP::STG_OFF, pc, [&] {
+        return tc::mbar_wait(acc_full(ab), (ti >> 1) & 1, status, 113);
+      });
+      if (!ready) { ok = false; break; }
       tc::tc_fence_before();
       tc::mbar_arrive_cluster(tc::map_to_cta(acc_empty(ab), 0));     // the leader's barrier, from either CTA
     }
@@ -889,10 +835,12 @@ cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int32_t* statu
     P.dot_with = (const __nv_bfloat16*)g.dot_with; P.dot_out = g.dot_out; P.dot_hd = g.dot_hd; P.dot_hq = g.dot_hq;
     P.epi = g.epi; P.aux1 = (const __nv_bfloat16*)g.aux1;
     if (g.epi != 0) {
-      if (g.epi < 1 || g.epi > 4 || g.ksplit > 1 || g.dot_with || (g.epi >= 2 && !g.residual) || (g.epi == 4 && !g.aux1) ||
-          (g.epi != 2 && !g.c2))
+      const bool rope = g.epi == 5, two_out = g.epi != 2 && !rope;
+      if (g.epi < 1 || g.epi > 5 || g.ksplit > 1 || g.dot_with || (g.epi >= 2 && !rope && !g.residual) || (g.epi == 4 && !g.aux1) ||
+          (two_out && !g.c2) || (rope && (!g.rope || g.residual || g.t_pad <= 0)))
         return cudaErrorInvalidValue;
-      if (g.epi != 2 && !fbl_encode_rtile_map(&P.tc2, g.c2, g.c_rpad, g.n / 64, 32, 1)) return cudaErrorInvalidValue;
+      P.rope = g.rope; P.rope_hd = g.rope_hd;
+      if (two_out && !fbl_encode_rtile_map(&P.tc2, g.c2, g.c_rpad, g.n / 64, 32, 1)) return cudaErrorInvalidValue;
     }
     P.ksplit = 1;
     if (g.ksplit > 1) {
@@ -907,44 +855,38 @@ cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int32_t* statu
   return cudaSuccess;
 }
 
+// Which fused epilogue a launch needs (activations and the rotation never meet in one).
+int group_epi(const GemmArgs* gs, int count) {
+  int epi = EPI_NONE;
+  for (int i = 0; i < count; ++i)
+    if (gs[i].epi != 0) epi = gs[i].epi == 5 ? EPI_ROPE : EPI_ACT;
+  return epi;
+}
+
+cudaError_t launch_group_kernel(void (*k)(const TcGroup), int grid, int threads, size_t smem, cudaStream_t st, int serial, const TcGroup& G) {
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return serial ? launch_serial(k, dim3(grid), dim3(threads), smem, st, G) : launch_pdl(k, dim3(grid), dim3(threads), smem, st, G);
+}
+
 template <int BN, int STAGES>
 cudaError_t launch_group_bn(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int esets_choice) {
   TcGroup G;
   int tiles = 0;
   cudaError_t e = fill_group(G, gs, count, status, BN, BM, BN, &tiles);
   if (e != cudaSuccess) return e;
-  using SP = SmemPlan<BN, STAGES>;
   const int grid = tiles < p->sm_count ? tiles : p->sm_count;
   // one tile per block at most: the epilogue is exposed, and the variant with two sets of epilogue warps halves it
   // (with several tiles per block the epilogues overlap the next main loops and the extra warps only cost)
   const int esets_knob = esets_choice ? esets_choice : p->knob_gemm_esets;
   const bool two_sets = esets_knob ? esets_knob == 2 : tiles <= p->sm_count;
-  bool epi = false;
-  for (int i = 0; i < count; ++i) epi = epi || gs[i].epi != 0;
-  if (epi) {                       // the variant with the fused activations (feed-forward block only)
-    if (two_sets) {
-      auto k = gemm_tc_kernel<BN, STAGES, 2, true>;
-      cudaError_t attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP::TOTAL);
-      if (attr_err != cudaSuccess) return attr_err;
-      return launch_pdl(k, dim3(grid), dim3(320), SP::TOTAL, st, G);
-    }
-    auto k = gemm_tc_kernel<BN, STAGES, 1, true>;
-    cudaError_t attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP::TOTAL);
-    if (attr_err != cudaSuccess) return attr_err;
-    return launch_pdl(k, dim3(grid), dim3(192), SP::TOTAL, st, G);
+  void (*k)(const TcGroup) = nullptr;
+  switch (group_epi(gs, count)) {
+    case EPI_ACT: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_ACT> : gemm_tc_kernel<BN, STAGES, 1, EPI_ACT>; break;
+    case EPI_ROPE: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_ROPE> : gemm_tc_kernel<BN, STAGES, 1, EPI_ROPE>; break;
+    default: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_NONE> : gemm_tc_kernel<BN, STAGES, 1, EPI_NONE>;
   }
-  if (two_sets) {
-    auto k = gemm_tc_kernel<BN, STAGES, 2>;
-    cudaError_t attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP::TOTAL);
-    if (attr_err != cudaSuccess) return attr_err;
-    return gs[0].serial ? launch_serial(k, dim3(grid), dim3(320), SP::TOTAL, st, G)
-                        : launch_pdl(k, dim3(grid), dim3(320), SP::TOTAL, st, G);
-  }
-  auto k = gemm_tc_kernel<BN, STAGES, 1>;
-  cudaError_t attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP::TOTAL);
-  if (attr_err != cudaSuccess) return attr_err;
-  return gs[0].serial ? launch_serial(k, dim3(grid), dim3(192), SP::TOTAL, st, G)
-                      : launch_pdl(k, dim3(grid), dim3(192), SP::TOTAL, st, G);
+  return launch_group_kernel(k, grid, two_sets ? 320 : 192, SmemPlan<BN, STAGES>::TOTAL, st, gs[0].serial, G);
 }
 
 cudaError_t launch_group_pair(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st) {
@@ -952,13 +894,9 @@ cudaError_t launch_group_pair(const fbl_plan* p, const GemmArgs* gs, int count, 
   int tiles = 0;
   cudaError_t e = fill_group(G, gs, count, status, 128, 256, 256, &tiles);   // each CTA loads 128 of the pair's 256 columns
   if (e != cudaSuccess) return e;
-  using SP = PairSmem;
-  auto k = gemm_tc_pair_kernel;
-  cudaError_t attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP::TOTAL);
-  if (attr_err != cudaSuccess) return attr_err;
-  const int pairs = tiles < p->sm_count / 2 ? tiles : p->sm_count / 2;
-  return gs[0].serial ? launch_serial(k, dim3(2 * pairs), dim3(192), SP::TOTAL, st, G)
-                      : launch_pdl(k, dim3(2 * pairs), dim3(192), SP::TOTAL, st, G);
+  const int epi = group_epi(gs, count), pairs = tiles < p->sm_count / 2 ? tiles : p->sm_count / 2;
+  auto k = epi == EPI_ACT ? gemm_tc_pair_kernel<EPI_ACT> : epi == EPI_ROPE ? gemm_tc_pair_kernel<EPI_ROPE> : gemm_tc_pair_kernel<EPI_NONE>;
+  return launch_group_kernel(k, 2 * pairs, 192, PairSmem::TOTAL, st, gs[0].serial, G);
 }
 
 namespace {
@@ -1009,11 +947,9 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
   if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
   fbl_plan::GemmChoice ch = {0, -1, 0};
   if (launch_id >= 0 && launch_id < FBL_GEMM_LAUNCH_COUNT) ch = p->choice[launch_id];
-  bool any_epi = false;
-  for (int i = 0; i < count; ++i) any_epi = any_epi || gs[i].epi != 0;
   // The tile whose slowest block finishes first; an offline choice for this launch, or the pair knob, comes before it.
   // (N need not be whole tiles: panels past it are loaded as zeros and not stored.)
-  const int pair_mode = any_epi ? 0 : ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 always, -1 by cost
+  const int pair_mode = ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 always, -1 by cost
   int kind = TILE_NARROW;
   if (pair_mode == 1) {
     kind = TILE_PAIR;

@@ -127,12 +127,14 @@ int fbl_layer_fwd_lora(const fbl_plan* p, const void* X, const float* gamma, con
   float* stats = (float*)(sv + p->sv_stats);
   void* Xn = sv + p->sv_xn; void* Q = sv + p->sv_q; void* K = sv + p->sv_k; void* V = sv + p->sv_v;
   void* A = sv + p->sv_a; float* lse = (float*)(sv + p->sv_lse); void* T = sv + p->sv_t;
+  float2* rope = (float2*)(sv + p->sv_rope);
+  bool rotated = false;
   const bool bias = p->d.has_bias;
   const int n = (int)p->n_pad, D = p->d.d_model;
   int k = 0;
 
   if (p->prof_on) { p->prof_n = 0; LORA_CUDA(cudaEventRecord(p->prof_ev[0], st)); }
-  LORA_STEP("norm_fwd", 1, launch_norm_fwd(p, X, gamma, beta, Xn, stats, status, st));
+  LORA_STEP("norm_fwd", 1, launch_norm_fwd(p, X, gamma, beta, Xn, stats, status, st, p->rope_base > 0.f ? rope : nullptr));
   {
     GemmArgs g = {};                       // T = Xn [Aq | Ak | Av]: one thin product for the three adapters
     g.m = n; g.n = RA; g.n_terms = 1;
@@ -159,11 +161,12 @@ int fbl_layer_fwd_lora(const fbl_plan* p, const void* X, const float* gamma, con
       g.c = O[i]; g.c_rpad = p->n_pad; g.bias = bias ? B[i] : nullptr;
       g.seq = p->d.seq; g.t_pad = p->t_pad;
     }
+    rotated = rope_in_projection(p, gs, rope);
     LORA_CUDA(run_gemm_group(p, gs, 3, status, st, -1, &k));
     LORA_STEP("proj_qkv", 0, cudaSuccess);
     p->launches += k;
   }
-  if (p->rope_base > 0.f) LORA_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
+  if (p->rope_base > 0.f && !rotated) LORA_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
   if (p->use_tc && attn_fwd_tc_supported(p)) LORA_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
   else if (p->d.dtype == FBL_DTYPE_FP32) LORA_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
   else LORA_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
@@ -228,10 +231,11 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     LORA_STEP("dA", 0, cudaSuccess);
     p->launches += k;
   }
-  if (p->use_tc && attn_bwd_tc_supported(p)) LORA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
+  if (p->use_tc && attn_bwd_tc_supported(p)) LORA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st,
+                                                  p->rope_base > 0.f ? (const float2*)(sv + p->sv_rope) : nullptr));
   else if (p->d.dtype == FBL_DTYPE_FP32) LORA_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
   else LORA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
-  if (p->rope_base > 0.f) LORA_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
+  if (p->rope_base > 0.f && !(p->use_tc && attn_bwd_tc_supported(p))) LORA_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   const void* G[3] = {dQ, dK, dV};
   {
     GemmArgs g = {};                       // dT = dQ Bq^T | dK Bk^T | dV Bv^T: B_all's column blocks read with swapped axes;

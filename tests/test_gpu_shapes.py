@@ -89,6 +89,11 @@ def test_fp32_gemm_tiles_and_slices(cfg):
     LayerConfig("rg1", 1, 300, 192, 5, 1, 64, "bf16", "layernorm", True, True, True, 1e-5, 241, 0.05),
     LayerConfig("rg2", 2, 500, 1088, 17, 17, 64, "bf16", "rmsnorm", True, False, False, 1e-5, 242, 0.02),
     MlpConfig("rg3", 3, 333, 448, 1216, "bf16", "layernorm", "gelu", True, True, 1e-5, 243, 0.03),
+    # activations with two outputs, and the rotary embedding (both head widths, with biases), in the projections' epilogues
+    MlpConfig("rg4", 2, 300, 256, 704, "bf16", "rmsnorm", "swiglu", True, True, 1e-5, 244, 0.03),
+    LayerConfig("rg5", 2, 300, 192, 5, 1, 64, "bf16", "rmsnorm", True, True, True, 1e-5, 245, 0.01, 0.0, 10000.0),
+    LayerConfig("rg6", 2, 141, 256, 3, 1, 128, "bf16", "layernorm", False, True, False, 1e-5, 246, 0.01, 0.0, 500.0),
+    LayerConfig("rg7", 3, 77, 256, 3, 3, 64, "bf16", "layernorm", True, True, False, 1e-5, 247, 0.01, 0.0, 500.0),
 ], ids=lambda c: getattr(c, "name", ""))
 def test_ragged_columns_on_every_gemm_tile(cfg, pair, monkeypatch):
     monkeypatch.setenv("FBL_GEMM_PAIR", pair)
