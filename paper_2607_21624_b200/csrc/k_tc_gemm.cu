@@ -287,8 +287,8 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
     bool bias_left = bias != nullptr;
     if constexpr (EPI == EPI_ROPE) {
       if (P.epi == 5) {
-        // rotation of a head's (i, i + hd / 2) column pairs; the table has a frequency's tokens next to each other, as
-        // the lanes have their rows
+        // Rotation of a head's (i, i + hd / 2) column pairs, of the rounded values, as where a pass of its own does it;
+        // the table has a frequency's tokens next to each other, as the lanes have their rows.
         const float2* tab = P.rope + row % P.t_pad;
         if (bias) {
 #pragma unroll
@@ -300,7 +300,7 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const float2 cs = tab[(long long)j * P.t_pad];
-            const float a = __uint_as_float(v[j]), b = __uint_as_float(v[j + 32]);
+            const float a = tc::round_bf16(__uint_as_float(v[j])), b = tc::round_bf16(__uint_as_float(v[j + 32]));
             v[j] = __float_as_uint(a * cs.x - b * cs.y);
             v[j + 32] = __float_as_uint(b * cs.x + a * cs.y);
           }
@@ -316,7 +316,7 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
               const float2 cs = tab[(long long)(hf * 32 + j) * P.t_pad];
               float b = __uint_as_float(w[j]);
               if (bias) b += __shfl_sync(0xffffffffu, bl[(hf * 32 + j) % (BN / 32)], ((pn ^ 1) * 64 + hf * 32 + j) / (BN / 32));
-              v[hf * 32 + j] = __float_as_uint(__uint_as_float(v[hf * 32 + j]) * cs.x + sign * b * cs.y);
+              v[hf * 32 + j] = __float_as_uint(tc::round_bf16(__uint_as_float(v[hf * 32 + j])) * cs.x + sign * tc::round_bf16(b) * cs.y);
             }
           }
         }
