@@ -199,6 +199,11 @@ def selftest_wait_timeout(scratch_ptr, limit_cycles, stream):
     _check(lib().fbl_selftest_wait_timeout(scratch_ptr, limit_cycles, stream))
 
 
+def raw_stream(torch, device) -> int:
+    """The current stream's handle, without building a stream object (0.2 instead of 2.2 us, twice per step)."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if device.index is None else device.index)
+
+
 GUARD_BYTE = 0xA5
 
 
@@ -283,7 +288,7 @@ class LayerRunner:
         return Plan(desc_from_config(cfg))
 
     def _stream(self):
-        return self.torch.cuda.current_stream(self.dev).cuda_stream
+        return raw_stream(self.torch, self.dev)
 
     def _shape(self, name):
         c = self.cfg

@@ -229,6 +229,7 @@ void fbl_plan_destroy(fbl_plan* plan) {
   if (!plan) return;
   if (plan->prof_on)
     for (int i = 0; i <= FBL_PROF_MAX; ++i) cudaEventDestroy(plan->prof_ev[i]);
+  for (FblMemoBase* m : plan->memo) delete m;
   delete plan;
 }
 

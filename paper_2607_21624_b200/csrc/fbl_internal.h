@@ -30,6 +30,9 @@ template <typename T> __device__ __forceinline__ T from_f(float v);
 template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+struct FblMemoBase { virtual ~FblMemoBase() {} };      // launch_memo.h
+enum { FBL_MEMO_TC_GEMM = 0, FBL_MEMO_FFMA_GEMM, FBL_MEMO_TC_FWD, FBL_MEMO_TC_BWD, FBL_MEMO_FFMA_ATTN, FBL_MEMO_COUNT };
+
 struct fbl_plan {
   fbl_layer_desc d;
   int e;        // bytes per element
@@ -74,8 +77,7 @@ struct fbl_plan {
   // bookkeeping of the enqueue calls (they take the plan as const): kernels enqueued so far, optional per-step
   // event timing.  Calls on one plan are not thread-safe; give each host thread its own plan.
   mutable int64_t launches;
-  static constexpr int TILE_MEMO = 16;      // GEMM launches by shape: the output tile chosen for each
-  mutable struct { uint64_t key; int kind; } tile_memo[TILE_MEMO];
+  mutable FblMemoBase* memo[FBL_MEMO_COUNT];
   mutable int prof_on, prof_n;
   mutable cudaEvent_t prof_ev[FBL_PROF_MAX + 1];
   mutable const char* prof_name[FBL_PROF_MAX];

@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "fbl_internal.h"
+#include "launch_memo.h"
 #include "pdl.cuh"
 #include "tc_common.cuh"
 
@@ -371,6 +372,8 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
   }
 }
 
+typedef LaunchMemo<FfmaAttnParams, 8, 12> AttnMemo;
+
 void fill(const fbl_plan* p, FfmaAttnParams& P, int32_t* status) {
   memset(&P, 0, sizeof(P));
   P.n_pad = p->n_pad; P.n_pad_k = p->n_pad_kv; P.seq = p->d.seq; P.t_pad = p->t_pad; P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;
@@ -379,24 +382,29 @@ void fill(const fbl_plan* p, FfmaAttnParams& P, int32_t* status) {
 
 template <int HD>
 cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse, int32_t* status, cudaStream_t st) {
-  FfmaAttnParams P;
+  auto k = attn_fwd_ffma_kernel<HD>;
+  auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
   if (!fbl_encode_f32_rtile_map(&P.tq, Q, p->n_pad, p->dq / 32, ROWS, HD / 32) ||
       !fbl_encode_f32_rtile_map(&P.tk, K, p->n_pad_kv, p->dkv / 32, FWD_KEYS, HD / 32) ||
       !fbl_encode_f32_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 32, FWD_KEYS, HD / 32))
     return cudaErrorInvalidValue;
   P.a = (float*)A; P.lse = lse;
-  auto k = attn_fwd_ffma_kernel<HD>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FfmaFwdSmem<HD>::TOTAL);
-  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FfmaFwdSmem<HD>::TOTAL);
+  };
+  LaunchKey key;
+  for (const void* q : {Q, K, V, (const void*)A, (const void*)lse, (const void*)status}) key.add(q);
+  return AttnMemo::run(p->memo[FBL_MEMO_FFMA_ATTN], key, make, [&](const FfmaAttnParams& P) {
   return launch_pdl(k, dim3((p->t_pad + ROWS - 1) / ROWS, p->d.n_q_heads, p->d.batch), dim3(THREADS), FfmaFwdSmem<HD>::TOTAL, st, P);
+  });
 }
 
 template <int HD>
 cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* dA, const float* lse, const float* dvec,
                        void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st) {
   constexpr int QT = FfmaBwdSmem<HD>::QT;
-  FfmaAttnParams P;
+  auto k = attn_bwd_ffma_kernel<HD>;
+  auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
   if (!fbl_encode_f32_rtile_map(&P.tq, Q, p->n_pad, p->dq / 32, QT, HD / 32) ||
       !fbl_encode_f32_rtile_map(&P.tdo, dA, p->n_pad, p->dq / 32, QT, HD / 32) ||
@@ -404,10 +412,14 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
       !fbl_encode_f32_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 32, ROWS, HD / 32))
     return cudaErrorInvalidValue;
   P.lse = const_cast<float*>(lse); P.dvec = dvec; P.dq = (float*)dQ; P.dk = (float*)dK; P.dv = (float*)dV;
-  auto k = attn_bwd_ffma_kernel<HD>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FfmaBwdSmem<HD>::TOTAL);
-  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FfmaBwdSmem<HD>::TOTAL);
+  };
+  LaunchKey key;
+  for (const void* q : {Q, K, V, dA, (const void*)lse, (const void*)dvec, (const void*)dQ, (const void*)dK, (const void*)dV, (const void*)status})
+    key.add(q);
+  return AttnMemo::run(p->memo[FBL_MEMO_FFMA_ATTN], key, make, [&](const FfmaAttnParams& P) {
   return launch_pdl(k, dim3((p->t_pad_kv + ROWS - 1) / ROWS, p->d.n_kv_heads, p->d.batch), dim3(THREADS), FfmaBwdSmem<HD>::TOTAL, st, P);
+  });
 }
 
 }  // namespace

@@ -21,6 +21,7 @@
 #include <string.h>
 
 #include "fbl_internal.h"
+#include "launch_memo.h"
 #include "pdl.cuh"
 #include "tc_common.cuh"
 
@@ -49,6 +50,8 @@ struct alignas(64) FfmaGroup {
   int count, slices;
   int32_t* status;
 };
+
+struct FfmaLaunch { FfmaGroup G; int grid; };      // a launch made ready
 
 struct Smem {
   static constexpr uint32_t A_BYTES = BM * BK * 4, B_BYTES = BN * BK * 4, STAGE = A_BYTES + B_BYTES;
@@ -279,9 +282,8 @@ bool gemm_ffma_supported(const fbl_plan* p, const GemmArgs& g) {
   return true;
 }
 
-cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st) {
-  if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
-  FfmaGroup G;
+static cudaError_t make_group(FfmaLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status) {
+  FfmaGroup& G = L.G;
   memset(&G, 0, sizeof(G));
   G.count = count;
   G.status = status;
@@ -307,9 +309,20 @@ cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int co
     tiles += P.tiles_m * P.tiles_n;
   }
   G.slices = choose_slices(p->sm_count, G);
-  cudaError_t e = cudaFuncSetAttribute(gemm_ffma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem::TOTAL);
-  if (e != cudaSuccess) return e;
-  return launch_pdl_cluster(gemm_ffma_kernel, dim3(tiles * G.slices), dim3(THREADS), Smem::TOTAL, st, G.slices, G);
+  L.grid = tiles * G.slices;
+  return cudaFuncSetAttribute(gemm_ffma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem::TOTAL);
+}
+
+cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st) {
+  if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
+  LaunchKey key;
+  gemm_group_key(key, gs, count, status);
+  return LaunchMemo<FfmaLaunch, 12, 248>::run(p->memo[FBL_MEMO_FFMA_GEMM], key,
+      [&](FfmaLaunch& L) { return make_group(L, p, gs, count, status); },
+      [&](const FfmaLaunch& L) {
+        if (L.G.slices == 1) return launch_pdl(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G);
+        return launch_pdl_cluster(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G.slices, L.G);
+      });
 }
 
 cudaError_t run_gemm_group(const fbl_plan* p, GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int launch_id, int* kernels) {

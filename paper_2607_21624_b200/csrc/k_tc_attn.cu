@@ -13,6 +13,7 @@
 
 #include "attn_common.cuh"
 #include "fbl_internal.h"
+#include "launch_memo.h"
 #include "pdl.cuh"
 #include "tc_common.cuh"
 
@@ -458,23 +459,33 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
   if (warp == 1) tc::tmem_dealloc(tmem_base, TMEM_COLS);
 }
 
+// A launch made ready: what the launchers remember.
+template <typename Params>
+struct AttnLaunch {
+  Params P;
+  void (*kernel)(const Params);
+  int grid, threads;
+  size_t smem;
+  cudaError_t set(void (*k)(const Params), int g, int t, size_t s) {
+    kernel = k; grid = g; threads = t; smem = s;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s);
+  }
+};
+
 template <int HD, int TILES>
-cudaError_t fwd_launch_t(const fbl_plan* p, AttnFwdParams& P, int n_qt, cudaStream_t st) {
-  auto k = attn_fwd_tc_kernel<HD, TILES>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FwdSmem<HD, TILES>::TOTAL);
-  if (e != cudaSuccess) return e;
+cudaError_t fwd_make_t(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, int n_qt) {
+  AttnFwdParams& P = L.P;
   if (TILES == 1) P.pair = 0;
   P.batch = p->d.batch;
   P.n_slots = P.pair ? (n_qt + 1) / 2 : n_qt;
   P.chunk = chunk_for((long long)p->seq_kv * HD * 4, p->d.n_q_heads * p->d.batch, 96ll << 20);   // K and V of one head
-  dim3 grid((unsigned)(P.n_slots * p->d.n_q_heads * p->d.batch));
-  return launch_pdl(k, grid, dim3(64 + 128 * TILES), FwdSmem<HD, TILES>::TOTAL, st, P);
+  return L.set(attn_fwd_tc_kernel<HD, TILES>, P.n_slots * p->d.n_q_heads * p->d.batch, 64 + 128 * TILES, FwdSmem<HD, TILES>::TOTAL);
 }
 
 template <int HD>
-cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
-                       int32_t* status, cudaStream_t st) {
-  AttnFwdParams P;
+cudaError_t fwd_make(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
+                     int32_t* status) {
+  AttnFwdParams& P = L.P;
   memset(&P, 0, sizeof(P));
   const int panels = HD / 64;
   if (!fbl_encode_rtile_map(&P.tq, Q, p->n_pad, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
@@ -490,9 +501,9 @@ cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   if (HD == 64) {
     // tuning knob: 1 = one query tile per block and two blocks per SM, 2 = two tiles per block; default by sequence length
     const int mode = p->knob_fwd_tiles;
-    if (mode == 1 || (mode == 0 && n_qt <= 4)) return fwd_launch_t<64, 1>(p, P, n_qt, st);
+    if (mode == 1 || (mode == 0 && n_qt <= 4)) return fwd_make_t<64, 1>(L, p, n_qt);
   }
-  return fwd_launch_t<HD, 2>(p, P, n_qt, st);
+  return fwd_make_t<HD, 2>(L, p, n_qt);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -1344,24 +1355,19 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) attn_bwd_short_kernel(const 
 
 
 template <int HD, bool DIRECT>
-cudaError_t bwd_launch_t(const fbl_plan* p, AttnBwdParams& P, cudaStream_t st) {
-  auto k = attn_bwd_tc_kernel<HD, DIRECT>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwdSmem<HD>::TOTAL);
-  if (e != cudaSuccess) return e;
+cudaError_t bwd_make_t(AttnLaunch<AttnBwdParams>& L, const fbl_plan* p) {
   // Q, dO (bf16) and the fp32 dQ accumulator of the query heads of one KV head.  The HD = 128 variant waits for
   // its single-buffered Q / dO tiles on the critical path, so it keeps the blocks that share those tiles close
   // together (small chunks: L2 hits); the pipelined HD = 64 variant hides that latency and prefers balance.
-  P.chunk = chunk_for((long long)p->group * p->d.seq * HD * 8, p->d.n_kv_heads * p->d.batch,
-                      BwdSmem<HD>::PIPE ? (96ll << 20) : (8ll << 20));
-  dim3 grid((unsigned)(((p->t_pad_kv + BKV - 1) / BKV) * p->d.n_kv_heads * p->d.batch));
-  return launch_pdl(k, grid, dim3(BWD_THREADS), BwdSmem<HD>::TOTAL, st, P);
+  L.P.chunk = chunk_for((long long)p->group * p->d.seq * HD * 8, p->d.n_kv_heads * p->d.batch,
+                        BwdSmem<HD>::PIPE ? (96ll << 20) : (8ll << 20));
+  return L.set(attn_bwd_tc_kernel<HD, DIRECT>, ((p->t_pad_kv + BKV - 1) / BKV) * p->d.n_kv_heads * p->d.batch, BWD_THREADS, BwdSmem<HD>::TOTAL);
 }
 
 template <int HD>
-cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* dA,
-                       const float* lse, const float* dvec, float* dqacc, void* dQ, void* dK, void* dV, int32_t* status,
-                       cudaStream_t st) {
-  AttnBwdParams P;
+cudaError_t bwd_make(AttnLaunch<AttnBwdParams>& L, const fbl_plan* p, const void* Q, const void* K, const void* V, const void* dA,
+                     const float* lse, const float* dvec, float* dqacc, void* dQ, void* dK, void* dV, int32_t* status) {
+  AttnBwdParams& P = L.P;
   memset(&P, 0, sizeof(P));
   const int panels = HD / 64;
   if (!fbl_encode_rtile_map(&P.tq, Q, p->n_pad, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
@@ -1375,11 +1381,9 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   P.causal = p->d.causal; P.dkv = p->dkv; P.scale = p->scale; P.status = status;
   P.n_pad_k = p->n_pad_kv; P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;
   P.batch = p->d.batch;
-  if (!direct) return bwd_launch_t<HD, false>(p, P, st);
-  if (p->t_pad_kv <= BKV) return bwd_launch_t<HD, true>(p, P, st);
-  cudaError_t e = cudaFuncSetAttribute(attn_bwd_short_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ShortSmem::TOTAL);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(attn_bwd_short_kernel, dim3((unsigned)(P.hq * P.batch)), dim3(SHORT_THREADS), ShortSmem::TOTAL, st, P);
+  if (!direct) return bwd_make_t<HD, false>(L, p);
+  if (p->t_pad_kv <= BKV) return bwd_make_t<HD, true>(L, p);
+  return L.set(attn_bwd_short_kernel, P.hq * P.batch, SHORT_THREADS, ShortSmem::TOTAL);
 }
 
 }  // namespace
@@ -1398,9 +1402,14 @@ bool attn_bwd_tc_supported(const fbl_plan* p) { return attn_fwd_tc_supported(p);
 
 cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                int32_t* status, cudaStream_t st) {
-  if (p->d.head_dim == 64) return fwd_launch<64>(p, Q, K, V, A, lse, status, st);
-  if (p->d.head_dim == 128) return fwd_launch<128>(p, Q, K, V, A, lse, status, st);
-  return cudaErrorInvalidValue;
+  typedef AttnLaunch<AttnFwdParams> Launch;
+  LaunchKey key;
+  for (const void* q : {Q, K, V, (const void*)A, (const void*)lse, (const void*)status}) key.add(q);
+  return LaunchMemo<Launch, 8, 8>::run(p->memo[FBL_MEMO_TC_FWD], key,
+      [&](Launch& L) {
+        return p->d.head_dim == 64 ? fwd_make<64>(L, p, Q, K, V, A, lse, status) : fwd_make<128>(L, p, Q, K, V, A, lse, status);
+      },
+      [&](const Launch& L) { return launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.P); });
 }
 
 cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,
@@ -1409,9 +1418,17 @@ cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, 
   // D = rowsum(dO * O) unless the dA GEMM's epilogue already produced it
   cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, dvec_ready, st);
   if (e != cudaSuccess) return e;
-  if (p->d.head_dim == 64) e = bwd_launch<64>(p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status, st);
-  else if (p->d.head_dim == 128) e = bwd_launch<128>(p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status, st);
-  else e = cudaErrorInvalidValue;
+  typedef AttnLaunch<AttnBwdParams> Launch;
+  LaunchKey key;
+  for (const void* q : {Q, K, V, dA, (const void*)lse, (const void*)dvec, (const void*)dqacc, (const void*)dQ, (const void*)dK, (const void*)dV,
+                        (const void*)status})
+    key.add(q);
+  e = LaunchMemo<Launch, 8, 12>::run(p->memo[FBL_MEMO_TC_BWD], key,
+      [&](Launch& L) {
+        return p->d.head_dim == 64 ? bwd_make<64>(L, p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status)
+                                   : bwd_make<128>(L, p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status);
+      },
+      [&](const Launch& L) { return launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.P); });
   if (e != cudaSuccess) return e;
   // dQ: fp32 accumulator -> storage dtype where the kernel has not written it; with the rotary embedding (`rope`: the
   // forward's table) dQ and dK are turned back by the opposite angle on the way

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "fbl_internal.h"
+#include "launch_memo.h"
 #include "pdl.cuh"
 #include "tc_common.cuh"
 
@@ -855,6 +856,8 @@ cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int32_t* statu
   return cudaSuccess;
 }
 
+namespace {
+
 // Which fused epilogue a launch needs (activations and the rotation never meet in one).
 int group_epi(const GemmArgs* gs, int count) {
   int epi = EPI_NONE;
@@ -863,17 +866,23 @@ int group_epi(const GemmArgs* gs, int count) {
   return epi;
 }
 
-cudaError_t launch_group_kernel(void (*k)(const TcGroup), int grid, int threads, size_t smem, cudaStream_t st, int serial, const TcGroup& G) {
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return serial ? launch_serial(k, dim3(grid), dim3(threads), smem, st, G) : launch_pdl(k, dim3(grid), dim3(threads), smem, st, G);
+// A launch made ready: what launch_gemm_tc_group remembers.
+struct GroupLaunch {
+  TcGroup G;
+  void (*kernel)(const TcGroup);
+  int grid, threads, serial;
+  size_t smem;
+};
+
+cudaError_t group_launch(GroupLaunch& L, void (*k)(const TcGroup), int grid, int threads, size_t smem, int serial) {
+  L.kernel = k; L.grid = grid; L.threads = threads; L.smem = smem; L.serial = serial;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 template <int BN, int STAGES>
-cudaError_t launch_group_bn(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int esets_choice) {
-  TcGroup G;
+cudaError_t make_group_bn(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, int esets_choice) {
   int tiles = 0;
-  cudaError_t e = fill_group(G, gs, count, status, BN, BM, BN, &tiles);
+  cudaError_t e = fill_group(L.G, gs, count, status, BN, BM, BN, &tiles);
   if (e != cudaSuccess) return e;
   const int grid = tiles < p->sm_count ? tiles : p->sm_count;
   // one tile per block at most: the epilogue is exposed, and the variant with two sets of epilogue warps halves it
@@ -886,18 +895,19 @@ cudaError_t launch_group_bn(const fbl_plan* p, const GemmArgs* gs, int count, in
     case EPI_ROPE: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_ROPE> : gemm_tc_kernel<BN, STAGES, 1, EPI_ROPE>; break;
     default: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_NONE> : gemm_tc_kernel<BN, STAGES, 1, EPI_NONE>;
   }
-  return launch_group_kernel(k, grid, two_sets ? 320 : 192, SmemPlan<BN, STAGES>::TOTAL, st, gs[0].serial, G);
+  return group_launch(L, k, grid, two_sets ? 320 : 192, SmemPlan<BN, STAGES>::TOTAL, gs[0].serial);
 }
 
-cudaError_t launch_group_pair(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st) {
-  TcGroup G;
+cudaError_t make_group_pair(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status) {
   int tiles = 0;
-  cudaError_t e = fill_group(G, gs, count, status, 128, 256, 256, &tiles);   // each CTA loads 128 of the pair's 256 columns
+  cudaError_t e = fill_group(L.G, gs, count, status, 128, 256, 256, &tiles);   // each CTA loads 128 of the pair's 256 columns
   if (e != cudaSuccess) return e;
   const int epi = group_epi(gs, count), pairs = tiles < p->sm_count / 2 ? tiles : p->sm_count / 2;
   auto k = epi == EPI_ACT ? gemm_tc_pair_kernel<EPI_ACT> : epi == EPI_ROPE ? gemm_tc_pair_kernel<EPI_ROPE> : gemm_tc_pair_kernel<EPI_NONE>;
-  return launch_group_kernel(k, 2 * pairs, 192, PairSmem::TOTAL, st, gs[0].serial, G);
+  return group_launch(L, k, 2 * pairs, 192, PairSmem::TOTAL, gs[0].serial);
 }
+
+}  // namespace
 
 namespace {
 
@@ -942,13 +952,9 @@ int best_tile(const TileWork* w, int count, int sm_count, bool pairs, double* cl
 
 }  // namespace
 
-cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st,
-                                 int launch_id) {
-  if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
-  fbl_plan::GemmChoice ch = {0, -1, 0};
-  if (launch_id >= 0 && launch_id < FBL_GEMM_LAUNCH_COUNT) ch = p->choice[launch_id];
-  // The tile whose slowest block finishes first; an offline choice for this launch, or the pair knob, comes before it.
-  // (N need not be whole tiles: panels past it are loaded as zeros and not stored.)
+// The tile whose slowest block finishes first; an offline choice for this launch, or the pair knob, comes before it.
+// (N need not be whole tiles: panels past it are loaded as zeros and not stored.)
+static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, const fbl_plan::GemmChoice& ch) {
   const int pair_mode = ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 always, -1 by cost
   int kind = TILE_NARROW;
   if (pair_mode == 1) {
@@ -956,27 +962,34 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
   } else if (ch.bn) {
     kind = ch.bn == 128 ? TILE_NARROW : TILE_WIDE;
   } else {
-    // the same few launches come again on every pass of a plan: their tiles are remembered by shape
     TileWork w[MAX_PROBLEMS];
-    uint64_t key = 1469598103934665603ull ^ (uint64_t)(pair_mode != 0);
     for (int i = 0; i < count; ++i) {
       w[i] = {gs[i].m, gs[i].n, 0, gs[i].ksplit > 1 ? gs[i].ksplit : 1};
       for (int t = 0; t < gs[i].n_terms; ++t) w[i].kb += (gs[i].t[t].k + BK - 1) / BK;
-      for (uint64_t v : {(uint64_t)w[i].m, (uint64_t)w[i].n, (uint64_t)w[i].kb, (uint64_t)w[i].split}) key = (key ^ v) * 1099511628211ull;
     }
-    int at = 0;
-    while (at < fbl_plan::TILE_MEMO && p->tile_memo[at].key && p->tile_memo[at].key != key) ++at;
-    if (at < fbl_plan::TILE_MEMO && p->tile_memo[at].key) {
-      kind = p->tile_memo[at].kind;
-    } else {
-      double clocks;
-      kind = best_tile(w, count, p->sm_count, pair_mode != 0, &clocks);
-      if (at < fbl_plan::TILE_MEMO) p->tile_memo[at] = {key, kind};
-    }
+    double clocks;
+    kind = best_tile(w, count, p->sm_count, pair_mode != 0, &clocks);
   }
-  if (kind == TILE_PAIR) return launch_group_pair(p, gs, count, status, st);
-  if (kind == TILE_WIDE) return launch_group_bn<256, 4>(p, gs, count, status, st, ch.esets);
-  return launch_group_bn<128, 6>(p, gs, count, status, st, ch.esets);
+  if (kind == TILE_PAIR) return make_group_pair(L, p, gs, count, status);
+  if (kind == TILE_WIDE) return make_group_bn<256, 4>(L, p, gs, count, status, ch.esets);
+  return make_group_bn<128, 6>(L, p, gs, count, status, ch.esets);
+}
+
+cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st,
+                                 int launch_id) {
+  if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
+  fbl_plan::GemmChoice ch = {0, -1, 0};
+  if (launch_id >= 0 && launch_id < FBL_GEMM_LAUNCH_COUNT) ch = p->choice[launch_id];
+  LaunchKey key;
+  gemm_group_key(key, gs, count, status);
+  key.add(ch.bn, ch.pair);
+  key.add(ch.esets, 0);
+  return LaunchMemo<GroupLaunch, 12, 248>::run(p->memo[FBL_MEMO_TC_GEMM], key,
+      [&](GroupLaunch& L) { return make_group(L, p, gs, count, status, ch); },
+      [&](const GroupLaunch& L) {
+        return L.serial ? launch_serial(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.G)
+                        : launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.G);
+      });
 }
 
 // How many slices to cut the reduction loops of the splittable problems of a group into (the same number for all

@@ -3,7 +3,7 @@ from __future__ import annotations
 
 import ctypes as C
 
-from .binding import DTYPES, NORMS, FblError, _check, aligned_bytes, guard_bands_intact, lib
+from .binding import DTYPES, NORMS, FblError, _check, aligned_bytes, guard_bands_intact, lib, raw_stream
 
 ACTS = {"gelu": 0, "swiglu": 1}
 MLP_TENSOR = {"X": 0, "H": 1, "W1": 2, "W2": 3}
@@ -136,7 +136,7 @@ class MlpRunner:
         self.vec = {k: v.view(torch.float32) for k, v in self._vec_raw.items()}
 
     def _stream(self):
-        return self.torch.cuda.current_stream(self.dev).cuda_stream
+        return raw_stream(self.torch, self.dev)
 
     def _shape(self, tid):
         c = self.cfg
