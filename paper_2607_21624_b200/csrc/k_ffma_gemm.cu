@@ -321,7 +321,7 @@ cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int co
       [&](FfmaLaunch& L) { return make_group(L, p, gs, count, status); },
       [&](const FfmaLaunch& L) {
         if (L.G.slices == 1) return launch_pdl(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G);
-        return launch_pdl_cluster(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G.slices, L.G);
+        return launch_cluster(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G.slices, true, L.G);
       });
 }
 

@@ -6,6 +6,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -54,6 +55,7 @@ struct alignas(64) TcProblem {
 struct alignas(64) TcGroup {
   TcProblem p[MAX_PROBLEMS];
   int count;
+  int slices;                                // gemm_tc_split_kernel: blocks of a cluster, which share a tile's reduction
   int32_t* status;
   // Optional chores for the epilogue warps while the first tile's main loop runs: zero-fill a buffer that a later
   // kernel of the pass adds into (16-byte units, dealt evenly to the blocks), and reset the pass's status word.
@@ -120,18 +122,25 @@ __device__ __forceinline__ float gelu_grad_fast(float u) {
 }
 __device__ __forceinline__ float sigmoid_fast(float g) { return __fdividef(1.f, 1.f + __expf(-g)); }
 
+// A warp's lanes of an accumulator in tensor memory.
+struct TmemAcc {
+  uint32_t addr;
+  __device__ __forceinline__ void load(int col, uint32_t (&v)[32]) const { tc::tmem_ld32(addr + col, v); }
+  __device__ __forceinline__ void wait() const { tc::tmem_ld_wait(); }
+};
+
 // One output tile of a CTA's 128 accumulator rows: TMEM -> registers -> swizzled staging -> bulk tensor store.  Each warp
 // owns the 32 rows of its TMEM lane quarter and its staging tiles, and issues its own stores: no block-wide hand-off per
-// panel, and the store of one panel overlaps the conversion of the next.  `acc`: the warp's lanes of the accumulator;
-// `wait`: waits until it is complete (what does not depend on it is requested first).
+// panel, and the store of one panel overlaps the conversion of the next.  `q`: which 32 rows; `acc`: reads 32 columns of
+// them (this lane's row); `wait`: waits until they are complete (what does not depend on them is requested first).
 // ESETS = 2 (launches in which every block has a single tile, so that nothing overlaps its epilogue): two sets of four
 // warps share the tile's 64-column panels, first and second half, and the epilogue takes half as long.  Each warp then
 // has one staging tile instead of two (the staging area is the same size).
 // EPI: what the instantiation can fuse besides bias, residual and the row reduction.
 enum { EPI_NONE = 0, EPI_ACT, EPI_ROPE };
-template <int BN, int ESETS, int EPI, typename Wait>
-__device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0, uint32_t acc, uint32_t stg0, int& pc, Wait wait) {
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, q = warp % 4, set = (warp - 2) / 4;
+template <int BN, int ESETS, int EPI, typename Acc, typename Wait>
+__device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0, int q, Acc acc, uint32_t stg0, int& pc, Wait wait) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, set = (warp - 2) / 4;
   constexpr int PPS = BN / 64 / ESETS;              // panels per set
   const int row = m0 + q * 32 + lane;               // row of the problem owned by this thread
   const bool pad = P.t_pad > 0 && (row % P.t_pad) >= P.seq;
@@ -172,9 +181,9 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
     const int n = n0 + pn * 64;
     if (n >= P.n) break;                           // uniform: N is whole 64-column panels
     uint32_t v[64];
-    tc::tmem_ld32(acc + pn * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-    tc::tmem_ld32(acc + pn * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-    tc::tmem_ld_wait();
+    acc.load(pn * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+    acc.load(pn * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+    acc.wait();
     if (P.ksplit > 1) {
       // partial sums of a reduction slice: two 32-column halves of the panel, fp32, added to the accumulation
       // buffer by bulk tensor reductions (same staging tiles and swizzle as the bf16 rows below)
@@ -310,8 +319,8 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
             uint32_t w[32];
-            tc::tmem_ld32(acc + (pn ^ 1) * 64 + hf * 32, w);
-            tc::tmem_ld_wait();
+            acc.load((pn ^ 1) * 64 + hf * 32, w);
+            acc.wait();
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
               const float2 cs = tab[(long long)(hf * 32 + j) * P.t_pad];
@@ -528,7 +537,7 @@ __global__ void __launch_bounds__(64 + 128 * ESETS, 1) gemm_tc_kernel(const __gr
     for (int w = blockIdx.x; ok && tile_at<BN>(G, w, &tcd); w += gridDim.x, ++ti) {
       const TcProblem& P = G.p[tcd.prob];
       const int ab = ti & 1;
-      const bool ready = epilogue_tile<BN, ESETS, EPI>(P, tcd.m0, tcd.n0, tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN, base + SP::STG_OFF, pc, [&] {
+      const bool ready = epilogue_tile<BN, ESETS, EPI>(P, tcd.m0, tcd.n0, q, TmemAcc{tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN}, base + SP::STG_OFF, pc, [&] {
         return tc::mbar_wait(acc_full(ab), (ti >> 1) & 1, status, 103);
       });
       if (!ready) { ok = false; break; }
@@ -694,7 +703,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair
       const TcProblem& P = G.p[tcd.prob];
       const int ab = ti & 1;
       const int m0 = tcd.m0 + (int)rank * 128;
-      const bool ready = epilogue_tile<BN, 1, EPI>(P, m0, tcd.n0, tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN, base + SP::STG_OFF, pc, [&] {
+      const bool ready = epilogue_tile<BN, 1, EPI>(P, m0, tcd.n0, q, TmemAcc{tmem_base + ((uint32_t)(q * 32) << 16) + ab * BN}, base + SP::STG_OFF, pc, [&] {
         return tc::mbar_wait(acc_full(ab), (ti >> 1) & 1, status, 113);
       });
       if (!ready) { ok = false; break; }
@@ -707,6 +716,193 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair
   __syncthreads();
   tc::cluster_sync_all();                        // neither CTA frees tensor memory or leaves while its peer may still
   if (warp == 1) tc::tmem_dealloc2(tmem_base, TMEM_COLS);   // read its shared memory or signal its barriers
+}
+
+// ---------------------------------------------------------------------------------------------------
+// Launches with few tiles and long reductions (few tokens: 50 x 768 outputs are six tiles for 148 SMs): the reduction of a
+// 128 x 128 tile is cut into 2 or 4 slices, one per block of a cluster.  Each block accumulates its slice in tensor
+// memory and leaves the fp32 sums in shared memory, over its operand stages; then it finishes its share of the tile's
+// rows, adding the slices through distributed shared memory in a fixed order.  One tile per cluster.  The bound is a
+// block's chain: first operands, its k-blocks at about 545 clk each, the exchange (about 2.5 us: distributed shared memory
+// gives a block some 15 bytes/clk), the epilogue.  Rank-16 adapter products of 4096 x 2048 (32 k-blocks, 32 row tiles):
+// 14.3 -> 12.0 us forward and 18.5 -> 13.0 us backward.
+// ---------------------------------------------------------------------------------------------------
+constexpr int SPLIT_STAGES = 6, SPLIT_LD = 132;        // pitch of a partial row, in floats: 16-byte accesses without conflicts
+__device__ __forceinline__ float4 ld_cluster(uint32_t a) {
+  float4 f;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f.x), "=f"(f.y), "=f"(f.z), "=f"(f.w) : "r"(a) : "memory");
+  return f;
+}
+struct PartialAcc {
+  uint32_t row;                                        // this lane's row in shared memory
+  __device__ __forceinline__ void load(int col, uint32_t (&v)[32]) const {
+#pragma unroll
+    for (int j = 0; j < 32; j += 4)
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[j]), "=r"(v[j + 1]), "=r"(v[j + 2]), "=r"(v[j + 3]) : "r"(row + (col + j) * 4) : "memory");
+  }
+  __device__ __forceinline__ void wait() const {}
+};
+
+template <int EPI>
+__global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_constant__ TcGroup G) {
+  constexpr int BN = 128, STAGES = SPLIT_STAGES;
+  using SP = SmemPlan<BN, STAGES>;
+  static_assert(128 * SPLIT_LD * 4 <= STAGES * (int)SP::STAGE, "a partial tile fits the operand stages");
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t bars = base + SP::BAR_OFF, slot = bars + 8 * SP::N_BARS, acc_full = bars + 8u * (2 * STAGES);
+  auto full = [&](int s) { return bars + 8u * s; };
+  auto empty = [&](int s) { return bars + 8u * (STAGES + s); };
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  int32_t* status = G.status;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      tc::mbar_init(full(s), 1);
+      tc::mbar_init(empty(s), 1);
+    }
+    tc::mbar_init(acc_full, 1);
+    tc::fence_barrier_init();
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(slot, BN);
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  uint32_t tmem_base;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  pdl_launch_dependents();
+
+  const int slice = blockIdx.x % G.slices;
+  TileCoord tcd;
+  tile_at<BN>(G, blockIdx.x / G.slices, &tcd);
+  const TcProblem& P = G.p[tcd.prob];
+  int total = 0;
+  for (int t = 0; t < P.n_terms; ++t) total += P.kblocks[t];
+  const int per = (total + G.slices - 1) / G.slices, begin = slice * per, end = min(total, begin + per);   // no slice is empty
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- TMA producer; the first weights before waiting for the kernel in front, as in gemm_tc_kernel ----
+      int prefilled = 0;
+      if (P.b_static && begin < P.kblocks[0]) {
+        prefilled = min(STAGES, min(end, P.kblocks[0]) - begin);
+        for (int i = 0; i < prefilled; ++i) {
+          const uint32_t sb = base + i * SP::STAGE + SP::A_BYTES;
+          tc::mbar_expect_tx(full(i), SP::STAGE);
+          if (P.b_mn[0]) tc::tma_load_3d(sb, &P.tb[0], full(i), 0, (begin + i) * BK, tcd.n0 / 64);
+          else tc::tma_load_3d(sb, &P.tb[0], full(i), 0, tcd.n0, begin + i);
+        }
+      }
+      pdl_wait();
+      int t = 0, first = 0;                              // term of the k-block, and its first k-block
+      for (int k = begin, it = 0; k < end; ++k, ++it) {
+        while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }
+        const int kb = k - first, s = it % STAGES;
+        const uint32_t sa = base + s * SP::STAGE, sb = sa + SP::A_BYTES;
+        if (it >= prefilled) {
+          if (!tc::mbar_wait(empty(s), ((it / STAGES) & 1) ^ 1, status, 141)) break;
+          tc::mbar_expect_tx(full(s), SP::STAGE);
+        }
+        if (P.a_mn[t]) tc::tma_load_3d(sa, &P.ta[t], full(s), 0, kb * BK, tcd.m0 / 64);
+        else tc::tma_load_3d(sa, &P.ta[t], full(s), 0, tcd.m0, kb);
+        if (it >= prefilled) {
+          if (P.b_mn[t]) tc::tma_load_3d(sb, &P.tb[t], full(s), 0, kb * BK, tcd.n0 / 64);
+          else tc::tma_load_3d(sb, &P.tb[t], full(s), 0, tcd.n0, kb);
+        }
+      }
+    }
+    __syncwarp();
+    tc::cluster_sync_all();
+    tc::cluster_arrive();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---- MMA issuer ----
+      const uint32_t hi = tc::smem_desc_hi(1024);
+      int t = 0, first = 0;
+      bool ok = true;
+      for (int k = begin, it = 0; k < end; ++k, ++it) {
+        while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }
+        const int s = it % STAGES;
+        if (!tc::mbar_wait(full(s), (it / STAGES) & 1, status, 142)) { ok = false; break; }
+        tc::tc_fence_after();
+        const uint32_t idesc = tc::idesc_bf16(BM, BN, P.a_mn[t], P.b_mn[t]), sa = base + s * SP::STAGE;
+        uint32_t a_lo = tc::smem_desc_lo(sa, P.a_mn[t] ? 8192u : 16u), b_lo = tc::smem_desc_lo(sa + SP::A_BYTES, P.b_mn[t] ? 8192u : 16u);
+        const uint32_t a_step = P.a_mn[t] ? 128u : 2u, b_step = P.b_mn[t] ? 128u : 2u;
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          tc::mma_bf16_ss_w(tmem_base, a_lo, hi, b_lo, hi, idesc, (it > 0 || kk > 0) ? 1u : 0u);
+          a_lo += a_step; b_lo += b_step;
+        }
+        tc::mma_commit(empty(s));
+      }
+      if (ok) tc::mma_commit(acc_full);
+    }
+    __syncwarp();
+    tc::cluster_sync_all();
+    tc::cluster_arrive();
+  } else {
+    // ---- epilogue warps: partial rows to shared memory, then this block's share of the row groups ----
+    pdl_wait();
+    group_chores(G, threadIdx.x - 64, 256);
+    const int q = warp % 4, set = (warp - 2) / 4, groups = 4 / G.slices;
+    auto exchange = [&]() -> bool {
+      const bool ok = tc::mbar_wait(acc_full, 0, status, 143);
+      tc::tc_fence_after();
+      if (ok && tcd.m0 + q * 32 < P.m) {
+        const uint32_t row = base + ((q * 32 + lane) * SPLIT_LD + set * 64) * 4;
+#pragma unroll 1
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t v[32];
+          tc::tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + set * 64 + hf * 32, v);
+          tc::tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; j += 4)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + (hf * 32 + j) * 4), "r"(v[j]), "r"(v[j + 1]), "r"(v[j + 2]), "r"(v[j + 3]) : "memory");
+        }
+      }
+      __syncwarp();
+      tc::cluster_sync_all();
+      // this block's rows: sixteen independent 16-byte loads a thread, their sums in place of its own partial rows
+      const int tid = threadIdx.x - 64, mine = 32 * min(32 * groups, P.m - tcd.m0 - slice * groups * 32);
+      for (int i = tid; i < mine; i += 512) {
+        const uint32_t at0 = base + (((slice * groups * 32) + i / 32) * SPLIT_LD + i % 32 * 4) * 4, at1 = at0 + 8 * SPLIT_LD * 4;
+        const bool two = i + 256 < mine;
+        float4 a[4], b[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c < G.slices) {
+            a[c] = ld_cluster(tc::map_to_cta(at0, c));
+            if (two) b[c] = ld_cluster(tc::map_to_cta(at1, c));
+          }
+#pragma unroll
+        for (int c = 1; c < 4; ++c)
+          if (c < G.slices) {
+            a[0].x += a[c].x; a[0].y += a[c].y; a[0].z += a[c].z; a[0].w += a[c].w;
+            b[0].x += b[c].x; b[0].y += b[c].y; b[0].z += b[c].z; b[0].w += b[c].w;
+          }
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at0), "f"(a[0].x), "f"(a[0].y), "f"(a[0].z), "f"(a[0].w) : "memory");
+        if (two)
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at1), "f"(b[0].x), "f"(b[0].y), "f"(b[0].z), "f"(b[0].w) : "memory");
+      }
+      __syncwarp();
+      tc::cluster_arrive();                              // the others' partial rows have been read
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      return ok;
+    };
+    const int rg = slice * groups + q;                   // the row group this warp finishes (the first `groups` warps of a set)
+    int pc = 0;
+    if (q < groups && tcd.m0 + rg * 32 < P.m)
+      epilogue_tile<BN, 2, EPI>(P, tcd.m0, tcd.n0, rg, PartialAcc{base + (rg * 32 + lane) * SPLIT_LD * 4}, base + SP::STG_OFF, pc, exchange);
+    else
+      exchange();
+    if (lane == 0) tc::bulk_wait_group0();
+    __syncwarp();
+  }
+  tc::tc_fence_before();
+  tc::cluster_wait();                                    // no block leaves while another may still read its partial rows
+  if (warp == 1) tc::tmem_dealloc(tmem_base, BN);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -870,11 +1066,12 @@ int group_epi(const GemmArgs* gs, int count) {
 struct GroupLaunch {
   TcGroup G;
   void (*kernel)(const TcGroup);
-  int grid, threads, serial;
+  int grid, threads, serial, cluster;        // cluster: blocks of a cluster where the launch says so, else 0
   size_t smem;
 };
 
-cudaError_t group_launch(GroupLaunch& L, void (*k)(const TcGroup), int grid, int threads, size_t smem, int serial) {
+cudaError_t group_launch(GroupLaunch& L, void (*k)(const TcGroup), int grid, int threads, size_t smem, int serial, int cluster = 0) {
+  L.cluster = cluster;
   L.kernel = k; L.grid = grid; L.threads = threads; L.smem = smem; L.serial = serial;
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
@@ -888,14 +1085,25 @@ cudaError_t make_group_bn(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs,
   // one tile per block at most: the epilogue is exposed, and the variant with two sets of epilogue warps halves it
   // (with several tiles per block the epilogues overlap the next main loops and the extra warps only cost)
   const int esets_knob = esets_choice ? esets_choice : p->knob_gemm_esets;
-  const bool two_sets = esets_knob ? esets_knob == 2 : tiles <= p->sm_count;
+  const bool two_sets = BN > 64 && (esets_knob ? esets_knob == 2 : tiles <= p->sm_count);
+  constexpr int SETS = BN > 64 ? 2 : 1;
   void (*k)(const TcGroup) = nullptr;
   switch (group_epi(gs, count)) {
-    case EPI_ACT: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_ACT> : gemm_tc_kernel<BN, STAGES, 1, EPI_ACT>; break;
-    case EPI_ROPE: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_ROPE> : gemm_tc_kernel<BN, STAGES, 1, EPI_ROPE>; break;
-    default: k = two_sets ? gemm_tc_kernel<BN, STAGES, 2, EPI_NONE> : gemm_tc_kernel<BN, STAGES, 1, EPI_NONE>;
+    case EPI_ACT: k = two_sets ? gemm_tc_kernel<BN, STAGES, SETS, EPI_ACT> : gemm_tc_kernel<BN, STAGES, 1, EPI_ACT>; break;
+    case EPI_ROPE: k = two_sets ? gemm_tc_kernel<BN, STAGES, SETS, EPI_ROPE> : gemm_tc_kernel<BN, STAGES, 1, EPI_ROPE>; break;
+    default: k = two_sets ? gemm_tc_kernel<BN, STAGES, SETS, EPI_NONE> : gemm_tc_kernel<BN, STAGES, 1, EPI_NONE>;
   }
   return group_launch(L, k, grid, two_sets ? 320 : 192, SmemPlan<BN, STAGES>::TOTAL, gs[0].serial);
+}
+
+cudaError_t make_group_split(GroupLaunch& L, const GemmArgs* gs, int count, int32_t* status, int slices) {
+  int tiles = 0;
+  cudaError_t e = fill_group(L.G, gs, count, status, 128, BM, 128, &tiles);
+  if (e != cudaSuccess) return e;
+  L.G.slices = slices;
+  const int epi = group_epi(gs, count);
+  auto k = epi == EPI_ACT ? gemm_tc_split_kernel<EPI_ACT> : epi == EPI_ROPE ? gemm_tc_split_kernel<EPI_ROPE> : gemm_tc_split_kernel<EPI_NONE>;
+  return group_launch(L, k, tiles * slices, 320, SmemPlan<128, SPLIT_STAGES>::TOTAL, gs[0].serial, slices);
 }
 
 cudaError_t make_group_pair(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status) {
@@ -911,13 +1119,13 @@ cudaError_t make_group_pair(GroupLaunch& L, const fbl_plan* p, const GemmArgs* g
 
 namespace {
 
-// Output tiles a launch may use: 128 x 128 or 128 x 256 on one CTA, 256 x 256 on a CTA pair.
-enum TileKind { TILE_NARROW = 0, TILE_WIDE, TILE_PAIR };
+// Output tiles a launch may use: 128 x 64 (slim), 128 x 128 or 128 x 256 on one CTA, 256 x 256 on a CTA pair.
+enum TileKind { TILE_NARROW = 0, TILE_WIDE, TILE_PAIR, TILE_SLIM };
 struct TileCost { int m, n; double kb, unit, epilogue, fixed; };      // extents; clocks per k-block, per unit, of an epilogue, per launch
 // Clocks from a sweep of the four launches of a layer over 64 to 6300 tokens and widths of 320 to 3264 columns.  A
 // k-block of a wide tile costs less than two of a narrow one (operands are re-read half as often per flop), a pair's
 // less still, but pairs start later; with few k-blocks the epilogue of the tile before is what a tile waits for.
-const TileCost TILE_COST[3] = {{128, 128, 545, 800, 1600, 0}, {128, 256, 710, 900, 3600, 0}, {256, 256, 675, 900, 3600, 3500}};
+const TileCost TILE_COST[4] = {{128, 128, 545, 800, 1600, 0}, {128, 256, 710, 900, 3600, 0}, {256, 256, 675, 900, 3600, 3500}, {128, 64, 400, 800, 1600, 0}};
 struct TileWork { long long m; int n, kb, split; };
 
 // Clocks of the longest block (pair) when the persistent kernel deals the units of a group's problems out in turn.
@@ -940,6 +1148,39 @@ double tile_makespan(const TileCost& c, const TileWork* w, int count, int slots)
   return longest + (dealt <= slots ? 0.5 : 1.0) * c.epilogue + c.fixed;
 }
 
+// Slices of gemm_tc_split_kernel (2 or 4; 0: that kernel is not the fastest) for a launch that takes `clocks` without.
+int best_slices(const TileWork* w, int count, int sm_count, double clocks) {
+  int pick = 0;
+  for (int S = 2; S <= 4; S *= 2) {
+    long long blocks = 0;
+    int longest = 0;
+    bool legal = true;
+    for (int i = 0; i < count; ++i) {
+      blocks += ((w[i].m + 127) / 128) * ((w[i].n + 127) / 128) * S;
+      legal = legal && w[i].split == 1 && w[i].kb >= 2 * S;
+      longest = std::max(longest, (w[i].kb + S - 1) / S);
+    }
+    if (!legal || blocks > sm_count) continue;
+    // against a tile of its own: the cluster's start, the partial rows' way through shared memory, two barriers
+    const double t = longest * TILE_COST[TILE_NARROW].kb + TILE_COST[TILE_NARROW].unit + 0.5 * TILE_COST[TILE_NARROW].epilogue + 5500;
+    if (t < clocks) { clocks = t; pick = S; }
+  }
+  return pick;
+}
+
+// 128 x 64 tiles: less to load per k-block, and more SMs loading, where there are fewer tiles than SMs (50 tokens of 768:
+// 20.0 -> 19.1 us a layer forward; 94 x 7 tokens of 320 x 640 gated: 57.8 -> 51.7 us a step).  With more tiles than SMs
+// they only add loads of A; and a row of a head of 128, which the rotation and the row reduction need whole, spans two.
+bool slim_legal(const GemmArgs* gs, int count, int sm_count) {
+  long long tiles = 0;
+  bool legal = true;
+  for (int i = 0; i < count; ++i) {
+    tiles += (long long)((gs[i].m + 127) / 128) * (gs[i].n / 64) * (gs[i].ksplit > 1 ? gs[i].ksplit : 1);
+    legal = legal && (!gs[i].dot_with || gs[i].dot_hd <= 64) && (gs[i].epi != 5 || gs[i].rope_hd <= 64);
+  }
+  return legal && tiles <= sm_count;
+}
+
 int best_tile(const TileWork* w, int count, int sm_count, bool pairs, double* clocks) {
   int kind = TILE_NARROW;
   *clocks = 1e300;
@@ -957,6 +1198,7 @@ int best_tile(const TileWork* w, int count, int sm_count, bool pairs, double* cl
 static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, const fbl_plan::GemmChoice& ch) {
   const int pair_mode = ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 always, -1 by cost
   int kind = TILE_NARROW;
+  GemmArgs by_length[MAX_PROBLEMS];
   if (pair_mode == 1) {
     kind = TILE_PAIR;
   } else if (ch.bn) {
@@ -969,8 +1211,32 @@ static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs*
     }
     double clocks;
     kind = best_tile(w, count, p->sm_count, pair_mode != 0, &clocks);
+    if (slim_legal(gs, count, p->sm_count)) {
+      const double t = tile_makespan(TILE_COST[TILE_SLIM], w, count, p->sm_count);
+      if (t < clocks) { clocks = t; kind = TILE_SLIM; }
+    }
+    const int slices = best_slices(w, count, p->sm_count, clocks);
+    if (slices) return make_group_split(L, gs, count, status, slices);
+    // The problems come with the token-axis reductions first; of few tokens those are the shortest, and the longest
+    // units should start first.
+    int order[MAX_PROBLEMS];
+    for (int i = 0; i < count; ++i) order[i] = i;
+    std::stable_sort(order, order + count, [&](int a, int b) { return w[a].kb / w[a].split > w[b].kb / w[b].split; });
+    TileWork sorted[MAX_PROBLEMS];
+    for (int i = 0; i < count; ++i) sorted[i] = w[order[i]];
+    double sorted_clocks;
+    const int sorted_kind = best_tile(sorted, count, p->sm_count, pair_mode != 0, &sorted_clocks);
+    if (kind != TILE_SLIM && sorted_clocks < 0.95 * clocks) {
+      kind = sorted_kind;
+      for (int i = 0; i < count; ++i) by_length[i] = gs[order[i]];
+      for (int i = 0; i < count; ++i) { by_length[i].zero_bytes = 0; by_length[i].reset_status = by_length[i].serial = 0; }
+      by_length[0].zero_ptr = gs[0].zero_ptr; by_length[0].zero_bytes = gs[0].zero_bytes;      // the launch's chores stay with its first problem
+      by_length[0].reset_status = gs[0].reset_status; by_length[0].serial = gs[0].serial;
+      gs = by_length;
+    }
   }
   if (kind == TILE_PAIR) return make_group_pair(L, p, gs, count, status);
+  if (kind == TILE_SLIM) return make_group_bn<64, 8>(L, p, gs, count, status, 1);
   if (kind == TILE_WIDE) return make_group_bn<256, 4>(L, p, gs, count, status, ch.esets);
   return make_group_bn<128, 6>(L, p, gs, count, status, ch.esets);
 }
@@ -987,6 +1253,7 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
   return LaunchMemo<GroupLaunch, 12, 248>::run(p->memo[FBL_MEMO_TC_GEMM], key,
       [&](GroupLaunch& L) { return make_group(L, p, gs, count, status, ch); },
       [&](const GroupLaunch& L) {
+        if (L.cluster) return launch_cluster(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.cluster, !L.serial, L.G);
         return L.serial ? launch_serial(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.G)
                         : launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.G);
       });

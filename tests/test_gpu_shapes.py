@@ -131,3 +131,21 @@ def test_attention_backward_of_short_sequences(cfg):
 ], ids=lambda c: c.name)
 def test_fp32_attention_tiles(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # few tokens and long reductions (cluster-split products): one to four row groups of a tile, two row tiles, remainders of
+    # the reduction over the slices, every epilogue (bias, residual, row reduction, activations, rotation at both widths)
+    LayerConfig("sp1", 1, 20, 1024, 16, 4, 64, "bf16", "layernorm", True, True, True, 1e-5, 281, 0.02),
+    LayerConfig("sp2", 3, 50, 1088, 7, 7, 128, "bf16", "rmsnorm", True, True, False, 1e-5, 282, 0.02, 0.0, 10000.0),
+    LayerConfig("sp3", 1, 101, 1216, 19, 1, 64, "bf16", "rmsnorm", False, False, True, 1e-5, 283, 0.02, 0.0, 10000.0),
+    MlpConfig("sp4", 1, 33, 1024, 2048, "bf16", "layernorm", "gelu", True, True, 1e-5, 284, 0.02),
+    MlpConfig("sp5", 2, 60, 1152, 1984, "bf16", "rmsnorm", "swiglu", True, True, 1e-5, 285, 0.02),
+    # short reductions (128 x 64 tiles): one panel, a ragged number of panels, tiles up to the number of SMs
+    LayerConfig("sp7", 2, 70, 448, 7, 7, 64, "bf16", "layernorm", True, True, True, 1e-5, 287, 0.02, 0.0, 10000.0),
+    MlpConfig("sp8", 3, 129, 192, 576, "bf16", "rmsnorm", "swiglu", True, True, 1e-5, 288, 0.02),
+    LayerConfig("sp9", 4, 250, 320, 5, 1, 64, "bf16", "rmsnorm", False, True, True, 1e-5, 289, 0.02),
+    XattnConfig("sp6", 2, 9, 60, 1024, 1280, 8, 8, 128, "bf16", "layernorm", True, True, 1e-5, 286, 0.02),
+], ids=lambda c: c.name)
+def test_few_tokens_long_reductions(cfg):
+    check(cfg)
