@@ -548,6 +548,16 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
   else FBL_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   // back through the rotation of Q and K: its transpose is the rotation by the opposite angle
   if (p->rope_base > 0.f && !(p->use_tc && attn_bwd_tc_supported(p))) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
+  // every bias gradient is a token-axis column sum: the four of them run beside the last products, or else in the norm
+  // backward's two launches
+  ColsumGroup sums = {};
+  float* cp = (float*)part;
+  if (bias) {
+    colsum_add(sums, dY, p->n_pad, D, dbo, &cp);
+    colsum_add(sums, dQ, p->n_pad, p->dq, dbq, &cp);
+    colsum_add(sums, dK, p->n_pad, p->dkv, dbk, &cp);
+    colsum_add(sums, dV, p->n_pad, p->dkv, dbv, &cp);
+  }
   {
     const void* G[3] = {dQ, dK, dV};
     void* DW[3] = {dWq, dWk, dWv};
@@ -569,7 +579,10 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     gx.t[2] = {dV, p->n_pad, 0, Wv, D, 1, p->dkv};
     gx.c = dXn; gx.c_rpad = p->n_pad; gx.seq = p->d.seq; gx.t_pad = p->t_pad;
     ConvertGroup cg = {};
-    if (gemm_group_tc(p, gs, 4)) {
+    int idle = 0;
+    const bool tc = gemm_group_tc(p, gs, 4), early = tc && colsum_early_pays(p, sums);
+    if (tc) {
+      if (early) gs[0].late_trigger = &idle;
       if (split_qkv) {
         float* acc = (float*)(sc + p->sb_acc_qkv);
         for (int i = 0; i < 3; ++i) {
@@ -586,6 +599,7 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
       }
     }
     FBL_GEMM_STEP("dWqkv+dXn", gs, 4, FBL_GEMM_DWQKV_DXN);
+    if (early) FBL_STEP("db", 1, launch_colsum_early(p, sums, idle, st));
     if (cg.count > 0) FBL_STEP("dW round", 1, launch_convert_f32_group(cg, st));     // one rounding launch for all sliced GEMMs
   }
   if (dwo_round) {
@@ -593,11 +607,7 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     cg.src[0] = (const float*)(sc + p->sb_acc_o); cg.dst[0] = dWo; cg.n[0] = up8(p->dq) * (int64_t)D; cg.count = 1;
     FBL_STEP("dW round", 1, launch_convert_f32_group(cg, st));
   }
-  // every bias gradient is a token-axis column sum: the four of them ride in the norm backward's two launches
-  const void* M4[4] = {dY, dQ, dK, dV};
-  float* O4[4] = {dbo, dbq, dbk, dbv};
-  const int C4[4] = {D, p->dq, p->dkv, p->dkv};
-  FBL_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, (float*)part, st, bias ? 4 : 0, M4, C4, O4));
+  FBL_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials((float*)part, cp), st, &sums));
   return FBL_OK;
 }
 

@@ -110,6 +110,10 @@ struct GemmArgs {
   // later kernel of the pass; reset the pass's status word), and `serial`: the launch may not start before
   // everything ahead of it on the stream has completed
   void* zero_ptr; size_t zero_bytes; int reset_status, serial;
+  // likewise, where not null (tensor-core kernels; see launch_colsum_early): the next launch on the stream may start only
+  // once everything ahead of this one has completed; receives the clocks an SM is expected to stand idle before the
+  // launch's slowest block ends, on average
+  int* late_trigger;
   // fused activation of the feed-forward block (tensor-core kernel only): 0 none, 1 GELU forward (c = U, c2 = gelu(U)),
   // 2 GELU backward (c = value * gelu'(U), U in `residual`), 3 gated forward (c = G, c2 = silu(G) * U, U in `residual`),
   // 4 gated backward (c = value * silu(G), c2 = value * U * silu'(G); U in `residual`, G in `aux1`)
@@ -166,16 +170,44 @@ cudaError_t launch_rope(const fbl_plan* p, void* A, int heads_a, void* B, int he
 // rope: where to leave the rotary embedding's table, [head_dim / 2][t_pad] (cosine, sine) of token t * base^(-2i/head_dim)
 cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma, const float* beta, void* Xn,
                             float* stats, int32_t* status, cudaStream_t st, float2* rope = nullptr);
-// counts its own launches in p->launches (one to three)
+// Token-axis column sums of up to four matrices: slabs of 256 rows are summed to one row of partials each (at part[i],
+// slabs x cols), which a second kernel adds up.
+struct ColsumGroup {
+  const void* m[4];
+  float* out[4];
+  float* part[4];
+  int64_t rows[4];
+  int cols[4], slabs[4];
+  int count;
+  int summed;               // the slabs' sums are under way already (launch_colsum_early)
+};
+// Adds a matrix; its partials come from *part, which moves on.
+void colsum_add(ColsumGroup& G, const void* m, int64_t rows, int cols, float* out, float** part);
+// Panels of slabs: the pieces of work of the first stage.
+static inline int64_t colsum_units(const fbl_plan* p, const ColsumGroup& G) {
+  int64_t units = 0;
+  for (int i = 0; i < G.count; ++i) units += (int64_t)G.slabs[i] * (G.cols[i] / p->tw);
+  return units;
+}
+// Whether the sums are better off beside the products than in the norm backward's launches, where up to about two pieces
+// per SM pass unnoticed (steps of 10 to 120 us: 1 to 4 % slower beside the products with up to 324 pieces on 148 SMs, 2 to
+// 5 % faster with 366 and more).
+static inline bool colsum_early_pays(const fbl_plan* p, const ColsumGroup& G) {
+  return G.count > 0 && 4 * colsum_units(p, G) > 9 * (int64_t)p->sm_count;
+}
+// The slabs' sums as a launch directly behind a tensor-core product launch with late_trigger (which gave `idle`), beside
+// which it runs: the matrices must have been complete before that product's launch.
+cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, cudaStream_t st);
+// Where the norm's own partial rows begin, behind column-sum partials from `part` to `end`.
+static inline float* norm_partials(float* part, const float* end) { return part + (end - part + 255) / 256 * 256; }
+// Norm backward with the column sums of `sums`; counts its own launches in p->launches (one to three).
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                             const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
-                            cudaStream_t st, int bias_count = 0, const void* const* bias_m = nullptr,
-                            const int* bias_cols = nullptr, float* const* bias_out = nullptr);
+                            cudaStream_t st, const ColsumGroup* sums = nullptr);
 cudaError_t launch_colsum(int dtype, const void* M, int64_t rows, int64_t cols, float* out, float* partials,
                           cudaStream_t st);
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols);
-cudaError_t launch_colsum_group(int dtype, int count, const void* const* M, int64_t rows, const int* cols,
-                                float* const* out, float* partials, cudaStream_t st);
+cudaError_t launch_colsum_group(int dtype, const ColsumGroup& G, cudaStream_t st);
 
 // fp32 storage (k_ffma_attn.cu); the backward adds into dQ, zeroed by the caller
 cudaError_t launch_attn_fwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,

@@ -342,25 +342,18 @@ __global__ void __launch_bounds__(256) rope_bwd_round_kernel(const float* __rest
 
 constexpr int COLSUM_SLAB = 256;
 
-struct ColsumGroup {
-  const void* m[4];
-  float* out[4];
-  int cols[4];
-  int64_t part_off[4];      // float offset of each matrix's partials inside the scratch area
-  int count;
-};
-
 // First stage of a token-axis column sum: the block's (128-byte column panel p, slab of 256 rows) of matrix `which`,
 // 32 storage tiles, reduced to one row of partials.  Any block of whole warps up to 512 threads; `red` has a row per warp.
 template <typename T>
-__device__ __forceinline__ void colsum_slab(const ColsumGroup& G, int64_t rows, float* __restrict__ part_base, int p,
-                                            int slab, int which, float (*red)[tile_w_of<T>::value + 1]) {
+__device__ __forceinline__ void colsum_slab(const ColsumGroup& G, int p, int slab, int which,
+                                            float (*red)[tile_w_of<T>::value + 1]) {
   constexpr int TW = tile_w_of<T>::value;
   constexpr int V = Vec16<T>::N;
   const int cols = G.cols[which];
-  if (p * TW >= cols) return;
+  if (p * TW >= cols || slab >= G.slabs[which]) return;
   const T* M = (const T*)G.m[which];
-  float* part = part_base + G.part_off[which];
+  const int64_t rows = G.rows[which];
+  float* part = G.part[which];
   const int rr = threadIdx.x / 8, l8 = threadIdx.x % 8, rstep = blockDim.x / 8;
   float acc[V];
 #pragma unroll
@@ -401,8 +394,7 @@ __global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn
                                                        const float* __restrict__ stats, const float* __restrict__ gamma,
                                                        T* __restrict__ dX, float* __restrict__ partials, int64_t n_pad, int d,
                                                        int tpr, int64_t per_block, int rms, int n_norm,
-                                                       const __grid_constant__ ColsumGroup CG,
-                                                       float* __restrict__ cs_part, int cs_panels, int cs_slabs) {
+                                                       const __grid_constant__ ColsumGroup CG, int cs_panels, int cs_slabs) {
   constexpr int V = Vec16<T>::N, TW = tile_w_of<T>::value;
   // exchange buffers of the row sums; the column-sum blocks use it as well
   __shared__ __align__(16) float s_ex[16 * (TW + 1) > 2 * NORM_EX ? 16 * (TW + 1) : 2 * NORM_EX];
@@ -412,7 +404,7 @@ __global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn
     pdl_launch_dependents();
     pdl_wait();
     const int idx = (int)blockIdx.x - n_norm;
-    colsum_slab<T>(CG, n_pad, cs_part, idx % cs_panels, (idx / cs_panels) % cs_slabs, idx / (cs_panels * cs_slabs),
+    colsum_slab<T>(CG, idx % cs_panels, (idx / cs_panels) % cs_slabs, idx / (cs_panels * cs_slabs),
                    reinterpret_cast<float(*)[TW + 1]>(s_ex));
     return;
   }
@@ -605,15 +597,14 @@ __global__ void __launch_bounds__(256) rope_kernel(T* __restrict__ A, int heads_
 // the step's two small final reductions share one launch.
 __global__ void __launch_bounds__(256) norm_bwd_reduce_kernel(const float* __restrict__ part, int blocks, int d,
                                                               float* __restrict__ dgamma, float* __restrict__ dbeta,
-                                                              int ny_norm, const __grid_constant__ ColsumGroup G, const float* __restrict__ cpart,
-                                                              int n_slabs) {
+                                                              int ny_norm, const __grid_constant__ ColsumGroup G) {
   __shared__ float red[8][33];
   pdl_launch_dependents();
   pdl_wait();
   if ((int)blockIdx.y >= ny_norm) {
     const int which = blockIdx.y - ny_norm;
-    const int cols = G.cols[which];
-    const float* cp = cpart + G.part_off[which];
+    const int cols = G.cols[which], n_slabs = G.slabs[which];
+    const float* cp = G.part[which];
     for (int c = blockIdx.x * 256 + threadIdx.x; c < cols; c += gridDim.x * 256) {
       float s = 0.f;
 #pragma unroll 8
@@ -648,11 +639,88 @@ __global__ void __launch_bounds__(256) norm_bwd_reduce_kernel(const float* __res
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) colsum_stage1(const __grid_constant__ ColsumGroup G, int64_t rows, float* __restrict__ part_base) {
+__global__ void __launch_bounds__(256) colsum_stage1(const __grid_constant__ ColsumGroup G) {
   __shared__ float red[8][tile_w_of<T>::value + 1];
   pdl_launch_dependents();
   pdl_wait();
-  colsum_slab<T>(G, rows, part_base, blockIdx.x, blockIdx.y, blockIdx.z, red);
+  colsum_slab<T>(G, blockIdx.x, blockIdx.y, blockIdx.z, red);
+}
+
+// The same sums beside a tensor-core product: that kernel starts its dependents only after its own wait, so everything in
+// front of it, the matrices among it, is complete when this one runs; the wait for the product comes last, for the kernels
+// behind this one.  A block takes a slab of a panel at a time; small as it is, and with at most one per SM, it fits beside
+// a product block.  Loads go to L2, whose data is current.  Bound by memory, and hidden by the product:
+// 2048 x 768 and 2048 x 3072 cost 5 us of a step of 114 us in a launch of their own; two of 3000 x 1280, with their
+// second stage, 7 us of 199 us.
+__global__ void __launch_bounds__(128, 8) colsum_early_kernel(const __grid_constant__ ColsumGroup G) {
+  using T = __nv_bfloat16;
+  constexpr int TW = tile_w_of<T>::value, V = Vec16<T>::N, B = 8, STEP = 16 * B;
+  __shared__ __align__(16) float red[3][TW];                            // 768 bytes: a product block leaves 1.9 KB, 1 KB of it reserved
+  pdl_launch_dependents();
+  const int warp = threadIdx.x / 32, rr = threadIdx.x / 8, l8 = threadIdx.x % 8;
+  // position of the next batch of 128 rows: unit (panel of a slab of a matrix), and its first row of this thread
+  int which = -1, left = (int)blockIdx.x, units = 0;
+  int64_t row = 0, r_end = 0;
+  const uint4* src = nullptr;
+  float* out = nullptr;
+  auto open_unit = [&]() {                                              // the first matrix that unit `left` falls into
+    while (left >= units) {
+      left -= units;
+      if (++which >= G.count) return;
+      units = G.cols[which] / TW * G.slabs[which];
+    }
+    const int cols = G.cols[which], panels = cols / TW, p = left % panels, slab = left / panels;
+    const int64_t rows = G.rows[which];
+    row = (int64_t)slab * COLSUM_SLAB + rr;
+    r_end = min((int64_t)(slab + 1) * COLSUM_SLAB, rows);
+    src = reinterpret_cast<const uint4*>((const T*)G.m[which] + (int64_t)p * rows * TW) + l8;
+    out = G.part[which] + (int64_t)slab * cols + p * TW + l8 * V;
+  };
+  open_unit();
+  uint4 u[B];                                                           // always a batch of loads in flight
+#pragma unroll
+  for (int k = 0; k < B; ++k) u[k] = which < G.count && row + k * 16 < r_end ? __ldcg(src + (row + k * 16) * 8) : make_uint4(0u, 0u, 0u, 0u);
+  float acc[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) acc[i] = 0.f;
+  while (which < G.count) {
+    float* const to = out;
+    const bool last = row - rr + STEP >= r_end;                         // uniform over the block
+    row += STEP;
+    if (last) {
+      left += gridDim.x;
+      open_unit();
+    }
+    const bool more = which < G.count;
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      float v[V];
+      load16(reinterpret_cast<const T*>(&u[k]), v);
+#pragma unroll
+      for (int i = 0; i < V; ++i) acc[i] += v[i];
+      u[k] = more && row + k * 16 < r_end ? __ldcg(src + (row + k * 16) * 8) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (last) {
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 8);
+        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+      }
+      if (warp > 0 && rr % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) red[warp - 1][l8 * V + i] = acc[i];
+      }
+      __syncthreads();
+      if (rr == 0) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) to[i] = acc[i] + red[0][l8 * V + i] + red[1][l8 * V + i] + red[2][l8 * V + i];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < V; ++i) acc[i] = 0.f;
+    }
+  }
+  pdl_wait();
 }
 
 template <typename T, int NV, int PF, int TPR>
@@ -671,7 +739,7 @@ cudaError_t norm_fwd_launch(const fbl_plan* p, const NormShape& s, const void* X
 template <typename T, int NV, int R>
 cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* dXn, const void* X, const void* dY,
                             const float* stats, const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
-                            const ColsumGroup& cg, float* cpart, int n_slabs, cudaStream_t st) {
+                            const ColsumGroup& cg, cudaStream_t st) {
   constexpr int V = Vec16<T>::N;
   const int d = p->d.d_model, rms = p->d.norm == FBL_NORM_RMSNORM;
   const int64_t pass = (int64_t)s.groups * R;
@@ -680,14 +748,17 @@ cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* d
   const int64_t per_block = ((p->n_pad + most - 1) / most + pass - 1) / pass * pass;
   const int blocks = (int)((p->n_pad + per_block - 1) / per_block);
   const size_t ring = (size_t)norm_stages(R, NV) * (dY ? 3 : 2) * R * NV * s.tpr * s.groups * 16;
-  int cs_panels = 0;
-  for (int i = 0; i < cg.count; ++i) cs_panels = cg.cols[i] / tile_w_of<T>::value > cs_panels ? cg.cols[i] / tile_w_of<T>::value : cs_panels;
+  int cs_panels = 0, n_slabs = 0;
+  for (int i = 0; i < cg.count && !cg.summed; ++i) {
+    cs_panels = max(cs_panels, cg.cols[i] / tile_w_of<T>::value);
+    n_slabs = max(n_slabs, cg.slabs[i]);
+  }
   // The column sums' first stage shares this launch while it is a few blocks for each that fits an SM beside the ring's
   // shared memory, which those blocks occupy without using it; beyond that a launch of its own is cheaper (91 us
   // together, 40 us apart for four 2977 x 2880 matrices; 4 us dearer apart for a 2048 x 768 and a 2048 x 3072 one).
   int cs_blocks = cs_panels * n_slabs * cg.count;
   if (cs_blocks > (ring <= 56 * 1024 ? 8 : 4) * p->sm_count) {
-    cudaError_t ce = launch_pdl(colsum_stage1<T>, dim3(cs_panels, n_slabs, cg.count), dim3(256), 0, st, cg, p->n_pad, cpart);
+    cudaError_t ce = launch_pdl(colsum_stage1<T>, dim3(cs_panels, n_slabs, cg.count), dim3(256), 0, st, cg);
     if (ce != cudaSuccess) return ce;
     p->launches++;
     cs_blocks = 0;
@@ -698,27 +769,28 @@ cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* d
   if (e != cudaSuccess) return e;
   e = launch_pdl(norm_bwd_kernel<T, NV, R>, dim3(blocks + cs_blocks), dim3(s.tpr * s.groups), smem, st,
                              (const T*)dXn, (const T*)X, (const T*)dY, stats, gamma, (T*)dX, dgamma ? part : (float*)nullptr, p->n_pad,
-                             d, s.tpr, per_block, rms, blocks, cg, cpart, cs_panels, n_slabs);
+                             d, s.tpr, per_block, rms, blocks, cg, cs_panels, n_slabs);
   if (e != cudaSuccess) return e;
   const int ny = !dgamma ? 0 : rms ? 1 : 2;
   p->launches += ny + cg.count == 0 ? 1 : 2;
   if (ny + cg.count == 0) return cudaSuccess;
   return launch_pdl(norm_bwd_reduce_kernel, dim3((d + 31) / 32, ny + cg.count), dim3(256), 0, st, (const float*)part,
-                    blocks, d, dgamma, dbeta, ny, cg, (const float*)cpart, n_slabs);
+                    blocks, d, dgamma, dbeta, ny, cg);
 }
 
 // ------------------------------------------------------------------------------------------
 // Token-axis column sums, two stages over tiles: (1) one block per (panel, slab of 256 rows)
 // reduces its 32 storage tiles to one row of partials, (2) a tree over slabs.
 // ------------------------------------------------------------------------------------------
-__global__ void colsum_stage2(const __grid_constant__ ColsumGroup G, const float* __restrict__ part_base, int n_slabs) {
+__global__ void colsum_stage2(const __grid_constant__ ColsumGroup G) {
   pdl_launch_dependents();
   pdl_wait();
   const int which = blockIdx.y;
   const int cols = G.cols[which];
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= cols) return;
-  const float* part = part_base + G.part_off[which];
+  const float* part = G.part[which];
+  const int n_slabs = G.slabs[which];
   float s = 0.f;
 #pragma unroll 8
   for (int k = 0; k < n_slabs; ++k) s += part[(int64_t)k * cols + c];
@@ -795,9 +867,9 @@ cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma
 template <typename T>
 cudaError_t norm_bwd_dispatch(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                               const float* gamma, void* dX, float* dgamma, float* dbeta, float* npart,
-                              const ColsumGroup& cg, float* cpart, int n_slabs, cudaStream_t st) {
+                              const ColsumGroup& cg, cudaStream_t st) {
   const NormShape s = norm_bwd_shape(p->d.d_model / Vec16<T>::N, p->n_pad, p->sm_count);
-#define FBL_CALL(NV_, R_) norm_bwd_launch<T, NV_, R_>(p, s, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, cpart, n_slabs, st)
+#define FBL_CALL(NV_, R_) norm_bwd_launch<T, NV_, R_>(p, s, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, st)
   switch (s.nv) {
     case 1: return s.r == 4 ? FBL_CALL(1, 4) : s.r == 2 ? FBL_CALL(1, 2) : FBL_CALL(1, 1);
     case 2: return s.r == 2 ? FBL_CALL(2, 2) : FBL_CALL(2, 1);
@@ -808,26 +880,36 @@ cudaError_t norm_bwd_dispatch(const fbl_plan* p, const void* dXn, const void* X,
 #undef FBL_CALL
 }
 
-// Norm backward (dgamma = nullptr: only dX, the norm's parameters are frozen), and with it (bias_count > 0) the bias
-// column sums of up to four matrices: their first stage runs as extra blocks of the first kernel, their second stage
-// inside the second.  `part` holds the column-sum slab partials first and the norm's per-block partial rows behind them.
+void colsum_add(ColsumGroup& G, const void* m, int64_t rows, int cols, float* out, float** part) {
+  const int i = G.count++;
+  G.m[i] = m; G.rows[i] = rows; G.cols[i] = cols; G.out[i] = out; G.part[i] = *part;
+  G.slabs[i] = (int)((rows + COLSUM_SLAB - 1) / COLSUM_SLAB);
+  *part += (int64_t)G.slabs[i] * cols;
+}
+
+cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, cudaStream_t st) {
+  int64_t bytes = 0;
+  for (int i = 0; i < G.count; ++i) bytes += G.rows[i] * G.cols[i] * 2;
+  // Where the product's SMs run out of work at different times, those that have (some 13 bytes/clk each) do the sums, and
+  // the ask for shared memory keeps them away from the busy ones: sharing those made a product of 46 us 2 us longer.  Where
+  // they all end together that is no help, and the sums share the SMs (47 MB of sums beside a product of 75 us: a step of
+  // 276 us that way, 251 us sharing).
+  const bool beside = (int64_t)idle * p->sm_count * 13 < bytes;
+  const dim3 grid((unsigned)min((int64_t)p->sm_count, colsum_units(p, G)));
+  G.summed = 1;
+  return launch_pdl(colsum_early_kernel, grid, dim3(128), beside ? 0 : 2048, st, G);
+}
+
+// Norm backward (dgamma = nullptr: only dX, the norm's parameters are frozen), and with it the bias column sums of up to
+// four matrices: their first stage, unless it ran beside the product in front, as extra blocks of the first kernel, their
+// second stage inside the second.  `part`: the norm's per-block partial rows.
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                             const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
-                            cudaStream_t st, int bias_count, const void* const* bias_m, const int* bias_cols,
-                            float* const* bias_out) {
-  ColsumGroup cg;
-  memset(&cg, 0, sizeof(cg));
-  const int n_slabs = (int)((p->n_pad + COLSUM_SLAB - 1) / COLSUM_SLAB);
-  if (bias_count > 4) return cudaErrorInvalidValue;
-  int64_t off = 0;
-  for (int i = 0; i < bias_count; ++i) {
-    cg.m[i] = bias_m[i]; cg.out[i] = bias_out[i]; cg.cols[i] = bias_cols[i]; cg.part_off[i] = off;
-    off += (int64_t)n_slabs * bias_cols[i];
-  }
-  cg.count = bias_count;
-  float* npart = part + (off + 255) / 256 * 256;
-  if (p->d.dtype == FBL_DTYPE_FP32) return norm_bwd_dispatch<float>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, part, n_slabs, st);
-  return norm_bwd_dispatch<__nv_bfloat16>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, part, n_slabs, st);
+                            cudaStream_t st, const ColsumGroup* sums) {
+  ColsumGroup cg = {};
+  if (sums) cg = *sums;
+  if (p->d.dtype == FBL_DTYPE_FP32) return norm_bwd_dispatch<float>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, st);
+  return norm_bwd_dispatch<__nv_bfloat16>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, st);
 }
 
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols) {
@@ -835,34 +917,25 @@ size_t colsum_scratch_bytes(int64_t rows, int64_t cols) {
   return (size_t)(slabs * cols) * sizeof(float);
 }
 
-// Column sums of up to four matrices that share a row count, in one pair of launches.
-cudaError_t launch_colsum_group(int dtype, int count, const void* const* M, int64_t rows, const int* cols, float* const* out,
-                                float* partials, cudaStream_t st) {
-  if (count < 1 || count > 4) return cudaErrorInvalidValue;
-  const int slabs = (int)((rows + COLSUM_SLAB - 1) / COLSUM_SLAB);
-  ColsumGroup G;
-  int max_cols = 0;
-  int64_t off = 0;
-  for (int i = 0; i < count; ++i) {
-    G.m[i] = M[i]; G.out[i] = out[i]; G.cols[i] = cols[i]; G.part_off[i] = off;
-    off += (int64_t)slabs * cols[i];
-    max_cols = cols[i] > max_cols ? cols[i] : max_cols;
-  }
-  G.count = count;
+// Column sums in a pair of launches of their own.
+cudaError_t launch_colsum_group(int dtype, const ColsumGroup& G, cudaStream_t st) {
+  if (G.count < 1) return cudaErrorInvalidValue;
+  int max_cols = 0, slabs = 0;
+  for (int i = 0; i < G.count; ++i) { max_cols = max(max_cols, G.cols[i]); slabs = max(slabs, G.slabs[i]); }
   const int tw = dtype == FBL_DTYPE_FP32 ? 32 : 64;
-  dim3 grid((unsigned)(max_cols / tw), slabs, count);
+  const dim3 grid((unsigned)(max_cols / tw), slabs, G.count);
   cudaError_t e;
-  if (dtype == FBL_DTYPE_FP32) e = launch_pdl(colsum_stage1<float>, grid, dim3(256), 0, st, G, rows, partials);
-  else e = launch_pdl(colsum_stage1<__nv_bfloat16>, grid, dim3(256), 0, st, G, rows, partials);
+  if (dtype == FBL_DTYPE_FP32) e = launch_pdl(colsum_stage1<float>, grid, dim3(256), 0, st, G);
+  else e = launch_pdl(colsum_stage1<__nv_bfloat16>, grid, dim3(256), 0, st, G);
   if (e != cudaSuccess) return e;
-  dim3 grid2((unsigned)((max_cols + 127) / 128), count);
-  return launch_pdl(colsum_stage2, grid2, dim3(128), 0, st, G, (const float*)partials, slabs);
+  return launch_pdl(colsum_stage2, dim3((unsigned)((max_cols + 127) / 128), G.count), dim3(128), 0, st, G);
 }
 
 cudaError_t launch_colsum(int dtype, const void* M, int64_t rows, int64_t cols, float* out, float* partials,
                           cudaStream_t st) {
-  const int c = (int)cols;
-  return launch_colsum_group(dtype, 1, &M, rows, &c, &out, partials, st);
+  ColsumGroup G = {};
+  colsum_add(G, M, rows, (int)cols, out, &partials);
+  return launch_colsum_group(dtype, G, st);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -55,6 +55,7 @@ struct alignas(64) TcProblem {
 struct alignas(64) TcGroup {
   TcProblem p[MAX_PROBLEMS];
   int count;
+  int late_trigger;                          // as in GemmArgs: the dependents' trigger comes after the wait
   int slices;                                // gemm_tc_split_kernel: blocks of a cluster, which share a tile's reduction
   int32_t* status;
   // Optional chores for the epilogue warps while the first tile's main loop runs: zero-fill a buffer that a later
@@ -407,7 +408,7 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
 // other accumulator (bias, residual, padding-row mask, bf16 rows in R-Tile order), so the epilogue of
 // one tile overlaps the main loop of the next.
 template <int BN, int STAGES, int ESETS, int EPI>
-__global__ void __launch_bounds__(64 + 128 * ESETS, 1) gemm_tc_kernel(const __grid_constant__ TcGroup G) {
+__global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_tc_kernel(const __grid_constant__ TcGroup G) {
   using SP = SmemPlan<BN, STAGES>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(64 + 128 * ESETS, 1) gemm_tc_kernel(const __gr
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
-  pdl_launch_dependents();
+  if (!G.late_trigger) pdl_launch_dependents();
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer ----------------------------------------------------------------------
@@ -465,6 +466,7 @@ __global__ void __launch_bounds__(64 + 128 * ESETS, 1) gemm_tc_kernel(const __gr
       prefilled = n;
     }
     pdl_wait();
+    if (G.late_trigger) pdl_launch_dependents();
     for (int w = blockIdx.x; ok && tile_at<BN>(G, w, &tcd); w += gridDim.x) {
       const TcProblem& P = G.p[tcd.prob];
       for (int t = 0; t < P.n_terms && ok; ++t) {
@@ -591,7 +593,7 @@ __device__ __forceinline__ bool pair_tile_at(const TcGroup& G, int w, TileCoord*
 }
 
 template <int EPI>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair_kernel(const __grid_constant__ TcGroup G) {
+__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224) gemm_tc_pair_kernel(const __grid_constant__ TcGroup G) {
   using SP = PairSmem;
   constexpr int STAGES = PAIR_STAGES, BN = PAIR_BN;
   extern __shared__ uint8_t smem_raw[];
@@ -629,7 +631,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
-  pdl_launch_dependents();
+  if (!G.late_trigger) pdl_launch_dependents();
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer (both CTAs): own A rows, own half of B's columns; bytes counted on the leader's barrier ----
@@ -637,6 +639,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1) gemm_tc_pair
     bool ok = true;
     TileCoord tcd;
     pdl_wait();
+    if (G.late_trigger) pdl_launch_dependents();
     for (int w = pair_id; ok && pair_tile_at(G, w, &tcd); w += n_pairs) {
       const TcProblem& P = G.p[tcd.prob];
       const int m0 = tcd.m0 + (int)rank * 128, n0 = tcd.n0 + (int)rank * 128;
@@ -772,7 +775,7 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
-  pdl_launch_dependents();
+  if (!G.late_trigger) pdl_launch_dependents();
 
   const int slice = blockIdx.x % G.slices;
   TileCoord tcd;
@@ -796,6 +799,7 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
         }
       }
       pdl_wait();
+      if (G.late_trigger) pdl_launch_dependents();
       int t = 0, first = 0;                              // term of the k-block, and its first k-block
       for (int k = begin, it = 0; k < end; ++k, ++it) {
         while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }
@@ -1004,6 +1008,7 @@ cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int32_t* statu
   memset(&G, 0, sizeof(G));
   G.count = count;
   G.status = status;
+  G.late_trigger = gs[0].late_trigger != nullptr;
   G.zero_ptr = (uint4*)gs[0].zero_ptr; G.zero_vec = (long long)(gs[0].zero_bytes / 16); G.reset_status = gs[0].reset_status;
   int tiles = 0;
   for (int i = 0; i < count; ++i) {
@@ -1067,6 +1072,7 @@ struct GroupLaunch {
   TcGroup G;
   void (*kernel)(const TcGroup);
   int grid, threads, serial, cluster;        // cluster: blocks of a cluster where the launch says so, else 0
+  int idle;                                  // what a late_trigger receives
   size_t smem;
 };
 
@@ -1129,7 +1135,7 @@ const TileCost TILE_COST[4] = {{128, 128, 545, 800, 1600, 0}, {128, 256, 710, 90
 struct TileWork { long long m; int n, kb, split; };
 
 // Clocks of the longest block (pair) when the persistent kernel deals the units of a group's problems out in turn.
-double tile_makespan(const TileCost& c, const TileWork* w, int count, int slots) {
+double tile_makespan(const TileCost& c, const TileWork* w, int count, int slots, double* idle = nullptr) {
   std::vector<double> load((size_t)slots, 0.0);
   long long dealt = 0;
   for (int i = 0; i < count; ++i) {
@@ -1143,8 +1149,9 @@ double tile_makespan(const TileCost& c, const TileWork* w, int count, int slots)
     }
     dealt += units;
   }
-  double longest = 0;
-  for (double l : load) longest = l > longest ? l : longest;
+  double longest = 0, sum = 0;
+  for (double l : load) { longest = l > longest ? l : longest; sum += l; }
+  if (idle) *idle = longest - sum / slots;
   return longest + (dealt <= slots ? 0.5 : 1.0) * c.epilogue + c.fixed;
 }
 
@@ -1199,16 +1206,16 @@ static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs*
   const int pair_mode = ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 always, -1 by cost
   int kind = TILE_NARROW;
   GemmArgs by_length[MAX_PROBLEMS];
+  TileWork w[MAX_PROBLEMS];
+  for (int i = 0; i < count; ++i) {
+    w[i] = {gs[i].m, gs[i].n, 0, gs[i].ksplit > 1 ? gs[i].ksplit : 1};
+    for (int t = 0; t < gs[i].n_terms; ++t) w[i].kb += (gs[i].t[t].k + BK - 1) / BK;
+  }
   if (pair_mode == 1) {
     kind = TILE_PAIR;
   } else if (ch.bn) {
     kind = ch.bn == 128 ? TILE_NARROW : TILE_WIDE;
   } else {
-    TileWork w[MAX_PROBLEMS];
-    for (int i = 0; i < count; ++i) {
-      w[i] = {gs[i].m, gs[i].n, 0, gs[i].ksplit > 1 ? gs[i].ksplit : 1};
-      for (int t = 0; t < gs[i].n_terms; ++t) w[i].kb += (gs[i].t[t].k + BK - 1) / BK;
-    }
     double clocks;
     kind = best_tile(w, count, p->sm_count, pair_mode != 0, &clocks);
     if (slim_legal(gs, count, p->sm_count)) {
@@ -1216,7 +1223,10 @@ static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs*
       if (t < clocks) { clocks = t; kind = TILE_SLIM; }
     }
     const int slices = best_slices(w, count, p->sm_count, clocks);
-    if (slices) return make_group_split(L, gs, count, status, slices);
+    if (slices) {
+      L.idle = 1 << 20;                              // fewer blocks than SMs, as a rule
+      return make_group_split(L, gs, count, status, slices);
+    }
     // The problems come with the token-axis reductions first; of few tokens those are the shortest, and the longest
     // units should start first.
     int order[MAX_PROBLEMS];
@@ -1228,13 +1238,16 @@ static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs*
     const int sorted_kind = best_tile(sorted, count, p->sm_count, pair_mode != 0, &sorted_clocks);
     if (kind != TILE_SLIM && sorted_clocks < 0.95 * clocks) {
       kind = sorted_kind;
-      for (int i = 0; i < count; ++i) by_length[i] = gs[order[i]];
-      for (int i = 0; i < count; ++i) { by_length[i].zero_bytes = 0; by_length[i].reset_status = by_length[i].serial = 0; }
+      for (int i = 0; i < count; ++i) { by_length[i] = gs[order[i]]; w[i] = sorted[i]; }
+      for (int i = 0; i < count; ++i) { by_length[i].zero_bytes = 0; by_length[i].reset_status = by_length[i].serial = 0; by_length[i].late_trigger = nullptr; }
       by_length[0].zero_ptr = gs[0].zero_ptr; by_length[0].zero_bytes = gs[0].zero_bytes;      // the launch's chores stay with its first problem
-      by_length[0].reset_status = gs[0].reset_status; by_length[0].serial = gs[0].serial;
+      by_length[0].reset_status = gs[0].reset_status; by_length[0].serial = gs[0].serial; by_length[0].late_trigger = gs[0].late_trigger;
       gs = by_length;
     }
   }
+  double idle;
+  tile_makespan(TILE_COST[kind], w, count, kind == TILE_PAIR ? p->sm_count / 2 : p->sm_count, &idle);
+  L.idle = (int)idle;
   if (kind == TILE_PAIR) return make_group_pair(L, p, gs, count, status);
   if (kind == TILE_SLIM) return make_group_bn<64, 8>(L, p, gs, count, status, 1);
   if (kind == TILE_WIDE) return make_group_bn<256, 4>(L, p, gs, count, status, ch.esets);
@@ -1253,6 +1266,7 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
   return LaunchMemo<GroupLaunch, 12, 248>::run(p->memo[FBL_MEMO_TC_GEMM], key,
       [&](GroupLaunch& L) { return make_group(L, p, gs, count, status, ch); },
       [&](const GroupLaunch& L) {
+        if (gs[0].late_trigger) *gs[0].late_trigger = L.idle;
         if (L.cluster) return launch_cluster(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.cluster, !L.serial, L.G);
         return L.serial ? launch_serial(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.G)
                         : launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.G);

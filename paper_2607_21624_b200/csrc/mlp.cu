@@ -405,6 +405,14 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
       MLP_STEP(1, act(p, true, dH, U, G, dU, dG, st));
     }
   }
+  // bias gradients: token-axis column sums of dY, dU (and dG), beside the last products or in the norm backward's launches
+  ColsumGroup sums = {};
+  float* cp = part;
+  if (bias) {
+    colsum_add(sums, dY, p->n_pad, D, db2, &cp);
+    colsum_add(sums, dU, p->n_pad, F, db1, &cp);
+    if (gated) colsum_add(sums, dG, p->n_pad, F, dbg, &cp);
+  }
   {
     GemmArgs gs[3];
     const void* Gr[2] = {dU, dG}; void* DW[2] = {dW1, dWg};
@@ -434,17 +442,15 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
         acc += up8(D) * (int64_t)F;
       }
     }
-    int k = 0;
+    int k = 0, idle = 0;
+    const bool early = all_tc && colsum_early_pays(bp, sums);
+    if (early) gs[0].late_trigger = &idle;
     MLP_CUDA(run_gemm_group(bp, gs, nw + 1, status, st, -1, &k));
     p->launches += k;
+    if (early) MLP_STEP(1, launch_colsum_early(bp, sums, idle, st));
   }
   if (cg.count > 0) MLP_STEP(1, launch_convert_f32_group(cg, st));
-  // bias gradients: token-axis column sums of dY, dU (and dG), riding in the norm backward's launches
-  const void* M3[3] = {dY, dU, dG};
-  float* O3[3] = {db2, db1, dbg};
-  const int C3[3] = {D, F, F};
-  const int nb = gated ? 3 : 2;
-  MLP_STEP(0, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st, bias ? nb : 0, M3, C3, O3));
+  MLP_STEP(0, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums));
   return FBL_OK;
 }
 

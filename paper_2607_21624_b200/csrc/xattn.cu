@@ -160,6 +160,14 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
   if (p->use_tc && attn_bwd_tc_supported(p)) XA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
   else if (p->d.dtype == FBL_DTYPE_FP32) XA_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
   else XA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
+  // bias gradients: column sums over the query tokens (dY, dQ) and over the memory's tokens (dK, dV), beside the last
+  // products or, the former, in the norm backward's launches
+  ColsumGroup sums = {};
+  float* cp = part;
+  if (bias) {
+    colsum_add(sums, dY, p->n_pad, D, dbo, &cp);
+    colsum_add(sums, dQ, p->n_pad, p->dq, dbq, &cp);
+  }
   {
     // query side: dWq = Xn^T dQ (token-axis reduction), dXn = dQ Wq^T
     // memory side: dWk = M^T dK, dWv = M^T dV (reductions over the memory's tokens), dM = dK Wk^T + dV Wv^T
@@ -203,18 +211,23 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
         acc += up8(Dm) * (int64_t)p->dkv;
       }
     }
+    int idle = 0;
+    if (bias && tc) all[0].late_trigger = &idle;
     XA_GEMM_STEP("dWqkv+dXn+dM", all, 5);
+    if (bias && tc) {
+      colsum_add(sums, dK, p->n_pad_kv, p->dkv, dbk, &part_kv);
+      colsum_add(sums, dV, p->n_pad_kv, p->dkv, dbv, &part_kv);
+      XA_STEP("db", 1, launch_colsum_early(p, sums, idle, st));
+    }
     if (cg.count > 0) XA_STEP("dW round", 1, launch_convert_f32_group(cg, st));
   }
-  // bias gradients: column sums over the query tokens (dY, dQ) and over the memory's tokens (dK, dV)
-  const void* Mq[2] = {dY, dQ};
-  float* Oq[2] = {dbo, dbq};
-  const int Cq[2] = {D, p->dq};
-  const void* Mk[2] = {dK, dV};
-  float* Ok[2] = {dbk, dbv};
-  const int Ck[2] = {p->dkv, p->dkv};
-  if (bias) XA_STEP("db_kv", 2, launch_colsum_group(p->d.dtype, 2, Mk, p->n_pad_kv, Ck, Ok, part_kv, st));
-  XA_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st, bias ? 2 : 0, Mq, Cq, Oq));
+  if (bias && !sums.summed) {
+    ColsumGroup kv = {};
+    colsum_add(kv, dK, p->n_pad_kv, p->dkv, dbk, &part_kv);
+    colsum_add(kv, dV, p->n_pad_kv, p->dkv, dbv, &part_kv);
+    XA_STEP("db_kv", 2, launch_colsum_group(p->d.dtype, kv, st));
+  }
+  XA_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums));
   return FBL_OK;
 }
 

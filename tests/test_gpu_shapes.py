@@ -149,3 +149,16 @@ def test_fp32_attention_tiles(cfg):
 ], ids=lambda c: c.name)
 def test_few_tokens_long_reductions(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # bias gradients summed beside the last products: ragged last slabs, one to three matrices' worth of pieces per block
+    LayerConfig("cs1", 2, 290, 2048, 16, 16, 128, "bf16", "layernorm", True, True, True, 1e-5, 291, 0.01),
+    LayerConfig("cs2", 9, 133, 1024, 16, 4, 64, "bf16", "rmsnorm", False, True, False, 1e-5, 292, 0.01, 0.0, 10000.0),
+    MlpConfig("cs3", 2, 270, 1024, 4096, "bf16", "rmsnorm", "swiglu", True, True, 1e-5, 293, 0.01),
+    MlpConfig("cs4", 5, 405, 768, 2048, "bf16", "layernorm", "gelu", True, False, 1e-5, 294, 0.01),
+    XattnConfig("cs5", 1, 8, 520, 512, 512, 8, 8, 64, "bf16", "layernorm", True, True, 1e-5, 295, 0.02),
+    XattnConfig("cs6", 2, 300, 300, 512, 256, 4, 4, 128, "bf16", "rmsnorm", True, True, 1e-5, 296, 0.02),
+], ids=lambda c: c.name)
+def test_bias_gradients_beside_products(cfg):
+    check(cfg)
