@@ -494,25 +494,7 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
   const bool bias = p->d.has_bias;
   const int n = (int)p->n_pad, D = p->d.d_model;
 
-  // One fill zeroes the status word and, behind it, every fp32 area the step adds into: the accumulation areas
-  // of sliced weight-gradient GEMMs and the dQ accumulator.  No fill then separates later kernels of the step,
-  // so each can start (programmatic dependent launch) while its predecessor drains.
   const bool split_o = p->use_tc && p->ksplit_o > 1, split_qkv = p->use_tc && p->ksplit_qkv > 1;
-  // Without sliced GEMMs on the tensor-core path (only the dQ accumulator and the status word to clear) the first
-  // GEMM launch does it instead: its idle epilogue warps zero the accumulator while its first tiles are computed.
-  // The fill node was also the barrier between the forward and the backward kernels, which the attention backward
-  // relies on when it requests forward-pass data (K, V, Q, LSE) before waiting for the kernel in front of it: that
-  // GEMM is therefore launched without programmatic overlap, i.e. only once the forward pass has completed.
-  bool first_gemm_fills = false;
-  // (Measured: 2 % on workload 2; for accumulators of tens of MB the stores delay the launch's own first tiles by
-  // more than the fill node costs, so large plans keep the node.)
-  if (p->use_tc && p->acc_bytes == 0 && attn_bwd_tc_supported(p) && bwd_zero_bytes(p) - p->sb_dqacc <= ((size_t)16 << 20)) {
-    GemmArgs gw = GemmArgs{}, ga = GemmArgs{};
-    gw.m = p->dq; gw.n = D; gw.n_terms = 1; gw.t[0] = {A, p->n_pad, 1, dY, p->n_pad, 0, n}; gw.c = dWo; gw.c_rpad = p->dq;
-    ga.m = n; ga.n = p->dq; ga.n_terms = 1; ga.t[0] = {dY, p->n_pad, 0, Wo, p->dq, 1, D}; ga.c = dA; ga.c_rpad = p->n_pad;
-    first_gemm_fills = gemm_tc_supported(p, gw) && gemm_tc_supported(p, ga);
-  }
-  if (!first_gemm_fills) FBL_CUDA(cudaMemsetAsync(status, 0, bwd_zero_bytes(p), st));
   FBL_PROF_BEGIN();
   bool dvec_ready = false, dwo_round = false;
   {
@@ -535,12 +517,9 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     }
     if (gemm_group_tc(p, gs, 2)) {
       if (split_o) { gw.ksplit = p->ksplit_o; gw.acc = (float*)(sc + p->sb_acc_o); }
-      if (first_gemm_fills) {
-        gs[0].zero_ptr = dqacc; gs[0].zero_bytes = bwd_zero_bytes(p) - p->sb_dqacc;
-        gs[0].reset_status = 1; gs[0].serial = 1;
-      }
       dwo_round = split_o;        // nothing in the step reads dWo: its rounding joins that of dWq, dWk, dWv below
     }
+    FBL_CUDA(start_backward(p, gs, 2, !split_o, true, status, bwd_zero_bytes(p), st));
     FBL_GEMM_STEP("dWo+dA", gs, 2, FBL_GEMM_DWO_DA);
   }
   if (p->use_tc && attn_bwd_tc_supported(p)) FBL_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope));   // dqacc: zero already

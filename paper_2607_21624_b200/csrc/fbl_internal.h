@@ -157,6 +157,12 @@ bool attn_bwd_tc_direct(const fbl_plan* p);    // the tensor-core backward write
 static inline size_t bwd_zero_bytes(const fbl_plan* p) {
   return p->use_tc && attn_bwd_tc_supported(p) && attn_bwd_tc_direct(p) ? p->sb_dqacc : p->zero_bytes;
 }
+// What a backward pass starts with: zero the first `bytes` of its scratch (the status word's block and the fp32 areas the
+// pass adds into).  `rides`: the pass's first products `gs` need nothing of it.  `serial`: no kernel of the pass may start
+// before the forward pass has completed (the attention backward requests that pass's results before waiting for the kernel
+// in front of it).  Counts a launch of its own.
+cudaError_t start_backward(const fbl_plan* p, GemmArgs* gs, int count, bool rides, bool serial, int32_t* status, size_t bytes, cudaStream_t st);
+
 static inline int attn_bwd_tc_launches(const fbl_plan* p, bool dvec_ready) {
   return (dvec_ready ? 1 : 2) + (attn_bwd_tc_direct(p) && !(p->rope_base > 0.f) ? 0 : 1);
 }

@@ -880,6 +880,29 @@ cudaError_t norm_bwd_dispatch(const fbl_plan* p, const void* dXn, const void* X,
 #undef FBL_CALL
 }
 
+// Zero-fill.  Bound by memory; a kernel and not a fill of the driver's, so that the products behind it are set up and their
+// first weights under way when it ends.
+static __global__ void __launch_bounds__(512) fill_kernel(uint4* __restrict__ out, int64_t n) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = z;
+}
+
+cudaError_t start_backward(const fbl_plan* p, GemmArgs* gs, int count, bool rides, bool serial, int32_t* status, size_t bytes, cudaStream_t st) {
+  // Idle epilogue warps of the first products clear what they can while the first tiles are computed; with tens of MB their
+  // stores delay those tiles by more than a launch costs.
+  if (rides && bytes <= (size_t)16 << 20 && gemm_group_tc(p, gs, count)) {
+    gs[0].zero_ptr = (char*)status + FBL_ALIGN; gs[0].zero_bytes = bytes - FBL_ALIGN;
+    gs[0].reset_status = 1; gs[0].serial = serial;
+    return cudaSuccess;
+  }
+  const int64_t n = (int64_t)(bytes / 16);
+  const dim3 grid((unsigned)min((int64_t)p->sm_count * 4, (n + 511) / 512));
+  p->launches++;
+  return serial ? launch_serial(fill_kernel, grid, dim3(512), 0, st, (uint4*)status, n) : launch_pdl(fill_kernel, grid, dim3(512), 0, st, (uint4*)status, n);
+}
+
 void colsum_add(ColsumGroup& G, const void* m, int64_t rows, int cols, float* out, float** part) {
   const int i = G.count++;
   G.m[i] = m; G.rows[i] = rows; G.cols[i] = cols; G.out[i] = out; G.part[i] = *part;

@@ -214,7 +214,6 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
   const int cols[3] = {p->dq, p->dkv, p->dkv};
   int k = 0;
 
-  LORA_CUDA(cudaMemsetAsync(status, 0, bwd_zero_bytes(p), st));    // status word and the dQ accumulator
   if (p->prof_on) { p->prof_n = 0; LORA_CUDA(cudaEventRecord(p->prof_ev[0], st)); }
   bool dvec_ready = false;
   {
@@ -227,6 +226,7 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
       ga.dot_with = A; ga.dot_out = dvec; ga.dot_hd = p->d.head_dim; ga.dot_hq = p->d.n_q_heads;
       dvec_ready = true;
     }
+    LORA_CUDA(start_backward(p, &ga, 1, true, true, status, bwd_zero_bytes(p), st));
     LORA_CUDA(run_gemm_group(p, &ga, 1, status, st, -1, &k));
     LORA_STEP("dA", 0, cudaSuccess);
     p->launches += k;

@@ -372,7 +372,6 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
   const bool tc = bp->use_tc != 0;
   const bool split2 = tc && p->ksplit_2 > 1, split1 = tc && p->ksplit_1 > 1;
 
-  MLP_CUDA(cudaMemsetAsync(status, 0, p->zero_bytes, st));     // status word + accumulation areas of sliced reductions
   ConvertGroup cg = {};
   {
     GemmArgs gs[2];
@@ -393,6 +392,7 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
       cg.src[cg.count] = gw.acc; cg.dst[cg.count] = dW2; cg.n[cg.count] = up8(F) * (int64_t)D; cg.count++;
     }
     int k = 0;
+    MLP_CUDA(start_backward(bp, gs, 2, !split2, false, status, p->zero_bytes, st));    // status word + accumulation areas of sliced reductions
     if (both_tc) {
       // the activation's derivative rides in the dH product's epilogue: dU (and dG) leave the accumulator tile, dH
       // itself is never stored

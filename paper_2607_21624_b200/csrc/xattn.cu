@@ -125,10 +125,6 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
   const bool bias = p->d.has_bias;
   const int n = (int)p->n_pad, nk = (int)p->n_pad_kv, D = p->d.d_model, Dm = p->d_mem;
 
-  // one fill: status word, the accumulation areas of sliced weight-gradient products, the dQ accumulator.  It is
-  // also the barrier between the forward pass's kernels and the backward's, which the attention backward relies on
-  // when it requests forward-pass data before waiting for the kernel in front of it.
-  XA_CUDA(cudaMemsetAsync(status, 0, bwd_zero_bytes(p), st));
   XA_PROF_BEGIN();
   const bool split_o = p->use_tc && p->ksplit_o > 1, split_q = p->use_tc && p->ksplit_qkv > 1,
              split_kv = p->use_tc && p->ksplit_kv > 1;
@@ -155,6 +151,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
       gw.ksplit = p->ksplit_o; gw.acc = (float*)(sc + p->sb_acc_o);
       cg.src[cg.count] = gw.acc; cg.dst[cg.count] = dWo; cg.n[cg.count] = up8(p->dq) * (int64_t)D; cg.count++;
     }
+    XA_CUDA(start_backward(p, gs, 2, !split_o, true, status, bwd_zero_bytes(p), st));
     XA_GEMM_STEP("dWo+dA", gs, 2);
   }
   if (p->use_tc && attn_bwd_tc_supported(p)) XA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
