@@ -496,7 +496,8 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
 
   const bool split_o = p->use_tc && p->ksplit_o > 1, split_qkv = p->use_tc && p->ksplit_qkv > 1;
   FBL_PROF_BEGIN();
-  bool dvec_ready = false, dwo_round = false;
+  bool dvec_ready = false;
+  ConvertGroup cg = {};                     // sliced products leave fp32 sums; the norm backward's second launch rounds them
   {
     GemmArgs gs[2];
     GemmArgs& gw = gs[0];   // dWo = A^T dY : token-axis reduction (longest reduction loop: first in the work list)
@@ -517,7 +518,9 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     }
     if (gemm_group_tc(p, gs, 2)) {
       if (split_o) { gw.ksplit = p->ksplit_o; gw.acc = (float*)(sc + p->sb_acc_o); }
-      dwo_round = split_o;        // nothing in the step reads dWo: its rounding joins that of dWq, dWk, dWv below
+      if (split_o) {
+        cg.src[0] = gw.acc; cg.dst[0] = dWo; cg.n[0] = up8(p->dq) * (int64_t)D; cg.count = 1;
+      }
     }
     FBL_CUDA(start_backward(p, gs, 2, !split_o, true, status, bwd_zero_bytes(p), st));
     FBL_GEMM_STEP("dWo+dA", gs, 2, FBL_GEMM_DWO_DA);
@@ -557,7 +560,6 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
     gx.t[1] = {dK, p->n_pad, 0, Wk, D, 1, p->dkv};
     gx.t[2] = {dV, p->n_pad, 0, Wv, D, 1, p->dkv};
     gx.c = dXn; gx.c_rpad = p->n_pad; gx.seq = p->d.seq; gx.t_pad = p->t_pad;
-    ConvertGroup cg = {};
     int idle = 0;
     const bool tc = gemm_group_tc(p, gs, 4), early = tc && colsum_early_pays(p, sums);
     if (tc) {
@@ -566,27 +568,15 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
         float* acc = (float*)(sc + p->sb_acc_qkv);
         for (int i = 0; i < 3; ++i) {
           gs[i].ksplit = p->ksplit_qkv; gs[i].acc = acc;
-          cg.src[i] = acc; cg.dst[i] = DW[i]; cg.n[i] = up8(D) * (int64_t)cols[i];
-          acc += cg.n[i];
+          cg.src[cg.count] = acc; cg.dst[cg.count] = DW[i]; cg.n[cg.count] = up8(D) * (int64_t)cols[i];
+          acc += cg.n[cg.count++];
         }
-        cg.count = 3;
-      }
-      if (dwo_round) {
-        cg.src[cg.count] = (const float*)(sc + p->sb_acc_o); cg.dst[cg.count] = dWo; cg.n[cg.count] = up8(p->dq) * (int64_t)D;
-        cg.count++;
-        dwo_round = false;
       }
     }
     FBL_GEMM_STEP("dWqkv+dXn", gs, 4, FBL_GEMM_DWQKV_DXN);
     if (early) FBL_STEP("db", 1, launch_colsum_early(p, sums, idle, st));
-    if (cg.count > 0) FBL_STEP("dW round", 1, launch_convert_f32_group(cg, st));     // one rounding launch for all sliced GEMMs
   }
-  if (dwo_round) {
-    ConvertGroup cg = {};
-    cg.src[0] = (const float*)(sc + p->sb_acc_o); cg.dst[0] = dWo; cg.n[0] = up8(p->dq) * (int64_t)D; cg.count = 1;
-    FBL_STEP("dW round", 1, launch_convert_f32_group(cg, st));
-  }
-  FBL_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials((float*)part, cp), st, &sums));
+  FBL_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials((float*)part, cp), st, &sums, &cg));
   return FBL_OK;
 }
 

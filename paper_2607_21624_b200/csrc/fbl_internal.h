@@ -206,10 +206,13 @@ static inline bool colsum_early_pays(const fbl_plan* p, const ColsumGroup& G) {
 cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, cudaStream_t st);
 // Where the norm's own partial rows begin, behind column-sum partials from `part` to `end`.
 static inline float* norm_partials(float* part, const float* end) { return part + (end - part + 255) / 256 * 256; }
-// Norm backward with the column sums of `sums`; counts its own launches in p->launches (one to three).
+// fp32 sums of sliced products, to be rounded to their bf16 places (n multiples of 4).
+struct ConvertGroup { const float* src[4]; void* dst[4]; int64_t n[4]; int count; };
+// Norm backward with the column sums of `sums` and the roundings of `round`; counts its own launches in p->launches (one to
+// three).
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                             const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
-                            cudaStream_t st, const ColsumGroup* sums = nullptr);
+                            cudaStream_t st, const ColsumGroup* sums = nullptr, const ConvertGroup* round = nullptr);
 cudaError_t launch_colsum(int dtype, const void* M, int64_t rows, int64_t cols, float* out, float* partials,
                           cudaStream_t st);
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols);
@@ -229,8 +232,6 @@ cudaError_t launch_attn_bwd_simt(const fbl_plan* p, const void* Q, const void* K
                                  void* dV, bool dvec_ready, cudaStream_t st);
 cudaError_t launch_attn_bwd_pre(const fbl_plan* p, const void* A, const void* dA, float* dvec, float* dqacc,
                                 bool dvec_ready, cudaStream_t st);
-struct ConvertGroup { const float* src[4]; void* dst[4]; int64_t n[4]; int count; };
-cudaError_t launch_convert_f32_group(const ConvertGroup& g, cudaStream_t st);   // bf16 destinations, n multiples of 4
 cudaError_t launch_attn_bwd_post(const fbl_plan* p, const float* dqacc, void* dQ, cudaStream_t st);
 cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                int32_t* status, cudaStream_t st);

@@ -394,21 +394,23 @@ __global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn
                                                        const float* __restrict__ stats, const float* __restrict__ gamma,
                                                        T* __restrict__ dX, float* __restrict__ partials, int64_t n_pad, int d,
                                                        int tpr, int64_t per_block, int rms, int n_norm,
-                                                       const __grid_constant__ ColsumGroup CG, int cs_panels, int cs_slabs) {
+                                                       const __grid_constant__ ColsumGroup CG, int cs_panels, int cs_slabs,
+                                                       int late) {
   constexpr int V = Vec16<T>::N, TW = tile_w_of<T>::value;
   // exchange buffers of the row sums; the column-sum blocks use it as well
   __shared__ __align__(16) float s_ex[16 * (TW + 1) > 2 * NORM_EX ? 16 * (TW + 1) : 2 * NORM_EX];
   // Blocks behind the first n_norm ones do the first stage of the bias gradients' column sums (one launch less):
   // block n_norm + (which * slabs + slab) * panels + p
   if ((int)blockIdx.x >= n_norm) {
-    pdl_launch_dependents();
+    if (!late) pdl_launch_dependents();
     pdl_wait();
+    if (late) pdl_launch_dependents();
     const int idx = (int)blockIdx.x - n_norm;
     colsum_slab<T>(CG, idx % cs_panels, (idx / cs_panels) % cs_slabs, idx / (cs_panels * cs_slabs),
                    reinterpret_cast<float(*)[TW + 1]>(s_ex));
     return;
   }
-  pdl_launch_dependents();
+  if (!late) pdl_launch_dependents();                        // late: what the second kernel rounds is complete when it starts
   const int group = threadIdx.x / tpr, lt = threadIdx.x % tpr, groups = blockDim.x / tpr;
   const float inv_d = 1.f / (float)d;
   int buf = 0;
@@ -423,6 +425,7 @@ __global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn
     for (int i = 0; i < V / 2; ++i) ag[j][i] = ab[j][i] = both(0.f);
   }
   pdl_wait();
+  if (late) pdl_launch_dependents();
   constexpr int S = norm_stages(R, NV);
   extern __shared__ __align__(16) uint8_t s_ring[];          // [stage][X, dXn, (dY)][row][vector][thread]
   const int arrays = dY ? 3 : 2;
@@ -594,12 +597,32 @@ __global__ void __launch_bounds__(256) rope_kernel(T* __restrict__ A, int heads_
 
 // dgamma[c] (y = 0) or dbeta[c] (y = 1) = sum over the first kernel's blocks of their partial rows.  Blocks with
 // y >= ny_norm finish the bias column sums instead (matrix y - ny_norm: the tree over its slab partials), so that
-// the step's two small final reductions share one launch.
+// the step's two small final reductions share one launch.  Blocks behind those (y >= ny_sums) round the fp32 sums of sliced
+// products, which are complete when this kernel starts: beside the first kernel, whose end they wait for only at their own
+// (four 768 x 768 matrices: a launch of 10 us in a step of 191 us before).
 __global__ void __launch_bounds__(256) norm_bwd_reduce_kernel(const float* __restrict__ part, int blocks, int d,
                                                               float* __restrict__ dgamma, float* __restrict__ dbeta,
-                                                              int ny_norm, const __grid_constant__ ColsumGroup G) {
+                                                              int ny_norm, const __grid_constant__ ColsumGroup G, int ny_sums,
+                                                              const __grid_constant__ ConvertGroup C) {
   __shared__ float red[8][33];
   pdl_launch_dependents();
+  if ((int)blockIdx.y >= ny_sums) {
+    const int64_t first = ((int64_t)((blockIdx.y - ny_sums) * gridDim.x + blockIdx.x) * 256 + threadIdx.x) * 4;
+    const int64_t step = (int64_t)(gridDim.y - ny_sums) * gridDim.x * 1024;
+    for (int k = 0; k < C.count; ++k) {
+      __nv_bfloat16* dst = (__nv_bfloat16*)C.dst[k];
+#pragma unroll 4
+      for (int64_t i = first; i < C.n[k]; i += step) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(C.src[k] + i));
+        __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+        uint2 o;
+        o.x = *reinterpret_cast<uint32_t*>(&lo); o.y = *reinterpret_cast<uint32_t*>(&hi);
+        *reinterpret_cast<uint2*>(dst + i) = o;
+      }
+    }
+    pdl_wait();
+    return;
+  }
   pdl_wait();
   if ((int)blockIdx.y >= ny_norm) {
     const int which = blockIdx.y - ny_norm;
@@ -739,7 +762,7 @@ cudaError_t norm_fwd_launch(const fbl_plan* p, const NormShape& s, const void* X
 template <typename T, int NV, int R>
 cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* dXn, const void* X, const void* dY,
                             const float* stats, const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
-                            const ColsumGroup& cg, cudaStream_t st) {
+                            const ColsumGroup& cg, const ConvertGroup& round, cudaStream_t st) {
   constexpr int V = Vec16<T>::N;
   const int d = p->d.d_model, rms = p->d.norm == FBL_NORM_RMSNORM;
   const int64_t pass = (int64_t)s.groups * R;
@@ -769,13 +792,17 @@ cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* d
   if (e != cudaSuccess) return e;
   e = launch_pdl(norm_bwd_kernel<T, NV, R>, dim3(blocks + cs_blocks), dim3(s.tpr * s.groups), smem, st,
                              (const T*)dXn, (const T*)X, (const T*)dY, stats, gamma, (T*)dX, dgamma ? part : (float*)nullptr, p->n_pad,
-                             d, s.tpr, per_block, rms, blocks, cg, cs_panels, n_slabs);
+                             d, s.tpr, per_block, rms, blocks, cg, cs_panels, n_slabs, (int)(round.count > 0));
   if (e != cudaSuccess) return e;
   const int ny = !dgamma ? 0 : rms ? 1 : 2;
-  p->launches += ny + cg.count == 0 ? 1 : 2;
-  if (ny + cg.count == 0) return cudaSuccess;
-  return launch_pdl(norm_bwd_reduce_kernel, dim3((d + 31) / 32, ny + cg.count), dim3(256), 0, st, (const float*)part,
-                    blocks, d, dgamma, dbeta, ny, cg);
+  const int nx = (d + 31) / 32, ny_sums = ny + cg.count;
+  int64_t rounded = 0;
+  for (int i = 0; i < round.count; ++i) rounded = max(rounded, round.n[i]);
+  const int ny_round = (int)((min((int64_t)p->sm_count * 4, (rounded + 1023) / 1024) + nx - 1) / nx);
+  p->launches += ny_sums + ny_round == 0 ? 1 : 2;
+  if (ny_sums + ny_round == 0) return cudaSuccess;
+  return launch_pdl(norm_bwd_reduce_kernel, dim3(nx, ny_sums + ny_round), dim3(256), 0, st, (const float*)part,
+                    blocks, d, dgamma, dbeta, ny, cg, ny_sums, round);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -867,9 +894,9 @@ cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma
 template <typename T>
 cudaError_t norm_bwd_dispatch(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                               const float* gamma, void* dX, float* dgamma, float* dbeta, float* npart,
-                              const ColsumGroup& cg, cudaStream_t st) {
+                              const ColsumGroup& cg, const ConvertGroup& round, cudaStream_t st) {
   const NormShape s = norm_bwd_shape(p->d.d_model / Vec16<T>::N, p->n_pad, p->sm_count);
-#define FBL_CALL(NV_, R_) norm_bwd_launch<T, NV_, R_>(p, s, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, st)
+#define FBL_CALL(NV_, R_) norm_bwd_launch<T, NV_, R_>(p, s, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, round, st)
   switch (s.nv) {
     case 1: return s.r == 4 ? FBL_CALL(1, 4) : s.r == 2 ? FBL_CALL(1, 2) : FBL_CALL(1, 1);
     case 2: return s.r == 2 ? FBL_CALL(2, 2) : FBL_CALL(2, 1);
@@ -928,11 +955,13 @@ cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, cud
 // second stage inside the second.  `part`: the norm's per-block partial rows.
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
                             const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
-                            cudaStream_t st, const ColsumGroup* sums) {
+                            cudaStream_t st, const ColsumGroup* sums, const ConvertGroup* round) {
   ColsumGroup cg = {};
+  ConvertGroup rg = {};
+  if (round) rg = *round;
   if (sums) cg = *sums;
-  if (p->d.dtype == FBL_DTYPE_FP32) return norm_bwd_dispatch<float>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, st);
-  return norm_bwd_dispatch<__nv_bfloat16>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, st);
+  if (p->d.dtype == FBL_DTYPE_FP32) return norm_bwd_dispatch<float>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, rg, st);
+  return norm_bwd_dispatch<__nv_bfloat16>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, rg, st);
 }
 
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols) {

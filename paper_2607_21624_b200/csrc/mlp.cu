@@ -372,7 +372,7 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
   const bool tc = bp->use_tc != 0;
   const bool split2 = tc && p->ksplit_2 > 1, split1 = tc && p->ksplit_1 > 1;
 
-  ConvertGroup cg = {};
+  ConvertGroup cg = {};       // sliced products leave fp32 sums; the norm backward's second launch rounds them
   {
     GemmArgs gs[2];
     GemmArgs& gw = gs[0];     // dW2 = H^T dY : token-axis reduction, H's tiles read MN-major
@@ -449,8 +449,7 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
     p->launches += k;
     if (early) MLP_STEP(1, launch_colsum_early(bp, sums, idle, st));
   }
-  if (cg.count > 0) MLP_STEP(1, launch_convert_f32_group(cg, st));
-  MLP_STEP(0, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums));
+  MLP_STEP(0, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums, &cg));
   return FBL_OK;
 }
 

@@ -128,7 +128,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
   XA_PROF_BEGIN();
   const bool split_o = p->use_tc && p->ksplit_o > 1, split_q = p->use_tc && p->ksplit_qkv > 1,
              split_kv = p->use_tc && p->ksplit_kv > 1;
-  ConvertGroup cg = {};                     // sliced products leave fp32 sums; one launch rounds them all at the end
+  ConvertGroup cg = {};                     // sliced products leave fp32 sums; the norm backward's second launch rounds them
   bool dvec_ready = false;
   {
     GemmArgs gs[2];
@@ -216,7 +216,6 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
       colsum_add(sums, dV, p->n_pad_kv, p->dkv, dbv, &part_kv);
       XA_STEP("db", 1, launch_colsum_early(p, sums, idle, st));
     }
-    if (cg.count > 0) XA_STEP("dW round", 1, launch_convert_f32_group(cg, st));
   }
   if (bias && !sums.summed) {
     ColsumGroup kv = {};
@@ -224,7 +223,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     colsum_add(kv, dV, p->n_pad_kv, p->dkv, dbv, &part_kv);
     XA_STEP("db_kv", 2, launch_colsum_group(p->d.dtype, kv, st));
   }
-  XA_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums));
+  XA_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums, &cg));
   return FBL_OK;
 }
 
