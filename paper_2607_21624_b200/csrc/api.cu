@@ -178,18 +178,18 @@ static int plan_build(const fbl_layer_desc* desc, int cross, int seq_kv_in, int 
   if (p->use_tc && cross) {
     const int kb_q = (int)((p->n_pad + 63) / 64), kb_k = (int)((p->n_pad_kv + 63) / 64);
     const GemmShape go[2] = {{p->dq, d.d_model, kb_q, 1}, {p->n_pad, p->dq, (d.d_model + 63) / 64, 0}};
-    p->ksplit_o = gemm_tc_choose_split(p->sm_count, go, 2);
+    p->ksplit_o = gemm_tc_choose_split(p->sm_count, go, 2, false);
     const GemmShape gq[2] = {{d.d_model, p->dq, kb_q, 1}, {p->n_pad, d.d_model, (p->dq + 63) / 64, 0}};
-    p->ksplit_qkv = gemm_tc_choose_split(p->sm_count, gq, 2);
+    p->ksplit_qkv = gemm_tc_choose_split(p->sm_count, gq, 2, true);
     const GemmShape gk[3] = {{d_mem, p->dkv, kb_k, 1}, {d_mem, p->dkv, kb_k, 1}, {p->n_pad_kv, d_mem, (2 * p->dkv + 63) / 64, 0}};
-    p->ksplit_kv = gemm_tc_choose_split(p->sm_count, gk, 3);
+    p->ksplit_kv = gemm_tc_choose_split(p->sm_count, gk, 3, true);
   } else if (p->use_tc) {
     const int kb_tok = (int)((p->n_pad + 63) / 64);
     const GemmShape go[2] = {{p->dq, d.d_model, kb_tok, 1}, {p->n_pad, p->dq, (d.d_model + 63) / 64, 0}};
-    p->ksplit_o = gemm_tc_choose_split(p->sm_count, go, 2);
+    p->ksplit_o = gemm_tc_choose_split(p->sm_count, go, 2, false);
     const GemmShape gq[4] = {{d.d_model, p->dq, kb_tok, 1}, {d.d_model, p->dkv, kb_tok, 1}, {d.d_model, p->dkv, kb_tok, 1},
                              {p->n_pad, d.d_model, (p->dq + 2 * p->dkv + 63) / 64, 0}};
-    p->ksplit_qkv = gemm_tc_choose_split(p->sm_count, gq, 4);
+    p->ksplit_qkv = gemm_tc_choose_split(p->sm_count, gq, 4, true);
   }
   if (p->use_tc && getenv("FBL_KSPLIT_O")) p->ksplit_o = atoi(getenv("FBL_KSPLIT_O"));          // tuning knobs
   if (p->use_tc && getenv("FBL_KSPLIT_QKV")) p->ksplit_qkv = atoi(getenv("FBL_KSPLIT_QKV"));

@@ -147,7 +147,7 @@ static inline bool rope_in_projection(const fbl_plan* p, GemmArgs* gs, const flo
   return true;
 }
 struct GemmShape { int64_t m; int n; int kblocks; int splittable; };
-int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count);
+int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count, bool zero_rides);
 cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles, cudaStream_t st);
 bool attn_fwd_tc_supported(const fbl_plan* p);
 bool attn_bwd_tc_supported(const fbl_plan* p);

@@ -1276,8 +1276,11 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
 // How many slices to cut the reduction loops of the splittable problems of a group into (the same number for all
 // of them).  The persistent kernel deals work units to its blocks round-robin, so a few long units beside many
 // short ones leave most SMs idle: this asks, for each candidate, when the longest block of the best tile finishes,
-// charging the fp32 detour (zero-fill, bulk reductions, rounding pass) as extra k-blocks and a fixed cost.
-int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count) {
+// charging the fp32 detour (zero-fill, bulk reductions, rounding) as extra k-blocks and a fixed cost.  `zero_rides`: a
+// launch in front of the group can do the zero-fill.  Each slice's tiles are read and written once more, so a small gain is
+// none: of five feed-forward and attention steps whose choice the figures below changed from a dearer rounding pass, two
+// gained 10 to 12 %, two 2 to 5 %, and the one that only the first group's lower price had changed lost 4 %.
+int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count, bool zero_rides) {
   static const int cand[] = {1, 2, 3, 4, 6, 8, 12, 16};
   double base_cost = 0.0, best_cost = 0.0;
   int best = 1;
@@ -1292,9 +1295,10 @@ int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count) {
     if (too_short || (S > 1 && !any_split)) continue;
     double cost;
     best_tile(w, count, sm_count, true, &cost);
-    if (S > 1) cost += 8000;                               // zero-fill and rounding pass
+    // zero-fill, in the launch in front or one of its own, and rounding beside the norm backward
+    if (S > 1) cost += zero_rides ? 4000 : 6000;
     if (S == 1) base_cost = best_cost = cost;
-    else if (cost < 0.85 * base_cost && cost < best_cost) { best = S; best_cost = cost; }   // worth it only with a clear gain
+    else if (cost < (zero_rides ? 0.9 : 0.85) * base_cost && cost < best_cost) { best = S; best_cost = cost; }   // worth it only with a clear gain
   }
   return best;
 }

@@ -191,11 +191,11 @@ int fbl_mlp_plan_create(const fbl_mlp_desc* desc, fbl_mlp_plan** out) {
   if (base->use_tc) {
     const int kb_tok = (int)((p->n_pad + 63) / 64);
     const GemmShape g2[2] = {{d.d_ff, d.d_model, kb_tok, 1}, {p->n_pad, d.d_ff, (d.d_model + 63) / 64, 0}};
-    p->ksplit_2 = gemm_tc_choose_split(base->sm_count, g2, 2);
+    p->ksplit_2 = gemm_tc_choose_split(base->sm_count, g2, 2, false);
     const GemmShape g1[3] = {{d.d_model, d.d_ff, kb_tok, 1}, {d.d_model, d.d_ff, kb_tok, 1},
                              {p->n_pad, d.d_model, (int)((gated ? 2 : 1) * ((d.d_ff + 63) / 64)), 0}};
-    if (gated) p->ksplit_1 = gemm_tc_choose_split(base->sm_count, g1, 3);
-    else { const GemmShape g1n[2] = {g1[0], g1[2]}; p->ksplit_1 = gemm_tc_choose_split(base->sm_count, g1n, 2); }
+    if (gated) p->ksplit_1 = gemm_tc_choose_split(base->sm_count, g1, 3, true);
+    else { const GemmShape g1n[2] = {g1[0], g1[2]}; p->ksplit_1 = gemm_tc_choose_split(base->sm_count, g1n, 2, true); }
     if (getenv("FBL_KSPLIT_MLP")) p->ksplit_2 = p->ksplit_1 = atoi(getenv("FBL_KSPLIT_MLP"));     // tuning / test knob
   }
   o = FBL_ALIGN;   // status word, then the fp32 accumulation areas of sliced reductions (zero-filled together)
