@@ -918,8 +918,8 @@ static __global__ void __launch_bounds__(512) fill_kernel(uint4* __restrict__ ou
 
 cudaError_t start_backward(const fbl_plan* p, GemmArgs* gs, int count, bool rides, bool serial, int32_t* status, size_t bytes, cudaStream_t st) {
   // Idle epilogue warps of the first products clear what they can while the first tiles are computed; with tens of MB their
-  // stores delay those tiles by more than a launch costs.
-  if (rides && bytes <= (size_t)16 << 20 && gemm_group_tc(p, gs, count)) {
+  // stores delay those tiles by more than a launch costs, but the fp32 kernels leave memory idle.
+  if (rides && (p->d.dtype == FBL_DTYPE_FP32 || (bytes <= (size_t)16 << 20 && gemm_group_tc(p, gs, count)))) {
     gs[0].zero_ptr = (char*)status + FBL_ALIGN; gs[0].zero_bytes = bytes - FBL_ALIGN;
     gs[0].reset_status = 1; gs[0].serial = serial;
     return cudaSuccess;

@@ -13,6 +13,7 @@
 // 64: forward 54 -> 38 us, backward with its dQ pass 120 -> 72 us (few warps per SM: 4 to 5 at this size).
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "fbl_internal.h"
@@ -39,6 +40,10 @@ __device__ __forceinline__ float4 lds4(uint32_t a) {
 }
 __device__ __forceinline__ void sts(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 
+__device__ __forceinline__ void sts4(uint32_t a, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 struct alignas(64) FfmaAttnParams {
   CUtensorMap tq, tk, tv, tdo;
   float* a;                     // forward: merged-head output [n_pad, dq]
@@ -48,6 +53,7 @@ struct alignas(64) FfmaAttnParams {
   float *dk, *dv;
   long long n_pad, n_pad_k;
   int seq, t_pad, seq_k, t_pad_k, hq, group, causal;
+  int slices;                   // backward: blocks of a cluster, which share a key tile's items
   float scale;
   int32_t* status;
 };
@@ -229,6 +235,9 @@ __global__ void __launch_bounds__(THREADS) attn_fwd_ffma_kernel(const __grid_con
 // ------------------------------------------------------------------------------------------
 // Backward: one block per (32-key tile, KV head, batch).  dK and dV stay in registers over the query tiles and the G
 // query heads of the group; dQ reduces over the key tiles and is added into its zeroed buffer with 16-byte reductions.
+// Where that makes fewer blocks than SMs (few sequences, few KV heads), a cluster of 2 to 8 blocks takes a key tile's
+// (query head, query tile) items in turn and adds its dK and dV through distributed shared memory in a fixed order: the
+// bound is the items' chain, some 6 us each.
 // ------------------------------------------------------------------------------------------
 template <int HD>
 struct FfmaBwdSmem {
@@ -245,7 +254,8 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u, bar_kv = base + SM::BAR_OFF, bar_q = bar_kv + 8, bar_do = bar_kv + 16;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, tm = lane % 4, tn = lane / 4;
-  const int j0 = blockIdx.x * ROWS, g = blockIdx.y, b = blockIdx.z;      // key tile 0 has the most queries: first
+  const int slices = P.slices, slice = blockIdx.x % slices;
+  const int j0 = blockIdx.x / slices * ROWS, g = blockIdx.y, b = blockIdx.z;      // key tile 0 has the most queries: first
   const int row0 = b * P.t_pad, row0k = b * P.t_pad_k;
   const int t0 = P.causal ? j0 / QT : 0, per_head = (P.seq + QT - 1) / QT - t0, n_it = max(0, per_head) * P.group;
   auto load = [&](const CUtensorMap* map, uint32_t dst, uint32_t bar, int it) {
@@ -261,9 +271,9 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
     tc::mbar_expect_tx(bar_kv, 2 * HD * ROWS * 4);
     tc::tma_load_3d(base + SM::K_OFF, &P.tk, bar_kv, 0, row0k + j0, g * PN);
     tc::tma_load_3d(base + SM::V_OFF, &P.tv, bar_kv, 0, row0k + j0, g * PN);
-    if (n_it > 0) {
-      load(&P.tq, base + SM::Q_OFF, bar_q, 0);
-      load(&P.tdo, base + SM::DO_OFF, bar_do, 0);
+    if (slice < n_it) {
+      load(&P.tq, base + SM::Q_OFF, bar_q, slice);
+      load(&P.tdo, base + SM::DO_OFF, bar_do, slice);
     }
   }
   __syncthreads();
@@ -278,7 +288,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
   const uint32_t p_row = base + SM::P_OFF + ra * LD * 4, s_row = base + SM::S_OFF + ra * LD * 4;
   bool ok = tc::mbar_wait(bar_kv, 0, P.status, 133);
   // JN: groups of eight queries of the tile that are worked through
-  auto tile = [&](auto jn_tag, int it) -> bool {
+  auto tile = [&](auto jn_tag, int it, int phase) -> bool {
     constexpr int JN = decltype(jn_tag)::value;
     const int h = g * P.group + it / per_head, i0 = (t0 + it % per_head) * QT;
     const bool need_mask = i0 + JN * 8 > P.seq || j0 + ROWS > P.seq_k || (P.causal && i0 < j0 + ROWS - 1);
@@ -290,7 +300,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
       lse[j] = gi < P.seq ? P.lse[at + gi] : 0.f;
       d[j] = gi < P.seq ? P.dvec[at + gi] : 0.f;
     }
-    ok = tc::mbar_wait(bar_q, it & 1, P.status, 134) && ok;
+    ok = tc::mbar_wait(bar_q, phase, P.status, 134) && ok;
     float p[4][JN], dp[4][JN];
     scores<HD, JN, ROWS, QT>(base + SM::K_OFF, base + SM::Q_OFF, ra, tn, p);
 #pragma unroll
@@ -301,7 +311,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
         p[i][j] = need_mask && (gi >= P.seq || gj >= P.seq_k || (P.causal && gj > gi)) ? 0.f : expf(p[i][j] * P.scale - lse[j]);
         sts(p_row + (4 * i * LD + tn + 8 * j) * 4, p[i][j]);
       }
-    ok = tc::mbar_wait(bar_do, it & 1, P.status, 135) && ok;
+    ok = tc::mbar_wait(bar_do, phase, P.status, 135) && ok;
     scores<HD, JN, ROWS, QT>(base + SM::V_OFF, base + SM::DO_OFF, ra, tn, dp);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -310,10 +320,10 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
     __syncwarp();
     weighted<HD, QT>(p_row, LD, base + SM::DO_OFF, tn, JN * 8, dv);
     if (__syncthreads_or(!ok)) return false;               // all warps are done with dO, and dS^T is complete
-    if (threadIdx.x == 0 && it + 1 < n_it) load(&P.tdo, base + SM::DO_OFF, bar_do, it + 1);
+    if (threadIdx.x == 0 && it + slices < n_it) load(&P.tdo, base + SM::DO_OFF, bar_do, it + slices);
     weighted<HD, QT>(s_row, LD, base + SM::Q_OFF, tn, JN * 8, dk);
     __syncthreads();                                       // ... and with Q
-    if (threadIdx.x == 0 && it + 1 < n_it) load(&P.tq, base + SM::Q_OFF, bar_q, it + 1);
+    if (threadIdx.x == 0 && it + slices < n_it) load(&P.tq, base + SM::Q_OFF, bar_q, it + slices);
     // dQ = dS K: 16 queries at a time per warp, four neighbouring ones per thread, reduced over the block's keys
 #pragma unroll 1
     for (int q0 = warp * 16; q0 < JN * 8; q0 += 16 * WARPS) {
@@ -354,22 +364,57 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
   };
   using Full = std::integral_constant<int, QT / 8>;
   using Half = std::integral_constant<int, QT / 16>;
-  for (int it = 0; it < n_it; ++it)
-    if (!(P.seq - (t0 + it % per_head) * QT > QT / 2 ? tile(Full{}, it) : tile(Half{}, it))) return;
+  for (int it = slice, phase = 0; it < n_it; it += slices, phase ^= 1)
+    if (!(P.seq - (t0 + it % per_head) * QT > QT / 2 ? tile(Full{}, it, phase) : tile(Half{}, it, phase))) break;
+  auto store = [&](float* out, int row, int col, float4 v, float f) {
+    if (j0 + row < P.t_pad_k) {
+      f = j0 + row < P.seq_k ? f : 0.f;
+      *reinterpret_cast<float4*>(out + rt_off<32>(P.n_pad_k, row0k + j0 + row, g * HD + col)) = make_float4(v.x * f, v.y * f, v.z * f, v.w * f);
+    }
+  };
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gj = j0 + ra + 4 * i;
-    if (gj >= P.t_pad_k) continue;
-    const float live = gj < P.seq_k ? 1.f : 0.f;
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int pn = 0; pn < PN; ++pn) {
-      const int64_t off = rt_off<32>(P.n_pad_k, row0k + gj, g * HD + pn * 32 + tn * 4);
+      const int row = ra + 4 * i, col = pn * 32 + tn * 4;
       const float2 x = unpack2(dk[i][2 * pn]), y = unpack2(dk[i][2 * pn + 1]), u = unpack2(dv[i][2 * pn]), w = unpack2(dv[i][2 * pn + 1]);
-      const float f = live * P.scale;
-      *reinterpret_cast<float4*>(P.dk + off) = make_float4(x.x * f, x.y * f, y.x * f, y.y * f);
-      *reinterpret_cast<float4*>(P.dv + off) = make_float4(u.x * live, u.y * live, w.x * live, w.y * live);
+      const float4 k4 = make_float4(x.x, x.y, y.x, y.y), v4 = make_float4(u.x, u.y, w.x, w.y);
+      if (slices == 1) {
+        store(P.dk, row, col, k4, P.scale);
+        store(P.dv, row, col, v4, 1.f);
+      } else {                                             // Q's and dO's places are free
+        sts4(base + SM::Q_OFF + (row * HD + col) * 4, k4);
+        sts4(base + SM::DO_OFF + (row * HD + col) * 4, v4);
+      }
     }
+  if (slices > 1) {
+    tc::cluster_sync_all();
+    const int per = ROWS / slices;                         // rows that this block finishes
+    for (int e = threadIdx.x; e < 2 * per * (HD / 4); e += THREADS) {
+      const int row = slice * per + e / (HD / 4) % per, col = e % (HD / 4) * 4;
+      const bool is_v = e >= per * (HD / 4);
+      const uint32_t at = base + (is_v ? SM::DO_OFF : SM::Q_OFF) + (row * HD + col) * 4;
+      float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int c = 0; c < slices; ++c) {
+        float4 f;
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f.x), "=f"(f.y), "=f"(f.z), "=f"(f.w) : "r"(tc::map_to_cta(at, c)) : "memory");
+        sum.x += f.x; sum.y += f.y; sum.z += f.z; sum.w += f.w;
+      }
+      store(is_v ? P.dv : P.dk, row, col, sum, is_v ? 1.f : P.scale);
+    }
+    __syncwarp();
+    tc::cluster_sync_all();                                // no block leaves while another may still read its sums
   }
+}
+
+// Shared memory to ask for: blocks that all fit the SMs at once spread evenly.  Launched while the kernel in front still
+// runs, they would crowd on the SMs that it frees first (84 blocks of the backward: 46 us spread, 61 us crowded; 78 longer
+// ones: 730 and 1050 us).  Two or three short ones (few `items` each) to an SM may as well start early.
+constexpr uint32_t ALONE = 114 * 1024;                     // with the 1 KB that a block has on top, half an SM's is less
+uint32_t spread(const fbl_plan* p, const dim3& grid, int items, uint32_t smem) {
+  const long long per_sm = ((long long)grid.x * grid.y * grid.z + p->sm_count - 1) / p->sm_count;
+  return per_sm == 1 || (per_sm <= 3 && items >= 4) ? std::max(smem, (uint32_t)(228 * 1024 / (per_sm + 1))) : smem;
 }
 
 typedef LaunchMemo<FfmaAttnParams, 8, 12> AttnMemo;
@@ -380,9 +425,13 @@ void fill(const fbl_plan* p, FfmaAttnParams& P, int32_t* status) {
   P.hq = p->d.n_q_heads; P.group = p->group; P.causal = p->d.causal; P.scale = p->scale; P.status = status;
 }
 
+static_assert(FfmaFwdSmem<128>::TOTAL <= ALONE && FfmaBwdSmem<128>::TOTAL <= ALONE, "");
+
 template <int HD>
 cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse, int32_t* status, cudaStream_t st) {
   auto k = attn_fwd_ffma_kernel<HD>;
+  const dim3 grid((p->t_pad + ROWS - 1) / ROWS, p->d.n_q_heads, p->d.batch);
+  const uint32_t smem = spread(p, grid, (p->t_pad_kv + FWD_KEYS - 1) / FWD_KEYS, FfmaFwdSmem<HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
   if (!fbl_encode_f32_rtile_map(&P.tq, Q, p->n_pad, p->dq / 32, ROWS, HD / 32) ||
@@ -390,12 +439,12 @@ cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
       !fbl_encode_f32_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 32, FWD_KEYS, HD / 32))
     return cudaErrorInvalidValue;
   P.a = (float*)A; P.lse = lse;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FfmaFwdSmem<HD>::TOTAL);
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
   };
   LaunchKey key;
   for (const void* q : {Q, K, V, (const void*)A, (const void*)lse, (const void*)status}) key.add(q);
   return AttnMemo::run(p->memo[FBL_MEMO_FFMA_ATTN], key, make, [&](const FfmaAttnParams& P) {
-  return launch_pdl(k, dim3((p->t_pad + ROWS - 1) / ROWS, p->d.n_q_heads, p->d.batch), dim3(THREADS), FfmaFwdSmem<HD>::TOTAL, st, P);
+  return launch_pdl(k, grid, dim3(THREADS), smem, st, P);
   });
 }
 
@@ -404,6 +453,13 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
                        void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st) {
   constexpr int QT = FfmaBwdSmem<HD>::QT;
   auto k = attn_bwd_ffma_kernel<HD>;
+  // slices of a key tile's items: an item each at least, and no more once there are two blocks per SM (of two warps each,
+  // for an SM's four schedulers)
+  const int key_tiles = (p->t_pad_kv + ROWS - 1) / ROWS, items = (p->d.seq + QT - 1) / QT * p->group;
+  int slices = 1;
+  while (slices < 8 && 2 * slices <= items && (long long)key_tiles * p->d.n_kv_heads * p->d.batch * slices <= 2 * p->sm_count) slices *= 2;
+  const dim3 grid(key_tiles * slices, p->d.n_kv_heads, p->d.batch);
+  const uint32_t smem = slices > 1 ? FfmaBwdSmem<HD>::TOTAL : spread(p, grid, items, FfmaBwdSmem<HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
   if (!fbl_encode_f32_rtile_map(&P.tq, Q, p->n_pad, p->dq / 32, QT, HD / 32) ||
@@ -412,13 +468,14 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
       !fbl_encode_f32_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 32, ROWS, HD / 32))
     return cudaErrorInvalidValue;
   P.lse = const_cast<float*>(lse); P.dvec = dvec; P.dq = (float*)dQ; P.dk = (float*)dK; P.dv = (float*)dV;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FfmaBwdSmem<HD>::TOTAL);
+  P.slices = slices;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
   };
   LaunchKey key;
   for (const void* q : {Q, K, V, dA, (const void*)lse, (const void*)dvec, (const void*)dQ, (const void*)dK, (const void*)dV, (const void*)status})
     key.add(q);
   return AttnMemo::run(p->memo[FBL_MEMO_FFMA_ATTN], key, make, [&](const FfmaAttnParams& P) {
-  return launch_pdl(k, dim3((p->t_pad_kv + ROWS - 1) / ROWS, p->d.n_kv_heads, p->d.batch), dim3(THREADS), FfmaBwdSmem<HD>::TOTAL, st, P);
+  return slices > 1 ? launch_cluster(k, grid, dim3(THREADS), smem, st, slices, true, P) : launch_pdl(k, grid, dim3(THREADS), smem, st, P);
   });
 }
 

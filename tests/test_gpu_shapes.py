@@ -162,3 +162,16 @@ def test_few_tokens_long_reductions(cfg):
 ], ids=lambda c: c.name)
 def test_bias_gradients_beside_products(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # fp32 attention backward with a key tile's items dealt over 2, 4 and 8 blocks: fewer items than blocks (causal ends),
+    # uneven shares, a ragged key tile, every head width
+    LayerConfig("fs1", 1, 70, 128, 4, 1, 32, "fp32", "layernorm", True, False, False, 1e-5, 301, 0.05),
+    LayerConfig("fs2", 2, 129, 128, 6, 2, 64, "fp32", "rmsnorm", False, False, True, 1e-5, 302, 0.05),
+    LayerConfig("fs3", 1, 100, 256, 3, 1, 128, "fp32", "rmsnorm", True, True, True, 1e-5, 303, 0.05, 0.0, 10000.0),
+    XattnConfig("fs4", 1, 150, 41, 96, 128, 3, 1, 64, "fp32", "layernorm", True, True, 1e-5, 304, 0.05),
+    XattnConfig("fs5", 3, 40, 33, 128, 64, 2, 1, 32, "fp32", "rmsnorm", False, False, 1e-5, 305, 0.05),
+], ids=lambda c: c.name)
+def test_fp32_attention_backward_slices(cfg):
+    check(cfg)
