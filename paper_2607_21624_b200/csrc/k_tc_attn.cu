@@ -464,10 +464,10 @@ template <typename Params>
 struct AttnLaunch {
   Params P;
   void (*kernel)(const Params);
-  int grid, threads;
+  int grid, threads, cluster;                              // cluster: blocks of one where the launch has any, else 0
   size_t smem;
-  cudaError_t set(void (*k)(const Params), int g, int t, size_t s) {
-    kernel = k; grid = g; threads = t; smem = s;
+  cudaError_t set(void (*k)(const Params), int g, int t, size_t s, int c = 0) {
+    kernel = k; grid = g; threads = t; smem = s; cluster = c;
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s);
   }
 };
@@ -528,6 +528,7 @@ struct alignas(64) AttnBwdParams {
   int seq, t_pad, hq, group, causal, dkv;
   int seq_k, t_pad_k;                // key-side sequence length and padded length
   int batch, chunk;      // grid = key tiles * KV heads * batch blocks, see decode_block
+  int slices;            // SLICED: blocks of a cluster, which share a key tile's items
   float scale;
   int32_t* status;
 };
@@ -583,7 +584,10 @@ constexpr int BWD_SM_THREADS = 512;
 
 // DIRECT: the sequence has a single key tile, so a block's dQ tile is complete and goes out rounded, without the fp32
 // accumulator, its zero-fill and the rounding pass.
-template <int HD, bool DIRECT>
+// SLICED: a cluster of `slices` blocks shares a key tile's (query head, query tile) items, in contiguous runs, and adds its
+// fp32 dK and dV through distributed shared memory in a fixed order.  For grouped heads whose key tiles, KV heads and
+// sequences make a fraction of 148 blocks: the bound is then the items' chain.
+template <int HD, bool DIRECT, bool SLICED>
 __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __grid_constant__ AttnBwdParams P) {
   using SM = BwdSmem<HD>;
   constexpr bool PIPE = SM::PIPE;
@@ -601,13 +605,16 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
   // under a causal mask key tile 0 has the most query tiles: it is slot 0
   const int n_kvh = P.hq / P.group;
   int slot_i, gb;
-  decode_block((int)blockIdx.x, (P.t_pad_k + BKV - 1) / BKV, n_kvh * P.batch, P.chunk, &slot_i, &gb);
+  const int slices = SLICED ? P.slices : 1, slice = SLICED ? (int)blockIdx.x % slices : 0;
+  decode_block((int)blockIdx.x / slices, (P.t_pad_k + BKV - 1) / BKV, n_kvh * P.batch, P.chunk, &slot_i, &gb);
   const int j0 = slot_i * BKV, g = gb % n_kvh, b = gb / n_kvh;
   const int row0 = b * P.t_pad, row0k = b * P.t_pad_k;
   const int n_qt = (P.seq + BQ - 1) / BQ;
   const int qt_begin = P.causal ? j0 / BQ : 0;
   const int per_head = n_qt - qt_begin;
-  const int n_it = P.group * per_head;
+  const int share = SLICED ? (P.group * per_head + slices - 1) / slices : P.group * per_head;
+  const int it0 = SLICED ? slice * share : 0, n_it = SLICED ? min(share, P.group * per_head - it0) : share;     // none: n_it <= 0
+  const int h0 = g * P.group + (SLICED && n_it > 0 ? it0 / per_head : 0), c0_q = SLICED && n_it > 0 ? it0 % per_head : 0;   // first item
   int32_t* status = P.status;
   if ((base & 1023u) != 0) {                    // the swizzled tiles need a 1024-byte aligned window
     if (threadIdx.x == 0) atomicCAS(status, 0, 399);
@@ -647,8 +654,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
     if (n_it > 0) {
       // LSE travels with Q and D with dO: 128 floats each, into the iteration's staging buffer
       tc::mbar_expect_tx(bar(BB_QFULL), SM::TILE + 512);
-      tc::tma_load_3d(base + SM::Q_OFF, &P.tq, bar(BB_QFULL), 0, row0 + qt_begin * BQ, g * P.group * (int)PANELS);
-      tc::bulk_load(base + SM::LSE_OFF, P.lse + ((long long)b * P.hq + g * P.group) * P.t_pad + qt_begin * BQ, 512, bar(BB_QFULL));
+      tc::tma_load_3d(base + SM::Q_OFF, &P.tq, bar(BB_QFULL), 0, row0 + (qt_begin + c0_q) * BQ, h0 * (int)PANELS);
+      tc::bulk_load(base + SM::LSE_OFF, P.lse + ((long long)b * P.hq + h0) * P.t_pad + (qt_begin + c0_q) * BQ, 512, bar(BB_QFULL));
     }
   }
   if (warp == 1) {
@@ -677,7 +684,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
     // (K, V and Q of the first tile were requested during set-up)
     bool waited = false;
     for (int it = 0; it < n_it; ++it) {
-      const int h = g * P.group + it / per_head, qt = qt_begin + it % per_head;
+      const int h = g * P.group + (it0 + it) / per_head, qt = qt_begin + (it0 + it) % per_head;
       // LSE travels with Q and D with dO, 128 floats each.  A stage's previous readers (the products, and for
       // LSE / D the softmax warps, which finish a tile before its dK and dV products are issued) are behind the
       // barrier that frees it.  Rows past the sequence end may hold anything: the softmax warps mask them.
@@ -812,7 +819,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
     if (lane == 0) {
       pdl_wait();                                    // the accumulator's zero-fill precedes the kernel before this one
       for (int dit = 0; dit < n_it; ++dit) {
-        const int h = g * P.group + dit / per_head, i0 = (qt_begin + dit % per_head) * BQ;
+        const int h = g * P.group + (it0 + dit) / per_head, i0 = (qt_begin + (it0 + dit) % per_head) * BQ;
         if (!tc::mbar_wait(bar(BB_DQSTAGED + (dit % NS)), (dit / (int)NS) & 1, status, 309)) break;   // one per buffer, like STAGEFREE
         const uint32_t stage = stage_addr(dit);
 #pragma unroll
@@ -856,7 +863,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       tc::tc_fence_before();
       tc::mbar_arrive(bar(BB_DQDRAINED));            // TMEM side done: the tensor pipe may reuse the columns
       if constexpr (DIRECT) {
-        const int h = g * P.group + dit / per_head, gi = (qt_begin + dit % per_head) * BQ + r;
+        const int h = g * P.group + (it0 + dit) / per_head, gi = (qt_begin + (it0 + dit) % per_head) * BQ + r;
         if (gi < P.t_pad) store_cols<NC>(P.dq, P.n_pad, row0 + gi, h * HD + c0, o, P.scale);
         return true;
       }
@@ -882,7 +889,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       return true;
     };
 
-    int c_q = 0;                                    // query tile within the head of the tile being processed
+    int c_q = c0_q;                                 // query tile within the head of the tile being processed
     for (int it = 0; it < n_it && ok; ++it) {
       const int i0 = (qt_begin + c_q) * BQ;
       if (++c_q == per_head) c_q = 0;
@@ -1068,7 +1075,30 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
     // it is behind us; HD = 128: the extra arrival above)
     if (!PIPE && ok && n_it > 0) ok = tc::mbar_wait(bar(BB_DVDONE), 0, status, 315);
     tc::tc_fence_after();
-    if (ok && n_it > 0) {
+    if constexpr (SLICED) {
+      // fp32 rows of dV, then of dK, over the operand tiles, which no product reads any more (without items: which have come)
+      if (n_it <= 0) ok = tc::mbar_wait(bar(BB_KVFULL), 0, status, 316);
+#pragma unroll 1
+      for (int which = 0; which < 2; ++which) {
+#pragma unroll 1
+        for (int cc = 0; cc < HD / 64; ++cc) {
+          const int c0 = part * (HD / 4) + cc * 16;
+          const uint32_t at = base + ((which * BKV + r) * (HD + 4) + c0) * 4;
+          if (n_it > 0) {
+            uint32_t o[16];
+            tc::tmem_ld16(lane_addr + (which ? DK_COL : DV_COL) + c0, o);
+            tc::tmem_ld_wait();
+#pragma unroll
+            for (int k = 0; k < 16; k += 4)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + k * 4), "r"(o[k]), "r"(o[k + 1]), "r"(o[k + 2]), "r"(o[k + 3]) : "memory");
+          } else {
+#pragma unroll
+            for (int k = 0; k < 16; k += 4)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(at + k * 4), "r"(0u) : "memory");
+          }
+        }
+      }
+    } else if (ok && n_it > 0) {
       const bool live = gj < P.seq_k;
 #pragma unroll 1
       for (int which = 0; which < 2; ++which) {
@@ -1086,6 +1116,35 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
         }
       }
     }
+  }
+  if constexpr (SLICED) {
+    __syncwarp();
+    tc::cluster_sync_all();
+    const int rows = BKV / slices;                        // of either matrix, that this block finishes
+    for (int e = threadIdx.x; e < 2 * rows * (HD / 8); e += BWD_THREADS) {
+      const bool is_k = e >= rows * (HD / 8);
+      const int row = slice * rows + e / (HD / 8) % rows, col = e % (HD / 8) * 8;
+      const uint32_t at = base + (((is_k ? BKV : 0) + row) * (HD + 4) + col) * 4;
+      float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+      for (int c = 0; c < slices; ++c) {
+        const uint32_t from = tc::map_to_cta(at, c);
+        float4 x, y;
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(from) : "memory");
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w) : "r"(from + 16) : "memory");
+        sum[0] += x.x; sum[1] += x.y; sum[2] += x.z; sum[3] += x.w;
+        sum[4] += y.x; sum[5] += y.y; sum[6] += y.z; sum[7] += y.w;
+      }
+      if (j0 + row >= P.t_pad_k) continue;
+      const float f = j0 + row < P.seq_k ? (is_k ? P.scale : 1.f) : 0.f;
+      uint4 v;
+      v.x = tc::pack_bf16(sum[0] * f, sum[1] * f); v.y = tc::pack_bf16(sum[2] * f, sum[3] * f);
+      v.z = tc::pack_bf16(sum[4] * f, sum[5] * f); v.w = tc::pack_bf16(sum[6] * f, sum[7] * f);
+      const int cg = g * HD + col;
+      *reinterpret_cast<uint4*>((is_k ? P.dk : P.dv) + ((long long)(cg / 64) * P.n_pad_k + row0k + j0 + row) * 64 + cg % 64) = v;
+    }
+    __syncwarp();
+    tc::cluster_sync_all();                               // no block leaves while another may still read its sums
   }
   tc::tc_fence_before();
   __syncthreads();
@@ -1361,7 +1420,14 @@ cudaError_t bwd_make_t(AttnLaunch<AttnBwdParams>& L, const fbl_plan* p) {
   // together (small chunks: L2 hits); the pipelined HD = 64 variant hides that latency and prefers balance.
   L.P.chunk = chunk_for((long long)p->group * p->d.seq * HD * 8, p->d.n_kv_heads * p->d.batch,
                         BwdSmem<HD>::PIPE ? (96ll << 20) : (8ll << 20));
-  return L.set(attn_bwd_tc_kernel<HD, DIRECT>, ((p->t_pad_kv + BKV - 1) / BKV) * p->d.n_kv_heads * p->d.batch, BWD_THREADS, BwdSmem<HD>::TOTAL);
+  // slices of a key tile's items: at least two items each, and no more blocks than seven eighths of the SMs, on which all
+  // clusters still find room at once
+  const int blocks = ((p->t_pad_kv + BKV - 1) / BKV) * p->d.n_kv_heads * p->d.batch, items = (p->d.seq + BQ - 1) / BQ * p->group;
+  int slices = 1;
+  while (slices < 8 && 4 * slices <= items && 16ll * blocks * slices <= 7 * p->sm_count) slices *= 2;
+  if (slices == 1) return L.set(attn_bwd_tc_kernel<HD, DIRECT, false>, blocks, BWD_THREADS, BwdSmem<HD>::TOTAL);
+  L.P.slices = slices;
+  return L.set(attn_bwd_tc_kernel<HD, DIRECT, true>, blocks * slices, BWD_THREADS, BwdSmem<HD>::TOTAL, slices);
 }
 
 template <int HD>
@@ -1428,7 +1494,10 @@ cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, 
         return p->d.head_dim == 64 ? bwd_make<64>(L, p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status)
                                    : bwd_make<128>(L, p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status);
       },
-      [&](const Launch& L) { return launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.P); });
+      [&](const Launch& L) {
+        return L.cluster ? launch_cluster(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.cluster, true, L.P)
+                         : launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.P);
+      });
   if (e != cudaSuccess) return e;
   // dQ: fp32 accumulator -> storage dtype where the kernel has not written it; with the rotary embedding (`rope`: the
   // forward's table) dQ and dK are turned back by the opposite angle on the way

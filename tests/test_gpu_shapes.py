@@ -175,3 +175,17 @@ def test_bias_gradients_beside_products(cfg):
 ], ids=lambda c: c.name)
 def test_fp32_attention_backward_slices(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # tensor-core attention backward with a key tile's items dealt over 2, 4 and 8 blocks: shares that do not divide, blocks
+    # without items (causal ends), one key tile (dQ written at once), ragged key tiles, the rotation behind it
+    LayerConfig("bs1", 1, 300, 256, 8, 1, 64, "bf16", "layernorm", True, False, False, 1e-5, 311, 0.02),
+    LayerConfig("bs2", 1, 420, 256, 5, 1, 128, "bf16", "rmsnorm", True, False, True, 1e-5, 312, 0.02, 0.0, 10000.0),
+    LayerConfig("bs3", 2, 100, 256, 12, 2, 64, "bf16", "layernorm", False, True, True, 1e-5, 313, 0.02),
+    LayerConfig("bs4", 1, 77, 256, 9, 1, 128, "bf16", "rmsnorm", True, False, True, 1e-5, 314, 0.02),
+    XattnConfig("bs5", 1, 640, 140, 256, 128, 3, 1, 64, "bf16", "layernorm", True, True, 1e-5, 315, 0.02),
+    XattnConfig("bs6", 3, 257, 520, 256, 128, 2, 1, 128, "bf16", "rmsnorm", False, False, 1e-5, 316, 0.02),
+], ids=lambda c: c.name)
+def test_attention_backward_slices(cfg):
+    check(cfg)
