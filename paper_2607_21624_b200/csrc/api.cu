@@ -411,6 +411,13 @@ int fbl_unpack(const fbl_plan* plan, int tensor_id, const void* tiled_dev, void*
   return pack_common(plan, tensor_id, tiled_dev, rowmajor_dev, stream, 1);
 }
 
+// With the rotary embedding dbk is what the rotation leaves of sums that cancel without it: little in a short sequence.
+// Rounding P and dS to bf16 for the tensor cores is 1 to 1.5 % of it for 8 to 15 tokens, 0.6 to 1 % for 23 to 64.  Less
+// than a tile of such tokens costs the fp32-arithmetic attention kernels little (a step of 30 tokens 67 -> 90 us).
+static bool cancelling_dbk(const fbl_plan* p) {
+  return p->rope_base > 0.f && p->d.has_bias && p->t_pad <= 64 && p->n_pad < 128;
+}
+
 int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const float* beta, const void* Wq,
                   const void* Wk, const void* Wv, const void* Wo, const float* bq, const float* bk, const float* bv,
                   const float* bo, void* Y, void* saved, void* scratch, void* stream) {
@@ -452,7 +459,7 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
     FBL_GEMM_STEP("proj_qkv", gs, 3, FBL_GEMM_PROJ_QKV);
   }
   if (p->rope_base > 0.f && !rotated) FBL_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
-  if (p->use_tc && attn_fwd_tc_supported(p)) FBL_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
+  if (p->use_tc && attn_fwd_tc_supported(p) && !cancelling_dbk(p)) FBL_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
   else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
   else FBL_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
   {
@@ -495,6 +502,7 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
   const int n = (int)p->n_pad, D = p->d.d_model;
 
   const bool split_o = p->use_tc && p->ksplit_o > 1, split_qkv = p->use_tc && p->ksplit_qkv > 1;
+  const bool tc_attn = p->use_tc && attn_bwd_tc_supported(p) && !cancelling_dbk(p);
   FBL_PROF_BEGIN();
   bool dvec_ready = false;
   ConvertGroup cg = {};                     // sliced products leave fp32 sums; the norm backward's second launch rounds them
@@ -522,14 +530,14 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
         cg.src[0] = gw.acc; cg.dst[0] = dWo; cg.n[0] = up8(p->dq) * (int64_t)D; cg.count = 1;
       }
     }
-    FBL_CUDA(start_backward(p, gs, 2, !split_o, true, status, bwd_zero_bytes(p), st));
+    FBL_CUDA(start_backward(p, gs, 2, !split_o, true, status, tc_attn ? bwd_zero_bytes(p) : p->zero_bytes, st));
     FBL_GEMM_STEP("dWo+dA", gs, 2, FBL_GEMM_DWO_DA);
   }
-  if (p->use_tc && attn_bwd_tc_supported(p)) FBL_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope));   // dqacc: zero already
+  if (tc_attn) FBL_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope));   // dqacc: zero already
   else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
   else FBL_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
   // back through the rotation of Q and K: its transpose is the rotation by the opposite angle
-  if (p->rope_base > 0.f && !(p->use_tc && attn_bwd_tc_supported(p))) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
+  if (p->rope_base > 0.f && !tc_attn) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   // every bias gradient is a token-axis column sum: the four of them run beside the last products, or else in the norm
   // backward's two launches
   ColsumGroup sums = {};

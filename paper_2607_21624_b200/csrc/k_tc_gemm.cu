@@ -1,8 +1,8 @@
 // Projection GEMMs on tcgen05 tensor cores (bf16 in, fp32 accumulate in TMEM, bf16 out), operands in
 // R-Tile order fetched by TMA.  One kernel serves all six projection steps and their transposed forms:
 // each operand is declared K-major or MN-major in the descriptors, so W / W^T and X / X^T are the same
-// tiles in HBM and in shared memory.  Up to three reduction loops feed one accumulator (dXn), and up
-// to four problems share one persistent launch (Q/K/V projections; dWo with dA; dWq/dWk/dWv with dXn).
+// tiles in HBM and in shared memory.  Up to four reduction loops feed one accumulator (dXn), and up
+// to five problems share one persistent launch (Q/K/V projections; dWo with dA; dWq/dWk/dWv with dXn).
 #include <stdlib.h>
 #include <string.h>
 
