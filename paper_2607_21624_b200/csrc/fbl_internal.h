@@ -117,8 +117,8 @@ struct GemmArgs {
   // fused activation of the feed-forward block (tensor-core kernel only): 0 none, 1 GELU forward (c = U, c2 = gelu(U)),
   // 2 GELU backward (c = value * gelu'(U), U in `residual`), 3 gated forward (c = G, c2 = silu(G) * U, U in `residual`),
   // 4 gated backward (c = value * silu(G), c2 = value * U * silu'(G); U in `residual`, G in `aux1`)
-  // 5 rotary embedding of whole heads of rope_hd columns, with the table launch_norm_fwd leaves (see there)
-  int epi; const void* aux1; void* c2; const float2* rope; int rope_hd;
+  // 5 rotary embedding of heads of 64 columns, with the table launch_norm_fwd leaves (see there)
+  int epi; const void* aux1; void* c2; const float2* rope;
 };
 
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
@@ -140,10 +140,12 @@ cudaError_t run_gemm_group(const fbl_plan* p, GemmArgs* gs, int count, int32_t* 
 static inline bool gemm_fuses_dot(const fbl_plan* p, const GemmArgs& ga) {
   return p->d.dtype == FBL_DTYPE_FP32 ? p->d.head_dim <= 64 && gemm_ffma_supported(p, ga) : p->use_tc && gemm_tc_supported(p, ga);
 }
-// The rotary embedding in the epilogue of the Q and K projections (gs[0], gs[1] of three): true if it goes there.
+// The rotary embedding in the epilogue of the Q and K projections (gs[0], gs[1] of three): true if it goes there.  A head of
+// 64 is one panel of the epilogue; one of 128 needs the neighbouring panel's accumulators and twice the table per element,
+// which took longer than a pass of its own (26900 tokens of 6 + 1 heads: 238 us against 61 and 34 us).
 static inline bool rope_in_projection(const fbl_plan* p, GemmArgs* gs, const float2* table) {
-  if (!(p->rope_base > 0.f) || !gemm_group_tc(p, gs, 3)) return false;
-  for (int i = 0; i < 2; ++i) { gs[i].epi = 5; gs[i].rope = table; gs[i].rope_hd = p->d.head_dim; }
+  if (!(p->rope_base > 0.f) || p->d.head_dim != 64 || !gemm_group_tc(p, gs, 3)) return false;
+  for (int i = 0; i < 2; ++i) { gs[i].epi = 5; gs[i].rope = table; }
   return true;
 }
 struct GemmShape { int64_t m; int n; int kblocks; int splittable; };

@@ -45,9 +45,8 @@ struct alignas(64) TcProblem {
   // operand U instead of a residual, `aux1` at the second one, G; `tc2` is the second output's map):
   //   1 GELU forward    C = v (U), C2 = gelu(v)           2 GELU backward    C = v gelu'(U)
   //   3 gated forward   C = v (G), C2 = silu(v) U          4 gated backward   C = v silu(G), C2 = v U silu'(G)
-  //   5 rotary embedding C = v with each head's (i, i + rope_hd / 2) pairs turned by the table's angle of the row's token
-  const float2* rope;      // [rope_hd / 2][t_pad] cosine and sine
-  int rope_hd;
+  //   5 rotary embedding C = v with each 64-column head's (i, i + 32) pairs turned by the table's angle of the row's token
+  const float2* rope;      // [32][t_pad] cosine and sine
   int epi;
   const __nv_bfloat16* aux1;
   CUtensorMap tc2;
@@ -146,9 +145,9 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
   const int row = m0 + q * 32 + lane;               // row of the problem owned by this thread
   const bool pad = P.t_pad > 0 && (row % P.t_pad) >= P.seq;
   const bool has_res = P.residual && row < P.m;
-  // a head of the fused row reduction, or of the rotation, must stay within one warp: where it spans more panels than a set has, the
-  // first set takes the whole tile
-  const bool whole = ESETS == 2 && ((P.dot_with && P.dot_hd > 64 * PPS) || (EPI == EPI_ROPE && P.epi == 5 && P.rope_hd > 64 * PPS));
+  // a head of the fused row reduction must stay within one warp: where it spans more panels than a set has, the first set
+  // takes the whole tile
+  const bool whole = ESETS == 2 && P.dot_with && P.dot_hd > 64 * PPS;
   const int pn_begin = set == 0 ? 0 : (whole ? BN / 64 : PPS);
   const int pn_end = ESETS == 1 ? BN / 64 : (set == 0 ? (whole ? BN / 64 : PPS) : BN / 64);
   uint4 rv[8];                                    // residual values of the next panel, requested a panel ahead
@@ -307,29 +306,12 @@ __device__ __forceinline__ bool epilogue_tile(const TcProblem& P, int m0, int n0
             v[j] = __float_as_uint(__uint_as_float(v[j]) + __shfl_sync(0xffffffffu, bl[j % (BN / 32)], (pn * 64 + j) / (BN / 32)));
           bias_left = false;
         }
-        if (P.rope_hd == 64) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float2 cs = tab[(long long)j * P.t_pad];
-            const float a = tc::round_bf16(__uint_as_float(v[j])), b = tc::round_bf16(__uint_as_float(v[j + 32]));
-            v[j] = __float_as_uint(a * cs.x - b * cs.y);
-            v[j + 32] = __float_as_uint(b * cs.x + a * cs.y);
-          }
-        } else {                                     // 128: the partner is the same column of the neighbouring panel
-          const float sign = (n / 64) & 1 ? 1.f : -1.f;
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            uint32_t w[32];
-            acc.load((pn ^ 1) * 64 + hf * 32, w);
-            acc.wait();
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const float2 cs = tab[(long long)(hf * 32 + j) * P.t_pad];
-              float b = __uint_as_float(w[j]);
-              if (bias) b += __shfl_sync(0xffffffffu, bl[(hf * 32 + j) % (BN / 32)], ((pn ^ 1) * 64 + hf * 32 + j) / (BN / 32));
-              v[hf * 32 + j] = __float_as_uint(tc::round_bf16(__uint_as_float(v[hf * 32 + j])) * cs.x + sign * tc::round_bf16(b) * cs.y);
-            }
-          }
+        for (int j = 0; j < 32; ++j) {
+          const float2 cs = tab[(long long)j * P.t_pad];
+          const float a = tc::round_bf16(__uint_as_float(v[j])), b = tc::round_bf16(__uint_as_float(v[j + 32]));
+          v[j] = __float_as_uint(a * cs.x - b * cs.y);
+          v[j + 32] = __float_as_uint(b * cs.x + a * cs.y);
         }
       }
     }
@@ -1041,7 +1023,7 @@ cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int32_t* statu
       if (g.epi < 1 || g.epi > 5 || g.ksplit > 1 || g.dot_with || (g.epi >= 2 && !rope && !g.residual) || (g.epi == 4 && !g.aux1) ||
           (two_out && !g.c2) || (rope && (!g.rope || g.residual || g.t_pad <= 0)))
         return cudaErrorInvalidValue;
-      P.rope = g.rope; P.rope_hd = g.rope_hd;
+      P.rope = g.rope;
       if (two_out && !fbl_encode_rtile_map(&P.tc2, g.c2, g.c_rpad, g.n / 64, 32, 1)) return cudaErrorInvalidValue;
     }
     P.ksplit = 1;
@@ -1177,13 +1159,13 @@ int best_slices(const TileWork* w, int count, int sm_count, double clocks) {
 
 // 128 x 64 tiles: less to load per k-block, and more SMs loading, where there are fewer tiles than SMs (50 tokens of 768:
 // 20.0 -> 19.1 us a layer forward; 94 x 7 tokens of 320 x 640 gated: 57.8 -> 51.7 us a step).  With more tiles than SMs
-// they only add loads of A; and a row of a head of 128, which the rotation and the row reduction need whole, spans two.
+// they only add loads of A; and a row of a head of 128, which the row reduction needs whole, spans two.
 bool slim_legal(const GemmArgs* gs, int count, int sm_count) {
   long long tiles = 0;
   bool legal = true;
   for (int i = 0; i < count; ++i) {
     tiles += (long long)((gs[i].m + 127) / 128) * (gs[i].n / 64) * (gs[i].ksplit > 1 ? gs[i].ksplit : 1);
-    legal = legal && (!gs[i].dot_with || gs[i].dot_hd <= 64) && (gs[i].epi != 5 || gs[i].rope_hd <= 64);
+    legal = legal && (!gs[i].dot_with || gs[i].dot_hd <= 64);
   }
   return legal && tiles <= sm_count;
 }

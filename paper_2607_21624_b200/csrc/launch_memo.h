@@ -73,7 +73,7 @@ inline void gemm_group_key(LaunchKey& k, const GemmArgs* gs, int count, const in
     }
     k.add(g.c); k.add((uint64_t)g.c_rpad); k.add(g.bias); k.add(g.residual); k.add(g.seq, g.t_pad);
     k.add(g.dot_with); k.add(g.dot_out); k.add(g.dot_hd, g.dot_hq);
-    k.add(g.acc); k.add(g.ksplit, g.epi); k.add(g.aux1); k.add(g.c2); k.add(g.rope); k.add(g.rope_hd, g.serial);
+    k.add(g.acc); k.add(g.ksplit, g.epi); k.add(g.aux1); k.add(g.c2); k.add(g.rope); k.add(g.serial, 0);
     if (i == 0) { k.add(g.late_trigger != nullptr, 0); k.add(g.zero_ptr); k.add((uint64_t)g.zero_bytes); k.add((uint64_t)g.reset_status); }
   }
 }
