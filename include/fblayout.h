@@ -293,6 +293,10 @@ int fbl_status_poll(const fbl_plan* plan, const void* scratch, int32_t* device_s
  * normal end). */
 int fbl_selftest_wait_timeout(void* scratch, int64_t limit_cycles, void* stream);
 
+/* Host code only, for tests: the 64-wide reduction blocks [*begin, *end) that block `slice` of a cluster of `slices` blocks
+ * works through where they share an output tile's reduction of `kblocks` (launches of few tiles and long reductions). */
+int fbl_gemm_slice_range(int kblocks, int slices, int slice, int* begin, int* end);
+
 /* ---------------------------------------------------------------------------------------------------------------
  * Offline tile selection (section 4.2, step 1 and Eq. 1, Eq. 2; Supplement Algorithm 1), restated for this GPU.
  *

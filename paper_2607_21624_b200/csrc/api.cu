@@ -619,6 +619,13 @@ int fbl_selftest_wait_timeout(void* scratch, int64_t limit_cycles, void* stream)
   return FBL_OK;
 }
 
+int fbl_gemm_slice_range(int kblocks, int slices, int slice, int* begin, int* end) {
+  if (kblocks < 0 || kblocks > 1 << 24 || slices < 1 || slices > 16 || slice < 0 || slice >= slices || !begin || !end) return FBL_ERR_INVALID_ARG;
+  *begin = gemm_slice_begin(kblocks, slices, slice);
+  *end = gemm_slice_begin(kblocks, slices, slice + 1);
+  return FBL_OK;
+}
+
 const char* fbl_strerror(int status) {
   switch (status) {
     case FBL_OK: return "ok";

@@ -148,6 +148,10 @@ static inline bool rope_in_projection(const fbl_plan* p, GemmArgs* gs, const flo
   for (int i = 0; i < 2; ++i) { gs[i].epi = 5; gs[i].rope = table; }
   return true;
 }
+// First k-block of a slice where a cluster shares a reduction of `total` k-blocks: shares differ by one at most, so none is
+// empty unless there are fewer k-blocks than slices.  (Shares rounded up leave the last ones short: nine k-blocks in four
+// make 3, 3, 3 and none.)
+__host__ __device__ __forceinline__ int gemm_slice_begin(int total, int slices, int slice) { return total * slice / slices; }
 struct GemmShape { int64_t m; int n; int kblocks; int splittable; };
 int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count, bool zero_rides);
 cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles, cudaStream_t st);

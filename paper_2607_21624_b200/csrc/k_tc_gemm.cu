@@ -707,7 +707,9 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
 // Launches with few tiles and long reductions (few tokens: 50 x 768 outputs are six tiles for 148 SMs): the reduction of a
 // 128 x 128 tile is cut into 2 or 4 slices, one per block of a cluster.  Each block accumulates its slice in tensor
 // memory and leaves the fp32 sums in shared memory, over its operand stages; then it finishes its share of the tile's
-// rows, adding the slices through distributed shared memory in a fixed order.  One tile per cluster.  The bound is a
+// rows, adding the slices through distributed shared memory in a fixed order.  One tile per cluster.  Every slice has a
+// k-block (gemm_slice_begin; make_group_split refuses a launch where one would not): what a block of none would add is what
+// its tensor memory held before.  The bound is a
 // block's chain: first operands, its k-blocks at about 545 clk each, the exchange (about 2.5 us: distributed shared memory
 // gives a block some 15 bytes/clk), the epilogue.  Rank-16 adapter products of 4096 x 2048 (32 k-blocks, 32 row tiles):
 // 14.3 -> 12.0 us forward and 18.5 -> 13.0 us backward.
@@ -765,7 +767,7 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
   const TcProblem& P = G.p[tcd.prob];
   int total = 0;
   for (int t = 0; t < P.n_terms; ++t) total += P.kblocks[t];
-  const int per = (total + G.slices - 1) / G.slices, begin = slice * per, end = min(total, begin + per);   // no slice is empty
+  const int begin = gemm_slice_begin(total, G.slices, slice), end = gemm_slice_begin(total, G.slices, slice + 1);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1089,6 +1091,11 @@ cudaError_t make_group_split(GroupLaunch& L, const GemmArgs* gs, int count, int3
   cudaError_t e = fill_group(L.G, gs, count, status, 128, BM, 128, &tiles);
   if (e != cudaSuccess) return e;
   L.G.slices = slices;
+  for (int i = 0; i < count; ++i) {
+    int kb = 0;
+    for (int t = 0; t < L.G.p[i].n_terms; ++t) kb += L.G.p[i].kblocks[t];
+    if (kb < slices) return cudaErrorInvalidValue;       // a slice without work
+  }
   const int epi = group_epi(gs, count);
   auto k = epi == EPI_ACT ? gemm_tc_split_kernel<EPI_ACT> : epi == EPI_ROPE ? gemm_tc_split_kernel<EPI_ROPE> : gemm_tc_split_kernel<EPI_NONE>;
   return group_launch(L, k, tiles * slices, 320, SmemPlan<128, SPLIT_STAGES>::TOTAL, gs[0].serial, slices);

@@ -5,6 +5,7 @@ import pytest
 from fbl_inputs import LayerConfig, MlpConfig, XattnConfig
 
 import test_gpu_layer
+import test_gpu_lora
 import test_gpu_mlp
 import test_gpu_xattn
 
@@ -189,3 +190,21 @@ def test_fp32_attention_backward_slices(cfg):
 ], ids=lambda c: c.name)
 def test_attention_backward_slices(cfg):
     check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    # cluster-split products with reductions of nine k-blocks, which four blocks do not share evenly, beside longer ones: the
+    # weight gradients of one launch or the other, the norm's output gradient, an adapter step's, both feed-forward forms
+    LayerConfig("ns1", 1, 520, 1536, 2, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 321, 0.02),
+    LayerConfig("ns2", 1, 576, 256, 8, 8, 64, "bf16", "layernorm", True, True, True, 1e-5, 322, 0.02),
+    LayerConfig("ns3", 7, 197, 192, 3, 3, 64, "bf16", "layernorm", False, True, True, 1e-5, 323, 0.02),
+    (LayerConfig("ns4", 1, 1345, 128, 2, 2, 64, "bf16", "rmsnorm", True, False, True, 1e-5, 324, 0.02), 16),
+    MlpConfig("ns5", 1, 520, 256, 1536, "bf16", "layernorm", "gelu", True, True, 1e-5, 325, 0.02),
+    MlpConfig("ns6", 1, 576, 128, 1024, "bf16", "rmsnorm", "swiglu", True, True, 1e-5, 326, 0.02),
+    XattnConfig("ns7", 1, 520, 64, 1536, 64, 2, 2, 64, "bf16", "layernorm", True, True, 1e-5, 327, 0.02),
+], ids=lambda c: getattr(c, "name", "ns4"))
+def test_cluster_slices_of_nine_k_blocks(cfg):
+    if isinstance(cfg, tuple):
+        test_gpu_lora.run_and_compare(cfg[0], cfg[1], guard_bytes=4096)
+    else:
+        check(cfg)

@@ -223,3 +223,19 @@ def test_cross_attention_plan_host_maps_follow_the_memory_side():
         Plan(desc_from_config(cfg), cross=(cfg.seq_kv, 100))
     with pytest.raises(FblError):
         Plan(desc_from_config(cfg), cross=(0, cfg.d_mem))
+
+
+def test_cluster_slices_of_a_reduction():
+    # the blocks of a cluster share a reduction: in order, none left out, shares at most one apart, so that no block of a
+    # reduction with a k-block for each is without work (nine over four as 3 + 3 + 3 + 0 was)
+    begin, end = ctypes.c_int(), ctypes.c_int()
+    for slices in (2, 4):
+        for kblocks in range(slices, 129):
+            at, shares = 0, []
+            for s in range(slices):
+                assert lib().fbl_gemm_slice_range(kblocks, slices, s, ctypes.byref(begin), ctypes.byref(end)) == 0
+                assert begin.value == at
+                at = end.value
+                shares.append(end.value - begin.value)
+            assert at == kblocks and min(shares) >= 1 and max(shares) - min(shares) <= 1, (kblocks, slices, shares)
+    assert lib().fbl_gemm_slice_range(9, 4, 4, ctypes.byref(begin), ctypes.byref(end)) != 0
