@@ -411,12 +411,27 @@ int fbl_unpack(const fbl_plan* plan, int tensor_id, const void* tiled_dev, void*
   return pack_common(plan, tensor_id, tiled_dev, rowmajor_dev, stream, 1);
 }
 
-// With the rotary embedding dbk is what the rotation leaves of sums that cancel without it: little in a short sequence.
-// Rounding P and dS to bf16 for the tensor cores is 1 to 1.5 % of it for 8 to 15 tokens, 0.6 to 1 % for 23 to 64.  Less
-// than a tile of such tokens costs the fp32-arithmetic attention kernels little (a step of 30 tokens 67 -> 90 us).
-static bool cancelling_dbk(const fbl_plan* p) {
-  return p->rope_base > 0.f && p->d.has_bias && p->t_pad <= 64 && p->n_pad < 128;
+}  // extern "C"
+
+cudaError_t run_attn_fwd(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse, int32_t* status, cudaStream_t st) {
+  switch (attn_fwd_kernels(p)) {
+    case ATTN_TC: return launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st);
+    case ATTN_FFMA: return launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st);
+    default: return launch_attn_fwd_simt(p, Q, K, V, A, lse, st);
+  }
 }
+
+cudaError_t run_attn_bwd(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A, const void* dA, const float* lse,
+                         float* dvec, float* dqacc, void* dQ, void* dK, void* dV, bool dvec_ready, int32_t* status, cudaStream_t st,
+                         const float2* rope) {
+  switch (attn_bwd_kernels(p)) {
+    case ATTN_TC: return launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope);
+    case ATTN_FFMA: return launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope);
+    default: return launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st);
+  }
+}
+
+extern "C" {
 
 int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const float* beta, const void* Wq,
                   const void* Wk, const void* Wv, const void* Wo, const float* bq, const float* bk, const float* bv,
@@ -459,9 +474,7 @@ int fbl_layer_fwd(const fbl_plan* p, const void* X, const float* gamma, const fl
     FBL_GEMM_STEP("proj_qkv", gs, 3, FBL_GEMM_PROJ_QKV);
   }
   if (p->rope_base > 0.f && !rotated) FBL_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
-  if (p->use_tc && attn_fwd_tc_supported(p) && !cancelling_dbk(p)) FBL_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
-  else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
-  else FBL_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
+  FBL_STEP("attn_fwd", 1, run_attn_fwd(p, Q, K, V, A, lse, status, st));
   {
     GemmArgs g = {};
     g.m = n; g.n = D; g.n_terms = 1;
@@ -502,7 +515,6 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
   const int n = (int)p->n_pad, D = p->d.d_model;
 
   const bool split_o = p->use_tc && p->ksplit_o > 1, split_qkv = p->use_tc && p->ksplit_qkv > 1;
-  const bool tc_attn = p->use_tc && attn_bwd_tc_supported(p) && !cancelling_dbk(p);
   FBL_PROF_BEGIN();
   bool dvec_ready = false;
   ConvertGroup cg = {};                     // sliced products leave fp32 sums; the norm backward's second launch rounds them
@@ -530,14 +542,12 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
         cg.src[0] = gw.acc; cg.dst[0] = dWo; cg.n[0] = up8(p->dq) * (int64_t)D; cg.count = 1;
       }
     }
-    FBL_CUDA(start_backward(p, gs, 2, !split_o, true, status, tc_attn ? bwd_zero_bytes(p) : p->zero_bytes, st));
+    FBL_CUDA(start_backward(p, gs, 2, !split_o, true, status, bwd_zero_bytes(p), st));
     FBL_GEMM_STEP("dWo+dA", gs, 2, FBL_GEMM_DWO_DA);
   }
-  if (tc_attn) FBL_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope));   // dqacc: zero already
-  else if (p->d.dtype == FBL_DTYPE_FP32) FBL_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
-  else FBL_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
+  FBL_STEP("attn_bwd", attn_bwd_launches(p, dvec_ready), run_attn_bwd(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope));
   // back through the rotation of Q and K: its transpose is the rotation by the opposite angle
-  if (p->rope_base > 0.f && !tc_attn) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
+  if (p->rope_base > 0.f && !attn_bwd_turns(p)) FBL_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   // every bias gradient is a token-axis column sum: the four of them run beside the last products, or else in the norm
   // backward's two launches
   ColsumGroup sums = {};

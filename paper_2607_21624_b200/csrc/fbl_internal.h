@@ -101,10 +101,10 @@ struct GemmArgs {
   const void* residual;           // same layout as C, or nullptr
   int seq, t_pad;                 // if t_pad > 0: rows with (row % t_pad) >= seq are written as zero
   int b_static;                   // 1: the first term's B operand is an input of the whole step (a weight)
-  // optional fused row reduction D[b,h,t] = sum_d C[row, h*hd+d] * dot_with[row, h*hd+d] (fp32 C, before rounding)
+  // optional fused row reduction D[b,h,t] = sum_d C[row, h*hd+d] * dot_with[row, h*hd+d] (C as stored, rounded)
   const void* dot_with; float* dot_out; int dot_hd, dot_hq;
   // reduction loop cut into ksplit slices whose fp32 partial tiles are added into `acc` (zeroed by the caller, same
-  // element order as C with 4-byte elements); C itself is then produced from acc by launch_convert_f32_group
+  // element order as C with 4-byte elements); the norm backward rounds them to C (ConvertGroup)
   int ksplit; float* acc;
   // of a group's first problem: chores of the launch (zero-fill zero_bytes, a multiple of 16, at zero_ptr for a
   // later kernel of the pass; reset the pass's status word), and `serial`: the launch may not start before
@@ -155,13 +155,22 @@ __host__ __device__ __forceinline__ int gemm_slice_begin(int total, int slices, 
 struct GemmShape { int64_t m; int n; int kblocks; int splittable; };
 int gemm_tc_choose_split(int sm_count, const GemmShape* sh, int count, bool zero_rides);
 cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles, cudaStream_t st);
-bool attn_fwd_tc_supported(const fbl_plan* p);
-bool attn_bwd_tc_supported(const fbl_plan* p);
+// With less than a tile of token rows on either side a bf16 layer keeps P and dS in fp32, or in two bf16 values: their rounding
+// is as large as that of the results there (dQ, dK, dV off by 2.3e-3 of their norm instead of 1.65e-3), and with the rotary
+// embedding dbk, what the rotation leaves of sums that cancel without it, is off by up to 1.5 %.  The line is where the caller's
+// results have always changed over; what it costs against P and dS in bf16 (us a step): 50 tokens of 12 heads 59 -> 72, 120
+// tokens of 16 heads over one KV head 69 -> 123, 8 queries over 1500 memory rows 115 -> 134, 4096 queries over 40 memory rows
+// 192 -> 348 (plain fp32 kernels: 87, 583, 338, 1330).
+static inline bool attn_fp32(const fbl_plan* p) { return p->n_pad < 128 || p->n_pad_kv < 128; }
+// The kernels that a plan's attention runs on.
+enum { ATTN_TC = 0, ATTN_FFMA, ATTN_SIMT };
+static inline int attn_fwd_kernels(const fbl_plan* p) { return p->d.dtype == FBL_DTYPE_FP32 ? ATTN_FFMA : p->use_tc ? ATTN_TC : ATTN_SIMT; }
+static inline int attn_bwd_kernels(const fbl_plan* p) { return p->use_tc && attn_fp32(p) ? ATTN_FFMA : attn_fwd_kernels(p); }
 bool attn_bwd_tc_direct(const fbl_plan* p);    // the tensor-core backward writes dQ itself: no fp32 accumulator to zero and round
 // Leading bytes of the backward scratch a step starts by zero-filling: status word and sliced products' accumulation areas,
 // and behind them the dQ accumulator where the attention backward adds into it.
 static inline size_t bwd_zero_bytes(const fbl_plan* p) {
-  return p->use_tc && attn_bwd_tc_supported(p) && attn_bwd_tc_direct(p) ? p->sb_dqacc : p->zero_bytes;
+  return attn_bwd_kernels(p) == ATTN_TC && attn_bwd_tc_direct(p) ? p->sb_dqacc : p->zero_bytes;
 }
 // What a backward pass starts with: zero the first `bytes` of its scratch (the status word's block and the fp32 areas the
 // pass adds into).  `rides`: the pass's first products `gs` need nothing of it.  `serial`: no kernel of the pass may start
@@ -169,8 +178,16 @@ static inline size_t bwd_zero_bytes(const fbl_plan* p) {
 // in front of it).  Counts a launch of its own.
 cudaError_t start_backward(const fbl_plan* p, GemmArgs* gs, int count, bool rides, bool serial, int32_t* status, size_t bytes, cudaStream_t st);
 
-static inline int attn_bwd_tc_launches(const fbl_plan* p, bool dvec_ready) {
-  return (dvec_ready ? 1 : 2) + (attn_bwd_tc_direct(p) && !(p->rope_base > 0.f) ? 0 : 1);
+// One launch forward.  Backward: D unless it is there, the attention, dQ's rounding where it was summed in fp32.  The rotation
+// of dQ and dK back goes with that rounding where `attn_bwd_turns`, else it is a step of its own.
+cudaError_t run_attn_fwd(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse, int32_t* status, cudaStream_t st);
+cudaError_t run_attn_bwd(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A, const void* dA, const float* lse,
+                         float* dvec, float* dqacc, void* dQ, void* dK, void* dV, bool dvec_ready, int32_t* status, cudaStream_t st,
+                         const float2* rope);
+static inline bool attn_bwd_turns(const fbl_plan* p) { return p->rope_base > 0.f && p->use_tc; }
+static inline int attn_bwd_launches(const fbl_plan* p, bool dvec_ready) {
+  const bool summed = attn_bwd_kernels(p) != ATTN_TC || !attn_bwd_tc_direct(p);
+  return (dvec_ready ? 1 : 2) + (p->d.dtype == FBL_DTYPE_BF16 && (summed || attn_bwd_turns(p)) ? 1 : 0);
 }
 void fbl_note_cuda_error(cudaError_t e, const char* where);
 
@@ -224,20 +241,20 @@ cudaError_t launch_colsum(int dtype, const void* M, int64_t rows, int64_t cols, 
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols);
 cudaError_t launch_colsum_group(int dtype, const ColsumGroup& G, cudaStream_t st);
 
-// fp32 storage (k_ffma_attn.cu); the backward adds into dQ, zeroed by the caller
+// fp32 arithmetic (k_ffma_attn.cu): fp32 storage, and the backward of bf16 storage.  The latter adds into dQ or, bf16, into dqacc,
+// zeroed by the caller; dqacc it rounds and, with `rope`, turns
 cudaError_t launch_attn_fwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                  int32_t* status, cudaStream_t st);
 cudaError_t launch_attn_bwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A, const void* dA,
-                                 const float* lse, float* dvec, void* dQ, void* dK, void* dV, bool dvec_ready, int32_t* status,
-                                 cudaStream_t st);
+                                 const float* lse, float* dvec, float* dqacc, void* dQ, void* dK, void* dV, bool dvec_ready,
+                                 int32_t* status, cudaStream_t st, const float2* rope);
 // bf16 storage in fp32 arithmetic (cross-check)
 cudaError_t launch_attn_fwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                  cudaStream_t st);
 cudaError_t launch_attn_bwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A,
                                  const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
                                  void* dV, bool dvec_ready, cudaStream_t st);
-cudaError_t launch_attn_bwd_pre(const fbl_plan* p, const void* A, const void* dA, float* dvec, float* dqacc,
-                                bool dvec_ready, cudaStream_t st);
+cudaError_t launch_attn_bwd_pre(const fbl_plan* p, const void* A, const void* dA, float* dvec, bool dvec_ready, cudaStream_t st);
 cudaError_t launch_attn_bwd_post(const fbl_plan* p, const float* dqacc, void* dQ, cudaStream_t st);
 cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                int32_t* status, cudaStream_t st);

@@ -1,5 +1,6 @@
-// fp32 attention on the FP32 pipe (plain FFMA, no tensor cores), operands in R-Tile order fetched by TMA into the swizzled
-// 128-byte rows they are stored as (see k_ffma_gemm.cu for the operand fragments).
+// Attention in fp32 arithmetic on the FP32 pipe (plain FFMA, no tensor cores), operands in R-Tile order fetched by TMA into
+// the swizzled 128-byte rows they are stored as (see k_ffma_gemm.cu for the operand fragments): fp32 storage, and the backward
+// of bf16 storage where P and dS stay in fp32 (attn_fp32), whose operands are widened on their way to registers.
 //
 // Both kernels give a warp 16 rows of the score tile and all its columns (lane = (row group tm of 4, column group tn of
 // 8), 4 x 8 scores per thread), so that the softmax needs only shuffles and the rows of P (forward) or of P^T and dS^T
@@ -44,13 +45,29 @@ __device__ __forceinline__ void sts4(uint32_t a, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
+// Four neighbouring columns (group c4) of a row of a tile of R rows, which lies in shared memory as TMA leaves it.
+template <typename T, int R>
+__device__ __forceinline__ void ld4(uint32_t tile, int row, int c4, f2& x, f2& y) {
+  if constexpr (sizeof(T) == 4) {
+    lds2x2(tile + (c4 / 8) * (R * 128) + row * 128 + (((c4 % 8) ^ (row & 7)) << 4), x, y);
+  } else {
+    uint32_t lo, hi;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi)
+                 : "r"(tile + (c4 / 16) * (R * 128) + row * 128 + (((c4 % 16 / 2) ^ (row & 7)) << 4) + c4 % 2 * 8) : "memory");
+    x = pack2(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u));
+    y = pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+  }
+}
+__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16* p, float4 v) { *reinterpret_cast<uint2*>(p) = make_uint2(tc::pack_bf16(v.x, v.y), tc::pack_bf16(v.z, v.w)); }
+
 struct alignas(64) FfmaAttnParams {
   CUtensorMap tq, tk, tv, tdo;
   float* a;                     // forward: merged-head output [n_pad, dq]
   float* lse;                   // [B, Hq, t_pad]
   const float* dvec;            // backward: D = rowsum(dO * O)
-  float* dq;                    // backward: zeroed dQ, added into
-  float *dk, *dv;
+  float* dq;                    // backward: zeroed dQ in fp32 (in the storage type's element order), added into
+  void *dk, *dv;
   long long n_pad, n_pad_k;
   int seq, t_pad, seq_k, t_pad_k, hq, group, causal;
   int slices;                   // backward: blocks of a cluster, which share a key tile's items
@@ -59,7 +76,7 @@ struct alignas(64) FfmaAttnParams {
 };
 
 // s[i][j] = rows a (row ra + 4 i) times rows b (row tn + 8 j), reduced over head_dim.
-template <int HD, int JN, int AR, int BR>
+template <typename T, int HD, int JN, int AR, int BR>
 __device__ __forceinline__ void scores(uint32_t a_tile, uint32_t b_tile, int ra, int tn, float (&s)[4][JN]) {
   f2 acc[4][JN];
 #pragma unroll
@@ -68,13 +85,11 @@ __device__ __forceinline__ void scores(uint32_t a_tile, uint32_t b_tile, int ra,
     for (int j = 0; j < JN; ++j) acc[i][j] = 0ull;
 #pragma unroll 2
   for (int kq = 0; kq < HD / 4; ++kq) {
-    const uint32_t at = a_tile + (kq / 8) * (AR * 128), bt = b_tile + (kq / 8) * (BR * 128);
-    const int kc = kq % 8;
     f2 a[4][2], b[JN][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) lds2x2(at + (ra + 4 * i) * 128 + ((kc ^ ((ra + 4 * i) & 7)) << 4), a[i][0], a[i][1]);
+    for (int i = 0; i < 4; ++i) ld4<T, AR>(a_tile, ra + 4 * i, kq, a[i][0], a[i][1]);
 #pragma unroll
-    for (int j = 0; j < JN; ++j) lds2x2(bt + (tn + 8 * j) * 128 + ((kc ^ tn) << 4), b[j][0], b[j][1]);
+    for (int j = 0; j < JN; ++j) ld4<T, BR>(b_tile, tn + 8 * j, kq, b[j][0], b[j][1]);
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
@@ -90,7 +105,7 @@ __device__ __forceinline__ void scores(uint32_t a_tile, uint32_t b_tile, int ra,
 
 // acc[i][..] += sum over n rows k of tile b of w[row i][k] b[k][columns of this thread]; w: this thread's four rows in
 // shared memory, four rows of pitch `ld` apart.
-template <int HD, int BR>
+template <typename T, int HD, int BR>
 __device__ __forceinline__ void weighted(uint32_t w, int ld, uint32_t b_tile, int tn, int n, f2 (&acc)[4][HD / 16]) {
 #pragma unroll 2
   for (int k0 = 0; k0 < n; k0 += 4) {
@@ -100,7 +115,7 @@ __device__ __forceinline__ void weighted(uint32_t w, int ld, uint32_t b_tile, in
     for (int k = 0; k < 4; ++k)
 #pragma unroll
       for (int p = 0; p < HD / 32; ++p)
-        lds2x2(b_tile + p * (BR * 128) + (k0 + k) * 128 + ((tn ^ ((k0 + k) & 7)) << 4), b[k][2 * p], b[k][2 * p + 1]);
+        ld4<T, BR>(b_tile, k0 + k, p * 8 + tn, b[k][2 * p], b[k][2 * p + 1]);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float4 v = lds4(w + (4 * i * ld + k0) * 4);
@@ -171,7 +186,7 @@ __global__ void __launch_bounds__(THREADS) attn_fwd_ffma_kernel(const __grid_con
     const int j0 = j * FWD_KEYS;
     ok = tc::mbar_wait(bar_k, j & 1, P.status, 131);
     float s[4][JN];
-    scores<HD, JN, ROWS, FWD_KEYS>(base + SM::Q_OFF, base + SM::K_OFF, warp * 16 + tm, tn, s);
+    scores<float, HD, JN, ROWS, FWD_KEYS>(base + SM::Q_OFF, base + SM::K_OFF, warp * 16 + tm, tn, s);
     if (__syncthreads_or(!ok)) return false;               // all warps are done with K
     if (threadIdx.x == 0 && j + 1 < n_tiles) load(&P.tk, base + SM::K_OFF, bar_k, j + 1);
     const bool need_mask = j0 + JN * 8 > P.seq_k || (P.causal && j0 + JN * 8 - 1 > i0);
@@ -207,7 +222,7 @@ __global__ void __launch_bounds__(THREADS) attn_fwd_ffma_kernel(const __grid_con
     }
     __syncwarp();
     ok = tc::mbar_wait(bar_v, j & 1, P.status, 132);
-    weighted<HD, FWD_KEYS>(p_row, FWD_LD, base + SM::V_OFF, tn, JN * 8, o);
+    weighted<float, HD, FWD_KEYS>(p_row, FWD_LD, base + SM::V_OFF, tn, JN * 8, o);
     if (__syncthreads_or(!ok)) return false;               // ... and with V
     if (threadIdx.x == 0 && j + 1 < n_tiles) load(&P.tv, base + SM::V_OFF, bar_v, j + 1);
     return true;
@@ -225,8 +240,8 @@ __global__ void __launch_bounds__(THREADS) attn_fwd_ffma_kernel(const __grid_con
 #pragma unroll
     for (int p = 0; p < PN; ++p) {
       const float2 x = unpack2(o[i][2 * p]), y = unpack2(o[i][2 * p + 1]);
-      *reinterpret_cast<float4*>(P.a + rt_off<32>(P.n_pad, row0 + gi, h * HD + p * 32 + tn * 4)) =
-          live ? make_float4(x.x * inv, x.y * inv, y.x * inv, y.y * inv) : make_float4(0.f, 0.f, 0.f, 0.f);
+      st4(P.a + rt_off<32>(P.n_pad, row0 + gi, h * HD + p * 32 + tn * 4),
+          live ? make_float4(x.x * inv, x.y * inv, y.x * inv, y.y * inv) : make_float4(0.f, 0.f, 0.f, 0.f));
     }
     if (tn == 0) P.lse[((long long)b * P.hq + h) * P.t_pad + gi] = live ? m[i] + logf(l[i]) : 0.f;
   }
@@ -239,18 +254,21 @@ __global__ void __launch_bounds__(THREADS) attn_fwd_ffma_kernel(const __grid_con
 // (query head, query tile) items in turn and adds its dK and dV through distributed shared memory in a fixed order: the
 // bound is the items' chain, some 6 us each.
 // ------------------------------------------------------------------------------------------
-template <int HD>
+template <typename T, int HD>
 struct FfmaBwdSmem {
   static constexpr int QT = HD == 128 ? 32 : 64, LD = QT + 8;            // queries of a tile; pitch of P^T and dS^T rows
-  static constexpr uint32_t K_OFF = 0, V_OFF = HD * ROWS * 4, Q_OFF = 2 * V_OFF, DO_OFF = Q_OFF + HD * QT * 4;
-  static constexpr uint32_t P_OFF = DO_OFF + HD * QT * 4, S_OFF = P_OFF + ROWS * LD * 4;
+  static constexpr uint32_t E = sizeof(T), K_OFF = 0, V_OFF = HD * ROWS * E, Q_OFF = 2 * V_OFF, DO_OFF = Q_OFF + HD * QT * E;
+  static constexpr uint32_t P_OFF = DO_OFF + HD * QT * E, S_OFF = P_OFF + ROWS * LD * 4;
+  // slices: a block's dK and dV in fp32, over the operand tiles when they are free
+  static constexpr uint32_t SUM_K = 0, SUM_V = HD * ROWS * 4;
+  static_assert(2 * SUM_V <= P_OFF, "");
   static constexpr uint32_t BAR_OFF = S_OFF + ROWS * LD * 4, TOTAL = BAR_OFF + 24 + 1024;
 };
 
-template <int HD>
+template <typename T, int HD>
 __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_constant__ FfmaAttnParams P) {
-  using SM = FfmaBwdSmem<HD>;
-  constexpr int PN = HD / 32, QT = SM::QT, LD = SM::LD;
+  using SM = FfmaBwdSmem<T, HD>;
+  constexpr int TW = tile_w_of<T>::value, PN = HD / TW, QT = SM::QT, LD = SM::LD;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u, bar_kv = base + SM::BAR_OFF, bar_q = bar_kv + 8, bar_do = bar_kv + 16;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, tm = lane % 4, tn = lane / 4;
@@ -259,7 +277,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
   const int row0 = b * P.t_pad, row0k = b * P.t_pad_k;
   const int t0 = P.causal ? j0 / QT : 0, per_head = (P.seq + QT - 1) / QT - t0, n_it = max(0, per_head) * P.group;
   auto load = [&](const CUtensorMap* map, uint32_t dst, uint32_t bar, int it) {
-    tc::mbar_expect_tx(bar, HD * QT * 4);
+    tc::mbar_expect_tx(bar, HD * QT * SM::E);
     tc::tma_load_3d(dst, map, bar, 0, row0 + (t0 + it % per_head) * QT, (g * P.group + it / per_head) * PN);
   };
   if (threadIdx.x == 0) {
@@ -268,7 +286,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
     tc::mbar_init(bar_do, 1);
     tc::fence_barrier_init();
     pdl_wait();
-    tc::mbar_expect_tx(bar_kv, 2 * HD * ROWS * 4);
+    tc::mbar_expect_tx(bar_kv, 2 * HD * ROWS * SM::E);
     tc::tma_load_3d(base + SM::K_OFF, &P.tk, bar_kv, 0, row0k + j0, g * PN);
     tc::tma_load_3d(base + SM::V_OFF, &P.tv, bar_kv, 0, row0k + j0, g * PN);
     if (slice < n_it) {
@@ -302,7 +320,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
     }
     ok = tc::mbar_wait(bar_q, phase, P.status, 134) && ok;
     float p[4][JN], dp[4][JN];
-    scores<HD, JN, ROWS, QT>(base + SM::K_OFF, base + SM::Q_OFF, ra, tn, p);
+    scores<T, HD, JN, ROWS, QT>(base + SM::K_OFF, base + SM::Q_OFF, ra, tn, p);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -312,16 +330,16 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
         sts(p_row + (4 * i * LD + tn + 8 * j) * 4, p[i][j]);
       }
     ok = tc::mbar_wait(bar_do, phase, P.status, 135) && ok;
-    scores<HD, JN, ROWS, QT>(base + SM::V_OFF, base + SM::DO_OFF, ra, tn, dp);
+    scores<T, HD, JN, ROWS, QT>(base + SM::V_OFF, base + SM::DO_OFF, ra, tn, dp);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < JN; ++j) sts(s_row + (4 * i * LD + tn + 8 * j) * 4, p[i][j] * (dp[i][j] - d[j]));
     __syncwarp();
-    weighted<HD, QT>(p_row, LD, base + SM::DO_OFF, tn, JN * 8, dv);
+    weighted<T, HD, QT>(p_row, LD, base + SM::DO_OFF, tn, JN * 8, dv);
     if (__syncthreads_or(!ok)) return false;               // all warps are done with dO, and dS^T is complete
     if (threadIdx.x == 0 && it + slices < n_it) load(&P.tdo, base + SM::DO_OFF, bar_do, it + slices);
-    weighted<HD, QT>(s_row, LD, base + SM::Q_OFF, tn, JN * 8, dk);
+    weighted<T, HD, QT>(s_row, LD, base + SM::Q_OFF, tn, JN * 8, dk);
     __syncthreads();                                       // ... and with Q
     if (threadIdx.x == 0 && it + slices < n_it) load(&P.tq, base + SM::Q_OFF, bar_q, it + slices);
     // dQ = dS K: 16 queries at a time per warp, four neighbouring ones per thread, reduced over the block's keys
@@ -336,8 +354,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
       for (int k = 0; k < ROWS; ++k) {
         f2 kb[HD / 16];
 #pragma unroll
-        for (int pn = 0; pn < PN; ++pn)
-          lds2x2(base + SM::K_OFF + pn * (ROWS * 128) + k * 128 + ((tn ^ (k & 7)) << 4), kb[2 * pn], kb[2 * pn + 1]);
+        for (int pn = 0; pn < HD / 32; ++pn) ld4<T, ROWS>(base + SM::K_OFF, k, pn * 8 + tn, kb[2 * pn], kb[2 * pn + 1]);
         const float4 v = lds4(base + SM::S_OFF + (k * LD + q0 + tm * 4) * 4);
         const float sv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -352,9 +369,9 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
         const int gi = i0 + q0 + tm * 4 + i;
         if (gi >= P.seq) continue;
 #pragma unroll
-        for (int pn = 0; pn < PN; ++pn) {
+        for (int pn = 0; pn < HD / 32; ++pn) {
           const float2 x = unpack2(dq[i][2 * pn]), y = unpack2(dq[i][2 * pn + 1]);
-          atomicAdd(reinterpret_cast<float4*>(P.dq + rt_off<32>(P.n_pad, row0 + gi, h * HD + pn * 32 + tn * 4)),
+          atomicAdd(reinterpret_cast<float4*>(P.dq + rt_off<TW>(P.n_pad, row0 + gi, h * HD + pn * 32 + tn * 4)),
                     make_float4(x.x * P.scale, x.y * P.scale, y.x * P.scale, y.y * P.scale));
         }
       }
@@ -366,25 +383,25 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
   using Half = std::integral_constant<int, QT / 16>;
   for (int it = slice, phase = 0; it < n_it; it += slices, phase ^= 1)
     if (!(P.seq - (t0 + it % per_head) * QT > QT / 2 ? tile(Full{}, it, phase) : tile(Half{}, it, phase))) break;
-  auto store = [&](float* out, int row, int col, float4 v, float f) {
+  auto store = [&](void* out, int row, int col, float4 v, float f) {
     if (j0 + row < P.t_pad_k) {
       f = j0 + row < P.seq_k ? f : 0.f;
-      *reinterpret_cast<float4*>(out + rt_off<32>(P.n_pad_k, row0k + j0 + row, g * HD + col)) = make_float4(v.x * f, v.y * f, v.z * f, v.w * f);
+      st4((T*)out + rt_off<TW>(P.n_pad_k, row0k + j0 + row, g * HD + col), make_float4(v.x * f, v.y * f, v.z * f, v.w * f));
     }
   };
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int pn = 0; pn < PN; ++pn) {
+    for (int pn = 0; pn < HD / 32; ++pn) {
       const int row = ra + 4 * i, col = pn * 32 + tn * 4;
       const float2 x = unpack2(dk[i][2 * pn]), y = unpack2(dk[i][2 * pn + 1]), u = unpack2(dv[i][2 * pn]), w = unpack2(dv[i][2 * pn + 1]);
       const float4 k4 = make_float4(x.x, x.y, y.x, y.y), v4 = make_float4(u.x, u.y, w.x, w.y);
       if (slices == 1) {
         store(P.dk, row, col, k4, P.scale);
         store(P.dv, row, col, v4, 1.f);
-      } else {                                             // Q's and dO's places are free
-        sts4(base + SM::Q_OFF + (row * HD + col) * 4, k4);
-        sts4(base + SM::DO_OFF + (row * HD + col) * 4, v4);
+      } else {
+        sts4(base + SM::SUM_K + (row * HD + col) * 4, k4);
+        sts4(base + SM::SUM_V + (row * HD + col) * 4, v4);
       }
     }
   if (slices > 1) {
@@ -393,7 +410,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
     for (int e = threadIdx.x; e < 2 * per * (HD / 4); e += THREADS) {
       const int row = slice * per + e / (HD / 4) % per, col = e % (HD / 4) * 4;
       const bool is_v = e >= per * (HD / 4);
-      const uint32_t at = base + (is_v ? SM::DO_OFF : SM::Q_OFF) + (row * HD + col) * 4;
+      const uint32_t at = base + (is_v ? SM::SUM_V : SM::SUM_K) + (row * HD + col) * 4;
       float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
       for (int c = 0; c < slices; ++c) {
@@ -425,7 +442,13 @@ void fill(const fbl_plan* p, FfmaAttnParams& P, int32_t* status) {
   P.hq = p->d.n_q_heads; P.group = p->group; P.causal = p->d.causal; P.scale = p->scale; P.status = status;
 }
 
-static_assert(FfmaFwdSmem<128>::TOTAL <= ALONE && FfmaBwdSmem<128>::TOTAL <= ALONE, "");
+static_assert(FfmaFwdSmem<128>::TOTAL <= ALONE && FfmaBwdSmem<float, 128>::TOTAL <= ALONE, "");
+
+template <typename T>
+bool encode(CUtensorMap* map, const void* base, int64_t r_pad, int cols, int rows, int hd) {
+  constexpr int TW = tile_w_of<T>::value;
+  return sizeof(T) == 4 ? fbl_encode_f32_rtile_map(map, base, r_pad, cols / TW, rows, hd / TW) : fbl_encode_rtile_map(map, base, r_pad, cols / TW, rows, hd / TW);
+}
 
 template <int HD>
 cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse, int32_t* status, cudaStream_t st) {
@@ -434,9 +457,8 @@ cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   const uint32_t smem = spread(p, grid, (p->t_pad_kv + FWD_KEYS - 1) / FWD_KEYS, FfmaFwdSmem<HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
-  if (!fbl_encode_f32_rtile_map(&P.tq, Q, p->n_pad, p->dq / 32, ROWS, HD / 32) ||
-      !fbl_encode_f32_rtile_map(&P.tk, K, p->n_pad_kv, p->dkv / 32, FWD_KEYS, HD / 32) ||
-      !fbl_encode_f32_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 32, FWD_KEYS, HD / 32))
+  if (!encode<float>(&P.tq, Q, p->n_pad, p->dq, ROWS, HD) || !encode<float>(&P.tk, K, p->n_pad_kv, p->dkv, FWD_KEYS, HD) ||
+      !encode<float>(&P.tv, V, p->n_pad_kv, p->dkv, FWD_KEYS, HD))
     return cudaErrorInvalidValue;
   P.a = (float*)A; P.lse = lse;
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
@@ -448,26 +470,24 @@ cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   });
 }
 
-template <int HD>
+template <typename T, int HD>
 cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* dA, const float* lse, const float* dvec,
-                       void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st) {
-  constexpr int QT = FfmaBwdSmem<HD>::QT;
-  auto k = attn_bwd_ffma_kernel<HD>;
+                       float* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st) {
+  constexpr int QT = FfmaBwdSmem<T, HD>::QT;
+  auto k = attn_bwd_ffma_kernel<T, HD>;
   // slices of a key tile's items: an item each at least, and no more once there are two blocks per SM (of two warps each,
   // for an SM's four schedulers)
   const int key_tiles = (p->t_pad_kv + ROWS - 1) / ROWS, items = (p->d.seq + QT - 1) / QT * p->group;
   int slices = 1;
   while (slices < 8 && 2 * slices <= items && (long long)key_tiles * p->d.n_kv_heads * p->d.batch * slices <= 2 * p->sm_count) slices *= 2;
   const dim3 grid(key_tiles * slices, p->d.n_kv_heads, p->d.batch);
-  const uint32_t smem = slices > 1 ? FfmaBwdSmem<HD>::TOTAL : spread(p, grid, items, FfmaBwdSmem<HD>::TOTAL);
+  const uint32_t smem = slices > 1 ? FfmaBwdSmem<T, HD>::TOTAL : spread(p, grid, items, FfmaBwdSmem<T, HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
-  if (!fbl_encode_f32_rtile_map(&P.tq, Q, p->n_pad, p->dq / 32, QT, HD / 32) ||
-      !fbl_encode_f32_rtile_map(&P.tdo, dA, p->n_pad, p->dq / 32, QT, HD / 32) ||
-      !fbl_encode_f32_rtile_map(&P.tk, K, p->n_pad_kv, p->dkv / 32, ROWS, HD / 32) ||
-      !fbl_encode_f32_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 32, ROWS, HD / 32))
+  if (!encode<T>(&P.tq, Q, p->n_pad, p->dq, QT, HD) || !encode<T>(&P.tdo, dA, p->n_pad, p->dq, QT, HD) ||
+      !encode<T>(&P.tk, K, p->n_pad_kv, p->dkv, ROWS, HD) || !encode<T>(&P.tv, V, p->n_pad_kv, p->dkv, ROWS, HD))
     return cudaErrorInvalidValue;
-  P.lse = const_cast<float*>(lse); P.dvec = dvec; P.dq = (float*)dQ; P.dk = (float*)dK; P.dv = (float*)dV;
+  P.lse = const_cast<float*>(lse); P.dvec = dvec; P.dq = dQ; P.dk = dK; P.dv = dV;
   P.slices = slices;
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
   };
@@ -492,14 +512,24 @@ cudaError_t launch_attn_fwd_ffma(const fbl_plan* p, const void* Q, const void* K
 }
 
 cudaError_t launch_attn_bwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A, const void* dA,
-                                 const float* lse, float* dvec, void* dQ, void* dK, void* dV, bool dvec_ready, int32_t* status,
-                                 cudaStream_t st) {
-  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, nullptr, dvec_ready, st);
+                                 const float* lse, float* dvec, float* dqacc, void* dQ, void* dK, void* dV, bool dvec_ready,
+                                 int32_t* status, cudaStream_t st, const float2* rope) {
+  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dvec_ready, st);
   if (e != cudaSuccess) return e;
-  switch (p->d.head_dim) {
-    case 32: return bwd_launch<32>(p, Q, K, V, dA, lse, dvec, dQ, dK, dV, status, st);
-    case 64: return bwd_launch<64>(p, Q, K, V, dA, lse, dvec, dQ, dK, dV, status, st);
-    case 128: return bwd_launch<128>(p, Q, K, V, dA, lse, dvec, dQ, dK, dV, status, st);
+#define FBL_CALL(T_, HD_, DQ_) e = bwd_launch<T_, HD_>(p, Q, K, V, dA, lse, dvec, DQ_, dK, dV, status, st)
+  if (p->d.dtype == FBL_DTYPE_BF16) {
+    if (p->d.head_dim == 64) FBL_CALL(__nv_bfloat16, 64, dqacc);
+    else if (p->d.head_dim == 128) FBL_CALL(__nv_bfloat16, 128, dqacc);
+    else e = cudaErrorInvalidValue;
+    if (e != cudaSuccess) return e;
+    return rope ? launch_rope_bwd_round(p, dqacc, dQ, dK, rope, st) : launch_attn_bwd_post(p, dqacc, dQ, st);
   }
-  return cudaErrorInvalidValue;
+  switch (p->d.head_dim) {
+    case 32: FBL_CALL(float, 32, (float*)dQ); break;
+    case 64: FBL_CALL(float, 64, (float*)dQ); break;
+    case 128: FBL_CALL(float, 128, (float*)dQ); break;
+    default: e = cudaErrorInvalidValue;
+  }
+  return e;
+#undef FBL_CALL
 }

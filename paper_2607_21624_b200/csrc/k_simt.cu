@@ -430,12 +430,9 @@ cudaError_t launch_attn_fwd_simt(const fbl_plan* p, const void* Q, const void* K
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_attn_bwd_pre(const fbl_plan* p, const void* A, const void* dA, float* dvec, float* dqacc,
-                                bool dvec_ready, cudaStream_t st) {
+cudaError_t launch_attn_bwd_pre(const fbl_plan* p, const void* A, const void* dA, float* dvec, bool dvec_ready, cudaStream_t st) {
   const int hd = p->d.head_dim;
   const int64_t total = p->n_pad * p->d.n_q_heads;
-  // dqacc was zero-filled with the status word at the start of the step
-  (void)dqacc;
   if (dvec_ready) return cudaSuccess;
   const unsigned rb = (unsigned)((total + 255) / 256);
   if (p->d.dtype == FBL_DTYPE_FP32)
@@ -455,7 +452,7 @@ cudaError_t launch_attn_bwd_simt(const fbl_plan* p, const void* Q, const void* K
                                  const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
                                  void* dV, bool dvec_ready, cudaStream_t st) {
   const int hd = p->d.head_dim;
-  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, dvec_ready, st);
+  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dvec_ready, st);
   if (e != cudaSuccess) return e;
   if (hd == 64) e = attn_bwd_launch<__nv_bfloat16, 64>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);
   else if (hd == 128) e = attn_bwd_launch<__nv_bfloat16, 128>(p, Q, K, V, dA, lse, dvec, dqacc, dK, dV, st);

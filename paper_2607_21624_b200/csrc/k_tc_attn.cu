@@ -35,6 +35,12 @@ struct alignas(64) AttnFwdParams {
   int32_t* status;
 };
 
+// Two values as packed bf16, and what the rounding leaves of them likewise.
+__device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
+  hi = tc::pack_bf16(x, y);
+  lo = tc::pack_bf16(x - __uint_as_float(hi << 16), y - __uint_as_float(hi & 0xffff0000u));
+}
+
 template <int HD, int TILES>
 struct FwdSmem {
   static constexpr uint32_t PANELS = HD / 64;
@@ -58,7 +64,11 @@ enum { B_QFULL = 0, B_KFULL = 1, B_KEMPTY = 3, B_VFULL = 5, B_VEMPTY = 7, B_SFUL
 // powers of two; until then the probabilities are computed against the stale max and stay below 2^8.
 constexpr float RESCALE_LOG2 = 8.f;
 
-template <int HD, int TILES>
+// SPLIT (attn_fp32): P goes to the tensor pipe as two bf16 values, its rounding and what that leaves, 16 bits and more in all:
+// A is off by 1.6414e-3 of its norm, the final rounding, as with P in fp32 (1.8e-3 with P in bf16; 60 layers of 1 to 120 rows
+// against 64 bits), for a second P V product: 19.2 -> 19.3 us a 50-token forward, 28.7 -> 30.2 us one of 120 tokens with heads
+// of 128 (on the FP32 pipe 24.3 and 47.7).
+template <int HD, int TILES, bool SPLIT>
 __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd_tc_kernel(const __grid_constant__ AttnFwdParams P) {
   using SM = FwdSmem<HD, TILES>;
   constexpr uint32_t PANELS = SM::PANELS;
@@ -72,6 +82,9 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
   constexpr int NBUF = ROT ? 3 : TILES;
   constexpr uint32_t O_COL = 128 * NBUF, TMEM_COLS = 256 * TILES;   // score buffer i at 128 i, O of tile g at O_COL + HD g
   static_assert(O_COL + TILES * HD <= TMEM_COLS, "tensor memory columns");
+  // the remainders: behind the packed P where a thread holds all its scores, else in columns of their own
+  constexpr uint32_t LO_COL = TILES == 1 ? O_COL + HD : 64;
+  static_assert(!SPLIT || (!ROT && LO_COL + 64 <= (TILES == 1 ? TMEM_COLS : 128)), "tensor memory columns");
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = tc::smem_u32(smem_raw);
   const uint32_t bars = base + SM::BAR_OFF;
@@ -182,6 +195,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
         // A operand from tensor memory: the packed bf16 P row of each lane, 16 keys = 8 columns per step
         tc::mma_bf16_ts_w(tmem_base + O_COL + w * HD, tmem_base + w * 128 + kk * 8, vl + kk * 128, hi, idesc_o,
                           (j > 0 || kk > 0) ? 1u : 0u);
+        if constexpr (SPLIT) tc::mma_bf16_ts_w(tmem_base + O_COL + w * HD, tmem_base + w * 128 + LO_COL + kk * 8, vl + kk * 128, hi, idesc_o, 1u);
       }
       tc::mma_commit(bar(B_PVDONE + w));
     };
@@ -335,11 +349,26 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
           const float2 x23 = __ffma2_rn(make_float2(sv[k + 2], sv[k + 3]), c2, nmc2);
           const float p0 = tc::fast_exp2(x01.x), p1 = tc::fast_exp2(x01.y), p2 = tc::fast_exp2(x23.x), p3 = tc::fast_exp2(x23.y);
           sum01 = __fadd2_rn(sum01, make_float2(p0, p1)); sum23 = __fadd2_rn(sum23, make_float2(p2, p3));
-          sr[k / 2] = tc::pack_bf16(p0, p1);
-          sr[k / 2 + 1] = tc::pack_bf16(p2, p3);
+          if constexpr (SPLIT) {
+            split_bf16(p0, p1, sr[k], sr[k + 1]);
+            split_bf16(p2, p3, sr[k + 2], sr[k + 3]);
+          } else {
+            sr[k / 2] = tc::pack_bf16(p0, p1);
+            sr[k / 2 + 1] = tc::pack_bf16(p2, p3);
+          }
         }
-        tc::tmem_st32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
-        tc::tmem_st32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
+        if constexpr (SPLIT) {
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {                // P's columns, first and second half, then the remainders'
+            uint32_t v[32];
+#pragma unroll
+            for (int k = 0; k < 32; ++k) v[k] = sr[(x & 1) * 64 + 2 * k + x / 2];
+            tc::tmem_st32(s_addr + 32 * x, v);
+          }
+        } else {
+          tc::tmem_st32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+          tc::tmem_st32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
+        }
       } else {
         // At most 128 registers here (two blocks per SM): two passes over the scores in tensor memory in 32-column
         // loads instead of holding the row, and only as many as the warp attends to.
@@ -402,21 +431,30 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
           tc::tmem_ld_wait();
           float* sc = reinterpret_cast<float*>(sr);
           if (need_mask) mask_chunk(sc, cc);
-          uint32_t pk[16];
+          uint32_t pk[16], lo[SPLIT ? 16 : 1];
 #pragma unroll
           for (int k = 0; k < 32; k += 4) {
             const float2 x01 = __ffma2_rn(make_float2(sc[k], sc[k + 1]), c2, nmc2);
             const float2 x23 = __ffma2_rn(make_float2(sc[k + 2], sc[k + 3]), c2, nmc2);
             const float p0 = tc::fast_exp2(x01.x), p1 = tc::fast_exp2(x01.y), p2 = tc::fast_exp2(x23.x), p3 = tc::fast_exp2(x23.y);
             sum01 = __fadd2_rn(sum01, make_float2(p0, p1)); sum23 = __fadd2_rn(sum23, make_float2(p2, p3));
-            pk[k / 2] = tc::pack_bf16(p0, p1);
-            pk[k / 2 + 1] = tc::pack_bf16(p2, p3);
+            if constexpr (SPLIT) {
+              split_bf16(p0, p1, pk[k / 2], lo[k / 2]);
+              split_bf16(p2, p3, pk[k / 2 + 1], lo[k / 2 + 1]);
+            } else {
+              pk[k / 2] = tc::pack_bf16(p0, p1);
+              pk[k / 2 + 1] = tc::pack_bf16(p2, p3);
+            }
           }
           tc::tmem_st16(s_addr + cc * 16, pk);
+          if constexpr (SPLIT) tc::tmem_st16(s_addr + LO_COL + cc * 16, lo);
         }
         const uint32_t zero[16] = {};
 #pragma unroll 1
-        for (int cc = n_ch; cc < 4; ++cc) tc::tmem_st16(s_addr + cc * 16, zero);
+        for (int cc = n_ch; cc < 4; ++cc) {
+          tc::tmem_st16(s_addr + cc * 16, zero);
+          if constexpr (SPLIT) tc::tmem_st16(s_addr + LO_COL + cc * 16, zero);
+        }
       }
       if (moved) l *= alpha;
       l += (sum01.x + sum01.y) + (sum23.x + sum23.y);
@@ -472,14 +510,14 @@ struct AttnLaunch {
   }
 };
 
-template <int HD, int TILES>
+template <int HD, int TILES, bool SPLIT = false>
 cudaError_t fwd_make_t(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, int n_qt) {
   AttnFwdParams& P = L.P;
   if (TILES == 1) P.pair = 0;
   P.batch = p->d.batch;
   P.n_slots = P.pair ? (n_qt + 1) / 2 : n_qt;
   P.chunk = chunk_for((long long)p->seq_kv * HD * 4, p->d.n_q_heads * p->d.batch, 96ll << 20);   // K and V of one head
-  return L.set(attn_fwd_tc_kernel<HD, TILES>, P.n_slots * p->d.n_q_heads * p->d.batch, 64 + 128 * TILES, FwdSmem<HD, TILES>::TOTAL);
+  return L.set(attn_fwd_tc_kernel<HD, TILES, SPLIT>, P.n_slots * p->d.n_q_heads * p->d.batch, 64 + 128 * TILES, FwdSmem<HD, TILES>::TOTAL);
 }
 
 template <int HD>
@@ -498,6 +536,7 @@ cudaError_t fwd_make(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, const void
   const int n_qt = (p->d.seq + BQ - 1) / BQ;
   // two query tiles per block when that still leaves at least one block per SM
   P.pair = (n_qt >= 2 && (long long)((n_qt + 1) / 2) * p->d.n_q_heads * p->d.batch >= p->sm_count) ? 1 : 0;
+  if (attn_fp32(p)) return fwd_make_t<HD, HD == 64 ? 1 : 2, true>(L, p, n_qt);
   if (HD == 64) {
     // tuning knob: 1 = one query tile per block and two blocks per SM, 2 = two tiles per block; default by sequence length
     const int mode = p->knob_fwd_tiles;
@@ -1461,11 +1500,6 @@ bool attn_bwd_tc_direct(const fbl_plan* p) {
   return p->d.head_dim == 64 && p->group == 1 && p->t_pad_kv <= 2 * BKV && p->t_pad <= 2 * BQ;
 }
 
-bool attn_fwd_tc_supported(const fbl_plan* p) {
-  return p->d.dtype == FBL_DTYPE_BF16 && (p->d.head_dim == 64 || p->d.head_dim == 128);   // boxes past the last row load zeros
-}
-bool attn_bwd_tc_supported(const fbl_plan* p) { return attn_fwd_tc_supported(p); }
-
 cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                int32_t* status, cudaStream_t st) {
   typedef AttnLaunch<AttnFwdParams> Launch;
@@ -1482,7 +1516,7 @@ cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, 
                                const void* dA, const float* lse, float* dvec, float* dqacc, void* dQ, void* dK,
                                void* dV, bool dvec_ready, int32_t* status, cudaStream_t st, const float2* rope) {
   // D = rowsum(dO * O) unless the dA GEMM's epilogue already produced it
-  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dqacc, dvec_ready, st);
+  cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dvec_ready, st);
   if (e != cudaSuccess) return e;
   typedef AttnLaunch<AttnBwdParams> Launch;
   LaunchKey key;

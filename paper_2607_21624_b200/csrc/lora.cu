@@ -167,9 +167,7 @@ int fbl_layer_fwd_lora(const fbl_plan* p, const void* X, const float* gamma, con
     p->launches += k;
   }
   if (p->rope_base > 0.f && !rotated) LORA_STEP("rope", 1, launch_rope(p, Q, p->d.n_q_heads, K, p->d.n_kv_heads, 0, st));
-  if (p->use_tc && attn_fwd_tc_supported(p)) LORA_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
-  else if (p->d.dtype == FBL_DTYPE_FP32) LORA_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
-  else LORA_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
+  LORA_STEP("attn_fwd", 1, run_attn_fwd(p, Q, K, V, A, lse, status, st));
   {
     GemmArgs g = {};
     g.m = n; g.n = D; g.n_terms = 1;
@@ -231,11 +229,9 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     LORA_STEP("dA", 0, cudaSuccess);
     p->launches += k;
   }
-  if (p->use_tc && attn_bwd_tc_supported(p)) LORA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st,
-                                                  p->rope_base > 0.f ? (const float2*)(sv + p->sv_rope) : nullptr));
-  else if (p->d.dtype == FBL_DTYPE_FP32) LORA_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
-  else LORA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
-  if (p->rope_base > 0.f && !(p->use_tc && attn_bwd_tc_supported(p))) LORA_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
+  LORA_STEP("attn_bwd", attn_bwd_launches(p, dvec_ready), run_attn_bwd(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st,
+                                                                       p->rope_base > 0.f ? (const float2*)(sv + p->sv_rope) : nullptr));
+  if (p->rope_base > 0.f && !attn_bwd_turns(p)) LORA_STEP("rope_bwd", 1, launch_rope(p, dQ, p->d.n_q_heads, dK, p->d.n_kv_heads, 1, st));
   const void* G[3] = {dQ, dK, dV};
   {
     GemmArgs g = {};                       // dT = dQ Bq^T | dK Bk^T | dV Bv^T: B_all's column blocks read with swapped axes;

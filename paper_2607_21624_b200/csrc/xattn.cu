@@ -83,9 +83,7 @@ int fbl_xattn_fwd(const fbl_plan* p, const void* X, const void* M, const float* 
     for (int i = 0; i < 3; ++i) gs[i].b_static = 1;
     XA_GEMM_STEP("proj_qkv", gs, 3);
   }
-  if (p->use_tc && attn_fwd_tc_supported(p)) XA_STEP("attn_fwd", 1, launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st));
-  else if (p->d.dtype == FBL_DTYPE_FP32) XA_STEP("attn_fwd", 1, launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st));
-  else XA_STEP("attn_fwd", 1, launch_attn_fwd_simt(p, Q, K, V, A, lse, st));
+  XA_STEP("attn_fwd", 1, run_attn_fwd(p, Q, K, V, A, lse, status, st));
   {
     GemmArgs g = {};
     g.m = n; g.n = D; g.n_terms = 1;
@@ -154,9 +152,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     XA_CUDA(start_backward(p, gs, 2, !split_o, true, status, bwd_zero_bytes(p), st));
     XA_GEMM_STEP("dWo+dA", gs, 2);
   }
-  if (p->use_tc && attn_bwd_tc_supported(p)) XA_STEP("attn_bwd", attn_bwd_tc_launches(p, dvec_ready), launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st));
-  else if (p->d.dtype == FBL_DTYPE_FP32) XA_STEP("attn_bwd", dvec_ready ? 1 : 2, launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st));
-  else XA_STEP("attn_bwd", dvec_ready ? 2 : 3, launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st));
+  XA_STEP("attn_bwd", attn_bwd_launches(p, dvec_ready), run_attn_bwd(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, nullptr));
   // bias gradients: column sums over the query tokens (dY, dQ) and over the memory's tokens (dK, dV), beside the last
   // products or, the former, in the norm backward's launches
   ColsumGroup sums = {};
