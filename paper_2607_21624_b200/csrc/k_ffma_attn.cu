@@ -151,11 +151,11 @@ __global__ void __launch_bounds__(THREADS) attn_fwd_ffma_kernel(const __grid_con
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, tm = lane % 4, tn = lane / 4;
   // later queries first: under a causal mask they have the most keys
   const int i0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * ROWS, h = blockIdx.y, b = blockIdx.z, g = h / P.group;
-  const int row0 = b * P.t_pad, row0k = b * P.t_pad_k;
+  const int row0 = b * P.t_pad;
   const int j_end = P.causal ? min(P.seq_k, i0 + ROWS) : P.seq_k, n_tiles = (j_end + FWD_KEYS - 1) / FWD_KEYS;
   auto load = [&](const CUtensorMap* map, uint32_t dst, uint32_t bar, int j) {
     tc::mbar_expect_tx(bar, HD * FWD_KEYS * 4);
-    tc::tma_load_3d(dst, map, bar, 0, row0k + j * FWD_KEYS, g * PN);
+    tc::tma_load_4d(dst, map, bar, 0, j * FWD_KEYS, b, g * PN);
   };
   if (threadIdx.x == 0) {
     tc::mbar_init(bar_k, 1);
@@ -163,8 +163,8 @@ __global__ void __launch_bounds__(THREADS) attn_fwd_ffma_kernel(const __grid_con
     tc::fence_barrier_init();
     pdl_wait();
     tc::mbar_expect_tx(bar_k, HD * (FWD_KEYS + ROWS) * 4);
-    tc::tma_load_3d(base + SM::Q_OFF, &P.tq, bar_k, 0, row0 + i0, h * PN);
-    tc::tma_load_3d(base + SM::K_OFF, &P.tk, bar_k, 0, row0k, g * PN);
+    tc::tma_load_4d(base + SM::Q_OFF, &P.tq, bar_k, 0, i0, b, h * PN);
+    tc::tma_load_4d(base + SM::K_OFF, &P.tk, bar_k, 0, 0, b, g * PN);
     load(&P.tv, base + SM::V_OFF, bar_v, 0);
   }
   __syncthreads();
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
   const int t0 = P.causal ? j0 / QT : 0, per_head = (P.seq + QT - 1) / QT - t0, n_it = max(0, per_head) * P.group;
   auto load = [&](const CUtensorMap* map, uint32_t dst, uint32_t bar, int it) {
     tc::mbar_expect_tx(bar, HD * QT * SM::E);
-    tc::tma_load_3d(dst, map, bar, 0, row0 + (t0 + it % per_head) * QT, (g * P.group + it / per_head) * PN);
+    tc::tma_load_4d(dst, map, bar, 0, (t0 + it % per_head) * QT, b, (g * P.group + it / per_head) * PN);
   };
   if (threadIdx.x == 0) {
     tc::mbar_init(bar_kv, 1);
@@ -287,8 +287,8 @@ __global__ void __launch_bounds__(THREADS) attn_bwd_ffma_kernel(const __grid_con
     tc::fence_barrier_init();
     pdl_wait();
     tc::mbar_expect_tx(bar_kv, 2 * HD * ROWS * SM::E);
-    tc::tma_load_3d(base + SM::K_OFF, &P.tk, bar_kv, 0, row0k + j0, g * PN);
-    tc::tma_load_3d(base + SM::V_OFF, &P.tv, bar_kv, 0, row0k + j0, g * PN);
+    tc::tma_load_4d(base + SM::K_OFF, &P.tk, bar_kv, 0, j0, b, g * PN);
+    tc::tma_load_4d(base + SM::V_OFF, &P.tv, bar_kv, 0, j0, b, g * PN);
     if (slice < n_it) {
       load(&P.tq, base + SM::Q_OFF, bar_q, slice);
       load(&P.tdo, base + SM::DO_OFF, bar_do, slice);
@@ -445,9 +445,9 @@ void fill(const fbl_plan* p, FfmaAttnParams& P, int32_t* status) {
 static_assert(FfmaFwdSmem<128>::TOTAL <= ALONE && FfmaBwdSmem<float, 128>::TOTAL <= ALONE, "");
 
 template <typename T>
-bool encode(CUtensorMap* map, const void* base, int64_t r_pad, int cols, int rows, int hd) {
+bool encode(CUtensorMap* map, const void* base, int t_pad, int batch, int cols, int rows, int hd) {
   constexpr int TW = tile_w_of<T>::value;
-  return sizeof(T) == 4 ? fbl_encode_f32_rtile_map(map, base, r_pad, cols / TW, rows, hd / TW) : fbl_encode_rtile_map(map, base, r_pad, cols / TW, rows, hd / TW);
+  return fbl_encode_seq_map(map, sizeof(T) == 4, base, t_pad, batch, cols / TW, rows, hd / TW);
 }
 
 template <int HD>
@@ -457,8 +457,8 @@ cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   const uint32_t smem = spread(p, grid, (p->t_pad_kv + FWD_KEYS - 1) / FWD_KEYS, FfmaFwdSmem<HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
-  if (!encode<float>(&P.tq, Q, p->n_pad, p->dq, ROWS, HD) || !encode<float>(&P.tk, K, p->n_pad_kv, p->dkv, FWD_KEYS, HD) ||
-      !encode<float>(&P.tv, V, p->n_pad_kv, p->dkv, FWD_KEYS, HD))
+  if (!encode<float>(&P.tq, Q, p->t_pad, p->d.batch, p->dq, ROWS, HD) || !encode<float>(&P.tk, K, p->t_pad_kv, p->d.batch, p->dkv, FWD_KEYS, HD) ||
+      !encode<float>(&P.tv, V, p->t_pad_kv, p->d.batch, p->dkv, FWD_KEYS, HD))
     return cudaErrorInvalidValue;
   P.a = (float*)A; P.lse = lse;
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
@@ -484,8 +484,8 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   const uint32_t smem = slices > 1 ? FfmaBwdSmem<T, HD>::TOTAL : spread(p, grid, items, FfmaBwdSmem<T, HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
   fill(p, P, status);
-  if (!encode<T>(&P.tq, Q, p->n_pad, p->dq, QT, HD) || !encode<T>(&P.tdo, dA, p->n_pad, p->dq, QT, HD) ||
-      !encode<T>(&P.tk, K, p->n_pad_kv, p->dkv, ROWS, HD) || !encode<T>(&P.tv, V, p->n_pad_kv, p->dkv, ROWS, HD))
+  if (!encode<T>(&P.tq, Q, p->t_pad, p->d.batch, p->dq, QT, HD) || !encode<T>(&P.tdo, dA, p->t_pad, p->d.batch, p->dq, QT, HD) ||
+      !encode<T>(&P.tk, K, p->t_pad_kv, p->d.batch, p->dkv, ROWS, HD) || !encode<T>(&P.tv, V, p->t_pad_kv, p->d.batch, p->dkv, ROWS, HD))
     return cudaErrorInvalidValue;
   P.lse = const_cast<float*>(lse); P.dvec = dvec; P.dq = dQ; P.dk = dK; P.dv = dV;
   P.slices = slices;

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
   int slot_i, hb;
   decode_block((int)blockIdx.x, P.n_slots, P.hq * P.batch, P.chunk, &slot_i, &hb);
   const int h = hb % P.hq, b = hb / P.hq, g = h / P.group;
-  const int row0 = b * P.t_pad, row0k = b * P.t_pad_k;     // first row of this sequence on the query and key sides
+  const int row0 = b * P.t_pad;                            // first row of this sequence
   int32_t* status = P.status;
   // with pairing a block owns two adjacent tiles, whose key ranges differ by one tile, so both warp groups stay
   // busy for the whole loop
@@ -136,13 +136,13 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
     tc::tma_prefetch_desc(&P.tv);
     pdl_wait();
     tc::mbar_expect_tx(bar(B_QFULL), (qt1 >= 0 ? 2u : 1u) * SM::TILE);
-    tc::tma_load_3d(base + SM::Q_OFF, &P.tq, bar(B_QFULL), 0, row0 + qt0 * BQ, h * (int)PANELS);
-    if (qt1 >= 0) tc::tma_load_3d(base + SM::Q_OFF + SM::TILE, &P.tq, bar(B_QFULL), 0, row0 + qt1 * BQ, h * (int)PANELS);
+    tc::tma_load_4d(base + SM::Q_OFF, &P.tq, bar(B_QFULL), 0, qt0 * BQ, b, h * (int)PANELS);
+    if (qt1 >= 0) tc::tma_load_4d(base + SM::Q_OFF + SM::TILE, &P.tq, bar(B_QFULL), 0, qt1 * BQ, b, h * (int)PANELS);
     if (n_kv_max > 0) {
       tc::mbar_expect_tx(bar(B_KFULL), SM::TILE);
-      tc::tma_load_3d(base + SM::K_OFF, &P.tk, bar(B_KFULL), 0, row0k, g * (int)PANELS);
+      tc::tma_load_4d(base + SM::K_OFF, &P.tk, bar(B_KFULL), 0, 0, b, g * (int)PANELS);
       tc::mbar_expect_tx(bar(B_VFULL), SM::TILE);
-      tc::tma_load_3d(base + SM::V_OFF, &P.tv, bar(B_VFULL), 0, row0k, g * (int)PANELS);
+      tc::tma_load_4d(base + SM::V_OFF, &P.tv, bar(B_VFULL), 0, 0, b, g * (int)PANELS);
     }
   }
   if (warp == 1) {
@@ -163,10 +163,10 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
       const uint32_t ph = (j >> 1) & 1;
       if (!tc::mbar_wait(bar(B_KEMPTY + s), ph ^ 1, status, 201)) break;
       tc::mbar_expect_tx(bar(B_KFULL + s), SM::TILE);
-      tc::tma_load_3d(base + SM::K_OFF + s * SM::TILE, &P.tk, bar(B_KFULL + s), 0, row0k + j * BKV, g * (int)PANELS);
+      tc::tma_load_4d(base + SM::K_OFF + s * SM::TILE, &P.tk, bar(B_KFULL + s), 0, j * BKV, b, g * (int)PANELS);
       if (!tc::mbar_wait(bar(B_VEMPTY + s), ph ^ 1, status, 202)) break;
       tc::mbar_expect_tx(bar(B_VFULL + s), SM::TILE);
-      tc::tma_load_3d(base + SM::V_OFF + s * SM::TILE, &P.tv, bar(B_VFULL + s), 0, row0k + j * BKV, g * (int)PANELS);
+      tc::tma_load_4d(base + SM::V_OFF + s * SM::TILE, &P.tv, bar(B_VFULL + s), 0, j * BKV, b, g * (int)PANELS);
     }
   } else if (warp == 1 && lane == 0) {
     // ---- MMA issuer --------------------------------------------------------------------------
@@ -526,9 +526,9 @@ cudaError_t fwd_make(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, const void
   AttnFwdParams& P = L.P;
   memset(&P, 0, sizeof(P));
   const int panels = HD / 64;
-  if (!fbl_encode_rtile_map(&P.tq, Q, p->n_pad, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
-  if (!fbl_encode_rtile_map(&P.tk, K, p->n_pad_kv, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
-  if (!fbl_encode_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
+  if (!fbl_encode_seq_map(&P.tq, false, Q, p->t_pad, p->d.batch, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
+  if (!fbl_encode_seq_map(&P.tk, false, K, p->t_pad_kv, p->d.batch, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
+  if (!fbl_encode_seq_map(&P.tv, false, V, p->t_pad_kv, p->d.batch, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
   P.a = (__nv_bfloat16*)A; P.lse = lse; P.n_pad = p->n_pad;
   P.seq = p->d.seq; P.t_pad = p->t_pad; P.hq = p->d.n_q_heads; P.group = p->group; P.causal = p->d.causal;
   P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;

@@ -945,6 +945,19 @@ static bool encode_panels(CUtensorMap* map, CUtensorMapDataType type, int width,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool fbl_encode_seq_map(CUtensorMap* map, bool f32, const void* base, int rows, int seqs, int panels, int box_rows, int box_panels) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint32_t width = f32 ? 32 : 64;
+  cuuint64_t dims[4] = {width, (cuuint64_t)rows, (cuuint64_t)seqs, (cuuint64_t)panels};
+  cuuint64_t strides[3] = {128, (cuuint64_t)rows * 128, (cuuint64_t)rows * seqs * 128};
+  cuuint32_t box[4] = {width, (cuuint32_t)box_rows, 1, (cuuint32_t)box_panels};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool fbl_encode_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels) {
   return encode_panels(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, base, r_pad, panels, box_rows, box_panels);
 }

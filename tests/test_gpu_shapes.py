@@ -238,3 +238,36 @@ def test_few_rows_keep_fp32_probabilities(cfg):
         same = (rounded == heads(name, want.shape[1])).mean()
         print(name, same)
         assert same >= 0.97, (name, same)
+
+
+@pytest.mark.parametrize("cfg", [
+    # a key and a query tile that reach past a sequence: fp32 at each head width and beside a cluster, bf16 of few rows
+    LayerConfig("iso1", 3, 20, 64, 2, 1, 32, "fp32", "layernorm", True, True, True, 1e-5, 341, 0.2),
+    LayerConfig("iso2", 3, 77, 128, 4, 2, 64, "fp32", "rmsnorm", False, False, True, 1e-5, 342, 0.1),
+    LayerConfig("iso3", 3, 41, 128, 8, 1, 128, "fp32", "rmsnorm", True, False, False, 1e-5, 343, 0.1),
+    LayerConfig("iso4", 3, 30, 128, 4, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 344, 0.1),
+    LayerConfig("iso5", 3, 33, 128, 2, 2, 128, "bf16", "rmsnorm", False, False, True, 1e-5, 345, 0.1),
+    XattnConfig("iso6", 3, 9, 50, 128, 64, 2, 1, 64, "bf16", "layernorm", True, True, 1e-5, 346, 0.1),
+    XattnConfig("iso7", 3, 50, 70, 64, 96, 2, 2, 64, "fp32", "layernorm", True, True, 1e-5, 347, 0.1),
+], ids=lambda c: c.name)
+def test_values_that_are_not_finite_stay_in_their_sequence(cfg):
+    import numpy as np
+    from fbl_inputs import make_inputs, make_xattn_inputs
+    from paper_2607_21624_b200 import LayerRunner, XattnRunner
+    cross = isinstance(cfg, XattnConfig)
+    inp = (make_xattn_inputs if cross else make_inputs)(cfg)
+    run = (XattnRunner if cross else LayerRunner)(cfg)
+    names = ("Y", "dX", "dM") if cross else ("Y", "dX")
+    run.load_inputs(inp)
+    run.step()
+    plain = {n: run.fetch(n) for n in names}
+    for n in ("X", "M") if cross else ("X",):
+        inp[n][1] = np.inf
+    run.load_inputs(inp)
+    run.step()
+    assert run.status() == 0
+    for n in names:
+        got = run.fetch(n)
+        assert not np.isfinite(got[1]).any(), n
+        for b in (0, 2):                  # the same sums, in an order that dQ's additions may change in the last place
+            assert np.abs(got[b] - plain[n][b]).max() <= (1e-5 if cfg.dtype == "fp32" else 1e-2) * np.abs(plain[n][b]).max(), (n, b)
