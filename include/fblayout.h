@@ -293,6 +293,13 @@ int fbl_status_poll(const fbl_plan* plan, const void* scratch, int32_t* device_s
  * normal end). */
 int fbl_selftest_wait_timeout(void* scratch, int64_t limit_cycles, void* stream);
 
+/* Self-test of the kernels that start beside the launch in front of them (no counterpart in the paper): behind a kernel
+ * that lets its dependents start at once, and fills M ([rows, cols], bf16, 1024-byte aligned, rows a multiple of 8, cols of 64)
+ * with ones only about 0.2 ms later, enqueues the bias gradients' early column sums of M.  Nothing vouches for M then, so the
+ * sums have to wait: out[cols] is `rows` in every place.  scratch: 1024 bytes + fbl_colsum_scratch_bytes, 1024-byte aligned. */
+int fbl_selftest_early_order(const fbl_plan* plan, void* M_dev, int64_t rows, int64_t cols, float* out_dev, void* scratch_dev,
+                             void* stream);
+
 /* Host code only, for tests: the 64-wide reduction blocks [*begin, *end) that block `slice` of a cluster of `slices` blocks
  * works through where they share an output tile's reduction of `kblocks` (launches of few tiles and long reductions). */
 int fbl_gemm_slice_range(int kblocks, int slices, int slice, int* begin, int* end);

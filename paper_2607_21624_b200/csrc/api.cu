@@ -592,9 +592,9 @@ int fbl_layer_bwd(const fbl_plan* p, const void* dY, const void* X, const float*
       }
     }
     FBL_GEMM_STEP("dWqkv+dXn", gs, 4, FBL_GEMM_DWQKV_DXN);
-    if (early) FBL_STEP("db", 1, launch_colsum_early(p, sums, idle, st));
+    if (early) FBL_STEP("db", 1, launch_colsum_early(p, sums, idle, status, st));
   }
-  FBL_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials((float*)part, cp), st, &sums, &cg));
+  FBL_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials((float*)part, cp), status, st, &sums, &cg));
   return FBL_OK;
 }
 
@@ -626,6 +626,17 @@ int fbl_selftest_wait_timeout(void* scratch, int64_t limit_cycles, void* stream)
   cudaStream_t st = as_stream(stream);
   FBL_CUDA(cudaMemsetAsync(scratch, 0, 8, st));
   FBL_CUDA(launch_wait_timeout_selftest((int32_t*)scratch, (long long)limit_cycles, st));
+  return FBL_OK;
+}
+
+int fbl_selftest_early_order(const fbl_plan* plan, void* M, int64_t rows, int64_t cols, float* out, void* scratch, void* stream) {
+  if (!plan || plan->d.dtype != FBL_DTYPE_BF16 || !M || !out || !scratch || rows <= 0 || rows % 8 != 0 || cols <= 0 || cols % 64 != 0 ||
+      cols > 16384 || rows > 1 << 20)
+    return FBL_ERR_INVALID_ARG;
+  if (misaligned(M) || misaligned(scratch)) return FBL_ERR_MISALIGNED;
+  cudaStream_t st = as_stream(stream);
+  FBL_CUDA(cudaMemsetAsync(scratch, 0, FBL_ALIGN, st));
+  FBL_CUDA(launch_early_order_selftest(plan, M, rows, (int)cols, out, (int32_t*)scratch, (float*)((char*)scratch + FBL_ALIGN), st));
   return FBL_OK;
 }
 

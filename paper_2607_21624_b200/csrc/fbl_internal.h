@@ -110,8 +110,8 @@ struct GemmArgs {
   // later kernel of the pass; reset the pass's status word), and `serial`: the launch may not start before
   // everything ahead of it on the stream has completed
   void* zero_ptr; size_t zero_bytes; int reset_status, serial;
-  // likewise, where not null (tensor-core kernels; see launch_colsum_early): the next launch on the stream may start only
-  // once everything ahead of this one has completed; receives the clocks an SM is expected to stand idle before the
+  // likewise, where not null (tensor-core kernels; see launch_colsum_early): the launch raises FBL_EARLY_COLSUM and lets the next
+  // one start once everything ahead of it has completed; receives the clocks an SM is expected to stand idle before the
   // launch's slowest block ends, on average
   int* late_trigger;
   // fused activation of the feed-forward block (tensor-core kernel only): 0 none, 1 GELU forward (c = U, c2 = gelu(U)),
@@ -172,6 +172,10 @@ bool attn_bwd_tc_direct(const fbl_plan* p);    // the tensor-core backward write
 static inline size_t bwd_zero_bytes(const fbl_plan* p) {
   return attn_bwd_kernels(p) == ATTN_TC && attn_bwd_tc_direct(p) ? p->sb_dqacc : p->zero_bytes;
 }
+// Flags of pdl_early in the first block of the backward scratch, as offsets in words from the status word; a pass clears them
+// with it.  FBL_EARLY_COLSUM: from the last products to the column sums beside them; FBL_EARLY_ROUND: from the norm backward's
+// first kernel to the roundings beside it.
+enum { FBL_EARLY_COLSUM = 64, FBL_EARLY_ROUND = 128 };
 // What a backward pass starts with: zero the first `bytes` of its scratch (the status word's block and the fp32 areas the
 // pass adds into).  `rides`: the pass's first products `gs` need nothing of it.  `serial`: no kernel of the pass may start
 // before the forward pass has completed (the attention backward requests that pass's results before waiting for the kernel
@@ -224,9 +228,11 @@ static inline int64_t colsum_units(const fbl_plan* p, const ColsumGroup& G) {
 static inline bool colsum_early_pays(const fbl_plan* p, const ColsumGroup& G) {
   return G.count > 0 && 4 * colsum_units(p, G) > 9 * (int64_t)p->sm_count;
 }
-// The slabs' sums as a launch directly behind a tensor-core product launch with late_trigger (which gave `idle`), beside
-// which it runs: the matrices must have been complete before that product's launch.
-cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, cudaStream_t st);
+// The slabs' sums as a launch behind a tensor-core product launch with late_trigger (which gave `idle`), beside which it runs:
+// the matrices must come from launches in front of that one.  `status`: of both launches.
+cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, int32_t* status, cudaStream_t st);
+cudaError_t launch_early_order_selftest(const fbl_plan* p, void* M, int64_t rows, int cols, float* out, int32_t* status, float* part,
+                                        cudaStream_t st);
 // Where the norm's own partial rows begin, behind column-sum partials from `part` to `end`.
 static inline float* norm_partials(float* part, const float* end) { return part + (end - part + 255) / 256 * 256; }
 // fp32 sums of sliced products, to be rounded to their bf16 places (n multiples of 4).
@@ -234,7 +240,7 @@ struct ConvertGroup { const float* src[4]; void* dst[4]; int64_t n[4]; int count
 // Norm backward with the column sums of `sums` and the roundings of `round`; counts its own launches in p->launches (one to
 // three).
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
-                            const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
+                            const float* gamma, void* dX, float* dgamma, float* dbeta, float* part, int32_t* status,
                             cudaStream_t st, const ColsumGroup* sums = nullptr, const ConvertGroup* round = nullptr);
 cudaError_t launch_colsum(int dtype, const void* M, int64_t rows, int64_t cols, float* out, float* partials,
                           cudaStream_t st);

@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn
                                                        T* __restrict__ dX, float* __restrict__ partials, int64_t n_pad, int d,
                                                        int tpr, int64_t per_block, int rms, int n_norm,
                                                        const __grid_constant__ ColsumGroup CG, int cs_panels, int cs_slabs,
-                                                       int late) {
+                                                       int32_t* __restrict__ late) {
   constexpr int V = Vec16<T>::N, TW = tile_w_of<T>::value;
   // exchange buffers of the row sums; the column-sum blocks use it as well
   __shared__ __align__(16) float s_ex[16 * (TW + 1) > 2 * NORM_EX ? 16 * (TW + 1) : 2 * NORM_EX];
@@ -404,13 +404,13 @@ __global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn
   if ((int)blockIdx.x >= n_norm) {
     if (!late) pdl_launch_dependents();
     pdl_wait();
-    if (late) pdl_launch_dependents();
+    if (late && threadIdx.x == 0) pdl_launch_dependents();
     const int idx = (int)blockIdx.x - n_norm;
     colsum_slab<T>(CG, idx % cs_panels, (idx / cs_panels) % cs_slabs, idx / (cs_panels * cs_slabs),
                    reinterpret_cast<float(*)[TW + 1]>(s_ex));
     return;
   }
-  if (!late) pdl_launch_dependents();                        // late: what the second kernel rounds is complete when it starts
+  if (!late) pdl_launch_dependents();                        // late: the flag under which the second kernel rounds beside this one
   const int group = threadIdx.x / tpr, lt = threadIdx.x % tpr, groups = blockDim.x / tpr;
   const float inv_d = 1.f / (float)d;
   int buf = 0;
@@ -425,7 +425,10 @@ __global__ void __launch_bounds__(512) norm_bwd_kernel(const T* __restrict__ dXn
     for (int i = 0; i < V / 2; ++i) ag[j][i] = ab[j][i] = both(0.f);
   }
   pdl_wait();
-  if (late) pdl_launch_dependents();
+  if (late && threadIdx.x == 0) {
+    if (blockIdx.x == 0) pdl_raise(late);
+    pdl_launch_dependents();
+  }
   constexpr int S = norm_stages(R, NV);
   extern __shared__ __align__(16) uint8_t s_ring[];          // [stage][X, dXn, (dY)][row][vector][thread]
   const int arrays = dY ? 3 : 2;
@@ -598,15 +601,16 @@ __global__ void __launch_bounds__(256) rope_kernel(T* __restrict__ A, int heads_
 // dgamma[c] (y = 0) or dbeta[c] (y = 1) = sum over the first kernel's blocks of their partial rows.  Blocks with
 // y >= ny_norm finish the bias column sums instead (matrix y - ny_norm: the tree over its slab partials), so that
 // the step's two small final reductions share one launch.  Blocks behind those (y >= ny_sums) round the fp32 sums of sliced
-// products, which are complete when this kernel starts: beside the first kernel, whose end they wait for only at their own
-// (four 768 x 768 matrices: a launch of 10 us in a step of 191 us before).
+// products, which launches in front of the first kernel left: beside that one (pdl_early), whose end they wait for only at
+// their own (four 768 x 768 matrices: a launch of 10 us in a step of 191 us before).
 __global__ void __launch_bounds__(256) norm_bwd_reduce_kernel(const float* __restrict__ part, int blocks, int d,
                                                               float* __restrict__ dgamma, float* __restrict__ dbeta,
                                                               int ny_norm, const __grid_constant__ ColsumGroup G, int ny_sums,
-                                                              const __grid_constant__ ConvertGroup C) {
+                                                              const __grid_constant__ ConvertGroup C, int32_t* early) {
   __shared__ float red[8][33];
   pdl_launch_dependents();
   if ((int)blockIdx.y >= ny_sums) {
+    pdl_early(early);
     const int64_t first = ((int64_t)((blockIdx.y - ny_sums) * gridDim.x + blockIdx.x) * 256 + threadIdx.x) * 4;
     const int64_t step = (int64_t)(gridDim.y - ny_sums) * gridDim.x * 1024;
     for (int k = 0; k < C.count; ++k) {
@@ -621,6 +625,7 @@ __global__ void __launch_bounds__(256) norm_bwd_reduce_kernel(const float* __res
       }
     }
     pdl_wait();
+    if (blockIdx.x == 0 && (int)blockIdx.y == ny_sums && threadIdx.x == 0) pdl_lower(early);
     return;
   }
   pdl_wait();
@@ -669,17 +674,17 @@ __global__ void __launch_bounds__(256) colsum_stage1(const __grid_constant__ Col
   colsum_slab<T>(G, blockIdx.x, blockIdx.y, blockIdx.z, red);
 }
 
-// The same sums beside a tensor-core product: that kernel starts its dependents only after its own wait, so everything in
-// front of it, the matrices among it, is complete when this one runs; the wait for the product comes last, for the kernels
-// behind this one.  A block takes a slab of a panel at a time; small as it is, and with at most one per SM, it fits beside
+// The same sums beside a tensor-core product, of matrices that launches in front of that one left (pdl_early); the wait for the
+// product comes last, for the kernels behind this one.  A block takes a slab of a panel at a time; small as it is, and with at most one per SM, it fits beside
 // a product block.  Loads go to L2, whose data is current.  Bound by memory, and hidden by the product:
 // 2048 x 768 and 2048 x 3072 cost 5 us of a step of 114 us in a launch of their own; two of 3000 x 1280, with their
 // second stage, 7 us of 199 us.
-__global__ void __launch_bounds__(128, 8) colsum_early_kernel(const __grid_constant__ ColsumGroup G) {
+__global__ void __launch_bounds__(128, 8) colsum_early_kernel(const __grid_constant__ ColsumGroup G, int32_t* early) {
   using T = __nv_bfloat16;
   constexpr int TW = tile_w_of<T>::value, V = Vec16<T>::N, B = 8, STEP = 16 * B;
   __shared__ __align__(16) float red[3][TW];                            // 768 bytes: a product block leaves 1.9 KB, 1 KB of it reserved
   pdl_launch_dependents();
+  pdl_early(early);
   const int warp = threadIdx.x / 32, rr = threadIdx.x / 8, l8 = threadIdx.x % 8;
   // position of the next batch of 128 rows: unit (panel of a slab of a matrix), and its first row of this thread
   int which = -1, left = (int)blockIdx.x, units = 0;
@@ -744,6 +749,7 @@ __global__ void __launch_bounds__(128, 8) colsum_early_kernel(const __grid_const
     }
   }
   pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) pdl_lower(early);
 }
 
 template <typename T, int NV, int PF, int TPR>
@@ -762,7 +768,7 @@ cudaError_t norm_fwd_launch(const fbl_plan* p, const NormShape& s, const void* X
 template <typename T, int NV, int R>
 cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* dXn, const void* X, const void* dY,
                             const float* stats, const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
-                            const ColsumGroup& cg, const ConvertGroup& round, cudaStream_t st) {
+                            int32_t* status, const ColsumGroup& cg, const ConvertGroup& round, cudaStream_t st) {
   constexpr int V = Vec16<T>::N;
   const int d = p->d.d_model, rms = p->d.norm == FBL_NORM_RMSNORM;
   const int64_t pass = (int64_t)s.groups * R;
@@ -792,7 +798,7 @@ cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* d
   if (e != cudaSuccess) return e;
   e = launch_pdl(norm_bwd_kernel<T, NV, R>, dim3(blocks + cs_blocks), dim3(s.tpr * s.groups), smem, st,
                              (const T*)dXn, (const T*)X, (const T*)dY, stats, gamma, (T*)dX, dgamma ? part : (float*)nullptr, p->n_pad,
-                             d, s.tpr, per_block, rms, blocks, cg, cs_panels, n_slabs, (int)(round.count > 0));
+                             d, s.tpr, per_block, rms, blocks, cg, cs_panels, n_slabs, round.count > 0 ? status + FBL_EARLY_ROUND : nullptr);
   if (e != cudaSuccess) return e;
   const int ny = !dgamma ? 0 : rms ? 1 : 2;
   const int nx = (d + 31) / 32, ny_sums = ny + cg.count;
@@ -802,7 +808,7 @@ cudaError_t norm_bwd_launch(const fbl_plan* p, const NormShape& s, const void* d
   p->launches += ny_sums + ny_round == 0 ? 1 : 2;
   if (ny_sums + ny_round == 0) return cudaSuccess;
   return launch_pdl(norm_bwd_reduce_kernel, dim3(nx, ny_sums + ny_round), dim3(256), 0, st, (const float*)part,
-                    blocks, d, dgamma, dbeta, ny, cg, ny_sums, round);
+                    blocks, d, dgamma, dbeta, ny, cg, ny_sums, round, status + FBL_EARLY_ROUND);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -893,10 +899,10 @@ cudaError_t launch_norm_fwd(const fbl_plan* p, const void* X, const float* gamma
 
 template <typename T>
 cudaError_t norm_bwd_dispatch(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
-                              const float* gamma, void* dX, float* dgamma, float* dbeta, float* npart,
+                              const float* gamma, void* dX, float* dgamma, float* dbeta, float* npart, int32_t* status,
                               const ColsumGroup& cg, const ConvertGroup& round, cudaStream_t st) {
   const NormShape s = norm_bwd_shape(p->d.d_model / Vec16<T>::N, p->n_pad, p->sm_count);
-#define FBL_CALL(NV_, R_) norm_bwd_launch<T, NV_, R_>(p, s, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, cg, round, st)
+#define FBL_CALL(NV_, R_) norm_bwd_launch<T, NV_, R_>(p, s, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, npart, status, cg, round, st)
   switch (s.nv) {
     case 1: return s.r == 4 ? FBL_CALL(1, 4) : s.r == 2 ? FBL_CALL(1, 2) : FBL_CALL(1, 1);
     case 2: return s.r == 2 ? FBL_CALL(2, 2) : FBL_CALL(2, 1);
@@ -937,7 +943,7 @@ void colsum_add(ColsumGroup& G, const void* m, int64_t rows, int cols, float* ou
   *part += (int64_t)G.slabs[i] * cols;
 }
 
-cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, cudaStream_t st) {
+cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, int32_t* status, cudaStream_t st) {
   int64_t bytes = 0;
   for (int i = 0; i < G.count; ++i) bytes += G.rows[i] * G.cols[i] * 2;
   // Where the product's SMs run out of work at different times, those that have (some 13 bytes/clk each) do the sums, and
@@ -947,21 +953,42 @@ cudaError_t launch_colsum_early(const fbl_plan* p, ColsumGroup& G, int idle, cud
   const bool beside = (int64_t)idle * p->sm_count * 13 < bytes;
   const dim3 grid((unsigned)min((int64_t)p->sm_count, colsum_units(p, G)));
   G.summed = 1;
-  return launch_pdl(colsum_early_kernel, grid, dim3(128), beside ? 0 : 2048, st, G);
+  return launch_pdl(colsum_early_kernel, grid, dim3(128), beside ? 0 : 2048, st, G, status + FBL_EARLY_COLSUM);
+}
+
+// Self-test of pdl_early: a kernel that lets its dependents start at once and writes what they read only after `clocks`.
+static __global__ void __launch_bounds__(256) slow_fill_kernel(uint4* __restrict__ out, int64_t n, uint4 v, long long clocks) {
+  pdl_launch_dependents();
+  pdl_wait();
+  for (const long long t0 = clock64(); clock64() - t0 < clocks;) {}
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = v;
+}
+
+cudaError_t launch_early_order_selftest(const fbl_plan* p, void* M, int64_t rows, int cols, float* out, int32_t* status, float* part,
+                                        cudaStream_t st) {
+  const uint32_t ones = 0x3f803f80u;                                    // two bf16 ones
+  const cudaError_t e = launch_pdl(slow_fill_kernel, dim3(8), dim3(256), 0, st, (uint4*)M, rows * cols / 8,
+                                   make_uint4(ones, ones, ones, ones), 400000ll);
+  if (e != cudaSuccess) return e;
+  ColsumGroup G = {};
+  colsum_add(G, M, rows, cols, out, &part);
+  const cudaError_t f = launch_colsum_early(p, G, 0, status, st);
+  if (f != cudaSuccess) return f;
+  return launch_pdl(colsum_stage2, dim3((unsigned)((cols + 127) / 128), 1), dim3(128), 0, st, G);
 }
 
 // Norm backward (dgamma = nullptr: only dX, the norm's parameters are frozen), and with it the bias column sums of up to
 // four matrices: their first stage, unless it ran beside the product in front, as extra blocks of the first kernel, their
 // second stage inside the second.  `part`: the norm's per-block partial rows.
 cudaError_t launch_norm_bwd(const fbl_plan* p, const void* dXn, const void* X, const void* dY, const float* stats,
-                            const float* gamma, void* dX, float* dgamma, float* dbeta, float* part,
+                            const float* gamma, void* dX, float* dgamma, float* dbeta, float* part, int32_t* status,
                             cudaStream_t st, const ColsumGroup* sums, const ConvertGroup* round) {
   ColsumGroup cg = {};
   ConvertGroup rg = {};
   if (round) rg = *round;
   if (sums) cg = *sums;
-  if (p->d.dtype == FBL_DTYPE_FP32) return norm_bwd_dispatch<float>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, rg, st);
-  return norm_bwd_dispatch<__nv_bfloat16>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, cg, rg, st);
+  if (p->d.dtype == FBL_DTYPE_FP32) return norm_bwd_dispatch<float>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, status, cg, rg, st);
+  return norm_bwd_dispatch<__nv_bfloat16>(p, dXn, X, dY, stats, gamma, dX, dgamma, dbeta, part, status, cg, rg, st);
 }
 
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols) {

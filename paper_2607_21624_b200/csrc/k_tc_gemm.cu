@@ -65,13 +65,19 @@ struct alignas(64) TcGroup {
 };
 
 __device__ __forceinline__ void group_chores(const TcGroup& G, int tid, int n_threads) {
-  if (G.reset_status && blockIdx.x == 0 && tid == 0) *G.status = 0;
+  if (G.reset_status && blockIdx.x == 0 && tid == 0) *G.status = G.status[FBL_EARLY_COLSUM] = G.status[FBL_EARLY_ROUND] = 0;
   if (G.zero_vec > 0) {
     const long long per = (G.zero_vec + gridDim.x - 1) / gridDim.x;
     const long long lo = (long long)blockIdx.x * per, hi = min(G.zero_vec, lo + per);
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
     for (long long i = lo + tid; i < hi; i += n_threads) G.zero_ptr[i] = z;
   }
+}
+
+// By the producer thread, after its pdl_wait(): whatever precedes the launch is complete for who sees the flag.
+__device__ __forceinline__ void late_trigger(const TcGroup& G) {
+  if (blockIdx.x == 0) pdl_raise(G.status + FBL_EARLY_COLSUM);
+  pdl_launch_dependents();
 }
 
 template <int BN, int STAGES>
@@ -448,7 +454,7 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
       prefilled = n;
     }
     pdl_wait();
-    if (G.late_trigger) pdl_launch_dependents();
+    if (G.late_trigger) late_trigger(G);
     for (int w = blockIdx.x; ok && tile_at<BN>(G, w, &tcd); w += gridDim.x) {
       const TcProblem& P = G.p[tcd.prob];
       for (int t = 0; t < P.n_terms && ok; ++t) {
@@ -621,7 +627,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
     bool ok = true;
     TileCoord tcd;
     pdl_wait();
-    if (G.late_trigger) pdl_launch_dependents();
+    if (G.late_trigger) late_trigger(G);
     for (int w = pair_id; ok && pair_tile_at(G, w, &tcd); w += n_pairs) {
       const TcProblem& P = G.p[tcd.prob];
       const int m0 = tcd.m0 + (int)rank * 128, n0 = tcd.n0 + (int)rank * 128;
@@ -783,7 +789,7 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
         }
       }
       pdl_wait();
-      if (G.late_trigger) pdl_launch_dependents();
+      if (G.late_trigger) late_trigger(G);
       int t = 0, first = 0;                              // term of the k-block, and its first k-block
       for (int k = begin, it = 0; k < end; ++k, ++it) {
         while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }

@@ -268,7 +268,7 @@ int fbl_layer_bwd_lora(const fbl_plan* p, const void* dY, const void* X, const f
     LORA_STEP("dB+dXn+dA", 0, cudaSuccess);
     p->launches += k;
   }
-  LORA_STEP("norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, st));
+  LORA_STEP("norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, part, status, st));
   return FBL_OK;
 }
 

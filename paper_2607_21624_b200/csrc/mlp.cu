@@ -447,9 +447,9 @@ int fbl_mlp_bwd(const fbl_mlp_plan* p, const void* dY, const void* X, const floa
     if (early) gs[0].late_trigger = &idle;
     MLP_CUDA(run_gemm_group(bp, gs, nw + 1, status, st, -1, &k));
     p->launches += k;
-    if (early) MLP_STEP(1, launch_colsum_early(bp, sums, idle, st));
+    if (early) MLP_STEP(1, launch_colsum_early(bp, sums, idle, status, st));
   }
-  MLP_STEP(0, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums, &cg));
+  MLP_STEP(0, launch_norm_bwd(bp, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), status, st, &sums, &cg));
   return FBL_OK;
 }
 

@@ -210,7 +210,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     if (bias && tc) {
       colsum_add(sums, dK, p->n_pad_kv, p->dkv, dbk, &part_kv);
       colsum_add(sums, dV, p->n_pad_kv, p->dkv, dbv, &part_kv);
-      XA_STEP("db", 1, launch_colsum_early(p, sums, idle, st));
+      XA_STEP("db", 1, launch_colsum_early(p, sums, idle, status, st));
     }
   }
   if (bias && !sums.summed) {
@@ -219,7 +219,7 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
     colsum_add(kv, dV, p->n_pad_kv, p->dkv, dbv, &part_kv);
     XA_STEP("db_kv", 2, launch_colsum_group(p->d.dtype, kv, st));
   }
-  XA_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), st, &sums, &cg));
+  XA_STEP(bias ? "db+norm_bwd" : "norm_bwd", 0, launch_norm_bwd(p, dXn, X, p->d.residual ? dY : nullptr, stats, gamma, dX, dgamma, dbeta, norm_partials(part, cp), status, st, &sums, &cg));
   return FBL_OK;
 }
 

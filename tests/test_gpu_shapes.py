@@ -271,3 +271,22 @@ def test_values_that_are_not_finite_stay_in_their_sequence(cfg):
         assert not np.isfinite(got[1]).any(), n
         for b in (0, 2):                  # the same sums, in an order that dQ's additions may change in the last place
             assert np.abs(got[b] - plain[n][b]).max() <= (1e-5 if cfg.dtype == "fp32" else 1e-2) * np.abs(plain[n][b]).max(), (n, b)
+
+
+@pytest.mark.parametrize("rows,cols", [(8, 64), (2048, 768), (1000, 4096)])
+def test_early_sums_wait_behind_a_launch_that_vouches_for_nothing(rows, cols):
+    import ctypes as C
+    import torch
+    from paper_2607_21624_b200.binding import Plan, _check, aligned_bytes, desc_from_config, lib
+    plan = Plan(desc_from_config(LayerConfig("eo", 1, 64, 64, 1, 1, 64, "bf16", "layernorm", True, True, False, 1e-5, 0, 0.02)))
+    fn = lib().fbl_selftest_early_order
+    fn.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p]
+    dev = torch.device("cuda:0")
+    m = aligned_bytes(torch, rows * cols * 2, dev)
+    scratch = aligned_bytes(torch, 1024 + plan.colsum_scratch_bytes(rows, cols), dev)
+    out = torch.zeros(cols, device=dev)
+    for _ in range(3):
+        m.zero_()
+        out.zero_()
+        _check(fn(plan._h, m.data_ptr(), rows, cols, out.data_ptr(), scratch.data_ptr(), torch.cuda.current_stream().cuda_stream))
+        assert (out == rows).all()
