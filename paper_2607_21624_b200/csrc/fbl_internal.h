@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "fblayout.h"
 
 #define FBL_TILE_H 8
@@ -78,6 +80,7 @@ struct fbl_plan {
   // event timing.  Calls on one plan are not thread-safe; give each host thread its own plan.
   mutable int64_t launches;
   mutable FblMemoBase* memo[FBL_MEMO_COUNT];
+  mutable std::mutex memo_lock;
   mutable int prof_on, prof_n;
   mutable cudaEvent_t prof_ev[FBL_PROF_MAX + 1];
   mutable const char* prof_name[FBL_PROF_MAX];

@@ -434,12 +434,12 @@ uint32_t spread(const fbl_plan* p, const dim3& grid, int items, uint32_t smem) {
   return per_sm == 1 || (per_sm <= 3 && items >= 4) ? std::max(smem, (uint32_t)(228 * 1024 / (per_sm + 1))) : smem;
 }
 
-typedef LaunchMemo<FfmaAttnParams, 8, 12> AttnMemo;
+typedef LaunchMemo<FfmaAttnParams, 4> AttnMemo;
 
-void fill(const fbl_plan* p, FfmaAttnParams& P, int32_t* status) {
+void fill(const fbl_plan* p, FfmaAttnParams& P) {
   memset(&P, 0, sizeof(P));
   P.n_pad = p->n_pad; P.n_pad_k = p->n_pad_kv; P.seq = p->d.seq; P.t_pad = p->t_pad; P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;
-  P.hq = p->d.n_q_heads; P.group = p->group; P.causal = p->d.causal; P.scale = p->scale; P.status = status;
+  P.hq = p->d.n_q_heads; P.group = p->group; P.causal = p->d.causal; P.scale = p->scale;
 }
 
 static_assert(FfmaFwdSmem<128>::TOTAL <= ALONE && FfmaBwdSmem<float, 128>::TOTAL <= ALONE, "");
@@ -456,17 +456,20 @@ cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   const dim3 grid((p->t_pad + ROWS - 1) / ROWS, p->d.n_q_heads, p->d.batch);
   const uint32_t smem = spread(p, grid, (p->t_pad_kv + FWD_KEYS - 1) / FWD_KEYS, FfmaFwdSmem<HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
-  fill(p, P, status);
-  if (!encode<float>(&P.tq, Q, p->t_pad, p->d.batch, p->dq, ROWS, HD) || !encode<float>(&P.tk, K, p->t_pad_kv, p->d.batch, p->dkv, FWD_KEYS, HD) ||
-      !encode<float>(&P.tv, V, p->t_pad_kv, p->d.batch, p->dkv, FWD_KEYS, HD))
-    return cudaErrorInvalidValue;
-  P.a = (float*)A; P.lse = lse;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
+    fill(p, P);
+    if (!encode<float>(&P.tq, Q, p->t_pad, p->d.batch, p->dq, ROWS, HD) || !encode<float>(&P.tk, K, p->t_pad_kv, p->d.batch, p->dkv, FWD_KEYS, HD) ||
+        !encode<float>(&P.tv, V, p->t_pad_kv, p->d.batch, p->dkv, FWD_KEYS, HD))
+      return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
+  };
+  auto point = [&](FfmaAttnParams& P) {
+    P.a = (float*)A; P.lse = lse; P.status = status;
+    return fbl_map_set_base(&P.tq, Q) && fbl_map_set_base(&P.tk, K) && fbl_map_set_base(&P.tv, V);
   };
   LaunchKey key;
-  for (const void* q : {Q, K, V, (const void*)A, (const void*)lse, (const void*)status}) key.add(q);
-  return AttnMemo::run(p->memo[FBL_MEMO_FFMA_ATTN], key, make, [&](const FfmaAttnParams& P) {
-  return launch_pdl(k, grid, dim3(THREADS), smem, st, P);
+  key.add(0, 0);                                           // the forward; the rest is the plan's
+  return AttnMemo::run(p, FBL_MEMO_FFMA_ATTN, key, make, point, [&](const FfmaAttnParams& P) {
+    return launch_pdl(k, grid, dim3(THREADS), smem, st, P);
   });
 }
 
@@ -483,19 +486,21 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
   const dim3 grid(key_tiles * slices, p->d.n_kv_heads, p->d.batch);
   const uint32_t smem = slices > 1 ? FfmaBwdSmem<T, HD>::TOTAL : spread(p, grid, items, FfmaBwdSmem<T, HD>::TOTAL);
   auto make = [&](FfmaAttnParams& P) {
-  fill(p, P, status);
-  if (!encode<T>(&P.tq, Q, p->t_pad, p->d.batch, p->dq, QT, HD) || !encode<T>(&P.tdo, dA, p->t_pad, p->d.batch, p->dq, QT, HD) ||
-      !encode<T>(&P.tk, K, p->t_pad_kv, p->d.batch, p->dkv, ROWS, HD) || !encode<T>(&P.tv, V, p->t_pad_kv, p->d.batch, p->dkv, ROWS, HD))
-    return cudaErrorInvalidValue;
-  P.lse = const_cast<float*>(lse); P.dvec = dvec; P.dq = dQ; P.dk = dK; P.dv = dV;
-  P.slices = slices;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
+    fill(p, P);
+    if (!encode<T>(&P.tq, Q, p->t_pad, p->d.batch, p->dq, QT, HD) || !encode<T>(&P.tdo, dA, p->t_pad, p->d.batch, p->dq, QT, HD) ||
+        !encode<T>(&P.tk, K, p->t_pad_kv, p->d.batch, p->dkv, ROWS, HD) || !encode<T>(&P.tv, V, p->t_pad_kv, p->d.batch, p->dkv, ROWS, HD))
+      return cudaErrorInvalidValue;
+    P.slices = slices;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ALONE);
+  };
+  auto point = [&](FfmaAttnParams& P) {
+    P.lse = const_cast<float*>(lse); P.dvec = dvec; P.dq = dQ; P.dk = dK; P.dv = dV; P.status = status;
+    return fbl_map_set_base(&P.tq, Q) && fbl_map_set_base(&P.tdo, dA) && fbl_map_set_base(&P.tk, K) && fbl_map_set_base(&P.tv, V);
   };
   LaunchKey key;
-  for (const void* q : {Q, K, V, dA, (const void*)lse, (const void*)dvec, (const void*)dQ, (const void*)dK, (const void*)dV, (const void*)status})
-    key.add(q);
-  return AttnMemo::run(p->memo[FBL_MEMO_FFMA_ATTN], key, make, [&](const FfmaAttnParams& P) {
-  return slices > 1 ? launch_cluster(k, grid, dim3(THREADS), smem, st, slices, true, P) : launch_pdl(k, grid, dim3(THREADS), smem, st, P);
+  key.add(1, 0);                                           // the backward
+  return AttnMemo::run(p, FBL_MEMO_FFMA_ATTN, key, make, point, [&](const FfmaAttnParams& P) {
+    return slices > 1 ? launch_cluster(k, grid, dim3(THREADS), smem, st, slices, true, P) : launch_pdl(k, grid, dim3(THREADS), smem, st, P);
   });
 }
 

@@ -287,12 +287,10 @@ bool gemm_ffma_supported(const fbl_plan* p, const GemmArgs& g) {
   return true;
 }
 
-static cudaError_t make_group(FfmaLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status) {
+static cudaError_t make_group(FfmaLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count) {
   FfmaGroup& G = L.G;
   memset(&G, 0, sizeof(G));
   G.count = count;
-  G.status = status;
-  G.zero_ptr = (uint4*)gs[0].zero_ptr; G.zero_vec = (long long)(gs[0].zero_bytes / 16); G.reset_status = gs[0].reset_status;
   int tiles = 0;
   for (int i = 0; i < count; ++i) {
     const GemmArgs& g = gs[i];
@@ -309,9 +307,7 @@ static cudaError_t make_group(FfmaLaunch& L, const fbl_plan* p, const GemmArgs* 
         return cudaErrorInvalidValue;
     }
     P.tiles_m = (g.m + BM - 1) / BM; P.tiles_n = (g.n + BN - 1) / BN;
-    P.c = (float*)g.c; P.c_rpad = g.c_rpad; P.bias = g.bias; P.residual = (const float*)g.residual;
-    P.seq = g.seq; P.t_pad = g.t_pad;
-    P.dot_with = (const float*)g.dot_with; P.dot_out = g.dot_out; P.dot_hd = g.dot_hd; P.dot_hq = g.dot_hq;
+    P.c_rpad = g.c_rpad; P.seq = g.seq; P.t_pad = g.t_pad; P.dot_hd = g.dot_hd; P.dot_hq = g.dot_hq;
     tiles += P.tiles_m * P.tiles_n;
   }
   G.slices = choose_slices(p->sm_count, G);
@@ -322,12 +318,27 @@ static cudaError_t make_group(FfmaLaunch& L, const fbl_plan* p, const GemmArgs* 
   return cudaFuncSetAttribute(gemm_ffma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem::TOTAL);
 }
 
+static bool point_group(FfmaGroup& G, const GemmArgs* gs, int32_t* status) {
+  G.status = status;
+  G.zero_ptr = (uint4*)gs[0].zero_ptr; G.zero_vec = (long long)(gs[0].zero_bytes / 16); G.reset_status = gs[0].reset_status;
+  bool ok = true;
+  for (int i = 0; i < G.count; ++i) {
+    const GemmArgs& g = gs[i];
+    FfmaProblem& P = G.p[i];
+    for (int t = 0; t < P.n_terms; ++t) ok = ok && fbl_map_set_base(&P.ta[t], g.t[t].a) && fbl_map_set_base(&P.tb[t], g.t[t].b);
+    P.c = (float*)g.c; P.bias = g.bias; P.residual = (const float*)g.residual;
+    P.dot_with = (const float*)g.dot_with; P.dot_out = g.dot_out;
+  }
+  return ok;
+}
+
 cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st) {
   if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
   LaunchKey key;
-  gemm_group_key(key, gs, count, status);
-  return LaunchMemo<FfmaLaunch, 12, 248>::run(p->memo[FBL_MEMO_FFMA_GEMM], key,
-      [&](FfmaLaunch& L) { return make_group(L, p, gs, count, status); },
+  gemm_group_key(key, gs, count);
+  return LaunchMemo<FfmaLaunch, 12>::run(p, FBL_MEMO_FFMA_GEMM, key,
+      [&](FfmaLaunch& L) { return make_group(L, p, gs, count); },
+      [&](FfmaLaunch& L) { return point_group(L.G, gs, status); },
       [&](const FfmaLaunch& L) {
         if (L.G.slices > 1) return launch_cluster(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G.slices, !L.serial, L.G);
         return L.serial ? launch_serial(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G)

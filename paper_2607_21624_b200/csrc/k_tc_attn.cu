@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
   if (warp == 1) tc::tmem_dealloc(tmem_base, TMEM_COLS);
 }
 
-// A launch made ready: what the launchers remember.
+// A launch made ready but for its addresses: what the launchers keep.
 template <typename Params>
 struct AttnLaunch {
   Params P;
@@ -521,18 +521,17 @@ cudaError_t fwd_make_t(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, int n_qt
 }
 
 template <int HD>
-cudaError_t fwd_make(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
-                     int32_t* status) {
+cudaError_t fwd_make(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, const void* Q, const void* K, const void* V) {
   AttnFwdParams& P = L.P;
   memset(&P, 0, sizeof(P));
   const int panels = HD / 64;
   if (!fbl_encode_seq_map(&P.tq, false, Q, p->t_pad, p->d.batch, p->dq / 64, BQ, panels)) return cudaErrorInvalidValue;
   if (!fbl_encode_seq_map(&P.tk, false, K, p->t_pad_kv, p->d.batch, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
   if (!fbl_encode_seq_map(&P.tv, false, V, p->t_pad_kv, p->d.batch, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
-  P.a = (__nv_bfloat16*)A; P.lse = lse; P.n_pad = p->n_pad;
+  P.n_pad = p->n_pad;
   P.seq = p->d.seq; P.t_pad = p->t_pad; P.hq = p->d.n_q_heads; P.group = p->group; P.causal = p->d.causal;
   P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;
-  P.scale = p->scale; P.status = status;
+  P.scale = p->scale;
   const int n_qt = (p->d.seq + BQ - 1) / BQ;
   // two query tiles per block when that still leaves at least one block per SM
   P.pair = (n_qt >= 2 && (long long)((n_qt + 1) / 2) * p->d.n_q_heads * p->d.batch >= p->sm_count) ? 1 : 0;
@@ -1471,7 +1470,7 @@ cudaError_t bwd_make_t(AttnLaunch<AttnBwdParams>& L, const fbl_plan* p) {
 
 template <int HD>
 cudaError_t bwd_make(AttnLaunch<AttnBwdParams>& L, const fbl_plan* p, const void* Q, const void* K, const void* V, const void* dA,
-                     const float* lse, const float* dvec, float* dqacc, void* dQ, void* dK, void* dV, int32_t* status) {
+                     float* dqacc) {
   AttnBwdParams& P = L.P;
   memset(&P, 0, sizeof(P));
   const int panels = HD / 64;
@@ -1481,9 +1480,8 @@ cudaError_t bwd_make(AttnLaunch<AttnBwdParams>& L, const fbl_plan* p, const void
   if (!fbl_encode_rtile_map(&P.tv, V, p->n_pad_kv, p->dkv / 64, BKV, panels)) return cudaErrorInvalidValue;
   const bool direct = attn_bwd_tc_direct(p);
   if (!direct && !fbl_encode_f32_panel_map(&P.tdq, dqacc, p->n_pad, p->dq / 64, BQ)) return cudaErrorInvalidValue;
-  P.lse = lse; P.dvec = dvec; P.dqacc = dqacc; P.dq = (__nv_bfloat16*)dQ; P.dk = (__nv_bfloat16*)dK; P.dv = (__nv_bfloat16*)dV;
   P.n_pad = p->n_pad; P.seq = p->d.seq; P.t_pad = p->t_pad; P.hq = p->d.n_q_heads; P.group = p->group;
-  P.causal = p->d.causal; P.dkv = p->dkv; P.scale = p->scale; P.status = status;
+  P.causal = p->d.causal; P.dkv = p->dkv; P.scale = p->scale;
   P.n_pad_k = p->n_pad_kv; P.seq_k = p->seq_kv; P.t_pad_k = p->t_pad_kv;
   P.batch = p->d.batch;
   if (!direct) return bwd_make_t<HD, false>(L, p);
@@ -1503,11 +1501,11 @@ bool attn_bwd_tc_direct(const fbl_plan* p) {
 cudaError_t launch_attn_fwd_tc(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                int32_t* status, cudaStream_t st) {
   typedef AttnLaunch<AttnFwdParams> Launch;
-  LaunchKey key;
-  for (const void* q : {Q, K, V, (const void*)A, (const void*)lse, (const void*)status}) key.add(q);
-  return LaunchMemo<Launch, 8, 8>::run(p->memo[FBL_MEMO_TC_FWD], key,
+  return LaunchMemo<Launch, 2>::run(p, FBL_MEMO_TC_FWD, LaunchKey(),                // its shape is the plan's
+      [&](Launch& L) { return p->d.head_dim == 64 ? fwd_make<64>(L, p, Q, K, V) : fwd_make<128>(L, p, Q, K, V); },
       [&](Launch& L) {
-        return p->d.head_dim == 64 ? fwd_make<64>(L, p, Q, K, V, A, lse, status) : fwd_make<128>(L, p, Q, K, V, A, lse, status);
+        L.P.a = (__nv_bfloat16*)A; L.P.lse = lse; L.P.status = status;
+        return fbl_map_set_base(&L.P.tq, Q) && fbl_map_set_base(&L.P.tk, K) && fbl_map_set_base(&L.P.tv, V);
       },
       [&](const Launch& L) { return launch_pdl(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.P); });
 }
@@ -1519,14 +1517,14 @@ cudaError_t launch_attn_bwd_tc(const fbl_plan* p, const void* Q, const void* K, 
   cudaError_t e = launch_attn_bwd_pre(p, A, dA, dvec, dvec_ready, st);
   if (e != cudaSuccess) return e;
   typedef AttnLaunch<AttnBwdParams> Launch;
-  LaunchKey key;
-  for (const void* q : {Q, K, V, dA, (const void*)lse, (const void*)dvec, (const void*)dqacc, (const void*)dQ, (const void*)dK, (const void*)dV,
-                        (const void*)status})
-    key.add(q);
-  e = LaunchMemo<Launch, 8, 12>::run(p->memo[FBL_MEMO_TC_BWD], key,
+  e = LaunchMemo<Launch, 2>::run(p, FBL_MEMO_TC_BWD, LaunchKey(),
+      [&](Launch& L) { return p->d.head_dim == 64 ? bwd_make<64>(L, p, Q, K, V, dA, dqacc) : bwd_make<128>(L, p, Q, K, V, dA, dqacc); },
       [&](Launch& L) {
-        return p->d.head_dim == 64 ? bwd_make<64>(L, p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status)
-                                   : bwd_make<128>(L, p, Q, K, V, dA, lse, dvec, dqacc, dQ, dK, dV, status);
+        AttnBwdParams& P = L.P;
+        P.lse = lse; P.dvec = dvec; P.dqacc = dqacc; P.dq = (__nv_bfloat16*)dQ; P.dk = (__nv_bfloat16*)dK; P.dv = (__nv_bfloat16*)dV;
+        P.status = status;
+        return fbl_map_set_base(&P.tq, Q) && fbl_map_set_base(&P.tdo, dA) && fbl_map_set_base(&P.tk, K) && fbl_map_set_base(&P.tv, V) &&
+               (attn_bwd_tc_direct(p) || fbl_map_set_base(&P.tdq, dqacc));
       },
       [&](const Launch& L) {
         return L.cluster ? launch_cluster(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.cluster, true, L.P)

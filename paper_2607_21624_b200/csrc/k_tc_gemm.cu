@@ -916,6 +916,21 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
+
+ReplaceAddressFn replace_fn() {
+  static ReplaceAddressFn fn = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapReplaceAddress", &p, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<ReplaceAddressFn>(p);
+  });
+  return fn;
+}
+
 // Self-test of the bounded wait every tensor-core kernel relies on: one block initialises an mbarrier that nothing
 // ever signals and waits on it through the same tc::mbar_wait, with a short limit.  The wait must give up, record
 // its code in the status word and let the block return normally.
@@ -936,6 +951,11 @@ __global__ void wait_timeout_selftest_kernel(int32_t* status, long long limit_cy
 cudaError_t launch_wait_timeout_selftest(int32_t* status, long long limit_cycles, cudaStream_t st) {
   wait_timeout_selftest_kernel<<<1, 64, 0, st>>>(status, limit_cycles);
   return cudaGetLastError();
+}
+
+bool fbl_map_set_base(CUtensorMap* map, const void* base) {
+  ReplaceAddressFn fn = replace_fn();
+  return fn && fn(map, const_cast<void*>(base)) == CUDA_SUCCESS;
 }
 
 static bool encode_panels(CUtensorMap* map, CUtensorMapDataType type, int width, const void* base, int64_t r_pad, int panels,
@@ -1002,17 +1022,14 @@ bool gemm_tc_supported(const fbl_plan* p, const GemmArgs& g) {
   return true;
 }
 
-// Problem set-up shared by the two kernels: tensor maps, operand orientations, epilogue extras and reduction
-// slices of every problem of a launch.  bn_box: columns of B one CTA loads per k-block; tile_m x tile_n: the output
+// Problem set-up shared by the kernels: tensor maps, operand orientations, epilogue extras and reduction
+// slices of every problem of a launch; addresses are point_group's.  bn_box: columns of B one CTA loads per k-block; tile_m x tile_n: the output
 // tile a work unit covers (the CTA pair's 256 x 256, or one CTA's 128 x BN).  Returns the number of work units in
 // *units.
-cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int32_t* status, int bn_box, int tile_m, int tile_n,
-                       int* units) {
+cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int bn_box, int tile_m, int tile_n, int* units) {
   memset(&G, 0, sizeof(G));
   G.count = count;
-  G.status = status;
   G.late_trigger = gs[0].late_trigger != nullptr;
-  G.zero_ptr = (uint4*)gs[0].zero_ptr; G.zero_vec = (long long)(gs[0].zero_bytes / 16); G.reset_status = gs[0].reset_status;
   int tiles = 0;
   for (int i = 0; i < count; ++i) {
     const GemmArgs& g = gs[i];
@@ -1034,17 +1051,13 @@ cudaError_t fill_group(TcGroup& G, const GemmArgs* gs, int count, int32_t* statu
     P.m = g.m; P.n = g.n;
     if (!fbl_encode_rtile_map(&P.tc, g.c, g.c_rpad, g.n / 64, 32, 1)) return cudaErrorInvalidValue;   // one warp's rows
     P.b_static = g.b_static;
-    P.c = (__nv_bfloat16*)g.c; P.c_rpad = g.c_rpad;
-    P.bias = g.bias; P.residual = (const __nv_bfloat16*)g.residual;
-    P.seq = g.seq; P.t_pad = g.t_pad;
-    P.dot_with = (const __nv_bfloat16*)g.dot_with; P.dot_out = g.dot_out; P.dot_hd = g.dot_hd; P.dot_hq = g.dot_hq;
-    P.epi = g.epi; P.aux1 = (const __nv_bfloat16*)g.aux1;
+    P.c_rpad = g.c_rpad; P.seq = g.seq; P.t_pad = g.t_pad;
+    P.dot_hd = g.dot_hd; P.dot_hq = g.dot_hq; P.epi = g.epi;
     if (g.epi != 0) {
       const bool rope = g.epi == 5, two_out = g.epi != 2 && !rope;
       if (g.epi < 1 || g.epi > 5 || g.ksplit > 1 || g.dot_with || (g.epi >= 2 && !rope && !g.residual) || (g.epi == 4 && !g.aux1) ||
           (two_out && !g.c2) || (rope && (!g.rope || g.residual || g.t_pad <= 0)))
         return cudaErrorInvalidValue;
-      P.rope = g.rope;
       if (two_out && !fbl_encode_rtile_map(&P.tc2, g.c2, g.c_rpad, g.n / 64, 32, 1)) return cudaErrorInvalidValue;
     }
     P.ksplit = 1;
@@ -1070,9 +1083,10 @@ int group_epi(const GemmArgs* gs, int count) {
   return epi;
 }
 
-// A launch made ready: what launch_gemm_tc_group remembers.
+// A launch made ready but for its addresses: what launch_gemm_tc_group keeps.
 struct GroupLaunch {
   TcGroup G;
+  int order[MAX_PROBLEMS];                   // the caller's problem that each of G's is
   void (*kernel)(const TcGroup);
   int grid, threads, serial, cluster;        // cluster: blocks of a cluster where the launch says so, else 0
   int idle;                                  // what a late_trigger receives
@@ -1085,10 +1099,29 @@ cudaError_t group_launch(GroupLaunch& L, void (*k)(const TcGroup), int grid, int
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+bool point_group(GroupLaunch& L, const GemmArgs* gs, int32_t* status) {
+  TcGroup& G = L.G;
+  G.status = status;
+  G.zero_ptr = (uint4*)gs[0].zero_ptr; G.zero_vec = (long long)(gs[0].zero_bytes / 16); G.reset_status = gs[0].reset_status;
+  bool ok = true;
+  for (int i = 0; i < G.count; ++i) {
+    const GemmArgs& g = gs[L.order[i]];
+    TcProblem& P = G.p[i];
+    for (int t = 0; t < P.n_terms; ++t) ok = ok && fbl_map_set_base(&P.ta[t], g.t[t].a) && fbl_map_set_base(&P.tb[t], g.t[t].b);
+    ok = ok && fbl_map_set_base(&P.tc, g.c);
+    if (P.epi != 0 && P.epi != 2 && P.epi != 5) ok = ok && fbl_map_set_base(&P.tc2, g.c2);
+    if (P.ksplit > 1 || g.ksplit > 1) ok = ok && fbl_map_set_base(&P.tacc, g.acc);
+    P.c = (__nv_bfloat16*)g.c; P.bias = g.bias; P.residual = (const __nv_bfloat16*)g.residual;
+    P.dot_with = (const __nv_bfloat16*)g.dot_with; P.dot_out = g.dot_out;
+    P.aux1 = (const __nv_bfloat16*)g.aux1; P.rope = g.rope;
+  }
+  return ok;
+}
+
 template <int BN, int STAGES>
-cudaError_t make_group_bn(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, int esets_choice) {
+cudaError_t make_group_bn(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int esets_choice) {
   int tiles = 0;
-  cudaError_t e = fill_group(L.G, gs, count, status, BN, BM, BN, &tiles);
+  cudaError_t e = fill_group(L.G, gs, count, BN, BM, BN, &tiles);
   if (e != cudaSuccess) return e;
   const int grid = tiles < p->sm_count ? tiles : p->sm_count;
   // one tile per block at most: the epilogue is exposed, and the variant with two sets of epilogue warps halves it
@@ -1105,9 +1138,9 @@ cudaError_t make_group_bn(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs,
   return group_launch(L, k, grid, two_sets ? 320 : 192, SmemPlan<BN, STAGES>::TOTAL, gs[0].serial);
 }
 
-cudaError_t make_group_split(GroupLaunch& L, const GemmArgs* gs, int count, int32_t* status, int slices) {
+cudaError_t make_group_split(GroupLaunch& L, const GemmArgs* gs, int count, int slices) {
   int tiles = 0;
-  cudaError_t e = fill_group(L.G, gs, count, status, 128, BM, 128, &tiles);
+  cudaError_t e = fill_group(L.G, gs, count, 128, BM, 128, &tiles);
   if (e != cudaSuccess) return e;
   L.G.slices = slices;
   for (int i = 0; i < count; ++i) {
@@ -1120,9 +1153,9 @@ cudaError_t make_group_split(GroupLaunch& L, const GemmArgs* gs, int count, int3
   return group_launch(L, k, tiles * slices, 320, SmemPlan<128, SPLIT_STAGES>::TOTAL, gs[0].serial, slices);
 }
 
-cudaError_t make_group_pair(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status) {
+cudaError_t make_group_pair(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count) {
   int tiles = 0;
-  cudaError_t e = fill_group(L.G, gs, count, status, 128, 256, 256, &tiles);   // each CTA loads 128 of the pair's 256 columns
+  cudaError_t e = fill_group(L.G, gs, count, 128, 256, 256, &tiles);   // each CTA loads 128 of the pair's 256 columns
   if (e != cudaSuccess) return e;
   const int epi = group_epi(gs, count), pairs = tiles < p->sm_count / 2 ? tiles : p->sm_count / 2;
   auto k = epi == EPI_ACT ? gemm_tc_pair_kernel<EPI_ACT> : epi == EPI_ROPE ? gemm_tc_pair_kernel<EPI_ROPE> : gemm_tc_pair_kernel<EPI_NONE>;
@@ -1210,12 +1243,13 @@ int best_tile(const TileWork* w, int count, int sm_count, bool pairs, double* cl
 
 // The tile whose slowest block finishes first; an offline choice for this launch, or the pair knob, comes before it.
 // (N need not be whole tiles: panels past it are loaded as zeros and not stored.)
-static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, const fbl_plan::GemmChoice& ch) {
+static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count, const fbl_plan::GemmChoice& ch) {
   const int pair_mode = ch.pair >= 0 ? ch.pair : p->knob_gemm_pair;       // 0 never, 1 always, -1 by cost
   int kind = TILE_NARROW;
   GemmArgs by_length[MAX_PROBLEMS];
   TileWork w[MAX_PROBLEMS];
   for (int i = 0; i < count; ++i) {
+    L.order[i] = i;
     w[i] = {gs[i].m, gs[i].n, 0, gs[i].ksplit > 1 ? gs[i].ksplit : 1};
     for (int t = 0; t < gs[i].n_terms; ++t) w[i].kb += (gs[i].t[t].k + BK - 1) / BK;
   }
@@ -1233,7 +1267,7 @@ static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs*
     const int slices = best_slices(w, count, p->sm_count, clocks);
     if (slices) {
       L.idle = 1 << 20;                              // fewer blocks than SMs, as a rule
-      return make_group_split(L, gs, count, status, slices);
+      return make_group_split(L, gs, count, slices);
     }
     // The problems come with the token-axis reductions first; of few tokens those are the shortest, and the longest
     // units should start first.
@@ -1246,20 +1280,18 @@ static cudaError_t make_group(GroupLaunch& L, const fbl_plan* p, const GemmArgs*
     const int sorted_kind = best_tile(sorted, count, p->sm_count, pair_mode != 0, &sorted_clocks);
     if (kind != TILE_SLIM && sorted_clocks < 0.95 * clocks) {
       kind = sorted_kind;
-      for (int i = 0; i < count; ++i) { by_length[i] = gs[order[i]]; w[i] = sorted[i]; }
-      for (int i = 0; i < count; ++i) { by_length[i].zero_bytes = 0; by_length[i].reset_status = by_length[i].serial = 0; by_length[i].late_trigger = nullptr; }
-      by_length[0].zero_ptr = gs[0].zero_ptr; by_length[0].zero_bytes = gs[0].zero_bytes;      // the launch's chores stay with its first problem
-      by_length[0].reset_status = gs[0].reset_status; by_length[0].serial = gs[0].serial; by_length[0].late_trigger = gs[0].late_trigger;
+      for (int i = 0; i < count; ++i) { by_length[i] = gs[order[i]]; w[i] = sorted[i]; L.order[i] = order[i]; }
+      by_length[0].serial = gs[0].serial; by_length[0].late_trigger = gs[0].late_trigger;      // the launch's own, not the problem's
       gs = by_length;
     }
   }
   double idle;
   tile_makespan(TILE_COST[kind], w, count, kind == TILE_PAIR ? p->sm_count / 2 : p->sm_count, &idle);
   L.idle = (int)idle;
-  if (kind == TILE_PAIR) return make_group_pair(L, p, gs, count, status);
-  if (kind == TILE_SLIM) return make_group_bn<64, 8>(L, p, gs, count, status, 1);
-  if (kind == TILE_WIDE) return make_group_bn<256, 4>(L, p, gs, count, status, ch.esets);
-  return make_group_bn<128, 6>(L, p, gs, count, status, ch.esets);
+  if (kind == TILE_PAIR) return make_group_pair(L, p, gs, count);
+  if (kind == TILE_SLIM) return make_group_bn<64, 8>(L, p, gs, count, 1);
+  if (kind == TILE_WIDE) return make_group_bn<256, 4>(L, p, gs, count, ch.esets);
+  return make_group_bn<128, 6>(L, p, gs, count, ch.esets);
 }
 
 cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st,
@@ -1268,11 +1300,12 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
   fbl_plan::GemmChoice ch = {0, -1, 0};
   if (launch_id >= 0 && launch_id < FBL_GEMM_LAUNCH_COUNT) ch = p->choice[launch_id];
   LaunchKey key;
-  gemm_group_key(key, gs, count, status);
+  gemm_group_key(key, gs, count);
   key.add(ch.bn, ch.pair);
   key.add(ch.esets, 0);
-  return LaunchMemo<GroupLaunch, 12, 248>::run(p->memo[FBL_MEMO_TC_GEMM], key,
-      [&](GroupLaunch& L) { return make_group(L, p, gs, count, status, ch); },
+  return LaunchMemo<GroupLaunch, 12>::run(p, FBL_MEMO_TC_GEMM, key,
+      [&](GroupLaunch& L) { return make_group(L, p, gs, count, ch); },
+      [&](GroupLaunch& L) { return point_group(L, gs, status); },
       [&](const GroupLaunch& L) {
         if (gs[0].late_trigger) *gs[0].late_trigger = L.idle;
         if (L.cluster) return launch_cluster(L.kernel, dim3(L.grid), dim3(L.threads), L.smem, st, L.cluster, !L.serial, L.G);

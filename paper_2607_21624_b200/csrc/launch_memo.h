@@ -1,79 +1,85 @@
-// What a launch of a plan is made of besides its arguments -- parameter block with its tensor maps, kernel, grid -- is
-// remembered by those arguments: a program calls with the same buffers pass after pass, and encoding ten to thirty tensor
-// maps, choosing tiles and setting function attributes is a tenth of a pass's host time (forward pass of four launches 19 ->
-// 17 us, ten-launch step 45 -> 41 us; passes of few tokens are host-bound: 21.7 -> 19.2 us for an adapter forward of 48
-// tokens).  Bounded per plan; the oldest entry makes room.
+// What a launch of a plan is made of besides addresses -- kernel, grid, and a parameter block whose tensor maps await their
+// addresses -- is kept in the plan under the launch's shape: choosing tiles, encoding ten to thirty tensor maps and setting
+// function attributes is host work that a pass of few tokens would wait for.  Addresses are put in on every launch (9 ns a
+// tensor map, against 46 to encode one), so a pass on new buffers costs what any other does, however many layers share the
+// plan (kept by address, twelve 50-token layers on one plan took 21.9 us a forward pass and one layer alone 19.0; now 19.5 and
+// 19.4).  A plan has less than a dozen shapes of launches of a kind; should there be more, the oldest makes room.
 #pragma once
+#include <cuda.h>
 #include <stdint.h>
 #include <string.h>
 
+#include <memory>
 #include <new>
 
 #include "fbl_internal.h"
 
 struct LaunchKey {
-  static constexpr int MAX = 256;
+  static constexpr int MAX = 128;          // five products of four terms are 99 words
   uint64_t v[MAX];
   int n = 0;
-  void add(uint64_t x) { if (n < MAX) v[n++] = x; }
-  void add(const void* p) { add((uint64_t)(uintptr_t)p); }
+  LaunchKey() {                            // function attributes are a device's
+    int dev = -1;
+    (void)cudaGetDevice(&dev);
+    add((uint64_t)(int64_t)dev);
+  }
+  void add(uint64_t x) { if (n < MAX) v[n] = x; ++n; }
   void add(int a, int b) { add(((uint64_t)(uint32_t)a << 32) | (uint32_t)b); }
 };
 
-template <typename Params, int N, int KEY>
+template <typename Params, int N>
 struct LaunchMemo : FblMemoBase {
-  struct Entry { Params params; uint64_t key[KEY]; int n; };
-  Entry entry[N];
+  struct Entry { Params params; uint64_t key[LaunchKey::MAX]; int n; };
+  std::unique_ptr<Entry> entry[N];
   int next = 0;
-  LaunchMemo() { for (Entry& e : entry) e.n = 0; }
 
-  // The entry of this key.  *hit = false: a fresh one, to be filled in (and dropped by `drop` if that fails).
-  Entry* find(const LaunchKey& k, bool* hit) {
-    for (Entry& e : entry)
-      if (e.n == k.n && memcmp(e.key, k.v, (size_t)k.n * sizeof(uint64_t)) == 0) { *hit = true; return &e; }
-    Entry& e = entry[next];
-    next = (next + 1) % N;
-    e.n = k.n;
-    memcpy(e.key, k.v, (size_t)k.n * sizeof(uint64_t));
-    *hit = false;
-    return &e;
-  }
-
-  // launch(params) with the parameters fill(params) makes for this key, remembered in `slot` of the plan.
-  template <typename Fill, typename Launch>
-  static cudaError_t run(FblMemoBase*& slot, const LaunchKey& k, Fill&& fill, Launch&& launch) {
-    if (!slot) slot = new (std::nothrow) LaunchMemo();
-    if (!slot || k.n > KEY || k.n >= LaunchKey::MAX) {
-      Params p;
-      const cudaError_t e = fill(p);
-      return e != cudaSuccess ? e : launch(p);
-    }
-    bool hit;
-    Entry* at = static_cast<LaunchMemo*>(slot)->find(k, &hit);
-    if (!hit) {
+  // launch(params) with what fill(params) makes for this key, kept in the plan's `slot`, and point(params) has given addresses.
+  template <typename Fill, typename Point, typename Launch>
+  static cudaError_t run(const fbl_plan* p, int slot, const LaunchKey& k, Fill&& fill, Point&& point, Launch&& launch) {
+    std::lock_guard<std::mutex> hold(p->memo_lock);
+    if (!p->memo[slot]) p->memo[slot] = new (std::nothrow) LaunchMemo();
+    LaunchMemo* memo = static_cast<LaunchMemo*>(p->memo[slot]);
+    Entry* at = nullptr;
+    std::unique_ptr<Entry> fresh;
+    if (memo && k.n <= LaunchKey::MAX)
+      for (int i = 0; i < N && !at; ++i) {
+        Entry* e = memo->entry[i].get();
+        if (e && e->n == k.n && memcmp(e->key, k.v, (size_t)k.n * sizeof(uint64_t)) == 0) at = e;
+      }
+    if (!at) {
+      fresh.reset(new (std::nothrow) Entry);
+      if (!fresh) return cudaErrorMemoryAllocation;
+      at = fresh.get();
       const cudaError_t e = fill(at->params);
-      if (e != cudaSuccess) { at->n = 0; return e; }
+      if (e != cudaSuccess) return e;
     }
-    return launch(at->params);
+    if (!point(at->params)) return cudaErrorInvalidValue;
+    const cudaError_t e = launch(at->params);
+    if (fresh && memo && k.n <= LaunchKey::MAX && e == cudaSuccess) {
+      fresh->n = k.n;
+      memcpy(fresh->key, k.v, (size_t)k.n * sizeof(uint64_t));
+      memo->entry[memo->next] = std::move(fresh);
+      memo->next = (memo->next + 1) % N;
+    }
+    return e;
   }
 };
 
-// Everything of a group of products that its parameter block depends on.
-inline void gemm_group_key(LaunchKey& k, const GemmArgs* gs, int count, const int32_t* status) {
-  k.add(status);
-  k.add((uint64_t)count);
+// What the parameter block of a group of products depends on besides addresses, in the order of the group.
+inline void gemm_group_key(LaunchKey& k, const GemmArgs* gs, int count) {
+  k.add(count, (gs[0].late_trigger != nullptr) * 2 + (gs[0].serial != 0));
   for (int i = 0; i < count; ++i) {
     const GemmArgs& g = gs[i];
     k.add(g.m, g.n);
     k.add(g.n_terms, g.b_static);
     for (int t = 0; t < g.n_terms; ++t) {
       const GemmTerm& m = g.t[t];
-      k.add(m.a); k.add((uint64_t)m.a_rpad); k.add(m.b); k.add((uint64_t)m.b_rpad);
+      k.add((uint64_t)m.a_rpad); k.add((uint64_t)m.b_rpad);
       k.add(m.k, m.a_trans * 2 + m.b_trans);
     }
-    k.add(g.c); k.add((uint64_t)g.c_rpad); k.add(g.bias); k.add(g.residual); k.add(g.seq, g.t_pad);
-    k.add(g.dot_with); k.add(g.dot_out); k.add(g.dot_hd, g.dot_hq);
-    k.add(g.acc); k.add(g.ksplit, g.epi); k.add(g.aux1); k.add(g.c2); k.add(g.rope); k.add(g.serial, 0);
-    if (i == 0) { k.add(g.late_trigger != nullptr, 0); k.add(g.zero_ptr); k.add((uint64_t)g.zero_bytes); k.add((uint64_t)g.reset_status); }
+    k.add((uint64_t)g.c_rpad); k.add(g.seq, g.t_pad); k.add(g.dot_hd, g.dot_hq); k.add(g.ksplit, g.epi);
+    // which operands there are: fill_group's checks look at them
+    k.add((g.bias != nullptr) | (g.residual != nullptr) << 1 | (g.dot_with != nullptr) << 2 | (g.aux1 != nullptr) << 3 |
+          (g.c2 != nullptr) << 4 | (g.rope != nullptr) << 5 | (g.acc != nullptr) << 6, 0);
   }
 }

@@ -322,6 +322,7 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 }  // namespace tc
 
 // Host side: encode a 3-D tensor map over an R-Tile bf16 matrix viewed as [panels][rows][64].
+bool fbl_map_set_base(CUtensorMap* map, const void* base);      // an encoded map at another address
 bool fbl_encode_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels);
 bool fbl_encode_f32_rtile_map(CUtensorMap* map, const void* base, int64_t r_pad, int panels, int box_rows, int box_panels);   // fp32: [panels][rows][32]
 // A matrix of `seqs` sequences of `rows` rows each, seen as [panels][seqs][rows][128 bytes]: a box that reaches past its sequence's

@@ -290,3 +290,38 @@ def test_early_sums_wait_behind_a_launch_that_vouches_for_nothing(rows, cols):
         out.zero_()
         _check(fn(plan._h, m.data_ptr(), rows, cols, out.data_ptr(), scratch.data_ptr(), torch.cuda.current_stream().cuda_stream))
         assert (out == rows).all()
+
+
+@pytest.mark.parametrize("cfg", [
+    LayerConfig("bs1", 2, 60, 256, 4, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 351, 0.05),
+    LayerConfig("bs2", 2, 300, 256, 4, 2, 64, "bf16", "rmsnorm", True, False, True, 1e-5, 352, 0.05, 0.0, 10000.0),
+    LayerConfig("bs3", 1, 70, 64, 2, 1, 32, "fp32", "layernorm", True, True, True, 1e-5, 353, 0.1),
+    MlpConfig("bs4", 1, 200, 256, 704, "bf16", "rmsnorm", "swiglu", True, True, 1e-5, 354, 0.05),
+    XattnConfig("bs5", 1, 140, 200, 128, 192, 2, 2, 64, "bf16", "layernorm", True, True, 1e-5, 355, 0.05),
+], ids=lambda c: c.name)
+def test_one_plan_over_many_sets_of_buffers(cfg):
+    # a model's layers share a plan: each pass goes to the buffers it is called with, whichever were before
+    import dataclasses
+    import numpy as np
+    from fbl_inputs import make_inputs, make_mlp_inputs, make_xattn_inputs
+    from paper_2607_21624_b200 import LayerRunner, MlpRunner, XattnRunner
+    make, Runner = (make_mlp_inputs, MlpRunner) if isinstance(cfg, MlpConfig) else (make_xattn_inputs, XattnRunner) if \
+        isinstance(cfg, XattnConfig) else (make_inputs, LayerRunner)
+    inputs = [make(dataclasses.replace(cfg, seed=cfg.seed + 1000 * i)) for i in range(4)]
+    alone = [Runner(cfg) for _ in inputs]
+    shared = [Runner(cfg) for _ in inputs]
+    for a, s, inp in zip(alone, shared, inputs):
+        a.load_inputs(inp)
+        s.load_inputs(inp)
+        a.step()
+    for s in shared:
+        s.plan = shared[0].plan
+    for order in ((0, 1, 2, 3), (3, 1, 0, 2)):
+        for i in order:
+            shared[i].step()
+    for a, s in zip(alone, shared):
+        assert s.status() == 0
+        for n in a.OUT_MATS:
+            if n in a.buf:                  # dQ's additions may come in another order
+                want = a.fetch(n)
+                assert np.abs(s.fetch(n) - want).max() <= (1e-5 if cfg.dtype == "fp32" else 1e-2) * np.abs(want).max(), n
