@@ -8,7 +8,6 @@
 
 #include <algorithm>
 #include <mutex>
-#include <vector>
 
 #include "fbl_internal.h"
 #include "launch_memo.h"
@@ -1175,9 +1174,13 @@ struct TileCost { int m, n; double kb, unit, epilogue, fixed; };      // extents
 const TileCost TILE_COST[4] = {{128, 128, 545, 800, 1600, 0}, {128, 256, 710, 900, 3600, 0}, {256, 256, 675, 900, 3600, 3500}, {128, 64, 400, 800, 1600, 0}};
 struct TileWork { long long m; int n, kb, split; };
 
-// Clocks of the longest block (pair) when the persistent kernel deals the units of a group's problems out in turn.
+// Clocks of the longest block (pair) when the persistent kernel deals the units of a group's problems out in turn.  (Of a
+// part with more SMs the first MAX_SLOTS stand for all; an enqueue call allocates nothing that could throw.)
+constexpr int MAX_SLOTS = 512;
 double tile_makespan(const TileCost& c, const TileWork* w, int count, int slots, double* idle = nullptr) {
-  std::vector<double> load((size_t)slots, 0.0);
+  double load[MAX_SLOTS];
+  slots = std::min(slots, MAX_SLOTS);
+  std::fill(load, load + slots, 0.0);
   long long dealt = 0;
   for (int i = 0; i < count; ++i) {
     const long long units = ((w[i].m + c.m - 1) / c.m) * ((w[i].n + c.n - 1) / c.n) * w[i].split;
@@ -1191,7 +1194,7 @@ double tile_makespan(const TileCost& c, const TileWork* w, int count, int slots,
     dealt += units;
   }
   double longest = 0, sum = 0;
-  for (double l : load) { longest = l > longest ? l : longest; sum += l; }
+  for (int s = 0; s < slots; ++s) { longest = std::max(longest, load[s]); sum += load[s]; }
   if (idle) *idle = longest - sum / slots;
   return longest + (dealt <= slots ? 0.5 : 1.0) * c.epilogue + c.fixed;
 }

@@ -204,6 +204,8 @@ int fbl_xattn_bwd(const fbl_plan* p, const void* dY, const void* X, const void* 
         acc += up8(Dm) * (int64_t)p->dkv;
       }
     }
+    // always beside the products: the memory side's sums, over other rows than the norm's, would take two launches of their own
+    // (5 to 11 % of a step of few tokens)
     int idle = 0;
     if (bias && tc) all[0].late_trigger = &idle;
     XA_GEMM_STEP("dWqkv+dXn+dM", all, 5);
