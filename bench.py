@@ -3,10 +3,10 @@
 
 One step = fbl_layer_fwd + fbl_layer_bwd over one batch of synthetic input.  Without --config the five
 workloads are timed one after the other in the same process; the JSON line's top-level figures are those of the
-largest one (workload 5, the Llama-7B-shaped long-sequence layer) and `per_config` carries all five.  Reported:
+largest one (workload 5, the Llama-7B-shaped long-sequence layer) and `per_config` has all of them.  Reported:
 algorithmic TFLOP/s (multiply-add = 2, causal pairs counted once, no recompute), tokens/s, the end-to-end figure
 with host buffers, a roofline object for the dominant kernel, the layer's memory efficiency and the float64
-oracle timed on the host cores.
+oracle timed on the host cores.  stdout gets one short line (`contract_line`), stderr the same with every figure.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--config i] [--impl reference]
 
@@ -581,6 +581,30 @@ def time_runner(run, cfg, workload, args, rep, flush_l2):
             "launches_per_step": launches}
 
 
+def rounded(v):
+    """Floats to six significant digits."""
+    if isinstance(v, dict):
+        return {k: rounded(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [rounded(x) for x in v]
+    return float(f"{v:.6g}") if isinstance(v, float) else v
+
+
+def contract_line(full):
+    """The line that goes to stdout: the headline's own figures and [ms per step, TFLOP/s] of everything timed, in less than
+    2800 characters, so that a reader who keeps the end of the output has all of it."""
+    line = {k: v for k, v in full.items() if k not in ("layer_roofline", "mem_efficiency", "activation_bytes", "roofline", "cpu_baseline",
+                                                      "peaks", "per_config")}
+    roof, cpu = full["roofline"], full["cpu_baseline"]
+    line["roofline"] = {k: roof[k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic", "kernel_share", "kernel_ms")}
+    line["frac_of_burst"] = full["layer_roofline"]["frac_of_measured_burst"]
+    line["mem_efficiency"] = full["mem_efficiency"]["value"]
+    line["activation_bytes"] = full["activation_bytes"]
+    line["cpu_baseline"] = cpu and {k: cpu[k] for k in ("value", "unit", "cores", "kind", "sample")}
+    line["per_config"] = {k: [v["ms_per_step"], v["tflops"]] for k, v in full["per_config"].items()}
+    return rounded(line)
+
+
 def run_rank(args):
     """Body of one rank (the only one at N = 1)."""
     rank = int(os.environ.get("RANK", "0"))
@@ -647,7 +671,7 @@ def run_rank(args):
                    "l2": "256 MiB written" + ("" if args.flush_write_only else ", then 256 MiB read (so that the write-back of the flush is over)") + " before every timed step",
                    "launch": "direct launches" if args.no_graph else "cuda graph replay",
                    "kernel_path": "default" if args.path == 0 else "ffma", "parallelism": "replicas only",
-                   "also_timed": "per_config holds all five workloads, each timed the same way in this process"},
+                   "also_timed": "per_config: [ms per step, TFLOP/s]"},
         "tokens_per_s": h["tokens_per_s"], "layer_roofline": h["layer_roofline"], "mem_efficiency": h["mem_efficiency"],
         "activation_bytes": h["activation_bytes"], "e2e": h["e2e"],
         "gpu_launches": (sum(r["launches_per_step"] for r in results.values())
@@ -660,7 +684,8 @@ def run_rank(args):
                        **{f"lora16_workload{i}": v for i, v in lora.items()},
                        **{f"xattn_{k}": v for k, v in xattn.items()}},
     }
-    print(json.dumps(line))
+    print(json.dumps(line), file=sys.stderr)           # every figure
+    print(json.dumps(contract_line(line)))
     rep.close()
 
 
