@@ -91,17 +91,16 @@ def min_bytes(cfg):
 # a weight share that does not grow, so they get no scaled entry.
 _MB = 1e6
 _NCU_MB = {
-    "cfg1-tiny-fp32": {"norm_fwd": 0.03, "proj_q": 0.10, "proj_k": 0.10, "proj_v": 0.10, "attn_fwd": 0.07, "proj_o": 0.10,
-                       "dA": 0.10, "dWo": 0.11, "attn_bwd": 0.04 + 0.11 + 0.02, "dXn": 0.16, "dWq": 0.11, "dWk": 0.11,
-                       "dWv": 0.11, "norm_bwd": 0.05},
-    "cfg2-gpt2-small": {"norm_fwd": 3.46, "proj_qkv": 6.76, "attn_fwd": 9.47, "proj_o": 4.39, "dWo+dA": 7.53,
-                        "attn_bwd": 19.12 + 6.30, "dWqkv+dXn": 16.18, "db+norm_bwd": 18.92 + 1.69},
-    "cfg3-vit-base": {"norm_fwd": 10.16, "proj_qkv": 13.43, "attn_fwd": 29.53, "proj_o": 11.07, "dWo+dA": 23.26,
-                      "attn_bwd": 59.97 + 19.67, "dWqkv+dXn": 50.12, "dW round": 11.06, "norm_bwd": 19.75 + 1.83},
-    "cfg4-llama1b-gqa": {"norm_fwd": 16.81, "proj_qkv": 29.42, "attn_fwd": 25.22, "proj_o": 25.23, "dWo+dA": 45.53,
-                         "attn_bwd": 77.46 + 33.56, "dWqkv+dXn": 62.33, "norm_bwd": 33.72 + 2.44},
-    "cfg5-llama7b-long-scaled": {"norm_fwd": 16.82, "proj_qkv": 147.11, "attn_fwd": 50.56, "proj_o": 50.49, "dWo+dA": 110.03,
-                                 "attn_bwd": 118.07 + 33.56, "dWqkv+dXn": 383.49, "norm_bwd": 33.91 + 4.87},
+    "cfg1-tiny-fp32": {"norm_fwd": 0.05, "proj_qkv": 0.10, "attn_fwd": 0.10, "proj_o": 0.06, "dWo+dA": 0.08, "attn_bwd": 0.15,
+                       "dWqkv+dXn": 0.14, "norm_bwd": 0.06 + 0.02},
+    "cfg2-gpt2-small": {"norm_fwd": 3.18, "proj_qkv": 6.76, "attn_fwd": 9.47, "proj_o": 4.39, "dWo+dA": 7.53,
+                        "attn_bwd": 19.12 + 6.30, "dWqkv+dXn": 16.18, "db": 12.60, "db+norm_bwd": 6.35 + 1.69},
+    "cfg3-vit-base": {"norm_fwd": 9.86, "proj_qkv": 13.44, "attn_fwd": 29.53, "proj_o": 11.07, "dWo+dA": 0.01 + 23.26,
+                      "attn_bwd": 40.02, "dWqkv+dXn": 50.33, "norm_bwd": 19.76 + 11.09},
+    "cfg4-llama1b-gqa": {"norm_fwd": 16.82, "proj_qkv": 29.43, "attn_fwd": 25.22, "proj_o": 25.23, "dWo+dA": 1.13 + 44.50,
+                         "attn_bwd": 77.78 + 33.56, "dWqkv+dXn": 96.17, "norm_bwd": 33.65 + 27.28},
+    "cfg5-llama7b-long-scaled": {"norm_fwd": 16.83, "proj_qkv": 147.03, "attn_fwd": 50.43, "proj_o": 50.73, "dWo+dA": 0.01 + 109.72,
+                                 "attn_bwd": 117.55 + 33.56, "dWqkv+dXn": 383.19, "norm_bwd": 33.65 + 4.21},
 }
 _NCU_MB["cfg5-llama7b-long"] = {k: 4.0 * v for k, v in _NCU_MB["cfg5-llama7b-long-scaled"].items()
                                 if k in ("norm_fwd", "attn_fwd", "attn_bwd", "norm_bwd")}     # the token-proportional kernels
@@ -415,6 +414,8 @@ def measure(cfg, args, rep, local_rank, flush_l2, want_cpu, lora_rank=0):
     flops = lora_flops(cfg, lora_rank) if lora_rank else cfg.flops()
     tfl = rep.whole_job_rate(flops, ms) / 1e12
     sf, sbytes = step_flops(cfg), step_bytes(cfg)
+    if "db" in kernel_ms:                                # the column sums have a step of their own
+        sbytes["db+norm_bwd"] = sbytes["norm_bwd"]
     if lora_rank:
         thin = 2.0 * cfg.n_tokens * lora_rank
         sf.update({"lora_T": thin * 3 * cfg.d_model, "lora_dA": thin * 3 * cfg.d_model, "lora_dT": thin * (cfg.d_q + 2 * cfg.d_kv),
