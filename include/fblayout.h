@@ -115,8 +115,9 @@ void fbl_plan_destroy(fbl_plan* plan);
 int fbl_tensor_bytes(const fbl_plan* plan, int tensor_id, size_t* bytes);
 
 /* Sizes of the three caller-owned work areas: `saved` carries forward tensors into the backward
- * (the E_reuse edges of the paper's graph, section 3.1: norm statistics, Xn, Q, K, V, A, LSE);
- * the scratch areas hold per-call temporaries. */
+ * (the E_reuse edges of the paper's graph, section 3.1: norm statistics, Xn, Q, K, V, A, LSE; in self-attention also
+ * room for the rotary embedding's table, seq x head_dim / 2 pairs of floats, which fbl_plan_enable_rope may call for after
+ * the sizes have been asked for); the scratch areas hold per-call temporaries. */
 int fbl_workspace_bytes(const fbl_plan* plan, size_t* saved, size_t* scratch_fwd, size_t* scratch_bwd);
 
 /* Where the step's intermediates live inside the caller's work areas (byte offset and size), so that a caller
@@ -404,8 +405,8 @@ int fbl_xattn_bwd(const fbl_plan* plan, const void* dY, const void* X, const voi
                   void* dWq, void* dWk, void* dWv, void* dWo, float* dbq, float* dbk, float* dbv, float* dbo,
                   float* dgamma, float* dbeta, void* scratch, void* stream);
 
-/* Kernel family used by later calls on this plan: 0 = default (tcgen05 tensor-core kernels for bf16
- * wherever one exists for the shape, FFMA kernels for fp32), 1 = FFMA kernels only (fp32 arithmetic on
+/* Kernel family used by later calls on this plan: 0 = default (tcgen05 tensor-core kernels for bf16, FFMA kernels for fp32
+ * and for the attention backward of bf16 layers with less than 128 token rows on either side), 1 = FFMA kernels only (fp32 arithmetic on
  * the same layout; lets a caller cross-check the tensor-core path on the device). */
 int fbl_plan_set_kernel_path(fbl_plan* plan, int path);
 
