@@ -142,9 +142,12 @@ static int plan_build(const fbl_layer_desc* desc, int cross, int seq_kv_in, int 
   auto env_int = [](const char* name, int dflt) { const char* v = getenv(name); return v ? atoi(v) : dflt; };
   p->knob_gemm_pair = env_int("FBL_GEMM_PAIR", -1);
   p->knob_gemm_esets = env_int("FBL_GEMM_ESETS", 0);
+  p->knob_f32_bn = env_int("FBL_F32_BN", 0);
+  p->knob_f32_slices = env_int("FBL_F32_SLICES", 0);
   p->knob_fwd_tiles = env_int("FBL_FWD_TILES", 0);
   for (int i = 0; i < FBL_GEMM_LAUNCH_COUNT; ++i) p->choice[i] = {0, -1, 0};
   p->use_tc = d.dtype == FBL_DTYPE_BF16 ? 1 : 0;
+  p->ffma_only = 0;
 
   const size_t n = (size_t)p->n_pad, nk = (size_t)p->n_pad_kv;
   auto mat = [&](size_t cols) { return fbl_align_up(n * cols * (size_t)e, FBL_ALIGN); };
@@ -275,6 +278,7 @@ int fbl_plan_enable_rope(fbl_plan* plan, float base) {
 int fbl_plan_set_kernel_path(fbl_plan* plan, int path) {
   if (!plan || (path != 0 && path != 1)) return FBL_ERR_INVALID_ARG;
   plan->use_tc = (path == 0 && plan->d.dtype == FBL_DTYPE_BF16) ? 1 : 0;
+  plan->ffma_only = path;
   return FBL_OK;
 }
 

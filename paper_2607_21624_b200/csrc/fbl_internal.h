@@ -33,7 +33,7 @@ template <> __device__ __forceinline__ float from_f<float>(float v) { return v; 
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 struct FblMemoBase { virtual ~FblMemoBase() {} };      // launch_memo.h
-enum { FBL_MEMO_TC_GEMM = 0, FBL_MEMO_FFMA_GEMM, FBL_MEMO_TC_FWD, FBL_MEMO_TC_BWD, FBL_MEMO_FFMA_ATTN, FBL_MEMO_COUNT };
+enum { FBL_MEMO_TC_GEMM = 0, FBL_MEMO_FFMA_GEMM, FBL_MEMO_TC_FWD, FBL_MEMO_TC_BWD, FBL_MEMO_FFMA_ATTN, FBL_MEMO_TC_F32_GEMM, FBL_MEMO_COUNT };
 
 struct fbl_plan {
   fbl_layer_desc d;
@@ -49,6 +49,7 @@ struct fbl_plan {
   float scale;
   int sm_count;
   int use_tc;   // 1: tensor-core (tcgen05) kernels where one exists for the shape; 0: FFMA kernels only
+  int ffma_only;   // kernel path 1: products of fp32 plans on the FP32 pipe instead of the tensor cores
   // byte offsets inside `saved`
   size_t sv_stats, sv_xn, sv_q, sv_k, sv_v, sv_a, sv_lse, sv_rope, saved_bytes;   // sv_rope: the rotary embedding's table
   // byte offsets inside the backward scratch
@@ -67,6 +68,7 @@ struct fbl_plan {
   // tuning knobs, read from the environment once, at plan creation (0 / -1 = the library's own choice)
   int knob_gemm_pair;       // -1 by size, 0 never the CTA-pair GEMM kernel, 1 wherever its tile shape is legal
   int knob_gemm_esets;      // 0 by tiles per block, 1 / 2 sets of epilogue warps
+  int knob_f32_bn, knob_f32_slices;   // 0 by size, 64 / 128 columns and 1, 2, 4, 8 slices of the fp32 products' tiles
   int knob_fwd_tiles;       // 0 by sequence length, 1 / 2 query tiles per forward-attention block at head_dim 64
   // low-rank adapters on Q, K, V (fbl_plan_enable_lora): rank, and the offsets of T = Xn [Aq|Ak|Av] inside `saved`,
   // of dT and of the unused norm-parameter gradients inside the backward scratch
@@ -130,6 +132,9 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
                                  int launch_id = -1);
 bool gemm_ffma_supported(const fbl_plan* p, const GemmArgs& g);
 cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st);
+// fp32 on the tensor cores: what gemm_ffma_supported accepts.  bn, slices: 0, or a tile width of 64 or 128 columns and 1, 2, 4 or 8
+// blocks that share a tile's reduction (measurements).
+cudaError_t launch_gemm_tc_f32_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int bn = 0, int slices = 0);
 // Every problem of the group can run on the tensor-core kernel and the plan wants it to.
 static inline bool gemm_group_tc(const fbl_plan* p, const GemmArgs* gs, int count) {
   bool tc = p->use_tc != 0;

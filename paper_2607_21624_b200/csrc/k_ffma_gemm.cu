@@ -1,5 +1,5 @@
-// fp32 GEMMs on the FP32 pipe (plain FFMA: single-pass TF32 cannot hold a 1e-4 relative bound), operands in R-Tile order
-// fetched by TMA: C[m,n] = sum_terms A_t[m,:] B_t[:,n] (+ bias[n]) (+ residual), up to five problems in one launch.
+// fp32 GEMMs on the FP32 pipe, the cross-check of the kernel that runs them on the tensor cores (k_tc_f32.cu; this one is what
+// fbl_plan_set_kernel_path(plan, 1) selects), operands in R-Tile order fetched by TMA: C[m,n] = sum_terms A_t[m,:] B_t[:,n] (+ bias[n]) (+ residual), up to five problems in one launch.
 //
 // A block owns a 64 x 64 tile of C: one producer warp and four compute warps, 4 x 8 results per thread.  Operand tiles
 // lie in shared memory exactly as the R-Tile panels store them (128-byte rows, 128-byte swizzle), and a transposed operand
@@ -18,40 +18,18 @@
 // 312 -> 79 us, 800 x 768 x 768 105 -> 34 us, the four products behind the attention backward at 800 x 768 591 -> 161 us;
 // 4096 x 1024 x 3072 47 TFLOP/s, 64 % of the pipe.  (8 x 8 results on two warps: 100, 52, 187 us; four blocks per SM at
 // 96 registers spill.)
-#include <string.h>
-
-#include "fbl_internal.h"
+#include "f32_gemm.cuh"
 #include "launch_memo.h"
 #include "pdl.cuh"
-#include "tc_common.cuh"
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 32, STAGES = 3;
-constexpr int MAX_TERMS = 4, MAX_PROBLEMS = 5;
-constexpr int COMPUTE = 128, THREADS = COMPUTE + 32;      // a compute thread holds 4 x 8 results
+using f32g::lds4;
+typedef f32g::Group FfmaGroup;
+typedef f32g::Problem FfmaProblem;
 
-struct alignas(64) FfmaProblem {
-  CUtensorMap ta[MAX_TERMS], tb[MAX_TERMS];
-  int n_terms, kblocks[MAX_TERMS];
-  int a_k[MAX_TERMS], b_k[MAX_TERMS];       // 1: the operand's stored rows are K indices
-  int m, n, tiles_m, tiles_n, total_kb;
-  float* c;
-  long long c_rpad;
-  const float* bias;
-  const float* residual;
-  int seq, t_pad;
-  const float* dot_with;                    // fused D = rowsum(C * dot_with) per head (head widths 32 and 64), or nullptr
-  float* dot_out;
-  int dot_hd, dot_hq;
-};
-struct alignas(64) FfmaGroup {
-  FfmaProblem p[MAX_PROBLEMS];
-  int count, slices, reset_status;
-  int32_t* status;
-  uint4* zero_ptr;                                  // chores of the launch, see GemmArgs
-  long long zero_vec;
-};
+constexpr int BM = 64, BN = 64, BK = 32, STAGES = 3;
+constexpr int COMPUTE = 128, THREADS = COMPUTE + 32;      // a compute thread holds 4 x 8 results
 
 struct FfmaLaunch { FfmaGroup G; int grid, serial; };      // a launch made ready
 
@@ -63,11 +41,6 @@ struct Smem {
 constexpr int OUT_LD = BN + 4;              // row pitch of the finished tile in shared memory (over the operand stages)
 static_assert(BM * OUT_LD * 4 <= STAGES * (int)Smem::STAGE, "the finished tile fits the stages");
 
-__device__ __forceinline__ float4 lds4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-  return v;
-}
 typedef unsigned long long f2;              // two fp32 values of one two-wide operation
 __device__ __forceinline__ f2 pack2(float x, float y) { f2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y)); return r; }
 __device__ __forceinline__ float2 unpack2(f2 v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
@@ -179,9 +152,7 @@ __global__ void __launch_bounds__(THREADS, 3) gemm_ffma_kernel(const __grid_cons
   __syncthreads();
   pdl_launch_dependents();
   pdl_wait();
-  if (G.reset_status && blockIdx.x == 0 && threadIdx.x == 0) *G.status = 0;
-  for (long long i = (long long)blockIdx.x * THREADS + threadIdx.x; i < G.zero_vec; i += (long long)gridDim.x * THREADS)
-    G.zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
+  f32g::group_chores(G, threadIdx.x, THREADS);
   // work unit: (problem, tile, slice); the slices of a tile are the blocks of a cluster
   const int slice = blockIdx.x % G.slices;
   int w = blockIdx.x / G.slices, pi = 0;
@@ -217,40 +188,7 @@ __global__ void __launch_bounds__(THREADS, 3) gemm_ffma_kernel(const __grid_cons
   }
   __syncwarp();
   if (G.slices > 1) tc::cluster_sync_all(); else __syncthreads();
-  // This block's share of the tile's rows: the slices' sums in slice order, bias, residual, padding rows, 16-byte stores
-  const int rows = BM / G.slices, r0 = slice * rows;
-  for (int v0 = 0; v0 < rows * (BN / 4); v0 += THREADS) {
-    const int v = v0 + threadIdx.x, m = m0 + r0 + v / (BN / 4), n = n0 + (v % (BN / 4)) * 4;
-    const bool live = v < rows * (BN / 4) && m < P.m && n < P.n;
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    float dot = 0.f;
-    if (live) {
-      const uint32_t addr = base + (uint32_t)((r0 + v / (BN / 4)) * OUT_LD + (v % (BN / 4)) * 4) * 4;
-      if (G.slices == 1) s = lds4(addr);
-      else
-        for (int c = 0; c < G.slices; ++c) {
-          float4 q;
-          asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "r"(tc::map_to_cta(addr, c)));
-          s.x += q.x; s.y += q.y; s.z += q.z; s.w += q.w;
-        }
-      const int64_t off = rt_off<32>(P.c_rpad, m, n);
-      if (P.bias) { s.x += P.bias[n]; s.y += P.bias[n + 1]; s.z += P.bias[n + 2]; s.w += P.bias[n + 3]; }
-      if (P.residual) {
-        const float4 q = *reinterpret_cast<const float4*>(P.residual + off);
-        s.x += q.x; s.y += q.y; s.z += q.z; s.w += q.w;
-      }
-      if (P.t_pad > 0 && m % P.t_pad >= P.seq) s = make_float4(0.f, 0.f, 0.f, 0.f);
-      *reinterpret_cast<float4*>(P.c + off) = s;
-      if (P.dot_with) {
-        const float4 q = *reinterpret_cast<const float4*>(P.dot_with + off);
-        dot = fmaf(s.x, q.x, fmaf(s.y, q.y, fmaf(s.z, q.z, s.w * q.w)));
-      }
-    }
-    if (P.dot_with) {                            // a head is 8 or 16 neighbouring threads (32 or 64 columns)
-      for (int o = P.dot_hd / 8; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      if (live && n % P.dot_hd == 0) P.dot_out[((int64_t)(m / P.t_pad) * P.dot_hq + n / P.dot_hd) * P.t_pad + m % P.t_pad] = dot;
-    }
-  }
+  f32g::finish_tile<BM, BN, OUT_LD, THREADS, false>(P, G.slices, slice, base, m0, n0);
   if (G.slices > 1) tc::cluster_sync_all();      // no block leaves while another may still read its partial tile
 }
 
@@ -289,27 +227,10 @@ bool gemm_ffma_supported(const fbl_plan* p, const GemmArgs& g) {
 
 static cudaError_t make_group(FfmaLaunch& L, const fbl_plan* p, const GemmArgs* gs, int count) {
   FfmaGroup& G = L.G;
-  memset(&G, 0, sizeof(G));
-  G.count = count;
+  const int order[f32g::MAX_PROBLEMS] = {0, 1, 2, 3, 4};
+  if (!f32g::fill_group(G, gs, count, order, BM, BN, BK)) return cudaErrorInvalidValue;
   int tiles = 0;
-  for (int i = 0; i < count; ++i) {
-    const GemmArgs& g = gs[i];
-    FfmaProblem& P = G.p[i];
-    P.n_terms = g.n_terms; P.m = g.m; P.n = g.n;
-    for (int t = 0; t < g.n_terms; ++t) {
-      const GemmTerm& tm = g.t[t];
-      P.kblocks[t] = (tm.k + BK - 1) / BK;
-      P.total_kb += P.kblocks[t];
-      P.a_k[t] = tm.a_trans ? 1 : 0;
-      P.b_k[t] = tm.b_trans ? 0 : 1;
-      if (!fbl_encode_f32_rtile_map(&P.ta[t], tm.a, tm.a_rpad, (tm.a_trans ? g.m : tm.k) / 32, P.a_k[t] ? BK : BM, P.a_k[t] ? 2 : 1) ||
-          !fbl_encode_f32_rtile_map(&P.tb[t], tm.b, tm.b_rpad, (tm.b_trans ? tm.k : g.n) / 32, P.b_k[t] ? BK : BN, P.b_k[t] ? 2 : 1))
-        return cudaErrorInvalidValue;
-    }
-    P.tiles_m = (g.m + BM - 1) / BM; P.tiles_n = (g.n + BN - 1) / BN;
-    P.c_rpad = g.c_rpad; P.seq = g.seq; P.t_pad = g.t_pad; P.dot_hd = g.dot_hd; P.dot_hq = g.dot_hq;
-    tiles += P.tiles_m * P.tiles_n;
-  }
+  for (int i = 0; i < count; ++i) tiles += G.p[i].tiles_m * G.p[i].tiles_n;
   G.slices = choose_slices(p->sm_count, G);
   L.grid = tiles * G.slices;
   // fp32 attention waits before it requests anything, so no launch has to be serial; but blocks that all fit the SMs at once
@@ -318,27 +239,13 @@ static cudaError_t make_group(FfmaLaunch& L, const fbl_plan* p, const GemmArgs* 
   return cudaFuncSetAttribute(gemm_ffma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem::TOTAL);
 }
 
-static bool point_group(FfmaGroup& G, const GemmArgs* gs, int32_t* status) {
-  G.status = status;
-  G.zero_ptr = (uint4*)gs[0].zero_ptr; G.zero_vec = (long long)(gs[0].zero_bytes / 16); G.reset_status = gs[0].reset_status;
-  bool ok = true;
-  for (int i = 0; i < G.count; ++i) {
-    const GemmArgs& g = gs[i];
-    FfmaProblem& P = G.p[i];
-    for (int t = 0; t < P.n_terms; ++t) ok = ok && fbl_map_set_base(&P.ta[t], g.t[t].a) && fbl_map_set_base(&P.tb[t], g.t[t].b);
-    P.c = (float*)g.c; P.bias = g.bias; P.residual = (const float*)g.residual;
-    P.dot_with = (const float*)g.dot_with; P.dot_out = g.dot_out;
-  }
-  return ok;
-}
-
 cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st) {
-  if (count < 1 || count > MAX_PROBLEMS) return cudaErrorInvalidValue;
+  if (count < 1 || count > f32g::MAX_PROBLEMS) return cudaErrorInvalidValue;
   LaunchKey key;
   gemm_group_key(key, gs, count);
   return LaunchMemo<FfmaLaunch, 12>::run(p, FBL_MEMO_FFMA_GEMM, key,
       [&](FfmaLaunch& L) { return make_group(L, p, gs, count); },
-      [&](FfmaLaunch& L) { return point_group(L.G, gs, status); },
+      [&](FfmaLaunch& L) { return f32g::point_group(L.G, gs, status); },
       [&](const FfmaLaunch& L) {
         if (L.G.slices > 1) return launch_cluster(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G.slices, !L.serial, L.G);
         return L.serial ? launch_serial(gemm_ffma_kernel, dim3(L.grid), dim3(THREADS), Smem::TOTAL, st, L.G)
@@ -351,6 +258,7 @@ cudaError_t run_gemm_group(const fbl_plan* p, GemmArgs* gs, int count, int32_t* 
   if (gemm_group_tc(p, gs, count)) return launch_gemm_tc_group(p, gs, count, status, st, launch_id);
   bool ffma = true;
   for (int i = 0; i < count; ++i) ffma = ffma && gemm_ffma_supported(p, gs[i]);
+  if (ffma && !p->ffma_only) return launch_gemm_tc_f32_group(p, gs, count, status, st);
   if (ffma) return launch_gemm_ffma_group(p, gs, count, status, st);
   if (p->d.dtype == FBL_DTYPE_FP32) return cudaErrorInvalidValue;      // no step forms such a product
   *kernels = count;

@@ -84,6 +84,65 @@ def test_fp32_gemm_tiles_and_slices(cfg):
     check(cfg)
 
 
+@pytest.mark.parametrize("slices", ["1", "2", "4", "8"])
+@pytest.mark.parametrize("bn", ["64", "128"])
+def test_fp32_products_on_every_tile(bn, slices, monkeypatch):
+    # tiles that end in the middle of a panel both ways, reductions of fewer 64-column blocks than slices and of a half one at
+    # the end, all operand orientations, fused row reduction, residual, padding rows
+    monkeypatch.setenv("FBL_F32_BN", bn)
+    monkeypatch.setenv("FBL_F32_SLICES", slices)
+    check(LayerConfig("ft1", 3, 67, 160, 5, 1, 32, "fp32", "rmsnorm", True, True, True, 1e-5, 228, 0.1))
+    check(LayerConfig("ft2", 1, 390, 352, 3, 3, 64, "fp32", "layernorm", False, False, False, 1e-5, 229, 0.05))
+
+
+def _mlp_outputs(cfg, inp, path):
+    import numpy as np
+    from paper_2607_21624_b200.mlp import MlpRunner
+    run = MlpRunner(cfg, guard_bytes=4096)
+    run.plan.set_kernel_path(path)
+    run.load_inputs(inp)
+    run.step()
+    assert run.status() == 0 and run.guards_intact() == []
+    return {n: np.asarray(run.fetch(n), dtype=np.float64) for n in ("Y", "dX", "dW1", "dW2", "db1", "db2", "dgamma")}
+
+
+def test_fp32_products_are_no_further_off_than_multiply_adds():
+    # against 64 bits; both kernels' sums are within a few units of the last place, so no element-wise bound is tighter than this
+    import numpy as np
+    from fbl_inputs import make_mlp_inputs
+    from oracle import mlp as orc
+    cfg = MlpConfig("fa1", 2, 300, 512, 768, "fp32", "layernorm", "gelu", True, False, 1e-5, 230, 0.05)
+    inp = make_mlp_inputs(cfg, affine_noise=True)
+    Y, _, grads = orc.mlp_fwd_bwd(cfg, inp)
+    ref = dict(grads, Y=Y)
+    off = lambda got, n: np.linalg.norm(got[n] - ref[n]) / np.linalg.norm(ref[n])
+    default, ffma = (_mlp_outputs(cfg, inp, path) for path in (0, 1))
+    for n in ("Y", "dX", "dW1", "dW2"):
+        assert off(default, n) <= off(ffma, n), (n, off(default, n), off(ffma, n))
+
+
+def test_fp32_products_of_operands_without_parts():
+    # infinities, NaN, and values that round to infinity in bf16: the same results as plain multiply-adds
+    import numpy as np
+    from fbl_inputs import make_mlp_inputs
+    cfg = MlpConfig("fa2", 1, 150, 160, 192, "fp32", "rmsnorm", "gelu", True, False, 1e-5, 231, 0.05)
+    inp = dict(make_mlp_inputs(cfg, affine_noise=True))
+    for n in ("W2", "dY"):
+        inp[n] = np.array(inp[n], copy=True)
+    inp["W2"][3, 5], inp["W2"][9, 7], inp["W2"][70, 130] = np.inf, -np.inf, 3.395e38
+    flat = inp["dY"].reshape(-1, cfg.d_model)
+    flat[11, 40], flat[77, 2] = np.nan, np.inf
+    default, ffma = (_mlp_outputs(cfg, inp, path) for path in (0, 1))
+    for n, want in ffma.items():
+        got = default[n]
+        assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want)), n
+        assert np.array_equal(got[np.isinf(got)], want[np.isinf(want)]), n
+        m = np.isfinite(want)
+        if m.any():
+            assert np.linalg.norm((got[m] - want[m]) / np.abs(want[m]).max()) <= 1e-5 * np.linalg.norm(want[m] / np.abs(want[m]).max()), n
+    assert np.isinf(ffma["Y"]).any() and np.isfinite(ffma["Y"]).any()
+
+
 @pytest.mark.parametrize("pair", ["-1", "1"], ids=["by-cost", "pairs"])
 @pytest.mark.parametrize("cfg", [
     # columns that are not whole tiles, on every tile shape: one to a few tiles of rows, an odd number of 64-wide panels
