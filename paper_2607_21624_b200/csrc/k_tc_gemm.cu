@@ -432,8 +432,13 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
   if (!G.late_trigger) pdl_launch_dependents();
 
   if (warp == 0 && lane == 0) {
-    // ---- TMA producer ----------------------------------------------------------------------
-    int it = 0;
+    // ---- TMA producer.  Its loop is kept short (stage, phase and coordinates advance by additions, nothing is decided per
+    // k-block): operands arrive from L2 about as fast as the products take them, so that a stage that is free and not yet
+    // requested is time lost, most of all with CTA pairs.  (With a case per operand, a division and a test for prefilled
+    // stages per k-block: gated feed-forward step of 4096 x 2048 x 8192 1131 us instead of 1088, 8192 x 4096 attention step
+    // 5190 instead of 5060, Whisper-shaped cross-attention step 189.8 instead of 186.8.)
+    int s = 0;
+    uint32_t ph = 1;
     bool ok = true;
     TileCoord tcd;
     // Weights do not depend on the kernel before this one: their tiles for the first stages of the first
@@ -457,22 +462,27 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
     for (int w = blockIdx.x; ok && tile_at<BN>(G, w, &tcd); w += gridDim.x) {
       const TcProblem& P = G.p[tcd.prob];
       for (int t = 0; t < P.n_terms && ok; ++t) {
-        const int kb_begin = t == 0 ? tcd.kb0 : 0, kb_end = t == 0 ? tcd.kb1 : P.kblocks[t];
-        for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
-          const uint32_t sa = base + s * SP::STAGE, sb = sa + SP::A_BYTES;
-          const bool pre = it < prefilled;                 // this stage's barrier is armed and its B tile on its way
-          if (!pre) {
-            if (!tc::mbar_wait(empty(s), ph ^ 1, status, 101)) { ok = false; break; }
-            tc::mbar_expect_tx(full(s), SP::STAGE);
-          }
-          if (P.a_mn[t]) tc::tma_load_3d(sa, &P.ta[t], full(s), 0, kb * BK, tcd.m0 / 64);
-          else tc::tma_load_3d(sa, &P.ta[t], full(s), 0, tcd.m0, kb);
-          if (!pre) {
-            if (P.b_mn[t]) tc::tma_load_3d(sb, &P.tb[t], full(s), 0, kb * BK, tcd.n0 / 64);
-            else tc::tma_load_3d(sb, &P.tb[t], full(s), 0, tcd.n0, kb);
-          }
+        int kb = t == 0 ? tcd.kb0 : 0;
+        const int kb_end = t == 0 ? tcd.kb1 : P.kblocks[t];
+        const CUtensorMap *ta = &P.ta[t], *tb = &P.tb[t];
+        const int a_mn = P.a_mn[t], b_mn = P.b_mn[t];
+        int ay = a_mn ? kb * BK : tcd.m0, az = a_mn ? tcd.m0 / 64 : kb, by = b_mn ? kb * BK : tcd.n0, bz = b_mn ? tcd.n0 / 64 : kb;
+        const int ady = a_mn ? BK : 0, adz = a_mn ? 0 : 1, bdy = b_mn ? BK : 0, bdz = b_mn ? 0 : 1;
+        auto advance = [&] {
+          ay += ady; az += adz; by += bdy; bz += bdz;
+          if (++s == STAGES) { s = 0; ph ^= 1; }
+        };
+        for (; prefilled > 0; --prefilled, ++kb) {         // the barrier is armed and the B tile on its way
+          tc::tma_load_3d(base + s * SP::STAGE, ta, full(s), 0, ay, az);
+          advance();
+        }
+        for (; kb < kb_end; ++kb) {
+          const uint32_t sa = base + s * SP::STAGE;
+          if (!tc::mbar_wait(empty(s), ph, status, 101)) { ok = false; break; }
+          tc::mbar_expect_tx(full(s), SP::STAGE);
+          tc::tma_load_3d(sa, ta, full(s), 0, ay, az);
+          tc::tma_load_3d(sa + SP::A_BYTES, tb, full(s), 0, by, bz);
+          advance();
         }
       }
     }
@@ -622,27 +632,31 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer (both CTAs): own A rows, own half of B's columns; bytes counted on the leader's barrier ----
-    int it = 0;
+    int s = 0;
+    uint32_t ph = 1;
     bool ok = true;
     TileCoord tcd;
+    const uint32_t full0 = tc::map_to_cta(full(0), 0);
     pdl_wait();
     if (G.late_trigger) late_trigger(G);
     for (int w = pair_id; ok && pair_tile_at(G, w, &tcd); w += n_pairs) {
       const TcProblem& P = G.p[tcd.prob];
       const int m0 = tcd.m0 + (int)rank * 128, n0 = tcd.n0 + (int)rank * 128;
       for (int t = 0; t < P.n_terms && ok; ++t) {
-        const int kb_begin = t == 0 ? tcd.kb0 : 0, kb_end = t == 0 ? tcd.kb1 : P.kblocks[t];
-        for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
-          const uint32_t sa = base + s * SP::STAGE, sb = sa + SP::A_BYTES;
-          if (!tc::mbar_wait(empty(s), ph ^ 1, status, 111)) { ok = false; break; }
+        int kb = t == 0 ? tcd.kb0 : 0;
+        const int kb_end = t == 0 ? tcd.kb1 : P.kblocks[t];
+        const CUtensorMap *ta = &P.ta[t], *tb = &P.tb[t];
+        const int a_mn = P.a_mn[t], b_mn = P.b_mn[t];
+        int ay = a_mn ? kb * BK : m0, az = a_mn ? m0 / 64 : kb, by = b_mn ? kb * BK : n0, bz = b_mn ? n0 / 64 : kb;
+        const int ady = a_mn ? BK : 0, adz = a_mn ? 0 : 1, bdy = b_mn ? BK : 0, bdz = b_mn ? 0 : 1;
+        for (; kb < kb_end; ++kb) {
+          const uint32_t sa = base + s * SP::STAGE, fb = full0 + 8u * s;
+          if (!tc::mbar_wait(empty(s), ph, status, 111)) { ok = false; break; }
           if (rank == 0) tc::mbar_expect_tx(full(s), 2 * SP::STAGE);
-          const uint32_t fb = tc::map_to_cta(full(s), 0);
-          if (P.a_mn[t]) tc::tma_load_3d_pair(sa, &P.ta[t], fb, 0, kb * BK, m0 / 64);
-          else tc::tma_load_3d_pair(sa, &P.ta[t], fb, 0, m0, kb);
-          if (P.b_mn[t]) tc::tma_load_3d_pair(sb, &P.tb[t], fb, 0, kb * BK, n0 / 64);
-          else tc::tma_load_3d_pair(sb, &P.tb[t], fb, 0, n0, kb);
+          tc::tma_load_3d_pair(sa, ta, fb, 0, ay, az);
+          tc::tma_load_3d_pair(sa + SP::A_BYTES, tb, fb, 0, by, bz);
+          ay += ady; az += adz; by += bdy; bz += bdz;
+          if (++s == STAGES) { s = 0; ph ^= 1; }
         }
       }
     }
