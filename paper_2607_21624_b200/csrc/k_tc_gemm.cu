@@ -568,7 +568,11 @@ struct PairSmem {
   static constexpr uint32_t TOTAL = BAR_OFF + 8 * N_BARS + 16 + 1024;
 };
 
-// work list in 256 x 256 tiles (ksplit slices as in tile_at); m0 / n0 are the pair's
+// work list in 256 x 256 tiles (ksplit slices as in tile_at); m0 / n0 are the pair's.  Tall problems go in bands of eight row
+// tiles: the 74 tiles at work then share eight row tiles and nine column tiles of operands instead of 32 and two or three, which
+// L2 holds (8192 x 4096 attention step: 5060 -> 4945 us, its four product launches 535, 172, 378, 1191 -> 505, 167, 364, 1131; bands
+// of 16 the same).  Up to 16 row tiles fit as they are (4096 x 2048 x 8192 feed-forward in bands of eight: 88 -> 92 us a launch).
+constexpr int PAIR_BAND = 8, PAIR_BAND_FROM = 16;
 __device__ __forceinline__ bool pair_tile_at(const TcGroup& G, int w, TileCoord* tc_out) {
   for (int p = 0; p < G.count; ++p) {
     const TcProblem& P = G.p[p];
@@ -577,8 +581,9 @@ __device__ __forceinline__ bool pair_tile_at(const TcGroup& G, int w, TileCoord*
     if (w < units) {
       const int slice = w % P.ksplit, t = w / P.ksplit;
       tc_out->prob = p;
-      tc_out->m0 = (t % tm) * 256;
-      tc_out->n0 = (t / tm) * 256;
+      const int band = tm > PAIR_BAND_FROM ? PAIR_BAND : tm, at = t / (band * tn), h = min(band, tm - at * band), u = t - at * band * tn;
+      tc_out->m0 = (at * band + u % h) * 256;
+      tc_out->n0 = (u / h) * 256;
       const int per = (P.kblocks[0] + P.ksplit - 1) / P.ksplit;
       tc_out->kb0 = slice * per;
       tc_out->kb1 = min(P.kblocks[0], (slice + 1) * per);

@@ -160,6 +160,12 @@ def test_ragged_columns_on_every_gemm_tile(cfg, pair, monkeypatch):
     check(cfg)
 
 
+def test_bands_of_row_tiles(monkeypatch):
+    # CTA pairs: 17 row tiles are two bands of eight and one of a single, partly filled tile; several column tiles
+    monkeypatch.setenv("FBL_GEMM_PAIR", "1")
+    check(MlpConfig("rb1", 1, 4300, 192, 576, "bf16", "rmsnorm", "gelu", False, True, 1e-5, 248, 0.05))
+
+
 @pytest.mark.parametrize("cfg", [
     # one key tile (dQ straight from the block), with one and several query tiles, grouped heads, both head widths
     LayerConfig("sa1", 2, 128, 128, 4, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 251, 0.05),
