@@ -19,8 +19,8 @@
 // 272 KB at 128 B/clk, where A's parts in shared memory would make it 416 KB (the products take 1536 clk).
 // Measured against the FP32 pipe (k_ffma_gemm.cu), us: 800 x 768 outputs, 768 columns to reduce: three problems 74 -> 22.8, one
 // 31 -> 15.3, dWo with dA 60 -> 23.8, dWq, dWk, dWv with dXn 159 -> 47.7; 2048 x 2048 x 2048 358 -> 93 (185 TFLOP/s); 64 x 64 x 64
-// 6.5 -> 5.5.  Error against 64 bits relative to the result's norm: 0.8e-7 to 1.9e-7 at 64 to 4096 columns, multiply-adds one after
-// another 1.4e-7 to 9.9e-7 (0.9 of theirs at most, over 56 products).
+// 6.5 -> 5.5.  Error against 64 bits relative to the result's norm: 0.4e-7 to 1.8e-7 at 32 to 4096 columns, multiply-adds one after
+// another 1.0e-7 to 9.9e-7; whole steps' outputs: 0.3 to 1.0 of theirs.
 #include "f32_gemm.cuh"
 #include "launch_memo.h"
 #include "pdl.cuh"
@@ -51,19 +51,8 @@ struct Smem {
 constexpr uint32_t TMEM_COLS = 512;
 template <int BN> __device__ constexpr uint32_t a_col(int set, int part) { return 2 * BN + 96 * set + 32 * part; }
 
-// Two fp32 values as three packed pairs of bf16.
-__device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-  const float2 minus = make_float2(-1.f, -1.f);
-  float2 v = make_float2(x, y);
-  hi = tc::pack_bf16(v.x, v.y);
-  v = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), minus, v);
-  mid = tc::pack_bf16(v.x, v.y);
-  v = __ffma2_rn(make_float2(__uint_as_float(mid << 16), __uint_as_float(mid & 0xffff0000u)), minus, v);
-  lo = tc::pack_bf16(v.x, v.y);
-}
-__device__ __forceinline__ void sts4(uint32_t a, const uint32_t* v) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
-}
+using tc::split3;
+using tc::sts4;
 
 template <int BN>
 __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_constant__ Group G) {
@@ -189,7 +178,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
         }
         uint32_t p[3][8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], p[0][k], p[1][k], p[2][k]);
+        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], tc::LIFT_4, p[0][k], p[1][k], p[2][k]);
 #pragma unroll
         for (int i = 0; i < 3; ++i) tc::tmem_st8(lane_addr + a_col<BN>(b, i) + 8 * h, p[i]);
       }
@@ -218,7 +207,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
         }
         uint32_t p[3][8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], p[0][k], p[1][k], p[2][k]);
+        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], 0.f, p[0][k], p[1][k], p[2][k]);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll

@@ -188,6 +188,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -259,6 +263,36 @@ __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(_
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// Two fp32 values as three packed pairs of bf16: the rounding, the rounding of what that leaves, and the rest (24 bits; `rest` is
+// not finite if and only if a value has no such parts).
+// `lift`: a share of the value that the rest is raised by.  The tensor core's additions round toward zero: a sum of products
+// (16 columns to an instruction, the small parts' first) comes out smaller by 6.0e-8 of itself, on average and for every size and
+// sign of the operands that was tried, after four full-size additions, 4.5e-8 after two, some 3.7e-8 after one.  Such losses
+// would add up from product to product, where rounding to nearest averages out.  So operands are raised by that much, between them
+// (products: error against 64 bits 7.7e-8 -> 4.9e-8 of the result's norm at 64 columns, 1.0e-7 -> 8e-8 at 768).
+constexpr float LIFT_4 = 6.03e-8f, LIFT_2 = 4.47e-8f, LIFT_1 = 3.7e-8f;
+__device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& hi, uint32_t& mid, uint32_t& lo, float2& rest) {
+  const float2 minus = make_float2(-1.f, -1.f), whole = make_float2(x, y);
+  hi = pack_bf16(x, y);
+  float2 v = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), minus, whole);
+  mid = pack_bf16(v.x, v.y);
+  v = __ffma2_rn(make_float2(__uint_as_float(mid << 16), __uint_as_float(mid & 0xffff0000u)), minus, v);
+  rest = __ffma2_rn(whole, make_float2(lift, lift), v);
+  lo = pack_bf16(rest.x, rest.y);
+}
+__device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  float2 rest;
+  split3(x, y, lift, hi, mid, lo, rest);
+}
+__device__ __forceinline__ void sts4(uint32_t a, const uint32_t* v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
 }
 
 // ---- CTA pairs (cta_group::2): one MMA over two SMs, each holding 128 rows of A and of the accumulator and half
