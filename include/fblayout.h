@@ -405,9 +405,9 @@ int fbl_xattn_bwd(const fbl_plan* plan, const void* dY, const void* X, const voi
                   void* dWq, void* dWk, void* dWv, void* dWo, float* dbq, float* dbk, float* dbv, float* dbo,
                   float* dgamma, float* dbeta, void* scratch, void* stream);
 
-/* Kernel family used by later calls on this plan: 0 = default (tcgen05 tensor-core kernels for bf16 and for the products of fp32,
- * whose operands they take in three bf16 parts; FFMA kernels for fp32 attention and for the attention backward of bf16 layers with
- * less than 128 token rows on either side), 1 = FFMA kernels only (fp32 arithmetic on the same layout; lets a caller cross-check
+/* Kernel family used by later calls on this plan: 0 = default (tcgen05 tensor-core kernels for bf16 and, with operands in three bf16
+ * parts, for fp32; FFMA kernels for fp32 attention of short sequences or heads of 128 and for the attention backward of bf16 layers
+ * with less than 128 token rows on either side), 1 = FFMA kernels only (fp32 arithmetic on the same layout; lets a caller cross-check
  * the tensor-core path on the device). */
 int fbl_plan_set_kernel_path(fbl_plan* plan, int path);
 

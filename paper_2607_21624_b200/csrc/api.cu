@@ -420,7 +420,9 @@ int fbl_unpack(const fbl_plan* plan, int tensor_id, const void* tiled_dev, void*
 cudaError_t run_attn_fwd(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse, int32_t* status, cudaStream_t st) {
   switch (attn_fwd_kernels(p)) {
     case ATTN_TC: return launch_attn_fwd_tc(p, Q, K, V, A, lse, status, st);
-    case ATTN_FFMA: return launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st);
+    case ATTN_FFMA:
+      if (attn_tc_f32_supported(p)) return launch_attn_fwd_tc_f32(p, Q, K, V, A, lse, status, st);
+      return launch_attn_fwd_ffma(p, Q, K, V, A, lse, status, st);
     default: return launch_attn_fwd_simt(p, Q, K, V, A, lse, st);
   }
 }
@@ -430,7 +432,9 @@ cudaError_t run_attn_bwd(const fbl_plan* p, const void* Q, const void* K, const 
                          const float2* rope) {
   switch (attn_bwd_kernels(p)) {
     case ATTN_TC: return launch_attn_bwd_tc(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope);
-    case ATTN_FFMA: return launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope);
+    case ATTN_FFMA:
+      if (attn_tc_f32_supported(p)) return launch_attn_bwd_tc_f32(p, Q, K, V, A, dA, lse, dvec, dQ, dK, dV, dvec_ready, status, st);
+      return launch_attn_bwd_ffma(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, status, st, rope);
     default: return launch_attn_bwd_simt(p, Q, K, V, A, dA, lse, dvec, dqacc, dQ, dK, dV, dvec_ready, st);
   }
 }

@@ -33,7 +33,7 @@ template <> __device__ __forceinline__ float from_f<float>(float v) { return v; 
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 struct FblMemoBase { virtual ~FblMemoBase() {} };      // launch_memo.h
-enum { FBL_MEMO_TC_GEMM = 0, FBL_MEMO_FFMA_GEMM, FBL_MEMO_TC_FWD, FBL_MEMO_TC_BWD, FBL_MEMO_FFMA_ATTN, FBL_MEMO_TC_F32_GEMM, FBL_MEMO_COUNT };
+enum { FBL_MEMO_TC_GEMM = 0, FBL_MEMO_FFMA_GEMM, FBL_MEMO_TC_FWD, FBL_MEMO_TC_BWD, FBL_MEMO_FFMA_ATTN, FBL_MEMO_TC_F32_GEMM, FBL_MEMO_TC_F32_FWD, FBL_MEMO_TC_F32_BWD, FBL_MEMO_COUNT };
 
 struct fbl_plan {
   fbl_layer_desc d;
@@ -255,13 +255,20 @@ cudaError_t launch_colsum(int dtype, const void* M, int64_t rows, int64_t cols, 
 size_t colsum_scratch_bytes(int64_t rows, int64_t cols);
 cudaError_t launch_colsum_group(int dtype, const ColsumGroup& G, cudaStream_t st);
 
-// fp32 arithmetic (k_ffma_attn.cu): fp32 storage, and the backward of bf16 storage.  The latter adds into dQ or, bf16, into dqacc,
+// fp32 arithmetic (k_ffma_attn.cu): fp32 storage where not attn_tc_f32_supported, and the backward of bf16 storage.  The latter adds into dQ or, bf16, into dqacc,
 // zeroed by the caller; dqacc it rounds and, with `rope`, turns
 cudaError_t launch_attn_fwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                  int32_t* status, cudaStream_t st);
 cudaError_t launch_attn_bwd_ffma(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A, const void* dA,
                                  const float* lse, float* dvec, float* dqacc, void* dQ, void* dK, void* dV, bool dvec_ready,
                                  int32_t* status, cudaStream_t st, const float2* rope);
+// fp32 storage on the tensor cores (k_tc_f32_attn.cu): heads of 32 and 64
+bool attn_tc_f32_supported(const fbl_plan* p);
+cudaError_t launch_attn_fwd_tc_f32(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
+                                   int32_t* status, cudaStream_t st);
+cudaError_t launch_attn_bwd_tc_f32(const fbl_plan* p, const void* Q, const void* K, const void* V, const void* A, const void* dA,
+                                   const float* lse, float* dvec, void* dQ, void* dK, void* dV, bool dvec_ready, int32_t* status,
+                                   cudaStream_t st);       // adds into dQ, zeroed by the caller
 // bf16 storage in fp32 arithmetic (cross-check)
 cudaError_t launch_attn_fwd_simt(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse,
                                  cudaStream_t st);

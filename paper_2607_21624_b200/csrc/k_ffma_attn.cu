@@ -1,6 +1,7 @@
 // Attention in fp32 arithmetic on the FP32 pipe (plain FFMA, no tensor cores), operands in R-Tile order fetched by TMA into
-// the swizzled 128-byte rows they are stored as (see k_ffma_gemm.cu for the operand fragments): fp32 storage, and the backward
-// of bf16 storage where P and dS stay in fp32 (attn_fp32), whose operands are widened on their way to registers.
+// the swizzled 128-byte rows they are stored as (see k_ffma_gemm.cu for the operand fragments): fp32 storage (short sequences
+// and heads of 128: the others run on the tensor cores, k_tc_f32_attn.cu), and the backward of bf16 storage where P and dS stay in
+// fp32 (attn_fp32), whose operands are widened on their way to registers.
 //
 // Both kernels give a warp 16 rows of the score tile and all its columns (lane = (row group tm of 4, column group tn of
 // 8), 4 x 8 scores per thread), so that the softmax needs only shuffles and the rows of P (forward) or of P^T and dS^T

@@ -95,6 +95,59 @@ def test_fp32_products_on_every_tile(bn, slices, monkeypatch):
     check(LayerConfig("ft2", 1, 390, 352, 3, 3, 64, "fp32", "layernorm", False, False, False, 1e-5, 229, 0.05))
 
 
+@pytest.mark.parametrize("cfg", [
+    # fp32 attention on the tensor cores: its shortest sequences, tiles of 64 and 128 rows that end early, at their edge and one
+    # past it on either side, grouped heads with one block and with a cluster to a key tile, both head widths, masks
+    LayerConfig("fc1", 2, 33, 128, 2, 2, 64, "fp32", "layernorm", True, True, True, 1e-5, 232, 0.1),
+    LayerConfig("fc2", 3, 65, 96, 4, 1, 32, "fp32", "rmsnorm", False, True, False, 1e-5, 233, 0.1),
+    LayerConfig("fc3", 1, 128, 128, 2, 1, 64, "fp32", "layernorm", True, False, False, 1e-5, 234, 0.1),
+    LayerConfig("fc4", 2, 129, 64, 3, 3, 32, "fp32", "rmsnorm", True, False, True, 1e-5, 235, 0.1),
+    LayerConfig("fc5", 1, 450, 192, 6, 2, 64, "fp32", "layernorm", True, True, False, 1e-5, 236, 0.1),
+    LayerConfig("fc6", 70, 192, 64, 3, 1, 64, "fp32", "layernorm", False, False, False, 1e-5, 237, 0.1),
+    XattnConfig("fc7", 2, 9, 200, 96, 64, 4, 2, 32, "fp32", "layernorm", True, True, 1e-5, 238, 0.1),
+    XattnConfig("fc8", 1, 260, 7, 64, 96, 2, 1, 64, "fp32", "rmsnorm", False, True, 1e-5, 239, 0.1),
+], ids=lambda c: c.name)
+def test_fp32_attention_on_tensor_cores(cfg):
+    check(cfg)
+
+
+@pytest.mark.parametrize("head_dim", [32, 64])
+def test_fp32_attention_of_operands_without_parts(head_dim):
+    # infinities among V and among dA: the same results as plain multiply-adds, and finite columns stay finite
+    import numpy as np
+    from fbl_inputs import make_inputs
+    from paper_2607_21624_b200 import LayerRunner
+    cfg = LayerConfig("fi1", 2, 150, 128, 4, 2, head_dim, "fp32", "layernorm", False, True, False, 1e-5, 240, 0.1)
+    inp = dict(make_inputs(cfg, affine_noise=True))
+    outs = {}
+    for path in (0, 1):
+        for case in ("V", "dA"):
+            run = LayerRunner(cfg, guard_bytes=4096)
+            run.plan.set_kernel_path(path)
+            changed = dict(inp)
+            if case == "V":
+                changed["bv"] = np.array(inp["bv"], copy=True)
+                changed["bv"][5], changed["bv"][head_dim + 9] = np.inf, -np.inf
+            else:
+                changed["dY"] = np.array(inp["dY"], copy=True)
+                changed["dY"].reshape(-1, cfg.d_model)[200, 7] = np.inf     # dA of one token is infinite
+            run.load_inputs(changed)
+            run.step()
+            assert run.status() == 0 and run.guards_intact() == []
+            outs[path, case] = {n: np.asarray(run.saved_view(n), dtype=np.float64) for n in ("A", "LSE", "dA", "dQ", "dK", "dV")}
+    for case, names in (("V", ("A", "LSE")), ("dA", ("A", "LSE", "dA", "dQ", "dK", "dV"))):
+        for n in names:
+            got, want = outs[0, case][n], outs[1, case][n]
+            assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want)), (case, n)
+            assert np.array_equal(got[np.isinf(got)], want[np.isinf(want)]), (case, n)
+            m = np.isfinite(want)
+            if not m.any():
+                continue
+            scale = np.abs(want[m]).max()
+            assert np.linalg.norm((got[m] - want[m]) / scale) <= 1e-5 * np.linalg.norm(want[m] / scale), (case, n)
+    assert np.isinf(outs[1, "V"]["A"]).any() and not np.isfinite(outs[1, "dA"]["dA"]).all()
+
+
 def _mlp_outputs(cfg, inp, path):
     import numpy as np
     from paper_2607_21624_b200.mlp import MlpRunner
