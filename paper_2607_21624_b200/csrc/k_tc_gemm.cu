@@ -1189,8 +1189,10 @@ enum TileKind { TILE_NARROW = 0, TILE_WIDE, TILE_PAIR, TILE_SLIM };
 struct TileCost { int m, n; double kb, unit, epilogue, fixed; };      // extents; clocks per k-block, per unit, of an epilogue, per launch
 // Clocks from a sweep of the four launches of a layer over 64 to 6300 tokens and widths of 320 to 3264 columns.  A
 // k-block of a wide tile costs less than two of a narrow one (operands are re-read half as often per flop), a pair's
-// less still, but pairs start later; with few k-blocks the epilogue of the tile before is what a tile waits for.
-const TileCost TILE_COST[4] = {{128, 128, 545, 800, 1600, 0}, {128, 256, 710, 900, 3600, 0}, {256, 256, 675, 900, 3600, 3500}, {128, 64, 400, 800, 1600, 0}};
+// less still (675 before their loading loop was shortened; with 640 in its place the ViT-Base step went from 181.3 to 179.9 us, the
+// Llama-1B-shaped one from 482 to 478; 640 with 2000 a launch, or 610 with 1000, cost the feed-forward and adapter steps 1 to 4 %),
+// but pairs start later; with few k-blocks the epilogue of the tile before is what a tile waits for.
+const TileCost TILE_COST[4] = {{128, 128, 545, 800, 1600, 0}, {128, 256, 710, 900, 3600, 0}, {256, 256, 640, 900, 3600, 3500}, {128, 64, 400, 800, 1600, 0}};
 struct TileWork { long long m; int n, kb, split; };
 
 // Clocks of the longest block (pair) when the persistent kernel deals the units of a group's problems out in turn.  (Of a
