@@ -405,7 +405,7 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
   auto acc_full = [&](int a) { return bars + 8u * (2 * STAGES + a); };
   auto acc_empty = [&](int a) { return bars + 8u * (2 * STAGES + 2 + a); };
   const uint32_t slot = bars + 8 * SP::N_BARS;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   int32_t* status = G.status;
   constexpr uint32_t TMEM_COLS = 2 * BN;                 // two fp32 accumulators of BN columns
 
@@ -429,9 +429,11 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   if (!G.late_trigger) pdl_launch_dependents();
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
+    const bool leader = tc::elect_one();
     // ---- TMA producer.  Its loop is kept short (stage, phase and coordinates advance by additions, nothing is decided per
     // k-block): operands arrive from L2 about as fast as the products take them, so that a stage that is free and not yet
     // requested is time lost, most of all with CTA pairs.  (With a case per operand, a division and a test for prefilled
@@ -446,11 +448,11 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
     int prefilled = 0;
     if (tile_at<BN>(G, blockIdx.x, &tcd) && G.p[tcd.prob].b_static && G.p[tcd.prob].ksplit == 1) {
       const TcProblem& P = G.p[tcd.prob];
-      tc::tma_prefetch_desc(&P.ta[0]);
-      tc::tma_prefetch_desc(&P.tb[0]);
+      if (leader) { tc::tma_prefetch_desc(&P.ta[0]); tc::tma_prefetch_desc(&P.tb[0]); }
       const int n = P.kblocks[0] < STAGES ? P.kblocks[0] : STAGES;
       for (int kb = 0; kb < n; ++kb) {
         const uint32_t sb = base + kb * SP::STAGE + SP::A_BYTES;
+        if (!leader) continue;
         tc::mbar_expect_tx(full(kb), SP::STAGE);
         if (P.b_mn[0]) tc::tma_load_3d(sb, &P.tb[0], full(kb), 0, kb * BK, tcd.n0 / 64);
         else tc::tma_load_3d(sb, &P.tb[0], full(kb), 0, tcd.n0, kb);
@@ -458,7 +460,7 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
       prefilled = n;
     }
     pdl_wait();
-    if (G.late_trigger) late_trigger(G);
+    if (G.late_trigger && leader) late_trigger(G);
     for (int w = blockIdx.x; ok && tile_at<BN>(G, w, &tcd); w += gridDim.x) {
       const TcProblem& P = G.p[tcd.prob];
       for (int t = 0; t < P.n_terms && ok; ++t) {
@@ -473,23 +475,26 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
           if (++s == STAGES) { s = 0; ph ^= 1; }
         };
         for (; prefilled > 0; --prefilled, ++kb) {         // the barrier is armed and the B tile on its way
-          tc::tma_load_3d(base + s * SP::STAGE, ta, full(s), 0, ay, az);
+          if (leader) tc::tma_load_3d(base + s * SP::STAGE, ta, full(s), 0, ay, az);
           advance();
         }
         for (; kb < kb_end; ++kb) {
           const uint32_t sa = base + s * SP::STAGE;
-          if (!tc::mbar_wait(empty(s), ph, status, 101)) { ok = false; break; }
-          tc::mbar_expect_tx(full(s), SP::STAGE);
-          tc::tma_load_3d(sa, ta, full(s), 0, ay, az);
-          tc::tma_load_3d(sa + SP::A_BYTES, tb, full(s), 0, by, bz);
+          if (!tc::mbar_wait_warp(empty(s), ph, status, 101)) { ok = false; break; }
+          if (leader) {
+            tc::mbar_expect_tx(full(s), SP::STAGE);
+            tc::tma_load_3d(sa, ta, full(s), 0, ay, az);
+            tc::tma_load_3d(sa + SP::A_BYTES, tb, full(s), 0, by, bz);
+          }
           advance();
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer: one thread.  Descriptor words are formed once per reduction loop; per instruction only
+  } else if (warp == 1) {
+    // ---- MMA issuer (a whole warp, see elect_one).  Descriptor words are formed once per reduction loop; per instruction only
     // the start-address field moves.  (The loop is not the limit: with 128 x 256 tiles a k-block's 48 KB of
     // operands take longer to arrive from L2, at about 64 B/clk per SM, than its four MMAs take to run.) ------
+    const bool leader = tc::elect_one();
     int s = 0, ti = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -498,7 +503,7 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
     for (int w = blockIdx.x; ok && tile_at<BN>(G, w, &tcd); w += gridDim.x, ++ti) {
       const TcProblem& P = G.p[tcd.prob];
       const int ab = ti & 1;
-      if (!tc::mbar_wait(acc_empty(ab), ((ti >> 1) & 1) ^ 1, status, 104)) { ok = false; break; }
+      if (!tc::mbar_wait_warp(acc_empty(ab), ((ti >> 1) & 1) ^ 1, status, 104)) { ok = false; break; }
       tc::tc_fence_after();
       const uint32_t d_tmem = tmem_base + ab * BN;
       uint32_t acc = 0;
@@ -510,20 +515,20 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
         const uint32_t b_lo0 = tc::smem_desc_lo(base + SP::A_BYTES, P.b_mn[t] ? 8192u : 16u), b_step = P.b_mn[t] ? 128u : 2u;
         const int nkb = t == 0 ? tcd.kb1 - tcd.kb0 : P.kblocks[t];
         for (int kb = 0; kb < nkb; ++kb) {
-          if (!tc::mbar_wait(full(s), ph, status, 102)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(full(s), ph, status, 102)) { ok = false; break; }
           tc::tc_fence_after();
-          uint32_t a_lo = a_lo0 + (uint32_t)s * (SP::STAGE >> 4), b_lo = b_lo0 + (uint32_t)s * (SP::STAGE >> 4);
+          const uint32_t a_lo = a_lo0 + (uint32_t)s * (SP::STAGE >> 4), b_lo = b_lo0 + (uint32_t)s * (SP::STAGE >> 4);
+          if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            tc::mma_bf16_ss_w(d_tmem, a_lo, hi, b_lo, hi, idesc, acc);
-            acc = 1;
-            a_lo += a_step; b_lo += b_step;
+            for (int kk = 0; kk < BK / 16; ++kk)
+              tc::mma_bf16_ss_w(d_tmem, a_lo + kk * a_step, hi, b_lo + kk * b_step, hi, idesc, kk > 0 ? 1u : acc);
+            tc::mma_commit(empty(s));              // frees the stage once these MMAs have read it
           }
-          tc::mma_commit(empty(s));              // frees the stage once these MMAs have read it
+          acc = 1;
           if (++s == STAGES) { s = 0; ph ^= 1; }
         }
       }
-      if (ok) tc::mma_commit(acc_full(ab));
+      if (ok && leader) tc::mma_commit(acc_full(ab));
     }
   } else if (warp >= 2) {
     // ---- epilogue warps ---------------------------------------------------------------------------
@@ -606,7 +611,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
   auto acc_full = [&](int a) { return bars + 8u * (2 * STAGES + a); };
   auto acc_empty = [&](int a) { return bars + 8u * (2 * STAGES + 2 + a); };
   const uint32_t slot = bars + 8 * SP::N_BARS;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   const uint32_t rank = tc::cluster_ctarank();
   const int pair_id = blockIdx.x / 2, n_pairs = gridDim.x / 2;
   int32_t* status = G.status;
@@ -633,9 +638,11 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   if (!G.late_trigger) pdl_launch_dependents();
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
+    const bool leader = tc::elect_one();
     // ---- TMA producer (both CTAs): own A rows, own half of B's columns; bytes counted on the leader's barrier ----
     int s = 0;
     uint32_t ph = 1;
@@ -643,7 +650,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
     TileCoord tcd;
     const uint32_t full0 = tc::map_to_cta(full(0), 0);
     pdl_wait();
-    if (G.late_trigger) late_trigger(G);
+    if (G.late_trigger && leader) late_trigger(G);
     for (int w = pair_id; ok && pair_tile_at(G, w, &tcd); w += n_pairs) {
       const TcProblem& P = G.p[tcd.prob];
       const int m0 = tcd.m0 + (int)rank * 128, n0 = tcd.n0 + (int)rank * 128;
@@ -656,17 +663,20 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
         const int ady = a_mn ? BK : 0, adz = a_mn ? 0 : 1, bdy = b_mn ? BK : 0, bdz = b_mn ? 0 : 1;
         for (; kb < kb_end; ++kb) {
           const uint32_t sa = base + s * SP::STAGE, fb = full0 + 8u * s;
-          if (!tc::mbar_wait(empty(s), ph, status, 111)) { ok = false; break; }
-          if (rank == 0) tc::mbar_expect_tx(full(s), 2 * SP::STAGE);
-          tc::tma_load_3d_pair(sa, ta, fb, 0, ay, az);
-          tc::tma_load_3d_pair(sa + SP::A_BYTES, tb, fb, 0, by, bz);
+          if (!tc::mbar_wait_warp(empty(s), ph, status, 111)) { ok = false; break; }
+          if (leader) {
+            if (rank == 0) tc::mbar_expect_tx(full(s), 2 * SP::STAGE);
+            tc::tma_load_3d_pair(sa, ta, fb, 0, ay, az);
+            tc::tma_load_3d_pair(sa + SP::A_BYTES, tb, fb, 0, by, bz);
+          }
           ay += ady; az += adz; by += bdy; bz += bdz;
           if (++s == STAGES) { s = 0; ph ^= 1; }
         }
       }
     }
-  } else if (warp == 1 && lane == 0 && rank == 0) {
+  } else if (warp == 1 && rank == 0) {
     // ---- MMA issuer (leader only) --------------------------------------------------------------
+    const bool leader = tc::elect_one();
     int s = 0, ti = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -675,7 +685,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
     for (int w = pair_id; ok && pair_tile_at(G, w, &tcd); w += n_pairs, ++ti) {
       const TcProblem& P = G.p[tcd.prob];
       const int ab = ti & 1;
-      if (!tc::mbar_wait(acc_empty(ab), ((ti >> 1) & 1) ^ 1, status, 114)) { ok = false; break; }
+      if (!tc::mbar_wait_warp(acc_empty(ab), ((ti >> 1) & 1) ^ 1, status, 114)) { ok = false; break; }
       tc::tc_fence_after();
       const uint32_t d_tmem = tmem_base + ab * BN;
       uint32_t acc = 0;
@@ -685,20 +695,20 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
         const uint32_t b_lo0 = tc::smem_desc_lo(base + SP::A_BYTES, P.b_mn[t] ? 8192u : 16u), b_step = P.b_mn[t] ? 128u : 2u;
         const int nkb = t == 0 ? tcd.kb1 - tcd.kb0 : P.kblocks[t];
         for (int kb = 0; kb < nkb; ++kb) {
-          if (!tc::mbar_wait(full(s), ph, status, 112)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(full(s), ph, status, 112)) { ok = false; break; }
           tc::tc_fence_after();
-          uint32_t a_lo = a_lo0 + (uint32_t)s * (SP::STAGE >> 4), b_lo = b_lo0 + (uint32_t)s * (SP::STAGE >> 4);
+          const uint32_t a_lo = a_lo0 + (uint32_t)s * (SP::STAGE >> 4), b_lo = b_lo0 + (uint32_t)s * (SP::STAGE >> 4);
+          if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            tc::mma_bf16_ss_w2(d_tmem, a_lo, hi, b_lo, hi, idesc, acc);
-            acc = 1;
-            a_lo += a_step; b_lo += b_step;
+            for (int kk = 0; kk < BK / 16; ++kk)
+              tc::mma_bf16_ss_w2(d_tmem, a_lo + kk * a_step, hi, b_lo + kk * b_step, hi, idesc, kk > 0 ? 1u : acc);
+            tc::mma_commit2_both(empty(s));        // frees the stage in both CTAs once these MMAs have read it
           }
-          tc::mma_commit2_both(empty(s));        // frees the stage in both CTAs once these MMAs have read it
+          acc = 1;
           if (++s == STAGES) { s = 0; ph ^= 1; }
         }
       }
-      if (ok) tc::mma_commit2_both(acc_full(ab));
+      if (ok && leader) tc::mma_commit2_both(acc_full(ab));
     }
   } else if (warp >= 2) {
     // ---- epilogue (both CTAs): this CTA's 128 accumulator rows, as in the single-CTA kernel -------------
@@ -764,7 +774,7 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
   const uint32_t bars = base + SP::BAR_OFF, slot = bars + 8 * SP::N_BARS, acc_full = bars + 8u * (2 * STAGES);
   auto full = [&](int s) { return bars + 8u * s; };
   auto empty = [&](int s) { return bars + 8u * (STAGES + s); };
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   int32_t* status = G.status;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -783,6 +793,7 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   if (!G.late_trigger) pdl_launch_dependents();
 
   const int slice = blockIdx.x % G.slices;
@@ -794,63 +805,63 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
   const int begin = gemm_slice_begin(total, G.slices, slice), end = gemm_slice_begin(total, G.slices, slice + 1);
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---- TMA producer; the first weights before waiting for the kernel in front, as in gemm_tc_kernel ----
-      int prefilled = 0;
-      if (P.b_static && begin < P.kblocks[0]) {
-        prefilled = min(STAGES, min(end, P.kblocks[0]) - begin);
-        for (int i = 0; i < prefilled; ++i) {
-          const uint32_t sb = base + i * SP::STAGE + SP::A_BYTES;
-          tc::mbar_expect_tx(full(i), SP::STAGE);
-          if (P.b_mn[0]) tc::tma_load_3d(sb, &P.tb[0], full(i), 0, (begin + i) * BK, tcd.n0 / 64);
-          else tc::tma_load_3d(sb, &P.tb[0], full(i), 0, tcd.n0, begin + i);
-        }
+    const bool leader = tc::elect_one();
+    // ---- TMA producer; the first weights before waiting for the kernel in front, as in gemm_tc_kernel ----
+    int prefilled = 0;
+    if (P.b_static && begin < P.kblocks[0]) {
+      prefilled = min(STAGES, min(end, P.kblocks[0]) - begin);
+      for (int i = 0; i < prefilled; ++i) {
+        const uint32_t sb = base + i * SP::STAGE + SP::A_BYTES;
+        if (!leader) continue;
+        tc::mbar_expect_tx(full(i), SP::STAGE);
+        if (P.b_mn[0]) tc::tma_load_3d(sb, &P.tb[0], full(i), 0, (begin + i) * BK, tcd.n0 / 64);
+        else tc::tma_load_3d(sb, &P.tb[0], full(i), 0, tcd.n0, begin + i);
       }
-      pdl_wait();
-      if (G.late_trigger) late_trigger(G);
-      int t = 0, first = 0;                              // term of the k-block, and its first k-block
-      for (int k = begin, it = 0; k < end; ++k, ++it) {
-        while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }
-        const int kb = k - first, s = it % STAGES;
-        const uint32_t sa = base + s * SP::STAGE, sb = sa + SP::A_BYTES;
-        if (it >= prefilled) {
-          if (!tc::mbar_wait(empty(s), ((it / STAGES) & 1) ^ 1, status, 141)) break;
-          tc::mbar_expect_tx(full(s), SP::STAGE);
-        }
-        if (P.a_mn[t]) tc::tma_load_3d(sa, &P.ta[t], full(s), 0, kb * BK, tcd.m0 / 64);
-        else tc::tma_load_3d(sa, &P.ta[t], full(s), 0, tcd.m0, kb);
-        if (it >= prefilled) {
-          if (P.b_mn[t]) tc::tma_load_3d(sb, &P.tb[t], full(s), 0, kb * BK, tcd.n0 / 64);
-          else tc::tma_load_3d(sb, &P.tb[t], full(s), 0, tcd.n0, kb);
-        }
+    }
+    pdl_wait();
+    if (G.late_trigger && leader) late_trigger(G);
+    int t = 0, first = 0;                              // term of the k-block, and its first k-block
+    for (int k = begin, it = 0; k < end; ++k, ++it) {
+      while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }
+      const int kb = k - first, s = it % STAGES;
+      const uint32_t sa = base + s * SP::STAGE, sb = sa + SP::A_BYTES;
+      if (it >= prefilled) {
+        if (!tc::mbar_wait_warp(empty(s), ((it / STAGES) & 1) ^ 1, status, 141)) break;
+        if (leader) tc::mbar_expect_tx(full(s), SP::STAGE);
+      }
+      if (!leader) continue;
+      if (P.a_mn[t]) tc::tma_load_3d(sa, &P.ta[t], full(s), 0, kb * BK, tcd.m0 / 64);
+      else tc::tma_load_3d(sa, &P.ta[t], full(s), 0, tcd.m0, kb);
+      if (it >= prefilled) {
+        if (P.b_mn[t]) tc::tma_load_3d(sb, &P.tb[t], full(s), 0, kb * BK, tcd.n0 / 64);
+        else tc::tma_load_3d(sb, &P.tb[t], full(s), 0, tcd.n0, kb);
       }
     }
     __syncwarp();
     tc::cluster_sync_all();
     tc::cluster_arrive();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- MMA issuer ----
-      const uint32_t hi = tc::smem_desc_hi(1024);
-      int t = 0, first = 0;
-      bool ok = true;
-      for (int k = begin, it = 0; k < end; ++k, ++it) {
-        while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }
-        const int s = it % STAGES;
-        if (!tc::mbar_wait(full(s), (it / STAGES) & 1, status, 142)) { ok = false; break; }
-        tc::tc_fence_after();
-        const uint32_t idesc = tc::idesc_bf16(BM, BN, P.a_mn[t], P.b_mn[t]), sa = base + s * SP::STAGE;
-        uint32_t a_lo = tc::smem_desc_lo(sa, P.a_mn[t] ? 8192u : 16u), b_lo = tc::smem_desc_lo(sa + SP::A_BYTES, P.b_mn[t] ? 8192u : 16u);
-        const uint32_t a_step = P.a_mn[t] ? 128u : 2u, b_step = P.b_mn[t] ? 128u : 2u;
+    // ---- MMA issuer ----
+    const bool leader = tc::elect_one();
+    const uint32_t hi = tc::smem_desc_hi(1024);
+    int t = 0, first = 0;
+    bool ok = true;
+    for (int k = begin, it = 0; k < end; ++k, ++it) {
+      while (k - first >= P.kblocks[t]) { first += P.kblocks[t]; ++t; }
+      const int s = it % STAGES;
+      if (!tc::mbar_wait_warp(full(s), (it / STAGES) & 1, status, 142)) { ok = false; break; }
+      tc::tc_fence_after();
+      const uint32_t idesc = tc::idesc_bf16(BM, BN, P.a_mn[t], P.b_mn[t]), sa = base + s * SP::STAGE;
+      const uint32_t a_lo = tc::smem_desc_lo(sa, P.a_mn[t] ? 8192u : 16u), b_lo = tc::smem_desc_lo(sa + SP::A_BYTES, P.b_mn[t] ? 8192u : 16u);
+      const uint32_t a_step = P.a_mn[t] ? 128u : 2u, b_step = P.b_mn[t] ? 128u : 2u;
+      if (leader) {
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-          tc::mma_bf16_ss_w(tmem_base, a_lo, hi, b_lo, hi, idesc, (it > 0 || kk > 0) ? 1u : 0u);
-          a_lo += a_step; b_lo += b_step;
-        }
+        for (int kk = 0; kk < BK / 16; ++kk)
+          tc::mma_bf16_ss_w(tmem_base, a_lo + kk * a_step, hi, b_lo + kk * b_step, hi, idesc, (it > 0 || kk > 0) ? 1u : 0u);
         tc::mma_commit(empty(s));
       }
-      if (ok) tc::mma_commit(acc_full);
     }
+    if (ok && leader) tc::mma_commit(acc_full);
     __syncwarp();
     tc::cluster_sync_all();
     tc::cluster_arrive();
