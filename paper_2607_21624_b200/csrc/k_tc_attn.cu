@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
   const uint32_t bars = base + SM::BAR_OFF;
   const uint32_t slot = bars + 8 * SM::N_BARS;
   auto bar = [&](int i) { return bars + 8u * i; };
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   const int n_qt = (P.seq + BQ - 1) / BQ;
   int slot_i, hb;
   decode_block((int)blockIdx.x, P.n_slots, P.hq * P.batch, P.chunk, &slot_i, &hb);
@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   pdl_launch_dependents();
 
   if (warp == 0 && lane == 0) {
@@ -168,7 +169,8 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
       tc::mbar_expect_tx(bar(B_VFULL + s), SM::TILE);
       tc::tma_load_4d(base + SM::V_OFF + s * SM::TILE, &P.tv, bar(B_VFULL + s), 0, j * BKV, b, g * (int)PANELS);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
+    const bool leader = tc::elect_one();
     // ---- MMA issuer --------------------------------------------------------------------------
     // Per key tile j: [P0(j) ready] PV0(j), S0(j+1), [P1(j) ready] PV1(j), S1(j+1): while one warp group works
     // on its scores the tensor pipe serves the other one.  S and P of a query tile share TMEM columns, so
@@ -180,6 +182,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
     const uint32_t q_lo = tc::smem_desc_lo(base + SM::Q_OFF, 16), k_lo = tc::smem_desc_lo(base + SM::K_OFF, 16);
     const uint32_t v_lo = tc::smem_desc_lo(base + SM::V_OFF, 16384);
     auto issue_s = [&](int w, int j) {
+      if (!leader) return;
       const uint32_t ql = q_lo + w * (SM::TILE >> 4), kl = k_lo + (j & 1) * (SM::TILE >> 4);
 #pragma unroll
       for (uint32_t kk = 0; kk < HD / 16; ++kk) {
@@ -189,6 +192,7 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
       tc::mma_commit(bar(B_SFULL + w));
     };
     auto issue_pv = [&](int w, int j) {
+      if (!leader) return;
       const uint32_t vl = v_lo + (j & 1) * (SM::TILE >> 4);
 #pragma unroll
       for (uint32_t kk = 0; kk < BKV / 16; ++kk) {
@@ -203,44 +207,52 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
       // Work items in issue order: (tile 0, j), (tile 1, j) while tile 1 has key tiles, then tile 0's remaining
       // ones (n_kv0 >= n_kv1: tile 0 is the later query tile).  Barriers of a score buffer are used once per
       // rotation, so neither side can run more than one phase ahead on any of them.
-      const int n_items = n_kv0 + n_kv1;
-      auto item = [&](int n, int& w, int& j) {
-        if (n < 2 * n_kv1) { w = n & 1; j = n >> 1; } else { w = 0; j = n - n_kv1; }
+      struct Item { int w, j, buf; uint32_t ph; };          // tile, key tile, score buffer and its phase
+      auto next = [&](Item& i) {
+        if (i.w == 0 && i.j < n_kv1) i.w = 1; else { i.w = 0; ++i.j; }
+        if (++i.buf == 3) { i.buf = 0; i.ph ^= 1; }
       };
-      auto issue_s_item = [&](int n) -> bool {
-        int w, j; item(n, w, j);
+      const int n_items = n_kv0 + n_kv1;
+      auto issue_s_item = [&](const Item& i) -> bool {
         // tile 0 is the first user of every key tile, and the last one where tile 1 has none
-        if (w == 0 && !tc::mbar_wait(bar(B_KFULL + (j & 1)), (j >> 1) & 1, status, 205)) return false;
-        const uint32_t ql = q_lo + w * (SM::TILE >> 4), kl = k_lo + (j & 1) * (SM::TILE >> 4);
-        const uint32_t d = tmem_base + (uint32_t)(n % 3) * 128;
+        if (i.w == 0 && !tc::mbar_wait_warp(bar(B_KFULL + (i.j & 1)), (i.j >> 1) & 1, status, 205)) return false;
+        const uint32_t ql = q_lo + i.w * (SM::TILE >> 4), kl = k_lo + (i.j & 1) * (SM::TILE >> 4);
+        const uint32_t d = tmem_base + (uint32_t)i.buf * 128;
+        if (leader) {
 #pragma unroll
-        for (uint32_t kk = 0; kk < HD / 16; ++kk) {
-          const uint32_t o = (kk / 4) * 1024 + (kk % 4) * 2;
-          tc::mma_bf16_ss_w(d, ql + o, hi, kl + o, hi, idesc_s, kk > 0);
+          for (uint32_t kk = 0; kk < HD / 16; ++kk) {
+            const uint32_t o = (kk / 4) * 1024 + (kk % 4) * 2;
+            tc::mma_bf16_ss_w(d, ql + o, hi, kl + o, hi, idesc_s, kk > 0);
+          }
+          tc::mma_commit(bar(B_SFULL + i.buf));
+          if (i.w == 1 || i.j >= n_kv1) tc::mma_commit(bar(B_KEMPTY + (i.j & 1)));
         }
-        tc::mma_commit(bar(B_SFULL + n % 3));
-        if (w == 1 || j >= n_kv1) tc::mma_commit(bar(B_KEMPTY + (j & 1)));
+        __syncwarp();
         return true;
       };
-      bool ok = tc::mbar_wait(bar(B_QFULL), 0, status, 203);
+      bool ok = tc::mbar_wait_warp(bar(B_QFULL), 0, status, 203);
       if (ok) tc::tc_fence_after();
-      for (int n = 0; n < 3 && n < n_items && ok; ++n) ok = issue_s_item(n);
+      Item now{0, 0, 0, 0}, ahead = now;
+      for (int n = 0; n < 3 && n < n_items && ok; ++n) { ok = issue_s_item(ahead); next(ahead); }
       for (int n = 0; n < n_items && ok; ++n) {
-        int w, j; item(n, w, j);
-        if (w == 0 && !tc::mbar_wait(bar(B_VFULL + (j & 1)), (j >> 1) & 1, status, 207)) { ok = false; break; }
-        if (!tc::mbar_wait(bar(B_PFULL + n % 3), (n / 3) & 1, status, 206)) { ok = false; break; }
+        if (now.w == 0 && !tc::mbar_wait_warp(bar(B_VFULL + (now.j & 1)), (now.j >> 1) & 1, status, 207)) break;
+        if (!tc::mbar_wait_warp(bar(B_PFULL + now.buf), now.ph, status, 206)) break;
         tc::tc_fence_after();
-        const uint32_t vl = v_lo + (j & 1) * (SM::TILE >> 4);
-        const uint32_t pa = tmem_base + (uint32_t)(n % 3) * 128, od = tmem_base + O_COL + w * HD;
+        const uint32_t vl = v_lo + (now.j & 1) * (SM::TILE >> 4);
+        const uint32_t pa = tmem_base + (uint32_t)now.buf * 128, od = tmem_base + O_COL + now.w * HD;
+        if (leader) {
 #pragma unroll
-        for (uint32_t kk = 0; kk < BKV / 16; ++kk)
-          tc::mma_bf16_ts_w(od, pa + kk * 8, vl + kk * 128, hi, idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
-        tc::mma_commit(bar(B_PVDONE + w));
-        if (w == 1 || j >= n_kv1) tc::mma_commit(bar(B_VEMPTY + (j & 1)));
-        if (n + 3 < n_items) ok = issue_s_item(n + 3);     // into the buffer whose P the product above has just read
+          for (uint32_t kk = 0; kk < BKV / 16; ++kk)
+            tc::mma_bf16_ts_w(od, pa + kk * 8, vl + kk * 128, hi, idesc_o, (now.j > 0 || kk > 0) ? 1u : 0u);
+          tc::mma_commit(bar(B_PVDONE + now.w));
+          if (now.w == 1 || now.j >= n_kv1) tc::mma_commit(bar(B_VEMPTY + (now.j & 1)));
+        }
+        __syncwarp();
+        next(now);
+        if (n + 3 < n_items) { ok = issue_s_item(ahead); next(ahead); }     // into the buffer whose P the product above has just read
       }
     } else {
-    bool ok = tc::mbar_wait(bar(B_QFULL), 0, status, 203) && tc::mbar_wait(bar(B_KFULL), 0, status, 204);
+    bool ok = tc::mbar_wait_warp(bar(B_QFULL), 0, status, 203) && tc::mbar_wait_warp(bar(B_KFULL), 0, status, 204);
     if (ok) {
       tc::tc_fence_after();
       if (n_kv0 > 0) issue_s(0, 0);
@@ -248,21 +260,23 @@ __global__ void __launch_bounds__(64 + 128 * TILES, TILES == 1 ? 2 : 1) attn_fwd
     }
     for (int j = 0; j < n_kv_max && ok; ++j) {
       const bool next = j + 1 < n_kv_max;
-      if (!tc::mbar_wait(bar(B_VFULL + (j & 1)), (j >> 1) & 1, status, 207)) { ok = false; break; }
-      if (next && !tc::mbar_wait(bar(B_KFULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, status, 205)) { ok = false; break; }
+      if (!tc::mbar_wait_warp(bar(B_VFULL + (j & 1)), (j >> 1) & 1, status, 207)) { ok = false; break; }
+      if (next && !tc::mbar_wait_warp(bar(B_KFULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, status, 205)) { ok = false; break; }
 #pragma unroll
       for (int w = 0; w < TILES; ++w) {
         const int nk = w ? n_kv1 : n_kv0;
         if (ok && j < nk) {
-          if (!tc::mbar_wait(bar(B_PFULL + w), j & 1, status, 206)) { ok = false; }
+          if (!tc::mbar_wait_warp(bar(B_PFULL + w), j & 1, status, 206)) { ok = false; }
           else { tc::tc_fence_after(); issue_pv(w, j); }
         }
         if (ok && j + 1 < nk) issue_s(w, j + 1);
       }
       if (!ok) break;
-      tc::mma_commit(bar(B_VEMPTY + (j & 1)));              // both P V products of this stage are behind us
-      if (next) tc::mma_commit(bar(B_KEMPTY + ((j + 1) & 1)));   // ... and both score products of the next stage
-      if (j == 0) tc::mma_commit(bar(B_KEMPTY));            // stage 0 scores were issued before the loop
+      if (leader) {
+        tc::mma_commit(bar(B_VEMPTY + (j & 1)));            // both P V products of this stage are behind us
+        if (next) tc::mma_commit(bar(B_KEMPTY + ((j + 1) & 1)));   // ... and both score products of the next stage
+        if (j == 0) tc::mma_commit(bar(B_KEMPTY));          // stage 0 scores were issued before the loop
+      }
     }
     }
   } else if (warp >= 2) {
@@ -639,7 +653,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
   const uint32_t bars = base + SM::BAR_OFF;
   const uint32_t slot = bars + 8 * SM::N_BARS;
   auto bar = [&](int i) { return bars + 8u * i; };
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   // under a causal mask key tile 0 has the most query tiles: it is slot 0
   const int n_kvh = P.hq / P.group;
   int slot_i, gb;
@@ -705,6 +719,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   pdl_launch_dependents();
   // Where a block's dQ tiles are staged for the bulk reduction: one staging tile; with the pipelined variant the
   // last tile goes to the dS^T buffer that the last iteration does not use (its readers, the dK and dQ products of
@@ -740,7 +755,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       tc::tma_load_3d(base + SM::DO_OFF + sd * SM::TILE, &P.tdo, bar(BB_DOFULL + sd), 0, row0 + qt * BQ, h * (int)PANELS);
       tc::bulk_load(base + SM::D_OFF + sd * 512, P.dvec + stat_off, 512, bar(BB_DOFULL + sd));
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
+    const bool leader = tc::elect_one();
     // ---- MMA issuer --------------------------------------------------------------------------
     const uint32_t idesc_s = tc::idesc_bf16(BKV, BQ, 0, 0);
     const uint32_t idesc_kv = tc::idesc_bf16(BKV, HD, 0, 1);
@@ -754,6 +770,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
     const uint32_t do_km = tc::smem_desc_lo(base + SM::DO_OFF, 16), do_mn = tc::smem_desc_lo(base + SM::DO_OFF, 16384);
     const uint32_t ds_km = tc::smem_desc_lo(base + SM::DS_OFF, 16), ds_mn = tc::smem_desc_lo(base + SM::DS_OFF, 16384);
     auto issue_s = [&](int it) {              // S^T = K Q^T of tile `it`
+      if (!leader) return;
       const uint32_t qs = q_km + (it % NQQ) * (SM::TILE >> 4);
 #pragma unroll
       for (uint32_t kk = 0; kk < HD / 16; ++kk) {
@@ -763,6 +780,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       if (!PIPE) tc::mma_commit(bar(BB_SFULL));     // HD = 128: the softmax warps start on the scores while dP^T is
     };                                              // still to come (it waits for the previous tile's dQ drain)
     auto issue_dp = [&](int it) {             // dP^T = V dO^T of tile `it`, announced on its own barrier
+      if (!leader) return;
       const uint32_t dos = do_km + (it % NDO) * (SM::TILE >> 4);
 #pragma unroll
       for (uint32_t kk = 0; kk < HD / 16; ++kk) {
@@ -772,6 +790,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       tc::mma_commit(bar(PIPE ? BB_SFULL : BB_DPFULL));      // HD = 64: one announcement for both score tiles
     };
     auto issue_dv = [&](int it) {             // dV += P^T dO, P^T read from tensor memory
+      if (!leader) return;
       const uint32_t dos = do_mn + (it % NDO) * (SM::TILE >> 4);
 #pragma unroll
       for (uint32_t kk = 0; kk < BQ / 16; ++kk)                      // dO: MN-major, 16 query rows per step;
@@ -779,6 +798,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
                           dos + kk * 128, hi, idesc_kv, (it > 0 || kk > 0) ? 1u : 0u);
     };
     auto issue_dk = [&](int it) {             // dK += dS^T Q
+      if (!leader) return;
       const uint32_t qs = q_mn + (it % NQQ) * (SM::TILE >> 4);
       const uint32_t dss = ds_km + (it % NP) * 2048;
 #pragma unroll
@@ -789,15 +809,16 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
       }
     };
     auto issue_dq = [&](int it) {             // dQ = dS K: the dS^T tile read MN-major, i.e. transposed by descriptor
+      if (!leader) return;
       const uint32_t dss = ds_mn + (it % NP) * 2048;
 #pragma unroll
       for (uint32_t kk = 0; kk < BKV / 16; ++kk)                     // both operands MN-major: 16 key rows per step
         tc::mma_bf16_ss_w(tmem_base + DQ_COL, dss + kk * 128, hi, k_mn + kk * 128, hi, idesc_dq, kk > 0);
       tc::mma_commit(bar(BB_DQFULL));
     };
-    bool ok = tc::mbar_wait(bar(BB_KVFULL), 0, status, 302);
+    bool ok = tc::mbar_wait_warp(bar(BB_KVFULL), 0, status, 302);
     if (ok && n_it > 0) {
-      ok = tc::mbar_wait(bar(BB_QFULL), 0, status, 303) && tc::mbar_wait(bar(BB_DOFULL), 0, status, 314);
+      ok = tc::mbar_wait_warp(bar(BB_QFULL), 0, status, 303) && tc::mbar_wait_warp(bar(BB_DOFULL), 0, status, 314);
       if (ok) { tc::tc_fence_after(); issue_s(0); issue_dp(0); }
     }
     if (PIPE) {
@@ -807,50 +828,50 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
         if (it + 1 < n_it) {
           // S^T(it+1) as soon as every softmax warp has copied S^T(it) to registers: it is computed while
           // they work on tile it
-          if (!tc::mbar_wait(bar(BB_SREAD), it & 1, status, 311)) { ok = false; break; }
-          if (!tc::mbar_wait(bar(BB_QFULL + ((it + 1) % NQQ)), ((it + 1) / NQQ) & 1, status, 303)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(bar(BB_SREAD), it & 1, status, 311)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(bar(BB_QFULL + ((it + 1) % NQQ)), ((it + 1) / NQQ) & 1, status, 303)) { ok = false; break; }
           tc::tc_fence_after();
           issue_s(it + 1);
         }
-        if (!tc::mbar_wait(bar(BB_PDSFULL), it & 1, status, 305)) { ok = false; break; }
+        if (!tc::mbar_wait_warp(bar(BB_PDSFULL), it & 1, status, 305)) { ok = false; break; }
         tc::tc_fence_after();
         if (it + 1 < n_it) {
-          if (!tc::mbar_wait(bar(BB_DOFULL + ((it + 1) % NDO)), ((it + 1) / NDO) & 1, status, 314)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(bar(BB_DOFULL + ((it + 1) % NDO)), ((it + 1) / NDO) & 1, status, 314)) { ok = false; break; }
           issue_dp(it + 1);                             // dP^T(it) has been read as well: announce tile it + 1
         }
         issue_dv(it);
-        tc::mma_commit(bar(BB_DVDONE));                 // P^T(it) has been read: P^T(it+1) may be stored
-        tc::mma_commit(bar(BB_DOEMPTY + (it % NDO)));   // ... and dO of this tile is not read again
+        if (leader) tc::mma_commit(bar(BB_DVDONE));                 // P^T(it) has been read: P^T(it+1) may be stored
+        if (leader) tc::mma_commit(bar(BB_DOEMPTY + (it % NDO)));   // ... and dO of this tile is not read again
         issue_dk(it);
-        tc::mma_commit(bar(BB_QEMPTY + (it % NQQ)));    // nor is Q
-        if (it > 0 && !tc::mbar_wait(bar(BB_DQDRAINED), (it - 1) & 1, status, 304)) { ok = false; break; }
+        if (leader) tc::mma_commit(bar(BB_QEMPTY + (it % NQQ)));    // nor is Q
+        if (it > 0 && !tc::mbar_wait_warp(bar(BB_DQDRAINED), (it - 1) & 1, status, 304)) { ok = false; break; }
         tc::tc_fence_after();
         issue_dq(it);
       }
     } else {
       for (int it = 0; it < n_it && ok; ++it) {
-        if (!tc::mbar_wait(bar(BB_PDSFULL), it & 1, status, 305)) { ok = false; break; }
+        if (!tc::mbar_wait_warp(bar(BB_PDSFULL), it & 1, status, 305)) { ok = false; break; }
         tc::tc_fence_after();
         // dQ first: its drain to shared memory (which frees the dP^T columns for the next tile) then overlaps
         // the dV and dK products
         issue_dq(it);
         issue_dk(it);
-        tc::mma_commit(bar(BB_QEMPTY));                 // Q of this tile is not read again: the next one is fetched
+        if (leader) tc::mma_commit(bar(BB_QEMPTY));                 // Q of this tile is not read again: the next one is fetched
         issue_dv(it);                                   // while dV runs
-        tc::mma_commit(bar(BB_DOEMPTY));                // ... and dO
+        if (leader) tc::mma_commit(bar(BB_DOEMPTY));                // ... and dO
         if (it + 1 < n_it) {
-          if (!tc::mbar_wait(bar(BB_QFULL), (it + 1) & 1, status, 303)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(bar(BB_QFULL), (it + 1) & 1, status, 303)) { ok = false; break; }
           tc::tc_fence_after();
           issue_s(it + 1);                   // the S^T columns (P^T by now) were last read by dV above
-          if (!tc::mbar_wait(bar(BB_DQDRAINED), it & 1, status, 304)) { ok = false; break; }
-          if (!tc::mbar_wait(bar(BB_DOFULL), (it + 1) & 1, status, 314)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(bar(BB_DQDRAINED), it & 1, status, 304)) { ok = false; break; }
+          if (!tc::mbar_wait_warp(bar(BB_DOFULL), (it + 1) & 1, status, 314)) { ok = false; break; }
           tc::tc_fence_after();
           issue_dp(it + 1);                  // the dP^T columns held dQ until it was drained
         }
       }
       // dQ is issued first here, so its barrier does not cover the last tile's dK and dV products: one more
       // arrival, on the barrier the pipelined variant uses for dV, tells the epilogue that they are complete
-      if (ok && n_it > 0) tc::mma_commit(bar(BB_DVDONE));
+      if (ok && n_it > 0 && leader) tc::mma_commit(bar(BB_DVDONE));
     }
   } else if (!DIRECT && warp == 18) {
     // ---- dQ reduction warp: adds each staged dQ tile to the fp32 accumulator with bulk tensor reductions ----
@@ -1216,7 +1237,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) attn_bwd_short_kernel(const 
   const uint32_t base = tc::smem_u32(smem_raw);
   const uint32_t bars = base + SM::BAR_OFF, slot = bars + 8 * SM::N_BARS;
   auto bar = [&](int i) { return bars + 8u * i; };
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   const int h = blockIdx.x % P.hq, b = blockIdx.x / P.hq;
   const int row0 = b * P.t_pad, row0k = b * P.t_pad_k;
   const int n_qt = (P.seq + BQ - 1) / BQ, n_kt = (P.seq_k + BKV - 1) / BKV;
@@ -1268,6 +1289,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) attn_bwd_short_kernel(const 
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   pdl_launch_dependents();
 
   if (warp == 0 && lane == 0) {
@@ -1277,7 +1299,8 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) attn_bwd_short_kernel(const 
       tc::tma_load_3d(base + SM::DO_OFF + t * SM::TILE, &P.tdo, bar(SB_DOFULL + t), 0, row0 + t * BQ, h);
       tc::bulk_load(base + SM::D_OFF + t * 512, P.dvec + ((long long)b * P.hq + h) * P.t_pad + t * BQ, 512, bar(SB_DOFULL + t));
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
+    const bool leader = tc::elect_one();
     // ---- MMA issuer ----
     const uint32_t idesc_s = tc::idesc_bf16(BKV, BQ, 0, 0), idesc_kv = tc::idesc_bf16(BKV, HD, 0, 1), idesc_dq = tc::idesc_bf16(BQ, HD, 1, 1);
     const uint32_t hi = tc::smem_desc_hi(1024), TW = SM::TILE >> 4;
@@ -1288,53 +1311,55 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) attn_bwd_short_kernel(const 
     const uint32_t ds_km = tc::smem_desc_lo(base + SM::DS_OFF, 16), ds_mn = tc::smem_desc_lo(base + SM::DS_OFF, 16384);
     const uint32_t p_km = tc::smem_desc_lo(base + SM::P_OFF, 16);
     auto scores = [&](uint32_t col, uint32_t a, uint32_t q) {            // S^T = K Q^T, dP^T = V dO^T
+      if (!leader) return;
 #pragma unroll
       for (uint32_t kk = 0; kk < 4; ++kk) tc::mma_bf16_ss_w(tmem_base + col, a + kk * 2, hi, q + kk * 2, hi, idesc_s, kk > 0);
     };
     auto product = [&](uint32_t col, uint32_t a, uint32_t q, bool more) {  // dV += P^T dO, dK += dS^T Q
+      if (!leader) return;
 #pragma unroll
       for (uint32_t kk = 0; kk < 8; ++kk)
         tc::mma_bf16_ss_w(tmem_base + col, a + (kk / 4) * 1024 + (kk % 4) * 2, hi, q + kk * 128, hi, idesc_kv, more || kk > 0);
     };
-    bool ok = tc::mbar_wait(bar(SB_KVFULL), 0, status, 321) && tc::mbar_wait(bar(SB_QFULL), 0, status, 322) &&
-              tc::mbar_wait(bar(SB_DOFULL), 0, status, 323);
+    bool ok = tc::mbar_wait_warp(bar(SB_KVFULL), 0, status, 321) && tc::mbar_wait_warp(bar(SB_QFULL), 0, status, 322) &&
+              tc::mbar_wait_warp(bar(SB_DOFULL), 0, status, 323);
     if (ok) {
       tc::tc_fence_after();
       scores(S_COL, k_km, q_km);
       scores(DP_COL, v_km, do_km);
-      tc::mma_commit(bar(SB_SFULL));
+      if (leader) tc::mma_commit(bar(SB_SFULL));
     }
     for (int it = 0; it < n_it && ok; ++it) {
       const int j = key_tile(it), i = query_tile(it);
       const bool next = it + 1 < n_it;
       const int jn = next ? key_tile(it + 1) : 0, in = next ? query_tile(it + 1) : 0;
       if (next) {                                        // S^T of the next pair once every warp holds this one's scores
-        if (!tc::mbar_wait(bar(SB_SREAD), it & 1, status, 324)) break;
-        if (!tc::mbar_wait(bar(SB_QFULL + in), 0, status, 322) || !tc::mbar_wait(bar(SB_KVFULL + jn), 0, status, 321)) break;
+        if (!tc::mbar_wait_warp(bar(SB_SREAD), it & 1, status, 324)) break;
+        if (!tc::mbar_wait_warp(bar(SB_QFULL + in), 0, status, 322) || !tc::mbar_wait_warp(bar(SB_KVFULL + jn), 0, status, 321)) break;
         tc::tc_fence_after();
         scores(S_COL, k_km + jn * TW, q_km + in * TW);
       }
-      if (!tc::mbar_wait(bar(SB_PDSFULL), it & 1, status, 325)) break;
+      if (!tc::mbar_wait_warp(bar(SB_PDSFULL), it & 1, status, 325)) break;
       tc::tc_fence_after();
       if (next) {
-        if (!tc::mbar_wait(bar(SB_DOFULL + in), 0, status, 323)) break;
+        if (!tc::mbar_wait_warp(bar(SB_DOFULL + in), 0, status, 323)) break;
         tc::tc_fence_after();
         scores(DP_COL, v_km + jn * TW, do_km + in * TW);
-        tc::mma_commit(bar(SB_SFULL));
+        if (leader) tc::mma_commit(bar(SB_SFULL));
       }
-      if (it == n0 && !tc::mbar_wait(bar(SB_KVDRAINED), 0, status, 326)) break;   // key tile 0's dV, dK are copied out
+      if (it == n0 && !tc::mbar_wait_warp(bar(SB_KVDRAINED), 0, status, 326)) break;   // key tile 0's dV, dK are copied out
       tc::tc_fence_after();
       const bool more = it != 0 && it != n0;
       product(DV_COL, p_km, do_mn + i * TW, more);
-      tc::mma_commit(bar(SB_DVDONE));
+      if (leader) tc::mma_commit(bar(SB_DVDONE));
       product(DK_COL, ds_km + (it & 1) * 2048, q_mn + i * TW, more);
-      if (it + 1 == n0) tc::mma_commit(bar(SB_DKDONE));
+      if (it + 1 == n0 && leader) tc::mma_commit(bar(SB_DKDONE));
 #pragma unroll
-      for (uint32_t kk = 0; kk < 8; ++kk)                // dQ += dS K: the dS^T tile read MN-major
+      for (uint32_t kk = 0; kk < 8 && leader; ++kk)      // dQ += dS K: the dS^T tile read MN-major
         tc::mma_bf16_ss_w(tmem_base + DQ_COL + i * 64, ds_mn + (it & 1) * 2048 + kk * 128, hi, k_mn + j * TW + kk * 128, hi, idesc_dq,
                           (j > 0 || kk > 0) ? 1u : 0u);
-      tc::mma_commit(bar(SB_DQDONE));
-      if (!next) tc::mma_commit(bar(SB_FINAL));
+      if (leader) tc::mma_commit(bar(SB_DQDONE));
+      if (!next && leader) tc::mma_commit(bar(SB_FINAL));
     }
   } else if (warp >= 2) {
     // ---- softmax warps: thread = (key row, one quarter of the 128 query columns) ----
