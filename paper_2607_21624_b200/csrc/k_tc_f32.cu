@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
   auto parts = [&](int b) { return bars + 8u * (2 * STAGES + b); };         // both operands' parts are in place
   auto done = [&](int b) { return bars + 8u * (2 * STAGES + 2 + b); };      // the products have read them: accumulator complete
   auto added = [&](int b) { return bars + 8u * (2 * STAGES + 4 + b); };     // the accumulator has been read
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   int32_t* status = G.status;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   pdl_launch_dependents();
   // work unit: (problem, tile, slice); the slices of a tile are the blocks of a cluster
   const int slice = blockIdx.x % G.slices;
@@ -128,27 +129,24 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t hi = tc::smem_desc_hi(1024);
-      const uint32_t idesc = tc::idesc_bf16(BM, BN, 0, P.b_k[0]);
-      const uint32_t b_lo = tc::smem_desc_lo(base + SM::PARTS_OFF, P.b_k[0] ? 8192u : 16u), b_step = P.b_k[0] ? 128u : 2u;
-      for (int it = 0; it < n_kb; ++it) {
-        const int b = it & 1;
-        const uint32_t ph = (it >> 1) & 1;
-        if (!tc::mbar_wait(added(b), ph ^ 1, status, 132) || !tc::mbar_wait(parts(b), ph, status, 133)) break;
-        tc::tc_fence_after();
-        const uint32_t d = tmem_base + b * BN, bs = b_lo + b * (3 * SM::PART >> 4);
-        uint32_t acc = 0;
-        auto product = [&](int pa, int pb) {
+    const bool leader = tc::elect_one();
+    const uint32_t hi = tc::smem_desc_hi(1024);
+    const uint32_t idesc = tc::idesc_bf16(BM, BN, 0, P.b_k[0]);
+    const uint32_t b_lo = tc::smem_desc_lo(base + SM::PARTS_OFF, P.b_k[0] ? 8192u : 16u), b_step = P.b_k[0] ? 128u : 2u;
+    for (int it = 0; it < n_kb; ++it) {
+      const int b = it & 1;
+      const uint32_t ph = (it >> 1) & 1;
+      if (!tc::mbar_wait_warp(added(b), ph ^ 1, status, 132) || !tc::mbar_wait_warp(parts(b), ph, status, 133)) break;
+      tc::tc_fence_after();
+      const uint32_t d = tmem_base + b * BN, bs = b_lo + b * (3 * SM::PART >> 4);
+      auto product = [&](int pa, int pb) {
+        if (!leader) return;
 #pragma unroll
-          for (uint32_t kk = 0; kk < BK / 16; ++kk) {
-            tc::mma_bf16_ts_w(d, tmem_base + a_col<BN>(b, pa) + kk * 8, bs + pb * (SM::PART >> 4) + kk * b_step, hi, idesc, acc);
-            acc = 1;
-          }
-        };
-        product(2, 0); product(0, 2); product(1, 1); product(1, 0); product(0, 1); product(0, 0);
-        tc::mma_commit(done(b));
-      }
+        for (uint32_t kk = 0; kk < BK / 16; ++kk)
+          tc::mma_bf16_ts_w(d, tmem_base + a_col<BN>(b, pa) + kk * 8, bs + pb * (SM::PART >> 4) + kk * b_step, hi, idesc, pa < 2 || kk > 0);
+      };
+      product(2, 0); product(0, 2); product(1, 1); product(1, 0); product(0, 1); product(0, 0);
+      if (leader) tc::mma_commit(done(b));
     }
   } else if (warp < 6) {
     // ---- A: a thread owns a row, 16 values at a time -> eight packed columns of each part

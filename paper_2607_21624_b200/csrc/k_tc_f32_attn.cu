@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
   auto bar = [&](int i) { return bars + 8u * i; };
   enum { KFULL = 0, KEMPTY = NB, VFULL = 2 * NB, VEMPTY = 3 * NB, KPARTS = 4 * NB, KFREE = 5 * NB, VPARTS = 6 * NB, VFREE = 7 * NB,
          SFULL = 8 * NB, SREAD = SFULL + NS, QFULL = SREAD + NS, QPARTS, PFULL, PVDONE, MEET };
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   // later queries first: under a causal mask they have the most keys
   const int i0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * QT, h = blockIdx.y, b = blockIdx.z, g = h / P.group;
   const int j_end = P.causal ? min(P.seq_k, i0 + QT) : P.seq_k, n_tiles = (j_end + KT - 1) / KT;
@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   pdl_launch_dependents();
 
   if (warp == 0) {
@@ -181,51 +182,52 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- products, the small ones first ----
-      const uint32_t hi = tc::smem_desc_hi(1024), idesc_s = tc::idesc_bf16(QT, KT, 0, 0), idesc_o = tc::idesc_bf16(QT, HD, 0, 1);
-      const uint32_t k_lo = tc::smem_desc_lo(base + SM::KP_OFF, 16), v_lo = tc::smem_desc_lo(base + SM::VP_OFF, 8192);
-      auto issue_s = [&](int j) -> bool {
-        const int s = j % NB, sb = j % NS;
-        if (!tc::mbar_wait(bar(KPARTS + s), (j / NB) & 1, status, 403) || !tc::mbar_wait(bar(SREAD + sb), ((j / NS) & 1) ^ 1, status, 404)) return false;
-        tc::tc_fence_after();
-        const uint32_t kl = k_lo + s * (SM::PARTS >> 4);
+    const bool leader = tc::elect_one();
+    // ---- products, the small ones first ----
+    const uint32_t hi = tc::smem_desc_hi(1024), idesc_s = tc::idesc_bf16(QT, KT, 0, 0), idesc_o = tc::idesc_bf16(QT, HD, 0, 1);
+    const uint32_t k_lo = tc::smem_desc_lo(base + SM::KP_OFF, 16), v_lo = tc::smem_desc_lo(base + SM::VP_OFF, 8192);
+    auto issue_s = [&](int j) -> bool {
+      const int s = j % NB, sb = j % NS;
+      if (!tc::mbar_wait_warp(bar(KPARTS + s), (j / NB) & 1, status, 403) || !tc::mbar_wait_warp(bar(SREAD + sb), ((j / NS) & 1) ^ 1, status, 404)) return false;
+      tc::tc_fence_after();
+      const uint32_t kl = k_lo + s * (SM::PARTS >> 4);
 #pragma unroll
-        for (uint32_t first = 0; first < HD / 16; first += HD / 32) {
-          const uint32_t d = tmem_base + SM::S_COL + sb * (2 * KT) + (first ? KT : 0);
-          uint32_t acc = 0;
-          auto product = [&](int pa, int pb) {
-#pragma unroll
-            for (uint32_t kk = first; kk < first + HD / 32; ++kk) {
-              tc::mma_bf16_ts_w(d, tmem_base + SM::QP_COL + pa * (HD / 2) + kk * 8, kl + pb * (SM::PART >> 4) + kk * 2, hi, idesc_s, acc);
-              acc = 1;
-            }
-          };
-          product(2, 0); product(0, 2); product(1, 1); product(1, 0); product(0, 1); product(0, 0);
-        }
-        tc::mma_commit(bar(SFULL + sb));
-        tc::mma_commit(bar(KFREE + s));
-        return true;
-      };
-      bool ok = tc::mbar_wait(bar(QPARTS), 0, status, 405) && issue_s(0);
-      for (int j = 0; j < n_tiles && ok; ++j) {
-        if (j + 1 < n_tiles && !issue_s(j + 1)) break;
-        const int s = j % NB;
-        if (!tc::mbar_wait(bar(VPARTS + s), (j / NB) & 1, status, 406) || !tc::mbar_wait(bar(PFULL), j & 1, status, 407)) break;
-        tc::tc_fence_after();
-        const uint32_t vl = v_lo + s * (SM::PARTS >> 4);
+      for (uint32_t first = 0; first < HD / 16; first += HD / 32) {
+        const uint32_t d = tmem_base + SM::S_COL + sb * (2 * KT) + (first ? KT : 0);
         uint32_t acc = 0;
         auto product = [&](int pa, int pb) {
+          if (!leader) return;
 #pragma unroll
-          for (uint32_t kk = 0; kk < KT / 16; ++kk) {
-            tc::mma_bf16_ts_w(tmem_base + SM::O_COL, tmem_base + SM::P_COL + pa * 32 + kk * 8, vl + pb * (SM::PART >> 4) + kk * 128, hi, idesc_o, acc);
+          for (uint32_t kk = first; kk < first + HD / 32; ++kk) {
+            tc::mma_bf16_ts_w(d, tmem_base + SM::QP_COL + pa * (HD / 2) + kk * 8, kl + pb * (SM::PART >> 4) + kk * 2, hi, idesc_s, acc);
             acc = 1;
           }
         };
         product(2, 0); product(0, 2); product(1, 1); product(1, 0); product(0, 1); product(0, 0);
-        tc::mma_commit(bar(PVDONE));
-        tc::mma_commit(bar(VFREE + s));
       }
+      if (leader) tc::mma_commit(bar(SFULL + sb));
+      if (leader) tc::mma_commit(bar(KFREE + s));
+      return true;
+    };
+    bool ok = tc::mbar_wait_warp(bar(QPARTS), 0, status, 405) && issue_s(0);
+    for (int j = 0; j < n_tiles && ok; ++j) {
+      if (j + 1 < n_tiles && !issue_s(j + 1)) break;
+      const int s = j % NB;
+      if (!tc::mbar_wait_warp(bar(VPARTS + s), (j / NB) & 1, status, 406) || !tc::mbar_wait_warp(bar(PFULL), j & 1, status, 407)) break;
+      tc::tc_fence_after();
+      const uint32_t vl = v_lo + s * (SM::PARTS >> 4);
+      uint32_t acc = 0;
+      auto product = [&](int pa, int pb) {
+        if (!leader) return;
+#pragma unroll
+        for (uint32_t kk = 0; kk < KT / 16; ++kk) {
+          tc::mma_bf16_ts_w(tmem_base + SM::O_COL, tmem_base + SM::P_COL + pa * 32 + kk * 8, vl + pb * (SM::PART >> 4) + kk * 128, hi, idesc_o, acc);
+          acc = 1;
+        }
+      };
+      product(2, 0); product(0, 2); product(1, 1); product(1, 0); product(0, 1); product(0, 0);
+      if (leader) tc::mma_commit(bar(PVDONE));
+      if (leader) tc::mma_commit(bar(VFREE + s));
     }
   } else if (warp >= 2 + SOFT_WARPS) {
     // ---- K and V into parts ----
@@ -481,7 +483,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
   const uint32_t bars = base + SM::BAR_OFF, slot = bars + 8 * SM::N_BARS, flag = slot + 8;
   auto bar = [&](int i) { return bars + 8u * i; };
   enum { KVFULL, QRAW, DORAW, QRAWE, DORAWE, KVPARTS, QPARTS, DOPARTS, SFULL, DPFULL, PREADY, DSREADY, DVDONE, DKDONE, DQDONE, DQREAD };
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   const int slices = P.slices, slice = blockIdx.x % slices;
   const int j0 = blockIdx.x / slices * BKT, g = blockIdx.y, b = blockIdx.z;      // key tile 0 has the most queries: first
   const int t0 = P.causal ? j0 / BQT : 0, per_head = max(0, (P.seq + BQT - 1) / BQT - t0), items = per_head * P.group;
@@ -511,6 +513,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
   tc::tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(slot));
+  tmem_base = tc::uniform(tmem_base);
   pdl_launch_dependents();
 
   if (warp == 0) {
@@ -530,66 +533,68 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- products, the small ones first (offsets in 16-byte units: 16 columns along a row 2, 16 rows 128) ----
-      const uint32_t hi = tc::smem_desc_hi(1024);
-      const uint32_t idesc_s = tc::idesc_bf16(BKT, BQT, 0, 0), idesc_kv = tc::idesc_bf16(BKT, HD, 0, 1), idesc_dq = tc::idesc_bf16(BQT, HD, 1, 1);
-      auto lo = [&](uint32_t off) { return tc::smem_desc_lo(base + off, 16); };  // tiles of one 64-column panel: no leading offset in use
-      auto six = [&](auto&& product) {
-        uint32_t acc = 0;
-        product(2, 0, acc); product(0, 2, acc); product(1, 1, acc); product(1, 0, acc); product(0, 1, acc); product(0, 0, acc);
-      };
-      auto scores = [&](uint32_t col, uint32_t a, uint32_t bq, uint32_t first) { // 128 keys x 64 queries, reduced over half of head_dim
-        six([&](int pb, int pa, uint32_t& acc) {                                 // (parts in the forward's order, where queries are operand A)
+    const bool leader = tc::elect_one();
+    // ---- products, the small ones first (offsets in 16-byte units: 16 columns along a row 2, 16 rows 128) ----
+    const uint32_t hi = tc::smem_desc_hi(1024);
+    const uint32_t idesc_s = tc::idesc_bf16(BKT, BQT, 0, 0), idesc_kv = tc::idesc_bf16(BKT, HD, 0, 1), idesc_dq = tc::idesc_bf16(BQT, HD, 1, 1);
+    auto lo = [&](uint32_t off) { return tc::smem_desc_lo(base + off, 16); };  // tiles of one 64-column panel: no leading offset in use
+    auto six = [&](auto&& product) {
+      uint32_t acc = 0;
+      product(2, 0, acc); product(0, 2, acc); product(1, 1, acc); product(1, 0, acc); product(0, 1, acc); product(0, 0, acc);
+    };
+    auto scores = [&](uint32_t col, uint32_t a, uint32_t bq, uint32_t first) { // 128 keys x 64 queries, reduced over half of head_dim
+      if (!leader) return;
+      six([&](int pb, int pa, uint32_t& acc) {                                 // (parts in the forward's order, where queries are operand A)
 #pragma unroll
-          for (uint32_t kk = 0; kk < HD / 32; ++kk, acc = 1)
-            tc::mma_bf16_ss_w(tmem_base + col, a + pa * (SM::KV_PART >> 4) + first + kk * 2, hi, bq + pb * (SM::Q_PART >> 4) + first + kk * 2, hi, idesc_s, acc);
-        });
-      };
-      auto weighted = [&](uint32_t col, uint32_t parts, uint32_t bq) {           // 128 keys x head_dim, reduced over 64 queries
-        six([&](int pa, int pb, uint32_t& acc) {
+        for (uint32_t kk = 0; kk < HD / 32; ++kk, acc = 1)
+          tc::mma_bf16_ss_w(tmem_base + col, a + pa * (SM::KV_PART >> 4) + first + kk * 2, hi, bq + pb * (SM::Q_PART >> 4) + first + kk * 2, hi, idesc_s, acc);
+      });
+    };
+    auto weighted = [&](uint32_t col, uint32_t parts, uint32_t bq) {           // 128 keys x head_dim, reduced over 64 queries
+      if (!leader) return;
+      six([&](int pa, int pb, uint32_t& acc) {
 #pragma unroll
-          for (uint32_t kk = 0; kk < BQT / 16; ++kk, acc = 1)
-            tc::mma_bf16_ts_w(tmem_base + col, tmem_base + parts + pa * 32 + kk * 8, bq + pb * (SM::Q_PART >> 4) + kk * 128, hi, idesc_kv, acc);
-        });
-      };
-      auto queries = [&](uint32_t col, uint32_t first) {                         // 64 queries x head_dim, reduced over 32 keys
-        six([&](int pa, int pb, uint32_t& acc) {
+        for (uint32_t kk = 0; kk < BQT / 16; ++kk, acc = 1)
+          tc::mma_bf16_ts_w(tmem_base + col, tmem_base + parts + pa * 32 + kk * 8, bq + pb * (SM::Q_PART >> 4) + kk * 128, hi, idesc_kv, acc);
+      });
+    };
+    auto queries = [&](uint32_t col, uint32_t first) {                         // 64 queries x head_dim, reduced over 32 keys
+      if (!leader) return;
+      six([&](int pa, int pb, uint32_t& acc) {
 #pragma unroll
-          for (uint32_t kk = 0; kk < 2; ++kk, acc = 1)
-            tc::mma_bf16_ss_w(tmem_base + col, lo(SM::DS_OFF) + pa * (SM::KV_PART >> 4) + first + kk * 128, hi,
-                              lo(SM::K_OFF) + pb * (SM::KV_PART >> 4) + first + kk * 128, hi, idesc_dq, acc);
-        });
-      };
-      bool ok = n_it > 0 && tc::mbar_wait(bar(KVPARTS), 0, status, 423);
-      for (int n = 0; n <= n_it && ok; ++n) {
-        if (n > 0) {
-          if (!tc::mbar_wait(bar(PREADY), (n - 1) & 1, status, 424)) break;
-          tc::tc_fence_after();
-          weighted(SM::DV_COL, SM::P_COL, lo(SM::DO_OFF));
-          tc::mma_commit(bar(DVDONE));
-          if (!tc::mbar_wait(bar(DSREADY), (n - 1) & 1, status, 428)) break;
-          tc::tc_fence_after();
-          weighted(SM::DK_COL, SM::DS_COL, lo(SM::Q_OFF));
-          tc::mma_commit(bar(DKDONE));
-          queries(SM::DQ_COL, 0);                            // and over dP^T, S^T and P^T, which have been read
-          queries(SM::DP_COL, 256);
-          queries(SM::S_COL, 512);
-          queries(SM::P_COL, 768);
-          tc::mma_commit(bar(DQDONE));
-        }
-        if (n == n_it) break;
-        if (!tc::mbar_wait(bar(QPARTS), n & 1, status, 425) || (n > 0 && !tc::mbar_wait(bar(DQREAD), (n - 1) & 1, status, 427))) break;
+        for (uint32_t kk = 0; kk < 2; ++kk, acc = 1)
+          tc::mma_bf16_ss_w(tmem_base + col, lo(SM::DS_OFF) + pa * (SM::KV_PART >> 4) + first + kk * 128, hi,
+                            lo(SM::K_OFF) + pb * (SM::KV_PART >> 4) + first + kk * 128, hi, idesc_dq, acc);
+      });
+    };
+    bool ok = n_it > 0 && tc::mbar_wait_warp(bar(KVPARTS), 0, status, 423);
+    for (int n = 0; n <= n_it && ok; ++n) {
+      if (n > 0) {
+        if (!tc::mbar_wait_warp(bar(PREADY), (n - 1) & 1, status, 424)) break;
         tc::tc_fence_after();
-        scores(SM::S_COL, lo(SM::K_OFF), lo(SM::Q_OFF), 0);
-        scores(SM::DV_COL, lo(SM::K_OFF), lo(SM::Q_OFF), HD / 16);       // over the dV and dK of the item before, which have been added
-        tc::mma_commit(bar(SFULL));
-        if (!tc::mbar_wait(bar(DOPARTS), n & 1, status, 426)) break;
+        weighted(SM::DV_COL, SM::P_COL, lo(SM::DO_OFF));
+        if (leader) tc::mma_commit(bar(DVDONE));
+        if (!tc::mbar_wait_warp(bar(DSREADY), (n - 1) & 1, status, 428)) break;
         tc::tc_fence_after();
-        scores(SM::DP_COL, lo(SM::V_OFF), lo(SM::DO_OFF), 0);
-        scores(SM::DK_COL, lo(SM::V_OFF), lo(SM::DO_OFF), HD / 16);
-        tc::mma_commit(bar(DPFULL));
+        weighted(SM::DK_COL, SM::DS_COL, lo(SM::Q_OFF));
+        if (leader) tc::mma_commit(bar(DKDONE));
+        queries(SM::DQ_COL, 0);                            // and over dP^T, S^T and P^T, which have been read
+        queries(SM::DP_COL, 256);
+        queries(SM::S_COL, 512);
+        queries(SM::P_COL, 768);
+        if (leader) tc::mma_commit(bar(DQDONE));
       }
+      if (n == n_it) break;
+      if (!tc::mbar_wait_warp(bar(QPARTS), n & 1, status, 425) || (n > 0 && !tc::mbar_wait_warp(bar(DQREAD), (n - 1) & 1, status, 427))) break;
+      tc::tc_fence_after();
+      scores(SM::S_COL, lo(SM::K_OFF), lo(SM::Q_OFF), 0);
+      scores(SM::DV_COL, lo(SM::K_OFF), lo(SM::Q_OFF), HD / 16);       // over the dV and dK of the item before, which have been added
+      if (leader) tc::mma_commit(bar(SFULL));
+      if (!tc::mbar_wait_warp(bar(DOPARTS), n & 1, status, 426)) break;
+      tc::tc_fence_after();
+      scores(SM::DP_COL, lo(SM::V_OFF), lo(SM::DO_OFF), 0);
+      scores(SM::DK_COL, lo(SM::V_OFF), lo(SM::DO_OFF), HD / 16);
+      if (leader) tc::mma_commit(bar(DPFULL));
     }
   } else {
     // ---- 16 warps: thread = (key row, a quarter of the queries and of the columns of dK, dV, dQ) ----
