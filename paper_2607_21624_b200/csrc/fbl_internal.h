@@ -69,7 +69,7 @@ struct fbl_plan {
   int knob_gemm_pair;       // -1 by size, 0 never the CTA-pair GEMM kernel, 1 wherever its tile shape is legal
   int knob_gemm_esets;      // 0 by tiles per block, 1 / 2 sets of epilogue warps
   int knob_f32_bn, knob_f32_slices;   // 0 by size, 64 / 128 columns and 1, 2, 4, 8 slices of the fp32 products' tiles
-  int knob_fwd_tiles;       // 0 by sequence length, 1 / 2 query tiles per forward-attention block at head_dim 64
+  int knob_fwd_tiles;       // 0 by shape, 1 / 2 query tiles per forward-attention block at head_dim 64
   // low-rank adapters on Q, K, V (fbl_plan_enable_lora): rank, and the offsets of T = Xn [Aq|Ak|Av] inside `saved`,
   // of dT and of the unused norm-parameter gradients inside the backward scratch
   float rope_base;          // > 0: rotary position embedding on Q and K (fbl_plan_enable_rope)

@@ -534,6 +534,25 @@ cudaError_t fwd_make_t(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, int n_qt
   return L.set(attn_fwd_tc_kernel<HD, TILES, SPLIT>, P.n_slots * p->d.n_q_heads * p->d.batch, 64 + 128 * TILES, FwdSmem<HD, TILES>::TOTAL);
 }
 
+// head_dim 64: one query tile a block and two blocks per SM, or two tiles (a single one where `pair` is 0) and one block per SM.
+// A block of two tiles takes 0.93 of the time of two blocks of one (it looks at a score once, and three score buffers rotate), a
+// tile alone on its SM 0.8 of what it takes in a block of one; blocks of one start and end faster and fill the SMs in
+// finer steps.  So, from forward passes of 200 to 2048 tokens, 8 to 128 heads and sequences (one / two tiles, us):
+//   short: one (5 x 16 heads of 384: 37.5 / 41.8; 1500 queries over 200 keys: 77.0 / 82.7);
+//   less than an SM's worth of pairs: a tile alone where all tiles fit at once (12 heads of 500: 25.3 / 23.2, of 1500 causal 41.8 /
+//   36.0), else one (2 x 20 heads of 830: 49.5 / 59.2), but for long causal chains (16 heads of 1536: 49.6 / 40.2);
+//   causal pairs: one up to nine tiles, eight aside (4 x 16 heads of 520: 33.1 / 38.0, 1020: 55.2 / 55.2, 1152: 59.5 / 62.4, 2048: 120.8 / 114.6);
+//   else rounds: one where the pairs' last round costs more (3 x 32 heads of 1150: 134 / 140, of 1500: 180 / 168); five rounds and more even out.
+bool fwd_one_tile(const fbl_plan* p, int n_qt, int pair) {
+  const int n_kt = (p->seq_kv + BKV - 1) / BKV;
+  if (n_qt <= 2 || n_kt <= 2) return true;
+  const long long sm = p->sm_count, heads = (long long)p->d.n_q_heads * p->d.batch, blocks = n_qt * heads, pairs = (n_qt + 1) / 2 * heads;
+  if (!pair) return blocks > sm && (!p->d.causal || n_qt <= 6);
+  if (n_qt <= 4 || n_kt <= 4) return true;
+  if (p->d.causal) return n_qt <= 9 && n_qt != 8;
+  return pairs <= 5 * sm && 1.08 * ((blocks + 2 * sm - 1) / (2 * sm)) < (pairs + sm - 1) / sm;
+}
+
 template <int HD>
 cudaError_t fwd_make(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, const void* Q, const void* K, const void* V) {
   AttnFwdParams& P = L.P;
@@ -551,9 +570,9 @@ cudaError_t fwd_make(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, const void
   P.pair = (n_qt >= 2 && (long long)((n_qt + 1) / 2) * p->d.n_q_heads * p->d.batch >= p->sm_count) ? 1 : 0;
   if (attn_fp32(p)) return fwd_make_t<HD, HD == 64 ? 1 : 2, true>(L, p, n_qt);
   if (HD == 64) {
-    // tuning knob: 1 = one query tile per block and two blocks per SM, 2 = two tiles per block; default by sequence length
+    // tuning knob: 1 = one query tile per block and two blocks per SM, 2 = two tiles per block; default by shape
     const int mode = p->knob_fwd_tiles;
-    if (mode == 1 || (mode == 0 && n_qt <= 4)) return fwd_make_t<64, 1>(L, p, n_qt);
+    if (mode == 1 || (mode == 0 && fwd_one_tile(p, n_qt, P.pair))) return fwd_make_t<64, 1>(L, p, n_qt);
   }
   return fwd_make_t<HD, 2>(L, p, n_qt);
 }

@@ -359,6 +359,20 @@ def test_few_rows_keep_fp32_probabilities(cfg):
 
 
 @pytest.mark.parametrize("cfg", [
+    # one or two query tiles a block of the forward: pairs of five causal tiles, tiles that just do not and just do fit the SMs at
+    # once, few key tiles, a round of pairs too many, long causal chains
+    LayerConfig("qt1", 13, 520, 256, 4, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 361, 0.05),
+    LayerConfig("qt2", 15, 515, 128, 2, 1, 64, "bf16", "rmsnorm", False, False, False, 1e-5, 362, 0.05),
+    LayerConfig("qt3", 1, 300, 256, 4, 4, 64, "bf16", "rmsnorm", True, False, True, 1e-5, 363, 0.05),
+    LayerConfig("qt4", 13, 520, 256, 4, 4, 64, "bf16", "rmsnorm", False, False, True, 1e-5, 364, 0.05),
+    LayerConfig("qt5", 11, 900, 128, 2, 1, 64, "bf16", "rmsnorm", True, False, True, 1e-5, 365, 0.05),
+    XattnConfig("qt6", 10, 700, 200, 256, 128, 4, 2, 64, "bf16", "layernorm", True, True, 1e-5, 366, 0.05),
+], ids=lambda c: c.name)
+def test_query_tiles_of_a_forward_block(cfg):
+    check(cfg)
+
+
+@pytest.mark.parametrize("cfg", [
     # a key and a query tile that reach past a sequence: fp32 at each head width and beside a cluster, bf16 of few rows
     LayerConfig("iso1", 3, 20, 64, 2, 1, 32, "fp32", "layernorm", True, True, True, 1e-5, 341, 0.2),
     LayerConfig("iso2", 3, 77, 128, 4, 2, 64, "fp32", "rmsnorm", False, False, True, 1e-5, 342, 0.1),
