@@ -51,7 +51,7 @@ __device__ __forceinline__ void lds2x2(uint32_t a, f2& x, f2& y) {
 
 // The slice's reduction loop and its partial tile, left in shared memory (row-major, OUT_LD) over the operand stages.
 template <bool AK, bool BKR>
-__device__ __forceinline__ void tile_loop(uint32_t base, uint32_t bars, int n_kb, int32_t* status) {
+__device__ __forceinline__ void tile_loop(uint32_t base, uint32_t bars, int n_kb, tc::Status status) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int tm = (warp % 2) * 8 + lane % 8, tn = (warp / 2) * 4 + lane / 8;    // 16 x 8 threads
   constexpr int NP = BKR ? 4 : 8;           // accumulator pairs per row: two columns, or even and odd K of one column
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(THREADS, 3) gemm_ffma_kernel(const __grid_cons
   auto full = [&](int s) { return bars + 8u * s; };
   auto empty = [&](int s) { return bars + 8u * (STAGES + s); };
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  int32_t* status = G.status;
+  const tc::Status status(G.status, G.reset_status);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       tc::mbar_init(full(s), 1);

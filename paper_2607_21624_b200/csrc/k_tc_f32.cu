@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
   auto done = [&](int b) { return bars + 8u * (2 * STAGES + 2 + b); };      // the products have read them: accumulator complete
   auto added = [&](int b) { return bars + 8u * (2 * STAGES + 4 + b); };     // the accumulator has been read
   const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
-  int32_t* status = G.status;
+  const tc::Status status(G.status, G.reset_status);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       tc::mbar_init(full(s), 1);

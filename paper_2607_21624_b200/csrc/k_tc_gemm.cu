@@ -406,7 +406,7 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
   auto acc_empty = [&](int a) { return bars + 8u * (2 * STAGES + 2 + a); };
   const uint32_t slot = bars + 8 * SP::N_BARS;
   const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
-  int32_t* status = G.status;
+  const tc::Status status(G.status, G.reset_status);
   constexpr uint32_t TMEM_COLS = 2 * BN;                 // two fp32 accumulators of BN columns
 
   if (threadIdx.x == 0) {
@@ -614,7 +614,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(EPI == EPI_ACT ? 255 : 224
   const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
   const uint32_t rank = tc::cluster_ctarank();
   const int pair_id = blockIdx.x / 2, n_pairs = gridDim.x / 2;
-  int32_t* status = G.status;
+  const tc::Status status(G.status, G.reset_status);
   constexpr uint32_t TMEM_COLS = 2 * BN;
 
   if (threadIdx.x == 0) {
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(320, 1) gemm_tc_split_kernel(const __grid_cons
   auto full = [&](int s) { return bars + 8u * s; };
   auto empty = [&](int s) { return bars + 8u * (STAGES + s); };
   const int warp = (int)tc::uniform(threadIdx.x / 32), lane = threadIdx.x % 32;
-  int32_t* status = G.status;
+  const tc::Status status(G.status, G.reset_status);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       tc::mbar_init(full(s), 1);

@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from fbl_inputs import LayerConfig, make_inputs
+from fbl_inputs import LayerConfig, MlpConfig, XattnConfig, make_inputs, make_mlp_inputs, make_xattn_inputs
 from tests.test_gpu_layer import run_and_compare
 
 pytestmark = pytest.mark.gpu
@@ -162,6 +162,39 @@ def test_bounded_wait_expires_and_the_context_stays_usable():
     ref = run.fetch("Y")
     run.step()
     assert run.status() == 0 and np.array_equal(ref, run.fetch("Y"))
+
+
+@pytest.mark.parametrize("cfg", [
+    LayerConfig("sw1", 2, 300, 256, 4, 2, 64, "bf16", "layernorm", True, True, True, 1e-5, 71, 0.02),
+    LayerConfig("sw2", 4, 300, 512, 8, 8, 64, "fp32", "layernorm", True, True, True, 1e-5, 72, 0.02),
+    LayerConfig("sw3", 1, 20, 64, 2, 2, 32, "fp32", "rmsnorm", True, False, True, 1e-5, 73, 0.02),
+    MlpConfig("sw4", 2, 600, 256, 1024, "bf16", "layernorm", "gelu", True, True, 1e-5, 74, 0.02),
+    MlpConfig("sw5", 1, 300, 256, 1024, "fp32", "rmsnorm", "swiglu", True, True, 1e-5, 75, 0.02),
+    XattnConfig("sw6", 2, 100, 300, 256, 128, 4, 2, 64, "fp32", "layernorm", True, True, 1e-5, 76, 0.02),
+], ids=lambda c: c.name)
+def test_a_code_that_an_earlier_pass_left_is_none_of_this_one(cfg):
+    # Each pass resets the status word itself, and its waits must not look at the word before: the scratch arrives with
+    # every word non-zero, behind launches that let the pass's first kernels start long before they end themselves.
+    import torch
+    from paper_2607_21624_b200 import LayerRunner, MlpRunner, XattnRunner
+    mlp = isinstance(cfg, MlpConfig)
+    run = MlpRunner(cfg) if mlp else XattnRunner(cfg) if isinstance(cfg, XattnConfig) else LayerRunner(cfg)
+    run.load_inputs(make_mlp_inputs(cfg) if mlp else make_xattn_inputs(cfg) if isinstance(cfg, XattnConfig) else make_inputs(cfg))
+    ahead = LayerRunner(LayerConfig("sw", 8, 1024, 2048, 32, 32, 64, "bf16", "layernorm", False, False, False, 1e-5, 0, 0.02))
+    names = ("Y", "dW1", "dW2") if mlp else ("Y", "dWo", "dWv")
+    run.step()
+    torch.cuda.synchronize()
+    want = {n: run.fetch(n) for n in names}
+    for _ in range(5):
+        run.scratch_fwd.fill_(0x7B)
+        run.scratch.fill_(0x7B)
+        ahead.forward()
+        run.forward()
+        ahead.forward()
+        run.backward()
+        assert run.status() == 0
+        for n in names:
+            assert np.array_equal(want[n], run.fetch(n)), n
 
 
 def test_forward_timeout_code_survives_the_backward():
