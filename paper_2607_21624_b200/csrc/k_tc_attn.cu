@@ -908,6 +908,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_kernel(const __gri
         tc::mbar_arrive(bar(BB_STAGEFREE + (dit % NS)));     // one barrier per staging buffer: a waiter is never
                                                              // more than one phase behind
       }
+      tc::bulk_wait_group0();                        // all sums are in global memory before the block exits, as in the products
     }
   } else if (warp >= 2 && warp < 18) {
     // ---- softmax warps: thread = (key row, one quarter of the 128 query columns) -----------------------
