@@ -1,7 +1,6 @@
 // What the two kernels for fp32 products share: the parameter block of a launch, and the end of a tile's work -- slices'
 // sums, bias, residual, padding rows, the fused row reduction.
 #pragma once
-#include <float.h>
 #include <string.h>
 
 #include "fbl_internal.h"
@@ -25,7 +24,7 @@ struct alignas(64) Problem {
   const float* dot_with;                    // fused D = rowsum(C * dot_with) per head (head widths 32 and 64), or nullptr
   float* dot_out;
   int dot_hd, dot_hq;
-  // the operands themselves, for results that the kernel on the tensor cores forms again (see there)
+  // the operands themselves, for tiles that the kernel on the tensor cores forms again (see there)
   const float* a[MAX_TERMS];
   const float* b[MAX_TERMS];
   long long a_rpad[MAX_TERMS], b_rpad[MAX_TERMS];
@@ -96,21 +95,10 @@ __device__ __forceinline__ float4 lds4(uint32_t a) {
   return v;
 }
 
-// One result from the operands in memory, one multiply-add after another.
-__device__ __forceinline__ float plain_result(const Problem& P, int m, int n) {
-  float s = 0.f;
-  for (int t = 0; t < P.n_terms; ++t)
-    for (int k = 0; k < P.k[t]; ++k)
-      s = fmaf(P.a[t][P.a_k[t] ? rt_off<32>(P.a_rpad[t], k, m) : rt_off<32>(P.a_rpad[t], m, k)],
-               P.b[t][P.b_k[t] ? rt_off<32>(P.b_rpad[t], k, n) : rt_off<32>(P.b_rpad[t], n, k)], s);
-  return s;
-}
-
 // This block's share of the tile's rows: the slices' sums (each block's at `base` of its shared memory, rows LD floats apart)
 // in slice order, bias, residual, padding rows, 16-byte stores.  A thread keeps its four columns and has two rows in flight (one
-// at a time, each waiting for its loads, an 800 x 768 x 768 product took 2 us longer).  AGAIN: results that are not finite
-// are formed again.
-template <int BM, int BN, int LD, int THREADS, bool AGAIN>
+// at a time, each waiting for its loads, an 800 x 768 x 768 product took 2 us longer).
+template <int BM, int BN, int LD, int THREADS>
 __device__ __forceinline__ void finish_tile(const Problem& P, int slices, int slice, uint32_t base, int m0, int n0) {
   constexpr int VECS = BN / 4, STEP = THREADS / VECS, U = 2;
   static_assert(THREADS % VECS == 0, "whole rows");
@@ -154,13 +142,6 @@ __device__ __forceinline__ void finish_tile(const Problem& P, int slices, int sl
       float dot = 0.f;
       if (live[u]) {
         float4 v = s[u];
-        if (AGAIN && !(fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + fabsf(v.w) <= FLT_MAX)) {
-#pragma unroll 1
-          for (int j = 0; j < 4; ++j) {
-            const float r = plain_result(P, m, n + j);
-            if (j == 0) v.x = r; else if (j == 1) v.y = r; else if (j == 2) v.z = r; else v.w = r;
-          }
-        }
         v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
         const int64_t off = rt_off<32>(P.c_rpad, m, n);
         if (P.residual) { v.x += extra[u].x; v.y += extra[u].y; v.z += extra[u].z; v.w += extra[u].w; }

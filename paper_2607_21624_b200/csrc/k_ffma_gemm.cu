@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(THREADS, 3) gemm_ffma_kernel(const __grid_cons
   }
   __syncwarp();
   if (G.slices > 1) tc::cluster_sync_all(); else __syncthreads();
-  f32g::finish_tile<BM, BN, OUT_LD, THREADS, false>(P, G.slices, slice, base, m0, n0);
+  f32g::finish_tile<BM, BN, OUT_LD, THREADS>(P, G.slices, slice, base, m0, n0);
   if (G.slices > 1) tc::cluster_sync_all();      // no block leaves while another may still read its partial tile
 }
 

@@ -7,8 +7,10 @@
 // Accuracy.  Every bf16 x bf16 product is exact in fp32; what is lost is the tensor core's own accumulation.  The accumulator
 // is therefore used for no more than 64 columns of a reduction, the small products first, and added to a sum that a thread
 // keeps in registers (rounded to nearest): no value passes more than four accumulations at its full size before such an addition.
-// Results that are not finite are formed again by plain multiply-adds, since an infinity has no parts (inf - inf is NaN),
-// so operands of any value give what the FP32 pipe gives.
+// An infinity has no parts (inf - inf is NaN), so a block whose part of a tile is not finite throughout forms it again by plain
+// multiply-adds: infinities and NaN go where the FP32 pipe puts them.  (ViT-shaped step of 4 x 197 tokens with an infinity in X,
+// which reaches every weight gradient: 840 us, all on the FP32 pipe 450, a thread to a result 20000; feed-forward step of 800 x 768 x
+// 3072 930, 630, 12000.)
 //
 // One block per 128 x BN tile, or per slice of its reduction (then a cluster shares the tile; partial tiles meet in distributed
 // shared memory in a fixed order: no atomics, the same bits every time).  18 warps: one loads fp32 operand tiles by TMA, four
@@ -43,7 +45,7 @@ struct Smem {
   static constexpr uint32_t A_BYTES = BM * BK * 4, B_BYTES = BN * BK * 4, STAGE = A_BYTES + B_BYTES;
   static constexpr uint32_t PART = BN * 128, PARTS_OFF = STAGES * STAGE;              // two sets of three parts of B
   static constexpr uint32_t BAR_OFF = PARTS_OFF + 6 * PART, N_BARS = 2 * STAGES + 6;
-  static constexpr uint32_t TOTAL = BAR_OFF + 8 * N_BARS + 16 + 1024;                 // + tensor memory slot + alignment slack
+  static constexpr uint32_t TOTAL = BAR_OFF + 8 * N_BARS + 16 + 1024;                 // + tensor memory slot, flag, alignment slack
   static constexpr int LD = BN + 4;                                                   // row pitch of the finished tile
   static_assert(BM * LD * 4 <= STAGES * STAGE, "the finished tile fits the stages");
 };
@@ -54,13 +56,81 @@ template <int BN> __device__ constexpr uint32_t a_col(int set, int part) { retur
 using tc::split3;
 using tc::sts4;
 
+// This block's part of its tile (k-blocks kb_begin .. kb_end) once more by multiply-adds, all threads of the block: where a result
+// is not finite, which an infinity makes of every product that it is in.  32 columns of the reduction at a time, at `stage` in shared memory as
+// [column][row]; a thread has four rows and BN / 16 columns of the tile, which goes to `tile` (rows LD floats apart).
+template <int BN>
+__device__ __noinline__ void plain_tile(const Problem& P, uint32_t tile, uint32_t stage, int m0, int n0, int kb_begin, int kb_end) {
+  constexpr int KS = 32, LDA = BM + 4, LDB = BN + 4, NV = BN / 64, GROUPS = 512;
+  static_assert(KS * (LDA + LDB) * 4 <= (int)(6 * Smem<BN>::PART) && GROUPS <= THREADS && GROUPS * 4 * 4 * NV == BM * BN, "parts' area, a thread's results");
+  const uint32_t sa = stage, sb = stage + KS * LDA * 4;
+  const int row = (int)(threadIdx.x / 16) * 4, col = (int)(threadIdx.x % 16) * 4;          // columns col, col + 64
+  float4 sum[4][NV];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) sum[i][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  // `rows` rows from r0 on (of `end`) of one operand, columns k0 .. k0 + 31 (of K) of the reduction; zeros beyond
+  auto fill = [&](uint32_t to, int ld, int rows, const float* m, long long r_pad, bool rows_are_k, int r0, int end, int k0, int K) {
+    for (int e = threadIdx.x; e < rows * (KS / 4); e += THREADS) {
+      if (rows_are_k) {
+        const int k = e / (rows / 4), r = e % (rows / 4) * 4;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r0 + r < end && k0 + k < K) x = *reinterpret_cast<const float4*>(m + rt_off<32>(r_pad, k0 + k, r0 + r));
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(to + (k * ld + r) * 4), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w) : "memory");
+      } else {
+        const int r = e % rows, k = e / rows * 4;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r0 + r < end && k0 + k < K) x = *reinterpret_cast<const float4*>(m + rt_off<32>(r_pad, r0 + r, k0 + k));
+        const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) asm volatile("st.shared.f32 [%0], %1;" ::"r"(to + ((k + i) * ld + r) * 4), "f"(v[i]) : "memory");
+      }
+    }
+  };
+  int t = 0, kb = kb_begin;
+#pragma unroll 1
+  for (int left = kb_end - kb_begin; left > 0; --left, ++kb) {
+    while (kb >= P.kblocks[t]) { kb -= P.kblocks[t]; ++t; }
+#pragma unroll 1
+    for (int k0 = kb * BK; k0 < min(kb * BK + BK, P.k[t]); k0 += KS) {
+      __syncthreads();
+      fill(sa, LDA, BM, P.a[t], P.a_rpad[t], P.a_k[t] != 0, m0, P.m, k0, P.k[t]);
+      fill(sb, LDB, BN, P.b[t], P.b_rpad[t], P.b_k[t] != 0, n0, P.n, k0, P.k[t]);
+      __syncthreads();
+      if (threadIdx.x < GROUPS) {
+#pragma unroll 4
+        for (int k = 0; k < KS; ++k) {
+          const float4 a4 = lds4(sa + (k * LDA + row) * 4);
+          const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const float4 b = lds4(sb + (k * LDB + col + 64 * v) * 4);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              sum[i][v].x = fmaf(a[i], b.x, sum[i][v].x); sum[i][v].y = fmaf(a[i], b.y, sum[i][v].y);
+              sum[i][v].z = fmaf(a[i], b.z, sum[i][v].z); sum[i][v].w = fmaf(a[i], b.w, sum[i][v].w);
+            }
+          }
+        }
+      }
+    }
+  }
+  if (threadIdx.x < GROUPS)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) sts4(tile + ((row + i) * Smem<BN>::LD + col + 64 * v) * 4, reinterpret_cast<const uint32_t*>(&sum[i][v]));
+  __syncthreads();
+}
+
 template <int BN>
 __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_constant__ Group G) {
   using SM = Smem<BN>;
   constexpr int STAGES = SM::STAGES;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t bars = base + SM::BAR_OFF, slot = bars + 8 * SM::N_BARS;
+  const uint32_t bars = base + SM::BAR_OFF, slot = bars + 8 * SM::N_BARS, flag = slot + 8;
   auto full = [&](int s) { return bars + 8u * s; };                         // fp32 tiles of a stage have arrived
   auto empty = [&](int s) { return bars + 8u * (STAGES + s); };             // ... have been read
   auto parts = [&](int b) { return bars + 8u * (2 * STAGES + b); };         // both operands' parts are in place
@@ -79,6 +149,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
       tc::mbar_init(added(b), 8);
     }
     tc::fence_barrier_init();
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(0u) : "memory");
   }
   if (warp == 1) {
     tc::tmem_alloc(slot, TMEM_COLS);
@@ -240,6 +311,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(added(b));
     }
+    float2 probe = make_float2(0.f, 0.f);     // NaN if and only if a sum is not finite
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) probe = __ffma2_rn(sum[i], make_float2(0.f, 0.f), probe);
+    if (!(probe.x == 0.f && probe.y == 0.f)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
     // the partial tile, over the stages: the last accumulator is complete, so every operand has been read
     const uint32_t row = base + (uint32_t)((q * 32 + lane) * SM::LD + half * N) * 4;
 #pragma unroll
@@ -248,9 +323,13 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
   __syncwarp();
   tc::tc_fence_before();
   pdl_wait();                                      // before anything is written
-  if (G.slices > 1) tc::cluster_sync_all(); else __syncthreads();
+  __syncthreads();
+  uint32_t again;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(again) : "r"(flag) : "memory");
+  if (again) plain_tile<BN>(P, base, base + SM::PARTS_OFF, m0, n0, kb_begin, kb_begin + n_kb);
+  if (G.slices > 1) tc::cluster_sync_all();
   if (warp == 1) tc::tmem_dealloc(tmem_base, TMEM_COLS);
-  f32g::finish_tile<BM, BN, SM::LD, THREADS, true>(P, G.slices, slice, base, m0, n0);
+  f32g::finish_tile<BM, BN, SM::LD, THREADS>(P, G.slices, slice, base, m0, n0);
   if (G.slices > 1) tc::cluster_sync_all();      // no block leaves while another may still read its partial tile
 }
 

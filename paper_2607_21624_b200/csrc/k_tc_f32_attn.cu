@@ -60,37 +60,101 @@ struct FwdSmem {
   static_assert(O_COL + HD <= 512, "tensor memory columns");
 };
 
-// Rows i0 .. of a head by plain arithmetic, a warp to a row: for blocks whose operands are not all finite.
+// A block's rows by plain arithmetic, where its operands are not all finite: the threads that are left when the others' work is
+// done, two to a query row (half of the keys' scores and of the output's columns each), tiles of 64 keys in shared memory.  A key
+// that the mask leaves out takes no part, whatever it holds.
 template <int HD>
-__device__ void plain_rows(const F32FwdParams& P, int b, int h, int g, int first, int last) {
-  const int lane = threadIdx.x % 32;
-  constexpr int N = HD / 32;
-#pragma unroll 1
-  for (int gi = first; gi < min(last, P.seq); ++gi) {
-    const long long row = (long long)b * P.t_pad + gi;
-    float q[N], o[N], m = -INFINITY, l = 0.f;
-#pragma unroll
-    for (int c = 0; c < N; ++c) { q[c] = P.q[rt_off<32>(P.n_pad, row, h * HD + c * 32 + lane)]; o[c] = 0.f; }
-    const int end = P.causal ? min(P.seq_k, gi + 1) : P.seq_k;
-#pragma unroll 1
-    for (int j = 0; j < end; ++j) {
-      const long long key = (long long)b * P.t_pad_k + j;
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < N; ++c) s = fmaf(q[c], P.k[rt_off<32>(P.n_pad_k, key, g * HD + c * 32 + lane)], s);
-#pragma unroll
-      for (int x = 16; x > 0; x /= 2) s += __shfl_xor_sync(0xffffffffu, s, x);
-      s *= P.scale;
-      const float m_new = fmaxf(m, s), alpha = m_new == -INFINITY ? 1.f : expf(m - m_new), p = m_new == -INFINITY ? 0.f : expf(s - m_new);
-      l = l * alpha + p;
-      m = m_new;
-#pragma unroll
-      for (int c = 0; c < N; ++c) o[c] = fmaf(p, P.v[rt_off<32>(P.n_pad_k, key, g * HD + c * 32 + lane)], o[c] * alpha);
+__device__ __noinline__ void plain_rows(const F32FwdParams& P, uint32_t base, int i0, int h, int b) {
+  constexpr int LD = HD + 4, LDP = KT + 1, N = HD / 4, HC = HD / 2;      // row pitches that keep a warp's rows on different banks
+  const uint32_t sq = base, sk = sq + QT * LD * 4, sv = sk + KT * HD * 4, sp = sv + KT * HD * 4, sm = sp + QT * LDP * 4;
+  static_assert((QT * LD + 2 * KT * HD + QT * LDP + 2 * QT) * 4 <= (int)FwdSmem<HD>::BAR_OFF, "shared memory");
+  const int r = threadIdx.x % QT, half = threadIdx.x / QT, gi = i0 + r, g = h / P.group;
+  const bool work = threadIdx.x < 2 * QT;
+  auto fill = [&](uint32_t to, int ld, int rows, const float* m, long long n_pad, int t_pad, int row0, int end, int col) {
+    for (int e = threadIdx.x; e < rows * N; e += FWD_THREADS) {
+      const int row = e / N, c = e % N * 4;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (row0 + row < end) x = *reinterpret_cast<const float4*>(m + rt_off<32>(n_pad, (long long)b * t_pad + row0 + row, col + c));
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(to + (row * ld + c) * 4), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w) : "memory");
     }
+  };
+  fill(sq, LD, QT, P.q, P.n_pad, P.t_pad, i0, P.seq, h * HD);
+  const int j_end = P.causal ? min(P.seq_k, i0 + QT) : P.seq_k, mine_end = P.causal ? min(P.seq_k, gi + 1) : P.seq_k;
+  float m = -INFINITY, l = 0.f, o[HC];
 #pragma unroll
-    for (int c = 0; c < N; ++c) P.a[rt_off<32>(P.n_pad, row, h * HD + c * 32 + lane)] = o[c] * (1.f / l);
-    if (lane == 0) P.lse[((long long)b * P.hq + h) * P.t_pad + gi] = m + logf(l);
+  for (int c = 0; c < HC; ++c) o[c] = 0.f;
+#pragma unroll 1
+  for (int j0 = 0; j0 < j_end; j0 += KT) {
+    __syncthreads();
+    fill(sk, HD, KT, P.k, P.n_pad_k, P.t_pad_k, j0, P.seq_k, g * HD);
+    fill(sv, HD, KT, P.v, P.n_pad_k, P.t_pad_k, j0, P.seq_k, g * HD);
+    __syncthreads();
+    float s[KT / 2], mx = -INFINITY;
+    if (work) {
+#pragma unroll
+      for (int k = 0; k < KT / 2; ++k) s[k] = 0.f;
+#pragma unroll 1
+      for (int d = 0; d < HD; d += 4) {
+        const float4 q = tc::lds4(sq + (r * LD + d) * 4);
+#pragma unroll
+        for (int k = 0; k < KT / 2; ++k) {
+          const float4 x = tc::lds4(sk + ((half * 32 + k) * HD + d) * 4);
+          s[k] = fmaf(q.x, x.x, fmaf(q.y, x.y, fmaf(q.z, x.z, fmaf(q.w, x.w, s[k]))));
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < KT / 2; ++k) {
+        s[k] = j0 + half * 32 + k < mine_end ? s[k] * P.scale : -INFINITY;
+        mx = fmaxf(mx, s[k]);
+      }
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(sm + threadIdx.x * 4), "f"(mx) : "memory");
+    }
+    __syncthreads();
+    float alpha = 1.f;
+    if (work) {
+      float mo;
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(mo) : "r"(sm + ((half ^ 1) * QT + r) * 4) : "memory");
+      const float m_new = fmaxf(m, fmaxf(mx, mo));
+      alpha = m_new == -INFINITY ? 1.f : expf(m - m_new);
+      m = m_new;
+      float sum = 0.f;
+#pragma unroll
+      for (int k = 0; k < KT / 2; ++k) {
+        const float p = m == -INFINITY || j0 + half * 32 + k >= mine_end ? 0.f : expf(s[k] - m);
+        sum += p;
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(sp + (r * LDP + half * 32 + k) * 4), "f"(p) : "memory");
+      }
+      l = l * alpha + sum;
+    }
+    __syncthreads();
+    if (work) {
+#pragma unroll
+      for (int c = 0; c < HC; ++c) o[c] *= alpha;
+#pragma unroll 1
+      for (int k = 0; k < min(KT, mine_end - j0); ++k) {
+        float p;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(p) : "r"(sp + (r * LDP + k) * 4) : "memory");
+#pragma unroll
+        for (int c = 0; c < HC; c += 4) {
+          const float4 v = tc::lds4(sv + (k * HD + half * HC + c) * 4);
+          o[c] = fmaf(p, v.x, o[c]); o[c + 1] = fmaf(p, v.y, o[c + 1]); o[c + 2] = fmaf(p, v.z, o[c + 2]); o[c + 3] = fmaf(p, v.w, o[c + 3]);
+        }
+      }
+    }
   }
+  __syncthreads();
+  if (work) asm volatile("st.shared.f32 [%0], %1;" ::"r"(sm + threadIdx.x * 4), "f"(l) : "memory");
+  __syncthreads();
+  if (!work || gi >= P.seq) return;
+  float lo;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(lo) : "r"(sm + ((half ^ 1) * QT + r) * 4) : "memory");
+  l = half ? lo + l : l + lo;
+  const float inv = 1.f / l;
+#pragma unroll
+  for (int c = 0; c < HC; c += 4)
+    *reinterpret_cast<float4*>(P.a + rt_off<32>(P.n_pad, (long long)b * P.t_pad + gi, h * HD + half * HC + c)) =
+        make_float4(o[c] * inv, o[c + 1] * inv, o[c + 2] * inv, o[c + 3] * inv);
+  if (half == 0) P.lse[((long long)b * P.hq + h) * P.t_pad + gi] = m + logf(l);
 }
 
 // One 16-value piece of a row of an fp32 tile as TMA leaves it (`rows` rows to a 32-column panel) -> three parts, each a bf16
@@ -365,8 +429,6 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
       if (lane == 0) tc::mbar_arrive(bar(PFULL));
     }
     if (ok && n_tiles > 0) ok = add_output(n_tiles - 1);
-    uint32_t again;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(again) : "r"(flag) : "memory");
     // the row's sum: both halves', where the next tile's maxima would go
     const uint32_t slot_l = (n_tiles & 1) * (2 * QT * 4);
     asm volatile("st.shared.f32 [%0], %1;" ::"r"(mine + slot_l), "f"(l) : "memory");
@@ -384,14 +446,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
       }
       if (half == 0) P.lse[((long long)b * P.hq + h) * P.t_pad + gi] = live ? m + logf(l) : 0.f;
     }
-    if (ok && again && meet()) {                             // these rows have been written
-      plain_rows<HD>(P, b, h, g, i0 + q * 32 + half * 16, i0 + q * 32 + half * 16 + 16);
-    }
   }
   __syncwarp();
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 1) tc::tmem_dealloc(tmem_base, 512);
+  uint32_t again;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(again) : "r"(flag) : "memory");
+  if (again) plain_rows<HD>(P, base, i0, h, b);
 }
 
 template <int HD>
@@ -456,22 +518,110 @@ struct BwdSmem {                                             // the same for bot
   static constexpr uint32_t S_COL = 0, DP_COL = 64, DV_COL = 128, DK_COL = 192, DQ_COL = 256, P_COL = 320, DS_COL = 416;
 };
 
-// One (query, key) pair by plain arithmetic, a warp to it: P and dS in all lanes.
+// A block's items by plain arithmetic, where an operand or a dS is not finite: dK and dV of all of them, left where the kernel leaves
+// its own, and dQ of those whose own was not added (even and odd items from the two numbers at `from_at` on).  16 warps, four threads to a key row (a quarter of
+// the queries, then of the columns of dK and dV), eight to a query row for dQ.  Pairs that the mask leaves out take no part.
 template <int HD>
-__device__ __forceinline__ void plain_pair(const F32BwdParams& P, const float* q, const float* dO, const float* k, const float* v, float lse, float d,
-                                           float& p, float& ds) {
-  float s = 0.f, dp = 0.f;
+__device__ __noinline__ void plain_items(const F32BwdParams& P, uint32_t base, uint32_t from_at, int n_it, int t0, int per_head) {
+  constexpr int LD = HD + 4, LDP = BQT + 1, N = HD / 4, HC = HD / 4, HQ = HD / 8;
+  const uint32_t sk = base, sv = sk + BKT * LD * 4, sq = sv + BKT * LD * 4, so = sq + BQT * HD * 4, sp = so + BQT * HD * 4, sd = sp + BKT * LDP * 4;
+  static_assert((2 * BKT * LD + 2 * BQT * HD + 2 * BKT * LDP) * 4 <= (int)BwdSmem::STAT_OFF, "shared memory");
+  const bool work = threadIdx.x < 4 * BKT;
+  const int slice = blockIdx.x % P.slices, j0 = blockIdx.x / P.slices * BKT, g = blockIdx.y, b = blockIdx.z;
+  int from[2];
+  for (int i = 0; i < 2; ++i) asm volatile("ld.shared.s32 %0, [%1];" : "=r"(from[i]) : "r"(from_at + 4 * i) : "memory");
+  const int r = threadIdx.x % BKT, quarter = threadIdx.x / BKT % 4, gj = j0 + r, i = threadIdx.x % BQT, eighth = threadIdx.x / BQT % 8;
+  auto fill = [&](uint32_t to, int ld, int rows, const float* m, long long n_pad, int t_pad, int row0, int end, int col) {
+    for (int e = threadIdx.x; e < rows * N; e += BWD_THREADS) {
+      const int row = e / N, c = e % N * 4;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (row0 + row < end) x = *reinterpret_cast<const float4*>(m + rt_off<32>(n_pad, (long long)b * t_pad + row0 + row, col + c));
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(to + (row * ld + c) * 4), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w) : "memory");
+    }
+  };
+  fill(sk, LD, BKT, P.k, P.n_pad_k, P.t_pad_k, j0, P.seq_k, g * HD);
+  fill(sv, LD, BKT, P.v, P.n_pad_k, P.t_pad_k, j0, P.seq_k, g * HD);
+  float dk[HC], dv[HC];
 #pragma unroll
-  for (int c = 0; c < HD / 32; ++c) { s = fmaf(k[c], q[c], s); dp = fmaf(v[c], dO[c], dp); }
+  for (int c = 0; c < HC; ++c) dk[c] = dv[c] = 0.f;
+#pragma unroll 1
+  for (int n = 0; n < n_it; ++n) {
+    const int item = slice + n * P.slices, h = g * P.group + item / per_head, i0 = (t0 + item % per_head) * BQT, gi = i0 + i;
+    const long long at = ((long long)b * P.hq + h) * P.t_pad;
+    __syncthreads();
+    fill(sq, HD, BQT, P.q, P.n_pad, P.t_pad, i0, P.seq, h * HD);
+    fill(so, HD, BQT, P.dO, P.n_pad, P.t_pad, i0, P.seq, h * HD);
+    __syncthreads();
+    // queries of this item that take part with this thread's key: first .. last - 1
+    const int first = P.causal ? max(0, gj - i0) : 0, last = gj < P.seq_k ? min(BQT, P.seq - i0) : 0;
+    if (work) {
+      float s[16], dp[16];
 #pragma unroll
-  for (int x = 16; x > 0; x /= 2) { s += __shfl_xor_sync(0xffffffffu, s, x); dp += __shfl_xor_sync(0xffffffffu, dp, x); }
-  p = expf(s * P.scale - lse);
-  ds = p * (dp - d);
-}
-template <int HD>
-__device__ __forceinline__ void plain_load(float* x, const float* m, long long n_pad, long long row, int col) {
+      for (int k = 0; k < 16; ++k) s[k] = dp[k] = 0.f;
+#pragma unroll 1
+      for (int d = 0; d < HD; d += 4) {
+        const float4 k4 = tc::lds4(sk + (r * LD + d) * 4), v4 = tc::lds4(sv + (r * LD + d) * 4);
 #pragma unroll
-  for (int c = 0; c < HD / 32; ++c) x[c] = m[rt_off<32>(n_pad, row, col + c * 32 + threadIdx.x % 32)];
+        for (int k = 0; k < 16; ++k) {
+          const float4 q4 = tc::lds4(sq + ((quarter * 16 + k) * HD + d) * 4), o4 = tc::lds4(so + ((quarter * 16 + k) * HD + d) * 4);
+          s[k] = fmaf(k4.x, q4.x, fmaf(k4.y, q4.y, fmaf(k4.z, q4.z, fmaf(k4.w, q4.w, s[k]))));
+          dp[k] = fmaf(v4.x, o4.x, fmaf(v4.y, o4.y, fmaf(v4.z, o4.z, fmaf(v4.w, o4.w, dp[k]))));
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const int c = quarter * 16 + k;
+        float p = 0.f, ds = 0.f;
+        if (c >= first && c < last) {
+          p = expf(s[k] * P.scale - P.lse[at + i0 + c]);
+          ds = p * (dp[k] - P.dvec[at + i0 + c]);
+        }
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(sp + (r * LDP + c) * 4), "f"(p) : "memory");
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(sd + (r * LDP + c) * 4), "f"(ds) : "memory");
+      }
+    }
+    __syncthreads();
+    if (!work) continue;
+#pragma unroll 1
+    for (int c = first; c < last; ++c) {
+      float p, ds;
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(p) : "r"(sp + (r * LDP + c) * 4) : "memory");
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(ds) : "r"(sd + (r * LDP + c) * 4) : "memory");
+#pragma unroll
+      for (int x = 0; x < HC; x += 4) {
+        const float4 o4 = tc::lds4(so + (c * HD + quarter * HC + x) * 4), q4 = tc::lds4(sq + (c * HD + quarter * HC + x) * 4);
+        dv[x] = fmaf(p, o4.x, dv[x]); dv[x + 1] = fmaf(p, o4.y, dv[x + 1]); dv[x + 2] = fmaf(p, o4.z, dv[x + 2]); dv[x + 3] = fmaf(p, o4.w, dv[x + 3]);
+        dk[x] = fmaf(ds, q4.x, dk[x]); dk[x + 1] = fmaf(ds, q4.y, dk[x + 1]); dk[x + 2] = fmaf(ds, q4.z, dk[x + 2]); dk[x + 3] = fmaf(ds, q4.w, dk[x + 3]);
+      }
+    }
+    if (n < from[n & 1] || gi >= P.seq) continue;
+    float dq[HQ];
+#pragma unroll
+    for (int x = 0; x < HQ; ++x) dq[x] = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < min(BKT, (P.causal ? min(P.seq_k, gi + 1) : P.seq_k) - j0); ++k) {
+      float ds;
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(ds) : "r"(sd + (k * LDP + i) * 4) : "memory");
+#pragma unroll
+      for (int x = 0; x < HQ; x += 4) {
+        const float4 k4 = tc::lds4(sk + (k * LD + eighth * HQ + x) * 4);
+        dq[x] = fmaf(ds, k4.x, dq[x]); dq[x + 1] = fmaf(ds, k4.y, dq[x + 1]); dq[x + 2] = fmaf(ds, k4.z, dq[x + 2]); dq[x + 3] = fmaf(ds, k4.w, dq[x + 3]);
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < HQ; x += 4)
+      atomicAdd(reinterpret_cast<float4*>(P.dq + rt_off<32>(P.n_pad, (long long)b * P.t_pad + gi, h * HD + eighth * HQ + x)),
+                make_float4(dq[x] * P.scale, dq[x + 1] * P.scale, dq[x + 2] * P.scale, dq[x + 3] * P.scale));
+  }
+  __syncthreads();
+  if (work) {
+#pragma unroll
+    for (int c = 0; c < HC; c += 4) {
+      tc::sts4(base + (r * LD + quarter * HC + c) * 4, reinterpret_cast<const uint32_t*>(&dk[c]));
+      tc::sts4(base + (BKT * LD + r * LD + quarter * HC + c) * 4, reinterpret_cast<const uint32_t*>(&dv[c]));
+    }
+  }
+  __syncthreads();
 }
 
 template <int HD>
@@ -491,11 +641,16 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
   auto head_of = [&](int n) { return g * P.group + (slice + n * slices) / per_head; };
   auto row_of = [&](int n) { return (t0 + (slice + n * slices) % per_head) * BQT; };
   int32_t* status = P.status;
+  auto raised = [&](int i) -> bool {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(flag + 4 * i) : "memory");
+    return v != 0;
+  };
   if (threadIdx.x == 0) {
     for (int i : {KVFULL, QRAW, DORAW, SFULL, DPFULL, DVDONE, DKDONE, DQDONE}) tc::mbar_init(bar(i), 1);
     for (int i : {QRAWE, DORAWE, KVPARTS, QPARTS, DOPARTS, PREADY, DSREADY, DQREAD}) tc::mbar_init(bar(i), WORK_WARPS);
     tc::fence_barrier_init();
-    for (int i = 0; i < 3; ++i) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag + 4 * i), "r"(0u) : "memory");
+    for (int i = 0; i < 5; ++i) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag + 4 * i), "r"(i < 3 ? 0u : 0x7fffffffu) : "memory");
     tc::tma_prefetch_desc(&P.tq); tc::tma_prefetch_desc(&P.tk); tc::tma_prefetch_desc(&P.tv); tc::tma_prefetch_desc(&P.tdo);
     pdl_wait();
     if (n_it > 0) {
@@ -609,11 +764,6 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
     auto raise = [&](const float2& probe, int i) {
       if (!(probe.x == 0.f && probe.y == 0.f)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag + 4 * i), "r"(1u) : "memory");
     };
-    auto raised = [&](int i) -> bool {
-      uint32_t v;
-      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(flag + 4 * i) : "memory");
-      return v != 0;
-    };
     auto convert = [&](uint32_t src, uint32_t dst, int rows, float lift, int flag_i) {
       float2 probe = make_float2(0.f, 0.f);
       for (int u = tid; u < rows * HD / 16; u += 32 * WORK_WARPS) convert_piece(src, dst, rows * 128, rows, u % rows, u / rows, lift, probe);
@@ -658,6 +808,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
 #pragma unroll
       for (int k = 0; k < HC / 2; ++k) sum[k] = __fadd2_rn(sum[k], make_float2(__uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1])));
     };
+    int plain_from[2] = {0x7fffffff, 0x7fffffff};              // even and odd items whose dQ is left to plain_items
     for (int n = 0; n < n_it && ok; ++n) {
       const int h = head_of(n), i0 = row_of(n);
       const uint32_t stat = base + SM::STAT_OFF + (n & 1) * 512;
@@ -743,81 +894,32 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
       const bool again = raised(n & 1) || raised(2);
       arrive(DQREAD);
       const int gi = i0 + q * 16 + lane;
-      if (!again) {
-        if (lane < 16 && gi < P.seq) {
+      if (again) {
+        if (warp == 2 && lane == 0 && n < plain_from[n & 1]) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag + 12 + 4 * (n & 1)), "r"(n) : "memory");
+        plain_from[n & 1] = min(plain_from[n & 1], n);
+      } else if (lane < 16 && gi < P.seq) {
 #pragma unroll
-          for (int c = 0; c < HC / 4; ++c)
-            atomicAdd(reinterpret_cast<float4*>(P.dq + rt_off<32>(P.n_pad, (long long)b * P.t_pad + gi, h * HD + quarter * HC + 4 * c)),
-                      make_float4(dq[2 * c].x * P.scale, dq[2 * c].y * P.scale, dq[2 * c + 1].x * P.scale, dq[2 * c + 1].y * P.scale));
-        }
-      } else {
-        // this block's keys' share of the item's dQ by plain arithmetic, a warp to a query
-#pragma unroll 1
-        for (int i = i0 + warp - 2; i < min(i0 + BQT, P.seq); i += WORK_WARPS) {
-          const long long row = (long long)b * P.t_pad + i, at = ((long long)b * P.hq + h) * P.t_pad + i;
-          float xq[PN], xo[PN], sum[PN] = {};
-          plain_load<HD>(xq, P.q, P.n_pad, row, h * HD);
-          plain_load<HD>(xo, P.dO, P.n_pad, row, h * HD);
-          const int end = min(j0 + BKT, P.causal ? min(P.seq_k, i + 1) : P.seq_k);
-#pragma unroll 1
-          for (int j = j0; j < end; ++j) {
-            float xk[PN], xv[PN], p, ds;
-            plain_load<HD>(xk, P.k, P.n_pad_k, (long long)b * P.t_pad_k + j, g * HD);
-            plain_load<HD>(xv, P.v, P.n_pad_k, (long long)b * P.t_pad_k + j, g * HD);
-            plain_pair<HD>(P, xq, xo, xk, xv, P.lse[at], P.dvec[at], p, ds);
-#pragma unroll
-            for (int c = 0; c < PN; ++c) sum[c] = fmaf(ds, xk[c], sum[c]);
-          }
-#pragma unroll
-          for (int c = 0; c < PN; ++c) atomicAdd(P.dq + rt_off<32>(P.n_pad, row, h * HD + c * 32 + lane), sum[c] * P.scale);
-        }
+        for (int c = 0; c < HC / 4; ++c)
+          atomicAdd(reinterpret_cast<float4*>(P.dq + rt_off<32>(P.n_pad, (long long)b * P.t_pad + gi, h * HD + quarter * HC + 4 * c)),
+                    make_float4(dq[2 * c].x * P.scale, dq[2 * c].y * P.scale, dq[2 * c + 1].x * P.scale, dq[2 * c + 1].y * P.scale));
       }
     }
     // dK and dV of this block's items to shared memory, over K's and V's parts, which no product reads any more
     const uint32_t out = base + (uint32_t)(r * (HD + 4) + quarter * HC) * 4;
     constexpr uint32_t SUM_V = BKT * (HD + 4) * 4;
-    if (!(ok && (raised(0) || raised(1) || raised(2)))) {
 #pragma unroll
-      for (int c = 0; c < HC / 2; c += 2) {
-        tc::sts4(out + c * 8, reinterpret_cast<const uint32_t*>(&dk[c]));
-        tc::sts4(out + SUM_V + c * 8, reinterpret_cast<const uint32_t*>(&dv[c]));
-      }
-    } else {
-#pragma unroll 1
-      for (int rr = warp - 2; rr < BKT; rr += WORK_WARPS) {  // by plain arithmetic, a warp to a key
-        const int j = j0 + rr;
-        float xk[PN], xv[PN], sk[PN] = {}, sv[PN] = {};
-        if (j < P.seq_k) {
-          plain_load<HD>(xk, P.k, P.n_pad_k, (long long)b * P.t_pad_k + j, g * HD);
-          plain_load<HD>(xv, P.v, P.n_pad_k, (long long)b * P.t_pad_k + j, g * HD);
-#pragma unroll 1
-          for (int n = 0; n < n_it; ++n) {
-            const int h = head_of(n), i0 = row_of(n);
-#pragma unroll 1
-            for (int i = P.causal ? max(i0, j) : i0; i < min(i0 + BQT, P.seq); ++i) {
-              const long long row = (long long)b * P.t_pad + i, at = ((long long)b * P.hq + h) * P.t_pad + i;
-              float xq[PN], xo[PN], p, ds;
-              plain_load<HD>(xq, P.q, P.n_pad, row, h * HD);
-              plain_load<HD>(xo, P.dO, P.n_pad, row, h * HD);
-              plain_pair<HD>(P, xq, xo, xk, xv, P.lse[at], P.dvec[at], p, ds);
-#pragma unroll
-              for (int c = 0; c < PN; ++c) { sk[c] = fmaf(ds, xq[c], sk[c]); sv[c] = fmaf(p, xo[c], sv[c]); }
-            }
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < PN; ++c) {
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + (rr * (HD + 4) + c * 32 + lane) * 4), "f"(sk[c]) : "memory");
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + SUM_V + (rr * (HD + 4) + c * 32 + lane) * 4), "f"(sv[c]) : "memory");
-        }
-      }
+    for (int c = 0; c < HC / 2; c += 2) {
+      tc::sts4(out + c * 8, reinterpret_cast<const uint32_t*>(&dk[c]));
+      tc::sts4(out + SUM_V + c * 8, reinterpret_cast<const uint32_t*>(&dv[c]));
     }
   }
   __syncwarp();
   tc::tc_fence_before();
   pdl_wait();
-  if (slices > 1) tc::cluster_sync_all(); else __syncthreads();
+  __syncthreads();
   if (warp == 1) tc::tmem_dealloc(tmem_base, 512);
+  if (raised(0) || raised(1) || raised(2)) plain_items<HD>(P, base, flag + 12, n_it, t0, per_head);
+  if (slices > 1) tc::cluster_sync_all();
   const int rows = BKT / slices;                             // of either matrix, that this block finishes
   for (int e = threadIdx.x; e < 2 * rows * (HD / 4); e += BWD_THREADS) {
     const bool is_v = e >= rows * (HD / 4);

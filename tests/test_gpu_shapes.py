@@ -148,6 +148,65 @@ def test_fp32_attention_of_operands_without_parts(head_dim):
     assert np.isinf(outs[1, "V"]["A"]).any() and not np.isfinite(outs[1, "dA"]["dA"]).all()
 
 
+@pytest.mark.parametrize("cfg", [
+    LayerConfig("np1", 2, 150, 128, 4, 2, 64, "fp32", "layernorm", True, True, False, 1e-5, 241, 0.1),
+    LayerConfig("np2", 1, 333, 96, 6, 6, 32, "fp32", "rmsnorm", True, False, True, 1e-5, 242, 0.1),
+], ids=lambda c: c.name)
+def test_fp32_attention_of_an_infinite_token_under_a_mask(cfg):
+    # one token infinite in Q, K and V: the queries before it are what they are without it
+    import numpy as np
+    from fbl_inputs import make_inputs
+    from paper_2607_21624_b200 import LayerRunner
+    inp, at = dict(make_inputs(cfg, affine_noise=True)), 70
+    outs = []
+    for poison in (False, True):
+        run = LayerRunner(cfg, guard_bytes=4096)
+        X = np.array(inp["X"], copy=True)
+        if poison:
+            X[0, at, 3] = np.inf
+        run.load_inputs(dict(inp, X=X))
+        run.step()
+        assert run.status() == 0 and run.guards_intact() == []
+        outs.append({n: np.asarray(run.saved_view(n), dtype=np.float64) for n in ("A", "LSE", "dQ")})
+    clean, got = outs
+    for n in ("A", "dQ"):
+        assert not np.isfinite(got[n][0, at:]).any(), n
+        assert np.linalg.norm(got[n][0, :at] - clean[n][0, :at]) <= 1e-5 * np.linalg.norm(clean[n][0, :at]), n
+        assert np.linalg.norm(got[n][1:] - clean[n][1:]) <= 1e-5 * np.linalg.norm(clean[n][1:]), n
+    assert np.abs(got["LSE"][0, :, :at] - clean["LSE"][0, :, :at]).max() <= 1e-5 * np.abs(clean["LSE"]).max()
+
+
+@pytest.mark.parametrize("cfg", [
+    LayerConfig("nt1", 4, 197, 768, 12, 12, 64, "fp32", "layernorm", False, True, True, 1e-6, 243, 0.02),
+    LayerConfig("nt2", 1, 1024, 512, 16, 4, 32, "fp32", "layernorm", True, False, True, 1e-6, 244, 0.02),
+    MlpConfig("nt3", 2, 400, 512, 2048, "fp32", "layernorm", "gelu", True, True, 1e-6, 245, 0.02),
+], ids=lambda c: c.name)
+def test_fp32_steps_with_an_infinity_take_no_other_time(cfg):
+    # an infinity reaches every weight gradient; the step must stay within a small factor of the multiply-adds that it falls
+    # back to (with a thread to a result it took 25 to 53 times as long)
+    import torch
+    from paper_2607_21624_b200 import LayerRunner, MlpRunner
+    us = {}
+    for path in (0, 1):
+        run = MlpRunner(cfg) if isinstance(cfg, MlpConfig) else LayerRunner(cfg)
+        run.plan.set_kernel_path(path)
+        for n, b in run.buf.items():
+            b.view(run.tdtype).normal_(std=0.02 if n[0] == "W" else 1.0)
+        run.vec["gamma"].fill_(1.0)
+        run.buf["X"].view(run.tdtype)[1000] = float("inf")
+        for _ in range(3):
+            run.step()
+        first, last = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        first.record()
+        for _ in range(5):
+            run.step()
+        last.record()
+        assert run.status() == 0
+        us[path] = first.elapsed_time(last) * 200
+        assert not torch.isfinite(run.buf["dW1" if isinstance(cfg, MlpConfig) else "dWq"].view(run.tdtype)).all()
+    assert us[0] <= 4 * us[1], us
+
+
 def _mlp_outputs(cfg, inp, path):
     import numpy as np
     from paper_2607_21624_b200.mlp import MlpRunner
