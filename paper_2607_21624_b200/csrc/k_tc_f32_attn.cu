@@ -26,7 +26,7 @@ struct Lift {
 
 struct alignas(64) F32FwdParams {
   CUtensorMap tq, tk, tv;
-  const float *q, *k, *v;       // the same operands, for blocks that are formed again
+  const float *q, *k, *v;       // the same operands, for blocks that are worked through by plain arithmetic
   float* a;                     // merged-head output [n_pad, dq]
   float* lse;                   // [B, Hq, t_pad]
   long long n_pad, n_pad_k;
@@ -60,7 +60,8 @@ struct FwdSmem {
   static_assert(O_COL + HD <= 512, "tensor memory columns");
 };
 
-// A block's rows by plain arithmetic, where its operands are not all finite: the threads that are left when the others' work is
+// A block's rows by plain arithmetic, where an operand is out of range (tc::probe_range), so that a score is never more than the
+// products can form: the threads that are left when the others' work is
 // done, two to a query row (half of the keys' scores and of the output's columns each), tiles of 64 keys in shared memory.  A key
 // that the mask leaves out takes no part, whatever it holds.
 template <int HD>
@@ -170,9 +171,8 @@ __device__ __forceinline__ void convert_piece(uint32_t src, uint32_t dst, uint32
   uint32_t p[3][8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    float2 rest;
-    tc::split3(x[2 * k], x[2 * k + 1], lift, p[0][k], p[1][k], p[2][k], rest);
-    probe = __ffma2_rn(rest, make_float2(0.f, 0.f), probe);
+    tc::split3(x[2 * k], x[2 * k + 1], lift, p[0][k], p[1][k], p[2][k]);
+    tc::probe_range(x[2 * k], x[2 * k + 1], probe);
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
           convert_piece(src, dst, SM::PART, KT, unit % KT, unit / KT, which ? 0.f : Lift<HD>::K, probe);
         }
         // the flag before anything that depends on these parts
-        if (!(probe.x == 0.f && probe.y == 0.f)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
+        if (tc::probe_failed(probe)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
         tc::fence_proxy_async();
         __syncwarp();
         if (lane == 0) { tc::mbar_arrive(bar((which ? VEMPTY : KEMPTY) + s)); tc::mbar_arrive(bar((which ? VPARTS : KPARTS) + s)); }
@@ -341,16 +341,15 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const float4 v = tc::lds4(row + (((piece % 2 * 4 + c) ^ (r & 7)) << 4));
-          float2 rest;
-          tc::split3(v.x, v.y, Lift<HD>::Q, p[0][2 * c], p[1][2 * c], p[2][2 * c], rest);
-          probe = __ffma2_rn(rest, make_float2(0.f, 0.f), probe);
-          tc::split3(v.z, v.w, Lift<HD>::Q, p[0][2 * c + 1], p[1][2 * c + 1], p[2][2 * c + 1], rest);
-          probe = __ffma2_rn(rest, make_float2(0.f, 0.f), probe);
+          tc::split3(v.x, v.y, Lift<HD>::Q, p[0][2 * c], p[1][2 * c], p[2][2 * c]);
+          tc::split3(v.z, v.w, Lift<HD>::Q, p[0][2 * c + 1], p[1][2 * c + 1], p[2][2 * c + 1]);
+          tc::probe_range(v.x, v.y, probe);
+          tc::probe_range(v.z, v.w, probe);
         }
 #pragma unroll
         for (int i = 0; i < 3; ++i) tc::tmem_st8(lane_addr + SM::QP_COL + i * (HD / 2) + piece * 8, p[i]);
       }
-      if (!(probe.x == 0.f && probe.y == 0.f)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
+      if (tc::probe_failed(probe)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
       tc::tmem_st_wait();
       tc::tc_fence_before();
       __syncwarp();
@@ -518,7 +517,7 @@ struct BwdSmem {                                             // the same for bot
   static constexpr uint32_t S_COL = 0, DP_COL = 64, DV_COL = 128, DK_COL = 192, DQ_COL = 256, P_COL = 320, DS_COL = 416;
 };
 
-// A block's items by plain arithmetic, where an operand or a dS is not finite: dK and dV of all of them, left where the kernel leaves
+// A block's items by plain arithmetic, where an operand or a dS is out of range (tc::probe_range): dK and dV of all of them, left where the kernel leaves
 // its own, and dQ of those whose own was not added (even and odd items from the two numbers at `from_at` on).  16 warps, four threads to a key row (a quarter of
 // the queries, then of the columns of dK and dV), eight to a query row for dQ.  Pairs that the mask leaves out take no part.
 template <int HD>
@@ -759,10 +758,10 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(bar(i));
     };
-    // A value without parts raises a flag, before what depends on it is announced: 0 and 1 for even and odd items, 2 for K and V.
+    // A value out of range (tc::probe_range) raises a flag, before what depends on it is announced: 0 and 1 for even and odd items, 2 for K and V.
     // (An item's flag is read when its products are complete, and raised for the item after next when all have read it.)
     auto raise = [&](const float2& probe, int i) {
-      if (!(probe.x == 0.f && probe.y == 0.f)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag + 4 * i), "r"(1u) : "memory");
+      if (tc::probe_failed(probe)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag + 4 * i), "r"(1u) : "memory");
     };
     auto convert = [&](uint32_t src, uint32_t dst, int rows, float lift, int flag_i) {
       float2 probe = make_float2(0.f, 0.f);
@@ -858,9 +857,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
       }
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        float2 rest;
-        tc::split3(p[2 * k], p[2 * k + 1], Lift<HD>::DS, part[0][k], part[1][k], part[2][k], rest);
-        probe = __ffma2_rn(rest, make_float2(0.f, 0.f), probe);
+        tc::split3(p[2 * k], p[2 * k + 1], Lift<HD>::DS, part[0][k], part[1][k], part[2][k]);
+        tc::probe_range(p[2 * k], p[2 * k + 1], probe);
       }
 #pragma unroll
       for (int i = 0; i < 3; ++i) {

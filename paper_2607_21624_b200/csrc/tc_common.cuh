@@ -296,27 +296,29 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Two fp32 values as three packed pairs of bf16: the rounding, the rounding of what that leaves, and the rest (24 bits; `rest` is
-// not finite if and only if a value has no such parts).
+// Two fp32 values as three packed pairs of bf16: the rounding, the rounding of what that leaves, and the rest (24 bits).
 // `lift`: a share of the value that the rest is raised by.  The tensor core's additions round toward zero: a sum of products
 // (16 columns to an instruction, the small parts' first) comes out smaller by 6.0e-8 of itself, on average and for every size and
 // sign of the operands that was tried, after four full-size additions, 4.5e-8 after two, some 3.7e-8 after one.  Such losses
 // would add up from product to product, where rounding to nearest averages out.  So operands are raised by that much, between them
 // (products: error against 64 bits 7.7e-8 -> 4.9e-8 of the result's norm at 64 columns, 1.0e-7 -> 8e-8 at 768).
 constexpr float LIFT_4 = 6.03e-8f, LIFT_2 = 4.47e-8f, LIFT_1 = 3.7e-8f;
-__device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& hi, uint32_t& mid, uint32_t& lo, float2& rest) {
+__device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
   const float2 minus = make_float2(-1.f, -1.f), whole = make_float2(x, y);
   hi = pack_bf16(x, y);
   float2 v = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), minus, whole);
   mid = pack_bf16(v.x, v.y);
   v = __ffma2_rn(make_float2(__uint_as_float(mid << 16), __uint_as_float(mid & 0xffff0000u)), minus, v);
-  rest = __ffma2_rn(whole, make_float2(lift, lift), v);
-  lo = pack_bf16(rest.x, rest.y);
+  v = __ffma2_rn(whole, make_float2(lift, lift), v);
+  lo = pack_bf16(v.x, v.y);
 }
-__device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-  float2 rest;
-  split3(x, y, lift, hi, mid, lo, rest);
+// Values that products of parts may meet: below 2^60, so that no sum of 128 products leaves the range of fp32.  A probe that has
+// seen others is not finite.  (Its sum may also leave the range with some values from 2^54 on, which costs time and nothing else.)
+constexpr float PROBE_SCALE = 2.9514790517935283e20f;      // 2^68
+__device__ __forceinline__ void probe_range(float x, float y, float2& probe) {
+  probe = __ffma2_rn(make_float2(x, y), make_float2(PROBE_SCALE, PROBE_SCALE), probe);
 }
+__device__ __forceinline__ bool probe_failed(const float2& probe) { return !(fabsf(probe.x) + fabsf(probe.y) < INFINITY); }
 __device__ __forceinline__ void sts4(uint32_t a, const uint32_t* v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
