@@ -7,10 +7,10 @@
 // Accuracy.  Every bf16 x bf16 product is exact in fp32; what is lost is the tensor core's own accumulation.  The accumulator
 // is therefore used for no more than 64 columns of a reduction, the small products first, and added to a sum that a thread
 // keeps in registers (rounded to nearest): no value passes more than four accumulations at its full size before such an addition.
-// An infinity has no parts (inf - inf is NaN), so a block whose part of a tile is not finite throughout forms it again by plain
-// multiply-adds: infinities and NaN go where the FP32 pipe puts them.  (ViT-shaped step of 4 x 197 tokens with an infinity in X,
-// which reaches every weight gradient: 840 us, all on the FP32 pipe 450, a thread to a result 20000; feed-forward step of 800 x 768 x
-// 3072 930, 630, 12000.)
+// An infinity has no parts (inf - inf is NaN), so a block whose part of a tile is not finite throughout (and so where an operand
+// is 2^111 or more, or a result 2^96) forms it again by plain multiply-adds: infinities and NaN go where the FP32 pipe puts them.
+// (ViT-shaped step of 4 x 197 tokens with an infinity in X, which reaches every weight gradient: 850 us, all on the FP32 pipe 450, a
+// thread to a result 20000; feed-forward step of 800 x 768 x 3072 950, 630, 12000.)
 //
 // One block per 128 x BN tile, or per slice of its reduction (then a cluster shares the tile; partial tiles meet in distributed
 // shared memory in a fixed order: no atomics, the same bits every time).  18 warps: one loads fp32 operand tiles by TMA, four
@@ -315,6 +315,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
 #pragma unroll
     for (int i = 0; i < N / 2; ++i) probe = __ffma2_rn(sum[i], make_float2(0.f, 0.f), probe);
     if (!(probe.x == 0.f && probe.y == 0.f)) asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) sum[i] = __fmul2_rn(sum[i], make_float2(tc::PARTS_BACK, tc::PARTS_BACK));
     // the partial tile, over the stages: the last accumulator is complete, so every operand has been read
     const uint32_t row = base + (uint32_t)((q * 32 + lane) * SM::LD + half * N) * 4;
 #pragma unroll

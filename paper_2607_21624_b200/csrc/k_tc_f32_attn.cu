@@ -323,6 +323,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
     // ---- softmax: thread = (query row, half) ----
     const int q = warp % 4, half = (warp - 2) / 4, r = q * 32 + lane, gi = i0 + r;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    const float scale = P.scale * tc::PARTS_BACK;             // of scores as they come out of the products
     const uint32_t mine = base + SM::MAX_OFF + (half * QT + r) * 4, other = base + SM::MAX_OFF + ((half ^ 1) * QT + r) * 4;
     uint32_t met = 0;
     auto meet = [&]() -> bool {                              // the two warps of these rows
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
       float mx = -INFINITY;
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
-        s[k] *= P.scale;
+        s[k] *= scale;
         if (need_mask && (j0 + k >= P.seq_k || (P.causal && j0 + k > gi))) s[k] = -INFINITY;
         mx = fmaxf(mx, s[k]);
       }
@@ -437,7 +438,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_tc_f32_kernel(const _
     l = half ? lo + l : l + lo;
     if (ok && gi < P.t_pad) {
       const bool live = gi < P.seq;
-      const float inv = live ? 1.f / l : 0.f;
+      const float inv = live ? 1.f / l * tc::PARTS_BACK : 0.f;
 #pragma unroll
       for (int c = 0; c < HC / 4; ++c) {
         const float4 v = live ? make_float4(o[2 * c].x * inv, o[2 * c].y * inv, o[2 * c + 1].x * inv, o[2 * c + 1].y * inv) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -769,6 +770,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
       raise(probe, flag_i);
       tc::fence_proxy_async();
     };
+    const float scale = P.scale * tc::PARTS_BACK;              // of S and dQ as they come out of the products
     pdl_wait();
     bool ok = true;
     auto next_do = [&](int n) {
@@ -834,7 +836,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
         const float4 l4 = tc::lds4(stat + (c0 + k) * 4);
         const float ls[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) p[k + u] = out >> (k + u) & 1 ? 0.f : expf((__uint_as_float(x[k + u]) + __uint_as_float(y[k + u])) * P.scale - ls[u]);
+        for (int u = 0; u < 4; ++u) p[k + u] = out >> (k + u) & 1 ? 0.f : expf((__uint_as_float(x[k + u]) + __uint_as_float(y[k + u])) * scale - ls[u]);
       }
 #pragma unroll
       for (int k = 0; k < 8; ++k) tc::split3(p[2 * k], p[2 * k + 1], Lift<HD>::P, part[0][k], part[1][k], part[2][k]);
@@ -853,7 +855,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
         const float4 d4 = tc::lds4(stat + 256 + (c0 + k) * 4);
         const float ds[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) p[k + u] = out >> (k + u) & 1 ? 0.f : p[k + u] * (__uint_as_float(x[k + u]) + __uint_as_float(y[k + u]) - ds[u]);
+        for (int u = 0; u < 4; ++u) p[k + u] = out >> (k + u) & 1 ? 0.f : p[k + u] * fmaf(__uint_as_float(x[k + u]) + __uint_as_float(y[k + u]), tc::PARTS_BACK, -ds[u]);
       }
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
@@ -899,12 +901,17 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
 #pragma unroll
         for (int c = 0; c < HC / 4; ++c)
           atomicAdd(reinterpret_cast<float4*>(P.dq + rt_off<32>(P.n_pad, (long long)b * P.t_pad + gi, h * HD + quarter * HC + 4 * c)),
-                    make_float4(dq[2 * c].x * P.scale, dq[2 * c].y * P.scale, dq[2 * c + 1].x * P.scale, dq[2 * c + 1].y * P.scale));
+                    make_float4(dq[2 * c].x * scale, dq[2 * c].y * scale, dq[2 * c + 1].x * scale, dq[2 * c + 1].y * scale));
       }
     }
     // dK and dV of this block's items to shared memory, over K's and V's parts, which no product reads any more
     const uint32_t out = base + (uint32_t)(r * (HD + 4) + quarter * HC) * 4;
     constexpr uint32_t SUM_V = BKT * (HD + 4) * 4;
+#pragma unroll
+    for (int c = 0; c < HC / 2; ++c) {
+      dk[c] = __fmul2_rn(dk[c], make_float2(tc::PARTS_BACK, tc::PARTS_BACK));
+      dv[c] = __fmul2_rn(dv[c], make_float2(tc::PARTS_BACK, tc::PARTS_BACK));
+    }
 #pragma unroll
     for (int c = 0; c < HC / 2; c += 2) {
       tc::sts4(out + c * 8, reinterpret_cast<const uint32_t*>(&dk[c]));

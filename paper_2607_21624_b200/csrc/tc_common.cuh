@@ -296,7 +296,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Two fp32 values as three packed pairs of bf16: the rounding, the rounding of what that leaves, and the rest (24 bits).
+// Two fp32 values times 2^16 as three packed pairs of bf16: the rounding, the rounding of what that leaves, and the rest (24 bits).
+// The power of two is for small values: the smallest step of fp32 is 2^-149, that of bf16 2^-133, and a value below 2^-109
+// (1.5e-33) would lose its last bits.  Products come out times 2^32, which is taken back from their sums, exactly.  Values from 2^111
+// on have no parts.
+constexpr float PARTS_SCALE = 65536.f, PARTS_BACK = 1.f / 4294967296.f;
 // `lift`: a share of the value that the rest is raised by.  The tensor core's additions round toward zero: a sum of products
 // (16 columns to an instruction, the small parts' first) comes out smaller by 6.0e-8 of itself, on average and for every size and
 // sign of the operands that was tried, after four full-size additions, 4.5e-8 after two, some 3.7e-8 after one.  Such losses
@@ -304,17 +308,17 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // (products: error against 64 bits 7.7e-8 -> 4.9e-8 of the result's norm at 64 columns, 1.0e-7 -> 8e-8 at 768).
 constexpr float LIFT_4 = 6.03e-8f, LIFT_2 = 4.47e-8f, LIFT_1 = 3.7e-8f;
 __device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-  const float2 minus = make_float2(-1.f, -1.f), whole = make_float2(x, y);
-  hi = pack_bf16(x, y);
+  const float2 minus = make_float2(-1.f, -1.f), whole = __fmul2_rn(make_float2(x, y), make_float2(PARTS_SCALE, PARTS_SCALE));
+  hi = pack_bf16(whole.x, whole.y);
   float2 v = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), minus, whole);
   mid = pack_bf16(v.x, v.y);
   v = __ffma2_rn(make_float2(__uint_as_float(mid << 16), __uint_as_float(mid & 0xffff0000u)), minus, v);
   v = __ffma2_rn(whole, make_float2(lift, lift), v);
   lo = pack_bf16(v.x, v.y);
 }
-// Values that products of parts may meet: below 2^60, so that no sum of 128 products leaves the range of fp32.  A probe that has
-// seen others is not finite.  (Its sum may also leave the range with some values from 2^54 on, which costs time and nothing else.)
-constexpr float PROBE_SCALE = 2.9514790517935283e20f;      // 2^68
+// Values that products of parts may meet: below 2^44, so that no sum of 128 products leaves the range of fp32.  A probe that has
+// seen others is not finite.  (Its sum may also leave the range with some values from 2^38 on, which costs time and nothing else.)
+constexpr float PROBE_SCALE = 1.9342813113834067e25f;      // 2^84
 __device__ __forceinline__ void probe_range(float x, float y, float2& probe) {
   probe = __ffma2_rn(make_float2(x, y), make_float2(PROBE_SCALE, PROBE_SCALE), probe);
 }

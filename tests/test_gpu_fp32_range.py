@@ -38,3 +38,30 @@ def test_scores_below_the_range(head_dim):
     for n in names:
         assert np.isfinite(want[n]).all() and np.isfinite(got[n]).all(), n
         assert off(got[n], want[n]) <= 1e-5, n
+
+
+def test_products_of_small_and_large_operands():
+    # values of 1e-36 have all their 24 bits in fp32, and their products with 1e30 are ordinary numbers
+    cfg = XattnConfig("fr2", 1, 70, 150, 128, 192, 4, 2, 32, "fp32", "layernorm", False, False, 1e-5, 412, 0.05)
+    inp = make_xattn_inputs(cfg)
+    inp["M"] = np.float32(inp["M"] * 1e-36).astype(np.float64)
+    inp["Wk"] = np.float32(inp["Wk"] * 1e30).astype(np.float64)
+    got, ffma = (outputs(cfg, inp, path, ("K", "V", "A")) for path in (0, 1))
+    exact = {"K": inp["M"] @ inp["Wk"], "V": inp["M"] @ inp["Wv"]}
+    for n, want in exact.items():
+        assert off(got[n], want) <= max(off(ffma[n], want), 1e-7), (n, off(got[n], want), off(ffma[n], want))
+    assert off(got["A"], ffma["A"]) <= 1e-6, off(got["A"], ffma["A"])
+
+
+@pytest.mark.parametrize("head_dim", [32, 64])
+def test_gradients_of_a_small_output_gradient(head_dim):
+    # they are linear in it; powers of two are exact, but for what fp32 itself loses of dS below 1e-38
+    cfg = LayerConfig("fr3", 2, 150, 128, 128 // head_dim, 64 // head_dim, head_dim, "fp32", "layernorm", True, False, False, 1e-5, 413, 0.1)
+    inp, names, small = make_inputs(cfg, affine_noise=True), ("dA", "dV", "dQ", "dK", "dWo", "dWv", "dX"), 2.0 ** -114
+    away = {}
+    for path in (0, 1):
+        plain = outputs(cfg, inp, path, names)
+        got = outputs(cfg, dict(inp, dY=inp["dY"] * small), path, names)
+        away[path] = {n: off(got[n] / small, plain[n]) for n in names}
+    for n in names:
+        assert away[0][n] <= 2 * away[1][n] + 2e-7, (n, away[0][n], away[1][n])
