@@ -54,6 +54,7 @@ constexpr uint32_t TMEM_COLS = 512;
 template <int BN> __device__ constexpr uint32_t a_col(int set, int part) { return 2 * BN + 96 * set + 32 * part; }
 
 using tc::split3;
+constexpr float LIFT = 2.7e-8f;       // of either operand: between them 0.9 of tc::LIFT_4, of one alone less than what brings up the next value
 using tc::sts4;
 
 // This block's part of its tile (k-blocks kb_begin .. kb_end) once more by multiply-adds, all threads of the block: where a result
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
         }
         uint32_t p[3][8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], tc::LIFT_4, p[0][k], p[1][k], p[2][k]);
+        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], LIFT, p[0][k], p[1][k], p[2][k]);
 #pragma unroll
         for (int i = 0; i < 3; ++i) tc::tmem_st8(lane_addr + a_col<BN>(b, i) + 8 * h, p[i]);
       }
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_f32_kernel(const __grid_co
         }
         uint32_t p[3][8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], 0.f, p[0][k], p[1][k], p[2][k]);
+        for (int k = 0; k < 8; ++k) split3(x[2 * k], x[2 * k + 1], LIFT, p[0][k], p[1][k], p[2][k]);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll

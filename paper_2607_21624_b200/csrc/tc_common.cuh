@@ -301,11 +301,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // (1.5e-33) would lose its last bits.  Products come out times 2^32, which is taken back from their sums, exactly.  Values from 2^111
 // on have no parts.
 constexpr float PARTS_SCALE = 65536.f, PARTS_BACK = 1.f / 4294967296.f;
-// `lift`: a share of the value that the rest is raised by.  The tensor core's additions round toward zero: a sum of products
-// (16 columns to an instruction, the small parts' first) comes out smaller by 6.0e-8 of itself, on average and for every size and
-// sign of the operands that was tried, after four full-size additions, 4.5e-8 after two, some 3.7e-8 after one.  Such losses
-// would add up from product to product, where rounding to nearest averages out.  So operands are raised by that much, between them
-// (products: error against 64 bits 7.7e-8 -> 4.9e-8 of the result's norm at 64 columns, 1.0e-7 -> 8e-8 at 768).
+// `lift`: a share of the value that the rest is raised by, unless the value has no more than 16 bits.  The tensor core's additions
+// round toward zero: a sum of products (16 columns to an instruction, the small parts' first) comes out smaller by 6.0e-8 of itself,
+// on average and for operands of every size and sign with 24 bits, after four full-size additions, 4.5e-8 after two, some 3.7e-8
+// after one.  Such losses would add up from product to product, where rounding to nearest averages out.  So operands are raised by
+// that much, between them (products: error against 64 bits 7.7e-8 -> 4.9e-8 of the result's norm at 64 columns, 1.0e-7 -> 8e-8 at
+// 768).  Where nothing is truncated a raised sum would be wrong, so values of up to 16 bits (zeros, ones, integers) stay as they are:
+// their products and sums are exact as far as fp32 holds them, and an operand raised by no more than 2.7e-8 that meets a single
+// one comes back as it was (raised by 6e-8, and whatever its bits, a fifth of the values came back one unit of the last
+// place larger).
 constexpr float LIFT_4 = 6.03e-8f, LIFT_2 = 4.47e-8f, LIFT_1 = 3.7e-8f;
 __device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
   const float2 minus = make_float2(-1.f, -1.f), whole = __fmul2_rn(make_float2(x, y), make_float2(PARTS_SCALE, PARTS_SCALE));
@@ -313,8 +317,13 @@ __device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& h
   float2 v = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), minus, whole);
   mid = pack_bf16(v.x, v.y);
   v = __ffma2_rn(make_float2(__uint_as_float(mid << 16), __uint_as_float(mid & 0xffff0000u)), minus, v);
-  v = __ffma2_rn(whole, make_float2(lift, lift), v);
-  lo = pack_bf16(v.x, v.y);
+  lo = pack_bf16(v.x, v.y);                    // exact
+  if (lift != 0.f) {
+    const __nv_bfloat162 rest = *reinterpret_cast<const __nv_bfloat162*>(&lo), up = __floats2bfloat162_rn(lift, lift);
+    const uint32_t of = hi & __hne2_mask(rest, __floats2bfloat162_rn(0.f, 0.f));
+    const __nv_bfloat162 raised = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&of), up, rest);
+    lo = *reinterpret_cast<const uint32_t*>(&raised);
+  }
 }
 // Values that products of parts may meet: below 2^44, so that no sum of 128 products leaves the range of fp32.  A probe that has
 // seen others is not finite.  (Its sum may also leave the range with some values from 2^38 on, which costs time and nothing else.)

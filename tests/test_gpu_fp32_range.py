@@ -65,3 +65,29 @@ def test_gradients_of_a_small_output_gradient(head_dim):
         away[path] = {n: off(got[n] / small, plain[n]) for n in names}
     for n in names:
         assert away[0][n] <= 2 * away[1][n] + 2e-7, (n, away[0][n], away[1][n])
+
+
+def test_exact_results_stay_exact():
+    # the operand itself where the other one is an identity or has one entry a row, sums of integers of either sign, and the first
+    # token under a causal mask, whose output is its own V
+    rng = np.random.default_rng(5)
+    cfg = XattnConfig("fr4", 1, 70, 192, 128, 192, 3, 3, 64, "fp32", "layernorm", False, False, 1e-5, 414, 0.05)
+    inp = make_xattn_inputs(cfg)
+    inp["Wk"] = np.eye(192)
+    inp["Wv"] = rng.integers(-900, 900, (192, 192)).astype(np.float64)
+    got = outputs(cfg, inp, 0, ("K",))
+    assert np.array_equal(got["K"], inp["M"])
+    inp = make_xattn_inputs(cfg)
+    inp["M"] = rng.integers(-3, 90, (1, 192, 192)).astype(np.float64)
+    inp["Wk"] = rng.integers(-900, 900, (192, 192)).astype(np.float64)
+    got = outputs(cfg, inp, 0, ("K",))
+    assert np.abs(inp["M"] @ inp["Wk"]).max() < 2 ** 24 and np.array_equal(got["K"], inp["M"] @ inp["Wk"])
+    inp["M"] = np.eye(192)[None, ::-1]
+    inp["Wv"] = np.float32(rng.standard_normal((192, 192)) * 10.0 ** rng.integers(-20, 20, (192, 192))).astype(np.float64)
+    got = outputs(cfg, inp, 0, ("V",))
+    assert np.array_equal(got["V"], inp["M"] @ inp["Wv"])
+    for head_dim in (32, 64):
+        cfg = LayerConfig("fr5", 2, 150, 128, 128 // head_dim, 64 // head_dim, head_dim, "fp32", "layernorm", True, True, False, 1e-5, 415, 0.1)
+        got = outputs(cfg, make_inputs(cfg, affine_noise=True), 0, ("A", "V"))
+        V = got["V"].reshape(2, 150, cfg.n_kv_heads, 1, head_dim).repeat(cfg.group, 3).reshape(2, 150, 128)
+        assert np.array_equal(got["A"][:, 0], V[:, 0])
