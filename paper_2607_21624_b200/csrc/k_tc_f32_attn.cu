@@ -988,13 +988,18 @@ cudaError_t bwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
 // pipe and fill an SM, so short sequences stay there.  Forward / backward against the FP32 pipe (us), causal, heads of 64: 8 heads
 // of 24 tokens x 16 sequences 7.7 / 13 and 6.3 / 9; of 64 tokens 8 / 14 and 10 / 22, x 64 sequences 29 / 52 and 22 / 45; 12 heads of
 // 197 tokens x 4 16 / 32 and 36 / 70; 4 heads of 2048 82 / 104 and 199 / 300; 8 x 100 queries over 8 rows x 16 8.6 / 19 and 8.6 / 25.
+// With half a tile of keys or less, and query blocks for several rounds, what counts is what a block takes by itself.  Steps over 16
+// memory rows, here / on the FP32 pipe: 96 x 8 heads of 80 queries 342 / 288, 32 x 16 heads of 200 queries 364 / 347, of 500 742 /
+// 738; 32 x 8 heads of 80 equal, of 200 with one KV head to four 251 / 266, 8 x 16 heads of 1500 572 / 616; over 48 rows from
+// equal to half of it.
 // Heads of 32: 64 tokens 6.5 / 10.4 and 7.1 / 9.9; 100 tokens of 8 heads x 32 19 / 33 and 22 / 45; 1500 queries over 16 rows x 4
 // 20 / 41 and 13 / 34, 16 over 1500 58 / 31 and 106 / 23.
 bool attn_tc_f32_supported(const fbl_plan* p) {
   if (p->d.dtype != FBL_DTYPE_FP32 || p->ffma_only || p->d.head_dim > 64) return false;
   const int longer = p->d.seq > p->seq_kv ? p->d.seq : p->seq_kv;
   if (p->d.head_dim == 32) return longer > 64 && p->seq_kv > 64;
-  return longer > 64 || (longer > 32 && (long long)p->d.batch * p->d.n_q_heads <= 2 * p->sm_count);
+  const bool rounds = (long long)p->d.batch * p->d.n_q_heads > 2 * p->sm_count;
+  return longer > 64 ? p->seq_kv > 32 || !rounds : longer > 32 && !rounds;
 }
 
 cudaError_t launch_attn_fwd_tc_f32(const fbl_plan* p, const void* Q, const void* K, const void* V, void* A, float* lse, int32_t* status,

@@ -111,6 +111,33 @@ def test_fp32_attention_on_tensor_cores(cfg):
     check(cfg)
 
 
+@pytest.mark.parametrize("cfg", [
+    XattnConfig("fm1", 96, 80, 16, 128, 128, 8, 8, 64, "fp32", "layernorm", False, True, 1e-5, 246, 0.1),
+    XattnConfig("fm2", 75, 70, 32, 128, 64, 4, 1, 64, "fp32", "rmsnorm", True, False, 1e-5, 247, 0.1),
+    XattnConfig("fm3", 74, 70, 32, 128, 64, 4, 1, 64, "fp32", "rmsnorm", True, False, 1e-5, 248, 0.1),
+], ids=lambda c: c.name)
+def test_fp32_attention_of_few_memory_rows(cfg):
+    # either side of the line between the two kernel families; neither takes longer than multiply-adds alone
+    import torch
+    from paper_2607_21624_b200 import XattnRunner
+    check(cfg)
+    us = {}
+    for path in (0, 1):
+        run = XattnRunner(cfg)
+        run.plan.set_kernel_path(path)
+        run.plan.profile_enable(True)
+        times = []
+        for _ in range(20):
+            total = 0.0
+            for part in (run.forward, run.backward):
+                part()
+                torch.cuda.synchronize()
+                total += sum(ms for name, ms in run.plan.profile_read() if name.startswith("attn"))
+            times.append(total)
+        us[path] = sorted(times)[10] * 1e3
+    assert us[0] <= 1.1 * us[1] + 2, us
+
+
 @pytest.mark.parametrize("head_dim", [32, 64])
 def test_fp32_attention_of_operands_without_parts(head_dim):
     # infinities among V and among dA: the same results as plain multiply-adds, and finite columns stay finite
