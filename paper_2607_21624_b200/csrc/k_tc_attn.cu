@@ -541,7 +541,10 @@ cudaError_t fwd_make_t(AttnLaunch<AttnFwdParams>& L, const fbl_plan* p, int n_qt
 //   short: one (5 x 16 heads of 384: 37.5 / 41.8; 1500 queries over 200 keys: 77.0 / 82.7);
 //   less than an SM's worth of pairs: a tile alone where all tiles fit at once (12 heads of 500: 25.3 / 23.2, of 1500 causal 41.8 /
 //   36.0), else one (2 x 20 heads of 830: 49.5 / 59.2), but for long causal chains (16 heads of 1536: 49.6 / 40.2);
-//   causal pairs: one up to nine tiles, eight aside (4 x 16 heads of 520: 33.1 / 38.0, 1020: 55.2 / 55.2, 1152: 59.5 / 62.4, 2048: 120.8 / 114.6);
+//   causal pairs: an odd count leaves a tile alone in its block, so odd counts change over later.  One up to six tiles (4 x 32 heads of
+//   760: 63.8 / 63.3, 16 x 32 219 / 234), two from eight on where the count is even (4 x 32 of 960: 84.6 / 82.0, 8 x 16 of 1020 93.2 /
+//   91.0, 3 x 40 83.5 / 84.5; 8 x 16 of 1260 124.7 / 120.9, of 1500 153.8 / 148.1), past nine where it is odd (16 x 12 of 890: 117 /
+//   124, 4 x 32 of 890 79.0 / 77.5; of 1150 96.5 / 100, 3 x 40 94.0 / 98.8; 11 and 13 tiles within 2 %);
 //   else rounds: one where the pairs' last round costs more (3 x 32 heads of 1150: 134 / 140, of 1500: 180 / 168); five rounds and more even out.
 bool fwd_one_tile(const fbl_plan* p, int n_qt, int pair) {
   const int n_kt = (p->seq_kv + BKV - 1) / BKV;
@@ -549,7 +552,7 @@ bool fwd_one_tile(const fbl_plan* p, int n_qt, int pair) {
   const long long sm = p->sm_count, heads = (long long)p->d.n_q_heads * p->d.batch, blocks = n_qt * heads, pairs = (n_qt + 1) / 2 * heads;
   if (!pair) return blocks > sm && (!p->d.causal || n_qt <= 6);
   if (n_qt <= 4 || n_kt <= 4) return true;
-  if (p->d.causal) return n_qt <= 9 && n_qt != 8;
+  if (p->d.causal) return n_qt <= (n_qt % 2 ? 9 : 6);
   return pairs <= 5 * sm && 1.08 * ((blocks + 2 * sm - 1) / (2 * sm)) < (pairs + sm - 1) / sm;
 }
 
