@@ -102,10 +102,11 @@ typedef struct fbl_plan fbl_plan; /* opaque: padded sizes, index-map constants, 
  * The plan also fixes, from the shapes alone, into how many slices the token-axis reductions of the weight
  * gradients are cut (1 for all but layers with few weight tiles and many tokens).  Environment variables
  * read here, for tuning and tests only: FBL_KSPLIT_O and FBL_KSPLIT_QKV override those slice counts,
- * FBL_VERBOSE prints the ones chosen to stderr.  Three more, again for tuning and tests only: FBL_GEMM_PAIR (0: never use the CTA-pair GEMM kernel, 1: use it wherever its tile shape is
+ * FBL_VERBOSE prints the ones chosen to stderr.  Five more, again for tuning and tests only: FBL_GEMM_PAIR (0: never use the CTA-pair GEMM kernel, 1: use it wherever its tile shape is
  * legal; unset: large launches only), FBL_GEMM_ESETS (1 or 2 sets of epilogue warps in the single-CTA GEMM kernel;
- * unset: 2 where every block of the launch has one tile) and FBL_FWD_TILES (1 or 2 query tiles per
- * forward-attention block at head_dim 64; unset: by shape). */
+ * unset: 2 where every block of the launch has one tile), FBL_FWD_TILES (1 or 2 query tiles per
+ * forward-attention block at head_dim 64; unset: by shape), FBL_F32_BN (64 or 128 columns of the fp32 products' tiles;
+ * unset: by size) and FBL_F32_SLICES (1, 2, 4 or 8 blocks that share such a tile's reduction; unset: by size). */
 int fbl_plan_create(const fbl_layer_desc* desc, fbl_plan** out);
 void fbl_plan_destroy(fbl_plan* plan);
 
@@ -406,8 +407,9 @@ int fbl_xattn_bwd(const fbl_plan* plan, const void* dY, const void* X, const voi
                   float* dgamma, float* dbeta, void* scratch, void* stream);
 
 /* Kernel family used by later calls on this plan: 0 = default (tcgen05 tensor-core kernels for bf16 and, with operands in three bf16
- * parts, for fp32; FFMA kernels for fp32 attention of short sequences or heads of 128 and for the attention backward of bf16 layers
- * with less than 128 token rows on either side), 1 = FFMA kernels only (fp32 arithmetic on the same layout; lets a caller cross-check
+ * parts, for fp32; FFMA kernels for fp32 attention of short sequences, of few memory rows or of heads of 128, for the attention
+ * backward of bf16 layers with less than 128 token rows on either side, and for fp32 tiles with operands or results that are not finite
+ * or beyond 2^44 in attention, 2^111 (results 2^96) in other products), 1 = FFMA kernels only (fp32 arithmetic on the same layout; lets a caller cross-check
  * the tensor-core path on the device). */
 int fbl_plan_set_kernel_path(fbl_plan* plan, int path);
 

@@ -89,11 +89,7 @@ inline bool point_group(Group& G, const GemmArgs* gs, int32_t* status) {
   return ok;
 }
 
-__device__ __forceinline__ float4 lds4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-  return v;
-}
+using tc::lds4;
 
 // This block's share of the tile's rows: the slices' sums (each block's at `base` of its shared memory, rows LD floats apart)
 // in slice order, bias, residual, padding rows, 16-byte stores.  A thread keeps its four columns and has two rows in flight (one

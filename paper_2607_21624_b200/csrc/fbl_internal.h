@@ -132,9 +132,8 @@ cudaError_t launch_gemm_tc_group(const fbl_plan* p, const GemmArgs* gs, int coun
                                  int launch_id = -1);
 bool gemm_ffma_supported(const fbl_plan* p, const GemmArgs& g);
 cudaError_t launch_gemm_ffma_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st);
-// fp32 on the tensor cores: what gemm_ffma_supported accepts.  bn, slices: 0, or a tile width of 64 or 128 columns and 1, 2, 4 or 8
-// blocks that share a tile's reduction (measurements).
-cudaError_t launch_gemm_tc_f32_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int bn = 0, int slices = 0);
+// fp32 on the tensor cores: what gemm_ffma_supported accepts
+cudaError_t launch_gemm_tc_f32_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st);
 // Every problem of the group can run on the tensor-core kernel and the plan wants it to.
 static inline bool gemm_group_tc(const fbl_plan* p, const GemmArgs* gs, int count) {
   bool tc = p->use_tc != 0;

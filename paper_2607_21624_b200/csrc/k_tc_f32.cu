@@ -390,17 +390,15 @@ Choice choose(const fbl_plan* p, const GemmArgs* gs, const int* order, int count
 
 }  // namespace
 
-cudaError_t launch_gemm_tc_f32_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st, int bn, int slices) {
+cudaError_t launch_gemm_tc_f32_group(const fbl_plan* p, const GemmArgs* gs, int count, int32_t* status, cudaStream_t st) {
   if (count < 1 || count > f32g::MAX_PROBLEMS) return cudaErrorInvalidValue;
   LaunchKey key;
-  key.add(bn, slices);
   gemm_group_key(key, gs, count);
   return LaunchMemo<Launch, 12>::run(p, FBL_MEMO_TC_F32_GEMM, key,
       [&](Launch& L) {
         int order[f32g::MAX_PROBLEMS];
         f32g::longest_first(gs, count, order);
-        Choice c = {bn, slices};
-        if (!bn) c = choose(p, gs, order, count);
+        const Choice c = choose(p, gs, order, count);
         if (!f32g::fill_group(L.G, gs, count, order, BM, c.bn, BK)) return cudaErrorInvalidValue;
         L.grid = 0;
         for (int i = 0; i < count; ++i) L.grid += L.G.p[i].tiles_m * L.G.p[i].tiles_n * c.slices;
