@@ -91,3 +91,23 @@ def test_exact_results_stay_exact():
         got = outputs(cfg, make_inputs(cfg, affine_noise=True), 0, ("A", "V"))
         V = got["V"].reshape(2, 150, cfg.n_kv_heads, 1, head_dim).repeat(cfg.group, 3).reshape(2, 150, 128)
         assert np.array_equal(got["A"][:, 0], V[:, 0])
+
+
+@pytest.mark.parametrize("cfg", [
+    LayerConfig("fr6", 2, 300, 256, 4, 4, 64, "fp32", "layernorm", False, True, False, 1e-5, 421, 0.05),
+    LayerConfig("fr7", 1, 700, 128, 4, 1, 32, "fp32", "rmsnorm", True, False, True, 1e-5, 422, 0.2),
+    LayerConfig("fr8", 3, 190, 192, 6, 2, 64, "fp32", "layernorm", True, True, True, 1e-5, 423, 0.3),
+    XattnConfig("fr9", 2, 130, 400, 128, 192, 4, 2, 32, "fp32", "rmsnorm", False, False, 1e-5, 424, 0.1),
+], ids=lambda c: c.name)
+def test_attention_is_no_further_off_than_multiply_adds(cfg):
+    # against 64 bits, the same inputs through both kernel families; 0.2 to 0.95 of it measured
+    from oracle import layer, xattn
+    cross = isinstance(cfg, XattnConfig)
+    inp = (make_xattn_inputs if cross else make_inputs)(cfg, affine_noise=True)
+    Y, saved, grads = (xattn.xattn_fwd_bwd if cross else layer.layer_fwd_bwd)(cfg, inp)
+    want = dict(grads, Y=Y, A=saved["A"])
+    names = ("A", "Y", "dQ", "dK", "dV", "dX", "dWo", "dWv", "dWq", "dWk")
+    got, ffma = (outputs(cfg, inp, path, names) for path in (0, 1))
+    print({n: round(off(got[n], want[n]) / off(ffma[n], want[n]), 2) for n in names})
+    for n in names:
+        assert off(got[n], want[n]) <= off(ffma[n], want[n]), (n, off(got[n], want[n]), off(ffma[n], want[n]))

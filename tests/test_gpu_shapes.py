@@ -383,6 +383,25 @@ def test_fp32_attention_backward_slices(cfg):
 
 
 @pytest.mark.parametrize("cfg", [
+    # the multiply-add kernels, which the tensor-core ones are compared with: products on partly filled 64 x 64 tiles, one to eight
+    # slices of a reduction, all operand orientations; attention of one to many tiles, groups, items dealt over a cluster
+    LayerConfig("ma1", 1, 5, 32, 1, 1, 32, "fp32", "layernorm", True, True, True, 1e-5, 431, 0.2),
+    LayerConfig("ma2", 3, 67, 160, 5, 1, 32, "fp32", "rmsnorm", True, True, False, 1e-5, 432, 0.1),
+    LayerConfig("ma3", 2, 129, 1056, 3, 3, 64, "fp32", "layernorm", False, False, True, 1e-5, 433, 0.03),
+    LayerConfig("ma4", 1, 224, 64, 2, 2, 64, "fp32", "rmsnorm", True, False, False, 1e-5, 434, 0.1),
+    LayerConfig("ma5", 2, 129, 128, 6, 2, 64, "fp32", "rmsnorm", False, False, True, 1e-5, 435, 0.05),
+    LayerConfig("ma6", 1, 70, 128, 4, 1, 32, "fp32", "layernorm", True, False, False, 1e-5, 436, 0.05, 0.0, 10000.0),
+    MlpConfig("ma7", 2, 70, 96, 416, "fp32", "layernorm", "swiglu", True, True, 1e-5, 437, 0.1),
+    MlpConfig("ma8", 1, 1100, 64, 256, "fp32", "rmsnorm", "gelu", True, False, 1e-5, 438, 0.1),
+    XattnConfig("ma9", 2, 33, 90, 64, 224, 4, 2, 32, "fp32", "layernorm", True, True, 1e-5, 439, 0.1),
+    XattnConfig("ma10", 1, 150, 41, 96, 128, 3, 1, 64, "fp32", "layernorm", True, True, 1e-5, 440, 0.05),
+], ids=lambda c: c.name)
+def test_fp32_multiply_add_kernels(cfg):
+    compare = test_gpu_mlp if isinstance(cfg, MlpConfig) else test_gpu_xattn if isinstance(cfg, XattnConfig) else test_gpu_layer
+    compare.run_and_compare(cfg, affine_noise=True, path=1, guard_bytes=4096)
+
+
+@pytest.mark.parametrize("cfg", [
     # tensor-core attention backward with a key tile's items dealt over 2, 4 and 8 blocks: shares that do not divide, blocks
     # without items (causal ends), one key tile (dQ written at once), ragged key tiles, the rotation behind it
     LayerConfig("bs1", 1, 300, 256, 8, 1, 64, "bf16", "layernorm", True, False, False, 1e-5, 311, 0.02),
