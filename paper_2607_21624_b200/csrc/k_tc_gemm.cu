@@ -492,8 +492,8 @@ __global__ void __maxnreg__(ESETS == 2 ? 168 : EPI == EPI_ACT ? 255 : 224) gemm_
     }
   } else if (warp == 1) {
     // ---- MMA issuer (a whole warp, see elect_one).  Descriptor words are formed once per reduction loop; per instruction only
-    // the start-address field moves.  (The loop is not the limit: with 128 x 256 tiles a k-block's 48 KB of
-    // operands take longer to arrive from L2, at about 64 B/clk per SM, than its four MMAs take to run.) ------
+    // the start-address field moves.  (With 128 x 256 tiles a k-block's 48 KB of operands take longer to arrive from
+    // L2, at about 64 B/clk per SM, than its four MMAs take to run.) ------
     const bool leader = tc::elect_one();
     int s = 0, ti = 0;
     uint32_t ph = 0;

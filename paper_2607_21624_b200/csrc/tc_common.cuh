@@ -326,7 +326,9 @@ __device__ __forceinline__ void split3(float x, float y, float lift, uint32_t& h
   }
 }
 // Values that products of parts may meet: below 2^44, so that no sum of 128 products leaves the range of fp32.  A probe that has
-// seen others is not finite.  (Its sum may also leave the range with some values from 2^38 on, which costs time and nothing else.)
+// seen others is not finite.  (Beside values of the other sign one of up to 2^45 may pass; the first of a thread's eight cannot, and the
+// 64 products of a sum, an eighth of them below 2^88, stay below 2^127.9 even so.  The probe may also leave the range with some values
+// from 2^38 on, which costs time and nothing else.)
 constexpr float PROBE_SCALE = 1.9342813113834067e25f;      // 2^84
 __device__ __forceinline__ void probe_range(float x, float y, float2& probe) {
   probe = __ffma2_rn(make_float2(x, y), make_float2(PROBE_SCALE, PROBE_SCALE), probe);
