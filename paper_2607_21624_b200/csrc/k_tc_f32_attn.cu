@@ -770,7 +770,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
       raise(probe, flag_i);
       tc::fence_proxy_async();
     };
-    const float scale = P.scale * tc::PARTS_BACK;              // of S and dQ as they come out of the products
+    // of S as it comes out of the products (where their product is below 1.2e-38 and loses bits, scores are below 1 and off by 2^-24)
+    const float scale = P.scale * tc::PARTS_BACK;
     pdl_wait();
     bool ok = true;
     auto next_do = [&](int n) {
@@ -899,9 +900,12 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) attn_bwd_tc_f32_kernel(const _
         plain_from[n & 1] = min(plain_from[n & 1], n);
       } else if (lane < 16 && gi < P.seq) {
 #pragma unroll
+        for (int c = 0; c < HC / 2; ++c)                       // the parts' power of two first: a small softmax scale times it is zero
+          dq[c] = __fmul2_rn(__fmul2_rn(dq[c], make_float2(tc::PARTS_BACK, tc::PARTS_BACK)), make_float2(P.scale, P.scale));
+#pragma unroll
         for (int c = 0; c < HC / 4; ++c)
           atomicAdd(reinterpret_cast<float4*>(P.dq + rt_off<32>(P.n_pad, (long long)b * P.t_pad + gi, h * HD + quarter * HC + 4 * c)),
-                    make_float4(dq[2 * c].x * scale, dq[2 * c].y * scale, dq[2 * c + 1].x * scale, dq[2 * c + 1].y * scale));
+                    make_float4(dq[2 * c].x, dq[2 * c].y, dq[2 * c + 1].x, dq[2 * c + 1].y));
       }
     }
     // dK and dV of this block's items to shared memory, over K's and V's parts, which no product reads any more

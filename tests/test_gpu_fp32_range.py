@@ -67,6 +67,20 @@ def test_gradients_of_a_small_output_gradient(head_dim):
         assert away[0][n] <= 2 * away[1][n] + 2e-7, (n, away[0][n], away[1][n])
 
 
+@pytest.mark.parametrize("head_dim", [32, 64])
+def test_gradients_under_a_small_softmax_scale(head_dim):
+    # scores are all but zero at scales this small, and dQ and dK linear in them: two of the same 24 bits, powers of two apart
+    names, away, bits = ("A", "dV", "dQ", "dK"), {}, float(np.float32(1.1))
+    for path in (0, 1):
+        runs = []
+        for scale in (bits * 2.0 ** -60, bits * 2.0 ** -105):
+            cfg = LayerConfig("fr10", 2, 150, 128, 128 // head_dim, 64 // head_dim, head_dim, "fp32", "layernorm", True, True, False, 1e-5, 416, 0.1, scale)
+            runs.append(outputs(cfg, make_inputs(cfg, affine_noise=True), path, names))
+        away[path] = {n: off(runs[1][n] * (2.0 ** 45 if n in ("dQ", "dK") else 1.0), runs[0][n]) for n in names}
+    for n in names:
+        assert away[0][n] <= 2 * away[1][n] + 2e-7, (n, away[0][n], away[1][n])
+
+
 def test_exact_results_stay_exact():
     # the operand itself where the other one is an identity or has one entry a row, sums of integers of either sign, and the first
     # token under a causal mask, whose output is its own V
