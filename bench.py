@@ -91,16 +91,16 @@ def min_bytes(cfg):
 # a weight share that does not grow, so they get no scaled entry.
 _MB = 1e6
 _NCU_MB = {
-    "cfg1-tiny-fp32": {"norm_fwd": 0.05, "proj_qkv": 0.10, "attn_fwd": 0.10, "proj_o": 0.06, "dWo+dA": 0.08, "attn_bwd": 0.15,
-                       "dWqkv+dXn": 0.14, "norm_bwd": 0.06 + 0.02},
-    "cfg2-gpt2-small": {"norm_fwd": 3.18, "proj_qkv": 6.76, "attn_fwd": 9.47, "proj_o": 4.39, "dWo+dA": 7.53,
-                        "attn_bwd": 19.12 + 6.30, "dWqkv+dXn": 16.18, "db": 12.60, "db+norm_bwd": 6.35 + 1.69},
-    "cfg3-vit-base": {"norm_fwd": 9.86, "proj_qkv": 13.44, "attn_fwd": 29.53, "proj_o": 11.07, "dWo+dA": 0.01 + 23.26,
-                      "attn_bwd": 40.02, "dWqkv+dXn": 50.33, "norm_bwd": 19.76 + 11.09},
-    "cfg4-llama1b-gqa": {"norm_fwd": 16.82, "proj_qkv": 29.43, "attn_fwd": 25.22, "proj_o": 25.23, "dWo+dA": 1.13 + 44.50,
-                         "attn_bwd": 77.78 + 33.56, "dWqkv+dXn": 96.17, "norm_bwd": 33.65 + 27.28},
-    "cfg5-llama7b-long-scaled": {"norm_fwd": 16.83, "proj_qkv": 147.03, "attn_fwd": 50.43, "proj_o": 50.73, "dWo+dA": 0.01 + 109.72,
-                                 "attn_bwd": 117.55 + 33.56, "dWqkv+dXn": 383.19, "norm_bwd": 33.65 + 4.21},
+    "cfg1-tiny-fp32": {"norm_fwd": 0.05, "proj_qkv": 0.12, "attn_fwd": 0.10, "proj_o": 0.09, "dWo+dA": 0.10, "attn_bwd": 0.15,
+                       "dWqkv+dXn": 0.17, "norm_bwd": 0.06 + 0.02},
+    "cfg2-gpt2-small": {"norm_fwd": 3.18, "proj_qkv": 6.76, "attn_fwd": 9.47, "proj_o": 4.39, "dWo+dA": 7.54,
+                        "attn_bwd": 19.12 + 6.30, "dWqkv+dXn": 16.19, "db": 12.60, "db+norm_bwd": 6.35 + 1.69},
+    "cfg3-vit-base": {"norm_fwd": 9.86, "proj_qkv": 13.43, "attn_fwd": 29.53, "proj_o": 11.07, "dWo+dA": 0.01 + 23.26,
+                      "attn_bwd": 40.01, "dWqkv+dXn": 50.17, "norm_bwd": 19.76 + 11.09},
+    "cfg4-llama1b-gqa": {"norm_fwd": 16.82, "proj_qkv": 29.44, "attn_fwd": 25.21, "proj_o": 25.23, "dWo+dA": 1.09 + 44.23,
+                         "attn_bwd": 77.88 + 33.56, "dWqkv+dXn": 95.87, "norm_bwd": 33.64 + 27.28},
+    "cfg5-llama7b-long-scaled": {"norm_fwd": 16.83, "proj_qkv": 146.92, "attn_fwd": 50.46, "proj_o": 50.58, "dWo+dA": 0.01 + 110.50,
+                                 "attn_bwd": 118.39 + 33.56, "dWqkv+dXn": 383.48, "norm_bwd": 33.63 + 4.21},
 }
 _NCU_MB["cfg5-llama7b-long"] = {k: 4.0 * v for k, v in _NCU_MB["cfg5-llama7b-long-scaled"].items()
                                 if k in ("norm_fwd", "attn_fwd", "attn_bwd", "norm_bwd")}     # the token-proportional kernels
