@@ -18,7 +18,8 @@
 // 128-byte-swizzled layout (K-major or MN-major as the operand lies: nothing is transposed on the way), one issues the products,
 // eight add the finished accumulators up.  A lies in tensor memory because shared memory is the bound: per 64 columns a
 // 128 x 128 tile moves 64 KB in, 64 KB out to the conversions, 48 KB of B's parts in and 96 KB of them out to the tensor core,
-// 272 KB at 128 B/clk, where A's parts in shared memory would make it 416 KB (the products take 1536 clk).
+// 272 KB at 128 B/clk, where A's parts in shared memory would make it 416 KB (the products take 1536 clk).  Counted: the tensor pipe
+// is active for 31 to 46 % of active cycles (800 x 768 outputs, 768 to 800 columns to reduce), conversions and waits for them the rest.
 // Measured against the FP32 pipe (k_ffma_gemm.cu), us: 800 x 768 outputs, 768 columns to reduce: three problems 74 -> 22.8, one
 // 31 -> 15.3, dWo with dA 60 -> 23.8, dWq, dWk, dWv with dXn 159 -> 47.7; 2048 x 2048 x 2048 358 -> 93 (185 TFLOP/s); 64 x 64 x 64
 // 6.5 -> 5.5.  Error against 64 bits relative to the result's norm: 0.4e-7 to 1.8e-7 at 32 to 4096 columns, multiply-adds one after

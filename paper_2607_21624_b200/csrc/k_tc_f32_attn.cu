@@ -40,7 +40,8 @@ struct alignas(64) F32FwdParams {
 // products, eight have two threads to a query row (half of the keys' scores and of the output's columns each; they meet for the
 // row maximum) and four turn K and V into bf16 parts in shared memory (K-major and MN-major as they lie).  Q's and P's parts are
 // operands in tensor memory.  The scores of the next tile and the output of this one are products under way while the softmax
-// works; the bound is the products: 24 + 24 instructions a tile at head_dim 64, some 2300 clk.
+// works; the products alone, 24 + 24 instructions a tile at head_dim 64, are some 2300 clk (counted on short chains, 48 heads of 197
+// tokens: tensor pipe active for 23 % of active cycles, the start and the conversions the rest).
 // ------------------------------------------------------------------------------------------
 constexpr int QT = 128, KT = 64;
 constexpr int SOFT_WARPS = 8, CONV_WARPS = 4, FWD_THREADS = 32 * (2 + SOFT_WARPS + CONV_WARPS);
@@ -489,7 +490,8 @@ cudaError_t fwd_launch(const fbl_plan* p, const void* Q, const void* K, const vo
 // rows lie in the first 16 of its lanes), 32 keys to an accumulator, whose sum goes to memory by 16-byte reductions.  18 warps: one
 // loads, one issues, 16 work (four threads to a key row): softmax, then the next queries' parts while this tile's products run.
 // Where that makes fewer blocks than SMs, a cluster of 2 to 8 blocks takes a key tile's items in turn and adds dK and dV through
-// distributed shared memory in a fixed order.  The bound is the products: 144 instructions an item, some 7000 clk.
+// distributed shared memory in a fixed order.  The products alone, 144 instructions an item, are some 7000 clk (48 heads of 197
+// tokens: tensor pipe active for 36 % of active cycles).
 // ------------------------------------------------------------------------------------------
 constexpr int BKT = 128, BQT = 64, WORK_WARPS = 16, BWD_THREADS = 32 * (2 + WORK_WARPS);
 

@@ -1198,7 +1198,8 @@ namespace {
 // Output tiles a launch may use: 128 x 64 (slim), 128 x 128 or 128 x 256 on one CTA, 256 x 256 on a CTA pair.
 enum TileKind { TILE_NARROW = 0, TILE_WIDE, TILE_PAIR, TILE_SLIM };
 struct TileCost { int m, n; double kb, unit, epilogue, fixed; };      // extents; clocks per k-block, per unit, of an epilogue, per launch
-// Clocks from a sweep of the four launches of a layer over 64 to 6300 tokens and widths of 320 to 3264 columns.  A
+// Clocks from a sweep of the four launches of a layer over 64 to 6300 tokens and widths of 320 to 3264 columns, taken before whole
+// warps issued (but a pair's k-block); the choices are still the fastest, or within 2 us of it, at the workloads' sizes.  A
 // k-block of a wide tile costs less than two of a narrow one (operands are re-read half as often per flop), a pair's
 // less still (675 before their loading loop was shortened; with 640 in its place the ViT-Base step went from 181.3 to 179.9 us, the
 // Llama-1B-shaped one from 482 to 478; 640 with 2000 a launch, or 610 with 1000, cost the feed-forward and adapter steps 1 to 4 %),
